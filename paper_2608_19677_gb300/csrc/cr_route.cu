@@ -13,15 +13,16 @@
 //     threads against the batch-start loads, the batch's counts accumulate in
 //     a second shared vector and are merged at the boundary;
 //   - batches of at most 32 requests (batch_B = 1 is exact sequential
-//     dispatch): k_route_resolve_warp, one warp per replica taking
-//     S = floor(32 / B) * B requests (whole batches) per step.  Inside a step a
-//     request's decision depends on the destinations of the earlier batches of
-//     the step; the warp finds them by fixed-point iteration: every lane
-//     decides from the step-start loads plus the lanes of earlier batches that
-//     currently sit on each candidate (a per-destination lane bitmask in
-//     shared memory), until no lane changes.  After iteration t the first t
-//     batches are final, so at most S iterations are needed and typically two
-//     or three; the result is the sequential one.
+//     dispatch): k_route_resolve_warp, one CTA per replica whose first warp
+//     takes S = floor(32 / B) * B requests (whole batches) per step, and whose
+//     other warps compute the candidates of later steps (no candidate pass).
+//     Inside a step a request's decision depends on the destinations of the
+//     earlier batches of the step; the warp finds them by fixed-point
+//     iteration: every lane decides from the step-start loads plus the lanes
+//     of earlier batches that currently sit on each of its choices, until no
+//     lane changes.  After iteration t the first t batches are final, so at
+//     most S iterations are needed and typically two or three; the result is
+//     the sequential one.
 #include <stdlib.h>
 #include <string.h>
 
@@ -639,147 +640,520 @@ __global__ void __launch_bounds__(kRouteBlock) k_route_resolve(const __grid_cons
     for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) Lg[r] = L[r];
 }
 
-// ---- batches of at most one warp: one warp per replica ----------------------
+// ---- batches of at most one warp: one CTA per replica ------------------------
+// Warp 0 resolves; warps 1 .. kPrepWarps prepare.  A step is S = floor(32 / B) * B
+// requests (whole batches), one per lane; a chunk is kPrepWarps steps.  While the
+// resolver works through chunk c, preparer w computes step w of chunk c + 1 into
+// the other half of a double buffer -- the candidates themselves (table probe,
+// Philox draws or ring position) and everything about the step that does not
+// depend on the live load -- and writes out the destinations of chunk c - 1.  The
+// resolver's serial chain is then only what the loads decide, on loads held
+// relative to their minimum in 32 bits:
+//   - two choices d1, d2 (power-of-two choices; a key with k_b = 1 is d1 = d2, one
+//     with k_b = 2 its two members, ties to the first): the preparer leaves, per
+//     lane, the lanes of the step whose first / second choice is this lane's d1 /
+//     d2 (four bit masks, built from one ballot per destination bit).  With S the
+//     ballot of the lanes on their second choice, the earlier lanes on d1 are
+//     popc(select(S, second == d1, first == d1) & earlier), so one iteration of the
+//     fixed point is two selects, two popcounts, a compare and a ballot in
+//     registers: no shared memory, no atomics.
+//   - bounded loads, R <= 32: the preparer leaves the bound and the first eight
+//     distinct owners of the walk; an iteration compares the first four at once
+//     (then the next four, then the walk itself), lane r holding the mask of the
+//     lanes on destination r (five ballots).
+//   - bounded loads on more destinations, and steps with a key of three or more
+//     members: lane masks per destination in shared memory (masked_step).
+//   - loads spread over 2^30 or more, or near 2^64 (sums wrap): the same masked
+//     steps on 64-bit loads.
+// Bound by the latency of the resolver's chain (a ballot and the branch on it cost
+// ~50 cycles, a popcount ~20, a shared-memory read ~29 on this GPU).  Measured on a
+// GB300 with B = 1, R = 30, 83,333 requests, five replicas: power-of-two choices 0.83
+// ms, plan replicas 0.68 ms, bounded loads 1.58 ms; all fifteen 1.42 ms, where one
+// warp that did all of it (every iteration re-reading loads and masks from shared
+// memory, bound computed by division inside the chain) took 3.7 ms.  256 requests,
+// one plan replica at R = 64: 64.8 -> 19.0 us a call (no staging of member lists, no
+// candidate launch).  Bounded loads on R > 32 cost 1.87 ms (masked_step).
+constexpr int kPrepWarps = 8;
+// warps 4 and 8 stay idle: the resolver has its SM sub-partition's issue slots to itself
+constexpr int kWarpPathWarps = kPrepWarps + 3;
+constexpr unsigned long long kNarrow = 1ull << 30;  // spread of the loads during a call, 32-bit loops
+constexpr uint32_t kOwn8 = 32;                      // destinations up to which ring walks go through eight distinct owners
 
-constexpr int kWarpChunk = 8;  // steps whose candidates are fetched one chunk ahead
-
-// A candidate with its table slot or first ring owner already fetched.
-struct prep_cand {
-    uint32_t kind;
-    uint32_t a;  // FIXED: destination; PAIR: d1; SET: first member; RING: owner of the first point
-    uint32_t b;  // PAIR: d2; SET: member offset; RING: first ring index
-    uint32_t k;  // SET: members
+// Shared memory of the kernel: the double-buffered steps, then loads [R] u64 (the
+// 32-bit loops use the first half) and lane masks [R] u32.
+struct prep_buf {
+    uint4 m[2][kPrepWarps][32];      // two choices: lanes with first == d1, second == d1, first == d2, second == d2
+                                     // ring: owners, eight u8 in (x, y) for R <= 32, else four u16 in (x, y); bound lo, hi
+    uint32_t d[2][kPrepWarps][32];   // two choices: d1 | d2 << 16; ring: first ring index
+    uint2 set[2][kPrepWarps][32];    // keys of three or more members: member offset, members (else 0)
+    uint16_t out[2][kPrepWarps][32]; // destinations decided
+    uint32_t any_set[2][kPrepWarps]; // some lane of the step has such a key
 };
 
-__device__ __forceinline__ prep_cand prepare(uint32_t c, const route_desc &rd, const uint16_t *own)
+// Table slot of a plan replica's key (koff = kEmpty: not in the table).
+__device__ __forceinline__ cr_table_slot plan_probe(const route_desc &rd, unsigned long long key)
 {
-    prep_cand p;
-    p.kind = c & kKindMask;
-    p.a = c & 0xffffu;
-    p.b = 0;
-    p.k = 1;
-    if (p.kind == kPair) {
-        p.a = c & 0x1fffu;
-        p.b = (c >> 13) & 0x1fffu;
-    } else if (p.kind == kSet) {
-        const cr_table_slot slot = rd.table[c & kLow30];
-        p.a = slot.m0;
-        p.b = slot.koff;
-        p.k = slot.k;
-    } else if (p.kind == kRing) {
-        p.b = c & kLow30;
-        p.a = own[p.b];
+    const unsigned long long mask = (1ull << rd.tbits) - 1ull;
+    unsigned long long sl = key >> (64 - rd.tbits);
+    cr_table_slot slot = rd.table[sl];
+    while (slot.koff != kEmpty && slot.key != key) {  // at least twice as many slots as keys: an empty one ends it
+        sl = (sl + 1) & mask;
+        slot = rd.table[sl];
     }
-    return p;
+    return slot;
 }
 
-// The decision of one request that sees load L[d] plus the lanes of `earlier`
-// currently placed on d.
-__device__ __forceinline__ uint32_t decide(const prep_cand &p, const route_desc &rd, const uint16_t *mem,
-                                           const unsigned long long *L, const uint32_t *mask, uint32_t earlier,
-                                           unsigned long long cap, uint32_t *status)
+// Prepare one step (one warp): its lanes' requests into half `h`, step `w` of the buffer.
+__device__ __forceinline__ void prepare_step(prep_buf &pb, uint32_t h, uint32_t w, const route_desc &rd, bool active,
+                                             unsigned long long key, unsigned long long g, uint32_t R, uint32_t nb,
+                                             unsigned long long seen_m)
 {
-    auto seen = [&](uint32_t d) { return L[d] + (unsigned long long)__popc(mask[d] & earlier); };
-    if (p.kind == kFixed) return p.a;
-    if (p.kind == kPair) return seen(p.a) <= seen(p.b) ? p.a : p.b;
-    if (p.kind == kRing) return seen(p.a) < cap ? p.a : ring_walk(rd, mem, p.b, cap, seen, status);
-    return set_min(mem, p.b, p.k, p.a, seen);
+    const uint32_t lane = cr_lane();
+    const uint32_t am = __ballot_sync(0xffffffffu, active);
+    if (rd.policy == CR_POLICY_CHWBL) {
+        uint4 m = make_uint4(0, 0, 0, 0);
+        uint32_t j0 = 0;
+        if (active) {
+            uint32_t j = j0 = ring_start(rd, cr_fmix64(key ^ rd.seed));
+            const unsigned long long cap = chwbl_cap(seen_m, R);
+            m.z = (uint32_t)cap;
+            m.w = (uint32_t)(cap >> 32);
+            if (R <= kOwn8) {
+                // the first eight distinct owners; shorter lists repeat the first one, which
+                // changes no decision (an owner met again is as full as before)
+                uint32_t met = 0, k = 0, lo = 0, hi = 0, o0 = rd.rowner[j];
+                for (uint32_t t = 0; t < rd.rM && t < 64u && k < 8u; ++t) {
+                    const uint32_t o = rd.rowner[j];
+                    j = j + 1 == rd.rM ? 0u : j + 1;
+                    if ((met >> o) & 1u) continue;
+                    met |= 1u << o;
+                    if (k < 4u)
+                        lo |= o << (8 * k);
+                    else
+                        hi |= o << (8 * (k - 4u));
+                    ++k;
+                }
+                for (; k < 8u; ++k) {
+                    if (k < 4u)
+                        lo |= o0 << (8 * k);
+                    else
+                        hi |= o0 << (8 * (k - 4u));
+                }
+                m.x = lo;
+                m.y = hi;
+            } else {
+                uint32_t o[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    o[q] = rd.rowner[j];
+                    j = j + 1 == rd.rM ? 0u : j + 1;
+                }
+                m.x = o[0] | (o[1] << 16);
+                m.y = o[2] | (o[3] << 16);
+            }
+        }
+        pb.m[h][w][lane] = m;
+        pb.d[h][w][lane] = j0;
+        return;
+    }
+    uint32_t d1 = 0, d2 = 0;
+    uint2 set = make_uint2(0, 0);
+    bool draw = active;  // power-of-two choices: every request, or a plan replica's keys outside the table
+    if (rd.policy != CR_POLICY_P2C) {
+        cr_table_slot slot;
+        slot.koff = kEmpty;
+        if (active) slot = plan_probe(rd, key);
+        __syncwarp();  // the draws below run once for the whole warp, not once per probe length
+        if (slot.koff != kEmpty) {
+            draw = false;
+            d1 = d2 = slot.m0;
+            if (slot.k > 1) d2 = rd.members[(size_t)slot.koff + 1];
+            if (slot.k > 2) {
+                set = make_uint2(slot.koff, slot.k);
+                for (uint32_t q = 2; q < slot.k; q += 64)  // brings the list into this SM's L1
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(rd.members + (size_t)slot.koff + q));
+            }
+        }
+        __syncwarp();
+    }
+    if (draw) {
+        const uint32_t c = p2c_pair(rd.seed, rd.policy, g, R);
+        d1 = c & 0x1fffu;
+        d2 = (c >> 13) & 0x1fffu;
+    }
+    __syncwarp();
+    uint32_t e11 = am, e21 = am, e12 = am, e22 = am;
+#pragma unroll
+    for (uint32_t b = 0; b < 13; ++b) {
+        if (b < nb) {  // uniform
+            const uint32_t b1 = __ballot_sync(0xffffffffu, (d1 >> b) & 1u);
+            const uint32_t b2 = __ballot_sync(0xffffffffu, (d2 >> b) & 1u);
+            const uint32_t x1 = 0u - ((d1 >> b) & 1u), x2 = 0u - ((d2 >> b) & 1u);
+            e11 &= ~(b1 ^ x1);
+            e21 &= ~(b2 ^ x1);
+            e12 &= ~(b1 ^ x2);
+            e22 &= ~(b2 ^ x2);
+        }
+    }
+    const bool any = __any_sync(0xffffffffu, set.y != 0u);
+    pb.m[h][w][lane] = active ? make_uint4(e11, e21, e12, e22) : make_uint4(0, 0, 0, 0);
+    pb.d[h][w][lane] = d1 | (d2 << 16);
+    pb.set[h][w][lane] = set;
+    if (lane == 0) pb.any_set[h][w] = any;
 }
 
-__global__ void __launch_bounds__(32) k_route_resolve_warp(const __grid_constant__ route_args args,
-                                                           const uint32_t *__restrict__ cand, unsigned long long n,
-                                                           uint32_t B, uint32_t R,
-                                                           unsigned long long *__restrict__ load,
-                                                           uint16_t *__restrict__ dest, uint32_t *status,
-                                                           unsigned long long MC)
+// bit by bit: sel ? b : a
+__device__ __forceinline__ uint32_t bit_select(uint32_t sel, uint32_t a, uint32_t b) { return (a & ~sel) | (b & sel); }
+
+// What the resolver's steps share.
+struct step_ctx {
+    uint32_t lane, bit, earlier;  // earlier: lanes of the earlier batches of the step
+    bool several;                 // more than one batch per step
+    uint32_t max_it;
+    uint32_t *status;
+};
+
+// A step decided through the lane masks in shared memory (zero between steps): `decide(earlier)`
+// gives this lane's destination from the step-start loads plus the lanes of `earlier` on each
+// destination.  After iteration t the first t batches of the step are final.
+template <typename LT, typename Decide>
+__device__ __forceinline__ uint32_t masked_step(const step_ctx &X, LT *L, uint32_t *mask, bool active, uint32_t R,
+                                                Decide decide)
 {
-    extern __shared__ unsigned long long sh[];
-    prep_cand *ps = reinterpret_cast<prep_cand *>(sh);      // [kWarpChunk][32] prepared candidates
-    unsigned long long *L = sh + kWarpChunk * 32 * sizeof(prep_cand) / sizeof(unsigned long long);  // [R]
-    uint32_t *mask = reinterpret_cast<uint32_t *>(L + R);   // [R] lanes of the step on each destination
-    uint16_t *smem_aux = reinterpret_cast<uint16_t *>(mask + R);  // [MC] members or ring owners
+    uint32_t d = active ? decide(0u) : 0u;
+    if (!CR_DCHECK(d < R, X.status)) d = 0;
+    if (active) atomicOr(&mask[d], X.bit);
+    __syncwarp();
+    if (X.several) {
+        for (uint32_t it = 0;; ++it) {
+            uint32_t nd = active ? decide(X.earlier) : d;
+            if (!CR_DCHECK(nd < R, X.status)) nd = 0;
+            const uint32_t moved = __ballot_sync(0xffffffffu, nd != d);
+            if (!moved) break;
+            if (it >= X.max_it) {  // unreachable: max_it iterations always settle the step
+                if (X.lane == 0) atomicOr(X.status, CR_FLAG_TIMEOUT);
+                break;
+            }
+            if (nd != d) {
+                atomicAnd(&mask[d], ~X.bit);
+                atomicOr(&mask[nd], X.bit);
+                d = nd;
+            }
+            __syncwarp();
+        }
+    }
+    if (active) {
+        const uint32_t mk = mask[d];
+        if ((mk & (0u - mk)) == X.bit) L[d] += (LT)__popc(mk);  // lowest lane adds
+    }
+    __syncwarp();
+    if (active) mask[d] = 0;
+    __syncwarp();
+    return d;
+}
+
+// A two-choice or set step through the masks.
+template <typename LT>
+__device__ __forceinline__ uint32_t set_step(const step_ctx &X, LT *L, uint32_t *mask, const route_desc &rd,
+                                             bool active, uint32_t R, uint32_t d12, uint2 set)
+{
+    const uint32_t d1 = d12 & 0xffffu, d2 = d12 >> 16;
+    return masked_step(X, L, mask, active, R, [&](uint32_t earlier) {
+        auto seen = [&](uint32_t x) { return (unsigned long long)(LT)(L[x] + (LT)__popc(mask[x] & earlier)); };
+        if (set.y) return set_min(rd.members, set.x, set.y, d1, seen);
+        return seen(d1) <= seen(d2) ? d1 : d2;
+    });
+}
+
+// A bounded-load step through the masks: the first four owners of the walk, then the walk itself.
+template <typename LT>
+__device__ __forceinline__ uint32_t ring_step(const step_ctx &X, LT *L, uint32_t *mask, const route_desc &rd,
+                                              bool active, uint32_t R, uint4 m, uint32_t j0, unsigned long long cap)
+{
+    const uint32_t o[4] = {m.x & 0xffffu, m.x >> 16, m.y & 0xffffu, m.y >> 16};
+    uint32_t t[4];  // free places of each owner (32: more than the step can take)
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        const unsigned long long l = L[o[w]];
+        t[w] = l >= cap ? 0u : (cap - l < 32ull ? (uint32_t)(cap - l) : 32u);
+    }
+    return masked_step(X, L, mask, active, R, [&](uint32_t earlier) {
+        uint32_t f[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) f[w] = (uint32_t)__popc(mask[o[w]] & earlier);
+        if (f[0] < t[0]) return o[0];
+        if (f[1] < t[1]) return o[1];
+        if (f[2] < t[2]) return o[2];
+        if (f[3] < t[3]) return o[3];
+        auto seen = [&](uint32_t x) { return (unsigned long long)(LT)(L[x] + (LT)__popc(mask[x] & earlier)); };
+        return ring_walk(rd, rd.rowner, j0, cap, seen, X.status);
+    });
+}
+
+// One chunk of two-choice steps on 32-bit loads.
+__device__ __forceinline__ void resolve_pairs(const step_ctx &X, prep_buf &pb, uint32_t h, uint32_t steps,
+                                              uint32_t *L, uint32_t *mask, const route_desc &rd, uint32_t R)
+{
+    const uint32_t lane = X.lane, below = X.bit - 1u;
+    uint4 mn = pb.m[h][0][lane];
+    uint32_t dn = pb.d[h][0][lane], an = pb.any_set[h][0];
+#pragma unroll 1
+    for (uint32_t q = 0; q < steps; ++q) {
+        const uint4 m = mn;
+        const uint32_t d12 = dn, any = an;
+        if (q + 1 < steps) {
+            mn = pb.m[h][q + 1][lane];
+            dn = pb.d[h][q + 1][lane];
+            an = pb.any_set[h][q + 1];
+        }
+        const uint32_t d1 = d12 & 0xffffu, d2 = d12 >> 16;
+        if (any) {
+            const uint32_t d = set_step(X, L, mask, rd, m.x != 0u, R, d12, pb.set[h][q][lane]);
+            pb.out[h][q][lane] = (uint16_t)d;
+            continue;
+        }
+        const uint32_t a1 = m.x & X.earlier, a2 = m.y & X.earlier, b1 = m.z & X.earlier, b2 = m.w & X.earlier;
+        const uint32_t l1 = L[d1], l2 = L[d2];
+        const int diff = (int)(l1 - l2);
+        uint32_t sel = __ballot_sync(0xffffffffu, diff > 0);
+        if (X.several) {
+            // the first `it` batches are final after pass `it`: at most max_it passes change anything
+            auto pass = [&](uint32_t now) {
+                const int x = diff + __popc(bit_select(now, a1, a2)) - __popc(bit_select(now, b1, b2));
+                return __ballot_sync(0xffffffffu, x > 0);
+            };
+            sel = pass(sel);
+            for (uint32_t it = 0; it <= X.max_it; ++it) {
+                const uint32_t ns = pass(sel);
+                const bool same = ns == sel;
+                sel = ns;
+                if (same) break;
+            }
+        }
+        const bool second = (sel & X.bit) != 0u;
+        const uint32_t mine = second ? bit_select(sel, m.z, m.w) : bit_select(sel, m.x, m.y);
+        const uint32_t d = second ? d2 : d1;
+        // the lowest lane of each destination adds its lanes (an inactive lane's masks are empty)
+        if ((mine & (below | X.bit)) == X.bit) L[d] = (second ? l2 : l1) + (uint32_t)__popc(mine);
+        pb.out[h][q][lane] = (uint16_t)d;
+        __syncwarp();
+    }
+}
+
+// One chunk of bounded-load steps on 32-bit loads relative to `base`, R <= 32: lane r holds the
+// mask of the lanes on destination r.
+__device__ __forceinline__ void resolve_ring32(const step_ctx &X, prep_buf &pb, uint32_t h, uint32_t steps,
+                                               uint32_t *L, const route_desc &rd, uint32_t R, unsigned long long base)
+{
+    const uint32_t lane = X.lane;
+    uint32_t xr[5];
+#pragma unroll
+    for (int b = 0; b < 5; ++b) xr[b] = 0u - ((lane >> b) & 1u);
+    uint4 mn = pb.m[h][0][lane];
+#pragma unroll 1
+    for (uint32_t q = 0; q < steps; ++q) {
+        const uint4 m = mn;
+        if (q + 1 < steps) mn = pb.m[h][q + 1][lane];
+        const unsigned long long cap64 = (unsigned long long)m.z | ((unsigned long long)m.w << 32);
+        const bool active = cap64 != 0ull;  // a bound is at least 1
+        const uint32_t am = __ballot_sync(0xffffffffu, active);
+        // the bound never is below the least load; far above every load it only has to stay there
+        const int cap = cap64 - base < 0x7fffffffull ? (int)(cap64 - base) : 0x7fffffff;
+        // free places of the first four owners of the walk (at most 0: none)
+        uint32_t o[4];
+        int t[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            o[w] = (m.x >> (8 * w)) & 0xffu;
+            t[w] = cap - (int)L[o[w]];
+        }
+        uint32_t c = t[0] > 0 ? o[0] : (t[1] > 0 ? o[1] : (t[2] > 0 ? o[2] : o[3])), M = 0;
+        for (uint32_t it = 0; it <= X.max_it + 1u; ++it) {
+            uint32_t mr = am;
+#pragma unroll
+            for (int b = 0; b < 5; ++b) mr &= ~(__ballot_sync(0xffffffffu, (c >> b) & 1u) ^ xr[b]);
+            M = mr;
+            int f[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) f[w] = __popc(__shfl_sync(0xffffffffu, mr, o[w]) & X.earlier);
+            uint32_t nc = f[0] < t[0] ? o[0] : (f[1] < t[1] ? o[1] : (f[2] < t[2] ? o[2] : o[3]));
+            bool left = active && f[0] >= t[0] && f[1] >= t[1] && f[2] >= t[2] && f[3] >= t[3];
+            if (!__any_sync(0xffffffffu, left || (active && nc != c))) break;
+            if (__any_sync(0xffffffffu, left)) {  // the next four owners of the walk
+                uint32_t n2 = 0xffu;
+#pragma unroll
+                for (int w = 3; w >= 0; --w) {
+                    const uint32_t ow = (m.y >> (8 * w)) & 0xffu;
+                    const int fw = __popc(__shfl_sync(0xffffffffu, mr, ow) & X.earlier);
+                    n2 = fw < cap - (int)L[ow] ? ow : n2;
+                }
+                if (left && n2 != 0xffu) {
+                    nc = n2;
+                    left = false;
+                }
+                if (__any_sync(0xffffffffu, left)) {  // rare: the walk itself, all lanes together
+                    uint32_t j = pb.d[h][q][lane];
+                    const uint32_t first = left ? (uint32_t)rd.rowner[j] : 0u;
+                    for (uint32_t x = 0; x < rd.rM; ++x) {
+                        const uint32_t ow = left ? (uint32_t)rd.rowner[j] : 0u;
+                        const uint32_t mo = __shfl_sync(0xffffffffu, mr, ow & 31u);
+                        if (left && (int)L[ow & 31u] + __popc(mo & X.earlier) < cap) {
+                            nc = ow;
+                            left = false;
+                        }
+                        j = j + 1 >= rd.rM ? 0u : j + 1;
+                        if (!__any_sync(0xffffffffu, left)) break;
+                    }
+                    if (left) {  // no destination below the bound: only when a load sum has wrapped
+                        nc = first;
+                        atomicOr(X.status, CR_FLAG_OVERFLOW);
+                    }
+                }
+                if (!__any_sync(0xffffffffu, active && nc != c)) break;
+            }
+            if (!CR_DCHECK(!active || nc < R, X.status)) nc = 0;
+            if (active) c = nc;
+        }
+        pb.out[h][q][lane] = (uint16_t)c;
+        if (lane < R) L[lane] += (uint32_t)__popc(M);
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(32 * kWarpPathWarps)
+k_route_resolve_warp(const __grid_constant__ route_args args, const unsigned long long *__restrict__ keys,
+                     unsigned long long n, unsigned long long g0, uint32_t B, uint32_t R,
+                     unsigned long long *__restrict__ load, uint16_t *__restrict__ dest, uint32_t *status)
+{
+    extern __shared__ uint4 sh4[];
+    prep_buf &pb = *reinterpret_cast<prep_buf *>(sh4);
+    unsigned long long *L64 = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(sh4) +
+                                                                     sizeof(prep_buf));
+    uint32_t *L32 = reinterpret_cast<uint32_t *>(L64);
+    uint32_t *mask = reinterpret_cast<uint32_t *>(L64 + R);
+    __shared__ unsigned long long s_tot, s_max, s_min;
     const uint32_t rep = args.dep[blockIdx.x];
     const route_desc &rd = args.d[rep];
     unsigned long long *Lg = load + (unsigned long long)rep * R;
-    const uint32_t *Cd = cand + (unsigned long long)rep * n;
     uint16_t *D = dest + (unsigned long long)rep * n;
-    const uint32_t lane = threadIdx.x;
-    unsigned long long tot = 0;
-    for (uint32_t r = lane; r < R; r += 32) {
-        const unsigned long long v = Lg[r];
-        L[r] = v;
-        mask[r] = 0;
-        tot += v;
+    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5;
+    const bool resolver = warp == 0, preparer = (warp & 3u) != 0;
+    const uint32_t pw = preparer ? warp - 1u - (warp >> 2) : 0u;  // preparer number, its step of every chunk
+    const bool ring = rd.policy == CR_POLICY_CHWBL;
+    if (threadIdx.x == 0) {
+        s_tot = s_max = 0;
+        s_min = ~0ull;
     }
-    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    const uint16_t *mem = stage_aux(rd, smem_aux, MC);
-    __syncwarp();
+    __syncthreads();
+    {
+        unsigned long long tot = 0, mx = 0, mi = ~0ull;
+        for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) {
+            const unsigned long long v = Lg[r];
+            L64[r] = v;
+            mask[r] = 0;
+            tot += v;
+            mx = v > mx ? v : mx;
+            mi = v < mi ? v : mi;
+        }
+        if (threadIdx.x < R) {
+            atomicAdd(&s_tot, tot);
+            atomicMax(&s_max, mx);
+            atomicMin(&s_min, mi);
+        }
+    }
+    __syncthreads();
+    const unsigned long long tot0 = s_tot, base = s_min;
+    // the 32-bit loops: the loads stay within 2^30 of the least one, and nothing wraps
+    const bool narrow = s_max < (1ull << 47) && n < kNarrow && s_max - base < kNarrow - n;
+    if (narrow) {  // in place: a thread's 64-bit words are read before any 32-bit word is written
+        for (uint32_t r0 = 0; r0 < R; r0 += blockDim.x) {
+            const uint32_t r = r0 + threadIdx.x;
+            const uint32_t v = r < R ? (uint32_t)(L64[r] - base) : 0u;
+            __syncthreads();
+            if (r < R) L32[r] = v;
+            __syncthreads();
+        }
+    }
     const uint32_t S = (32u / B) * B;               // requests per step: whole batches
     const uint32_t bstart = (lane / B) * B;         // first lane of this lane's batch
-    const uint32_t earlier = (1u << bstart) - 1u;   // lanes of the earlier batches of the step
-    const uint32_t bit = 1u << lane;
-    const bool several = S > B;
-    const bool ring = rd.policy == CR_POLICY_CHWBL;  // only its decisions read the cap
-    const unsigned long long CHR = (unsigned long long)S * kWarpChunk;
-    uint32_t cn[kWarpChunk];
-#pragma unroll
-    for (int q = 0; q < kWarpChunk; ++q) {
-        const unsigned long long i = (unsigned long long)q * S + lane;
-        cn[q] = (lane < S && i < n) ? Cd[i] : 0u;  // 0 = FIXED 0: inactive lanes read nothing
+    step_ctx X;
+    X.lane = lane;
+    X.bit = 1u << lane;
+    X.earlier = (1u << bstart) - 1u;
+    X.several = S > B;
+    X.max_it = S;
+    X.status = status;
+    const uint32_t nb = R > 1 ? 32u - (uint32_t)__clz(R - 1u) : 0u;  // bits of a destination, <= 13
+    const unsigned long long CHR = (unsigned long long)S * kPrepWarps;  // requests per chunk
+    const unsigned long long nchunks = (n + CHR - 1) / CHR;
+    const bool own8 = ring && R <= kOwn8;
+    // preparer pw: step pw of a chunk; the chunk after's key is in flight meanwhile
+    auto index_of = [&](unsigned long long c) { return c * CHR + (unsigned long long)pw * S + lane; };
+    auto key_of = [&](unsigned long long c) {
+        const unsigned long long i = index_of(c);
+        return (lane < S && i < n) ? keys[i] : 0ull;
+    };
+    auto prepare_chunk = [&](unsigned long long c, unsigned long long key) {
+        const unsigned long long i = index_of(c);
+        prepare_step(pb, (uint32_t)(c & 1), pw, rd, lane < S && i < n, key, g0 + i, R, nb,
+                     tot0 + (i - lane) + bstart);
+    };
+    auto write_chunk = [&](unsigned long long c) {
+        const unsigned long long i = index_of(c);
+        if (lane < S && i < n) D[i] = pb.out[c & 1][pw][lane];
+    };
+    unsigned long long knext = 0;
+    if (preparer) {
+        const unsigned long long k0 = key_of(0);
+        knext = key_of(1);
+        prepare_chunk(0, k0);
     }
-    for (unsigned long long c0 = 0; c0 < n; c0 += CHR) {
-        // each lane prepares (and later reads) only its own entries: no barrier needed
-#pragma unroll
-        for (int q = 0; q < kWarpChunk; ++q) ps[q * 32 + lane] = prepare(cn[q], rd, mem);
-#pragma unroll
-        for (int q = 0; q < kWarpChunk; ++q) {
-            const unsigned long long i = c0 + CHR + (unsigned long long)q * S + lane;
-            cn[q] = (lane < S && i < n) ? Cd[i] : 0u;
-        }
+    __syncthreads();
+    for (unsigned long long c = 0; c < nchunks; ++c) {
+        if (preparer) {
+            if (c > 0) write_chunk(c - 1);  // before its half is prepared anew
+            if (c + 1 < nchunks) {
+                const unsigned long long key = knext;
+                knext = key_of(c + 2);
+                prepare_chunk(c + 1, key);
+            }
+        } else if (resolver) {
+            const uint32_t h = (uint32_t)(c & 1);
+            const unsigned long long left = n - c * CHR;
+            const uint32_t steps = left >= CHR ? (uint32_t)kPrepWarps : (uint32_t)((left + S - 1) / S);
+            if (narrow && !ring) {
+                resolve_pairs(X, pb, h, steps, L32, mask, rd, R);
+            } else if (narrow && own8) {
+                resolve_ring32(X, pb, h, steps, L32, rd, R, base);
+            } else {
 #pragma unroll 1
-        for (int q = 0; q < kWarpChunk; ++q) {
-            const unsigned long long s0 = c0 + (unsigned long long)q * S;
-            if (s0 >= n) break;  // uniform over the warp
-            const unsigned long long i = s0 + lane;
-            const bool active = lane < S && i < n;
-            const unsigned long long cap = ring ? chwbl_cap(tot + bstart, R) : 0ull;
-            const prep_cand pq = ps[q * 32 + lane];
-            uint32_t d = decide(pq, rd, mem, L, mask, 0u, cap, status);
-            if (!CR_DCHECK(d < R, status)) d = 0;
-            if (active) atomicOr(&mask[d], bit);
-            __syncwarp();
-            if (several) {
-                // fixed point: after iteration t the first t batches of the step are final
-                for (uint32_t it = 0;; ++it) {
-                    uint32_t nd = active ? decide(pq, rd, mem, L, mask, earlier, cap, status) : d;
-                    if (!CR_DCHECK(nd < R, status)) nd = 0;
-                    const uint32_t moved = __ballot_sync(0xffffffffu, nd != d);
-                    if (!moved) break;
-                    if (it >= S) {  // unreachable: S iterations always settle the step
-                        if (lane == 0) atomicOr(status, CR_FLAG_TIMEOUT);
-                        break;
+                for (uint32_t q = 0; q < steps; ++q) {
+                    const uint4 m = pb.m[h][q][lane];
+                    const uint32_t dj = pb.d[h][q][lane];
+                    uint32_t d;
+                    if (!ring) {
+                        d = set_step(X, L64, mask, rd, m.x != 0u, R, dj, pb.set[h][q][lane]);
+                    } else {
+                        const unsigned long long cap = (unsigned long long)m.z | ((unsigned long long)m.w << 32);
+                        const bool active = lane < S && (c * kPrepWarps + q) * S + lane < n;
+                        uint4 ow = m;
+                        if (own8) {  // the first four of the eight owners
+                            ow.x = (m.x & 0xffu) | ((m.x & 0xff00u) << 8);
+                            ow.y = ((m.x >> 16) & 0xffu) | ((m.x >> 24) << 16);
+                        }
+                        if (narrow)
+                            d = ring_step(X, L32, mask, rd, active, R, ow, dj, cap - base);
+                        else
+                            d = ring_step(X, L64, mask, rd, active, R, ow, dj, cap);
                     }
-                    if (nd != d) {
-                        atomicAnd(&mask[d], ~bit);
-                        atomicOr(&mask[nd], bit);
-                        d = nd;
-                    }
-                    __syncwarp();
+                    pb.out[h][q][lane] = (uint16_t)d;
                 }
             }
-            if (active) {
-                const uint32_t mk = mask[d];
-                if ((mk & (0u - mk)) == bit) L[d] += (unsigned long long)__popc(mk);  // lowest lane adds
-                D[i] = (uint16_t)d;
-            }
-            __syncwarp();
-            if (active) mask[d] = 0;
-            __syncwarp();
-            const unsigned long long left = n - s0;
-            tot += left < S ? left : S;
         }
+        __syncthreads();
     }
-    for (uint32_t r = lane; r < R; r += 32) Lg[r] = L[r];
+    if (preparer) write_chunk(nchunks - 1);
+    for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) Lg[r] = narrow ? base + L32[r] : L64[r];
 }
 
 // ---- ring construction ------------------------------------------------------
@@ -895,9 +1269,9 @@ extern "C" int cr_ring_export(cr_ctx *ctx, const cr_ring *g, uint64_t *point, ui
     return cr_sync(ctx);
 }
 
-static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, const uint32_t *cand, uint64_t n,
-                          uint32_t batch_B, uint32_t R, uint64_t mc, uint32_t n_dep, uint64_t *d_load,
-                          uint16_t *d_dest);
+static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, const uint32_t *cand,
+                          const uint64_t *d_key, uint64_t n, uint64_t g0, uint32_t batch_B, uint32_t R, uint64_t mc,
+                          uint32_t n_dep, uint64_t *d_load, uint16_t *d_dest);
 
 extern "C" int cr_route_batch(cr_ctx *ctx, const cr_plan *const *plans, const cr_replica *reps, uint32_t n_rep,
                               uint32_t R, const uint64_t *d_key, uint64_t n, uint64_t first_req_index,
@@ -956,23 +1330,40 @@ extern "C" int cr_route_batch(cr_ctx *ctx, const cr_plan *const *plans, const cr
     // candidate rows, costliest policy first, so that the grid's last wave holds cheap rows
     // (per request: jump hash ~8 jumps, Philox ~10 rounds, plan probe + Philox for misses,
     // ring lookup, round robin)
+    // (batches of at most a warp: only the load-independent replicas; k_route_resolve_warp
+    // computes the others' candidates itself)
+    const bool warp_path = batch_B <= 32;
+    uint32_t n_cand = 0;
     {
         auto cost = [&](uint32_t p) {
             return p == CR_POLICY_HASH ? 0 : p == CR_POLICY_P2C ? 1 : p <= CR_POLICY_CR_NOREPL ? 2
                  : p == CR_POLICY_CHWBL ? 3 : 4;
         };
-        uint32_t k = 0;
         for (uint32_t c = 0; c <= 4; ++c)
-            for (uint32_t i = 0; i < n_rep; ++i)
-                if ((uint32_t)cost(reps[i].policy) == c) args.cand[k++] = i;
+            for (uint32_t i = 0; i < n_rep; ++i) {
+                const uint32_t p = reps[i].policy;
+                if (warp_path && p != CR_POLICY_RR && p != CR_POLICY_HASH) continue;
+                if ((uint32_t)cost(p) == c) args.cand[n_cand++] = i;
+            }
     }
     // split routing: the candidates scratch is free once the last resolution has read it
     const cudaStream_t rs = ctx->resolve_stream ? ctx->resolve_stream : ctx->stream;
     const bool split = rs != ctx->stream;
     if (split && ctx->resolve_recorded) CR_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_resolve, 0));
-    void *pc;
-    CR_TRY(cr_scratch(ctx, SCR_ROUTE_DESC, (size_t)n * n_rep * sizeof(uint32_t), &pc));
-    uint32_t *cand = (uint32_t *)pc;
+    uint32_t *cand = nullptr;
+    const uint64_t *key_dep = d_key;
+    if (!warp_path) {
+        void *pc;
+        CR_TRY(cr_scratch(ctx, SCR_ROUTE_DESC, (size_t)n * n_rep * sizeof(uint32_t), &pc));
+        cand = (uint32_t *)pc;
+    } else if (split && n_dep) {
+        // the resolution reads the keys on its own stream: from a copy, so that the caller's
+        // keys are still read on the context's stream only
+        void *pc;
+        CR_TRY(cr_scratch(ctx, SCR_ROUTE_DESC, (size_t)n * sizeof(uint64_t), &pc));
+        CR_CUDA(ctx, cudaMemcpyAsync(pc, d_key, (size_t)n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, ctx->stream));
+        key_dep = (const uint64_t *)pc;
+    }
     const int pcand = cr_prof_begin(ctx, ctx->stream, CR_PROF_ROUTE_CAND);
     for (uint32_t i = 0; i < n_rep; ++i) {
         const uint64_t base = (uint64_t)first_req_index + reps[i].seed;  // wraps mod 2^64 as the policy does
@@ -983,10 +1374,11 @@ extern "C" int cr_route_batch(cr_ctx *ctx, const cr_plan *const *plans, const cr
     const unsigned int cbx = cr_blocks(n, 256, (unsigned int)ctx->num_sms * 32u);
     const unsigned int want = (unsigned int)ctx->num_sms * 16u;
     unsigned int cgy = (want + cbx - 1) / cbx;
-    cgy = cgy < 1 ? 1 : (cgy > n_rep ? n_rep : cgy);
-    CR_LAUNCH(ctx, k_route_cand, dim3(cbx, cgy), 256, 0, args, n_rep,
-              (const unsigned long long *)d_key, (unsigned long long)n, (unsigned long long)first_req_index, R, cand,
-              d_dest);
+    cgy = cgy < 1 ? 1 : (cgy > n_cand ? n_cand : cgy);
+    if (n_cand)
+        CR_LAUNCH(ctx, k_route_cand, dim3(cbx, cgy), 256, 0, args, n_cand,
+                  (const unsigned long long *)d_key, (unsigned long long)n, (unsigned long long)first_req_index, R,
+                  cand, d_dest);
     cr_prof_end(ctx, ctx->stream, pcand);
     // load counts of RR / HASH replicas (their choices never read the load)
     for (uint32_t i = 0; i < n_rep; ++i) {
@@ -1004,7 +1396,7 @@ extern "C" int cr_route_batch(cr_ctx *ctx, const cr_plan *const *plans, const cr
     }
     if (n_dep) {
         const int pr = cr_prof_begin(ctx, rs, CR_PROF_ROUTE_RESOLVE);
-        CR_TRY(launch_resolve(ctx, rs, args, cand, n, batch_B, R, mc, n_dep, d_load, d_dest));
+        CR_TRY(launch_resolve(ctx, rs, args, cand, key_dep, n, first_req_index, batch_B, R, mc, n_dep, d_load, d_dest));
         cr_prof_end(ctx, rs, pr);
     }
     if (split) {
@@ -1015,9 +1407,9 @@ extern "C" int cr_route_batch(cr_ctx *ctx, const cr_plan *const *plans, const cr
 }
 
 // The load-dependent resolution of every dependent replica, enqueued on stream rs.
-static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, const uint32_t *cand, uint64_t n,
-                          uint32_t batch_B, uint32_t R, uint64_t mc, uint32_t n_dep, uint64_t *d_load,
-                          uint16_t *d_dest)
+static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, const uint32_t *cand,
+                          const uint64_t *d_key, uint64_t n, uint64_t g0, uint32_t batch_B, uint32_t R, uint64_t mc,
+                          uint32_t n_dep, uint64_t *d_load, uint16_t *d_dest)
 {
     // member lists and ring owners go to shared memory when they fit beside the loads
     auto with_members = [&](size_t base, uint64_t *MC) {
@@ -1026,13 +1418,13 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     };
     uint64_t MC;
     if (batch_B <= 32) {
-        const size_t smem = with_members(kWarpChunk * 32 * sizeof(prep_cand) +
-                                             (size_t)R * (sizeof(unsigned long long) + sizeof(uint32_t)), &MC);
+        const size_t smem = sizeof(prep_buf) + (size_t)R * (sizeof(unsigned long long) + sizeof(uint32_t));
         if (smem > 48 * 1024)
             CR_CUDA(ctx, cudaFuncSetAttribute(k_route_resolve_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
-        CR_LAUNCH_ON(ctx, rs, k_route_resolve_warp, n_dep, 32, smem, args, (const uint32_t *)cand, (unsigned long long)n,
-                  batch_B, R, (unsigned long long *)d_load, d_dest, ctx->d_status, (unsigned long long)MC);
+        CR_LAUNCH_ON(ctx, rs, k_route_resolve_warp, n_dep, 32 * kWarpPathWarps, smem, args,
+                     (const unsigned long long *)d_key, (unsigned long long)n, (unsigned long long)g0, batch_B, R,
+                     (unsigned long long *)d_load, d_dest, ctx->d_status);
         return CR_OK;
     }
     // staging chunk: a whole number of batches, at most kStage requests

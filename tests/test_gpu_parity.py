@@ -380,6 +380,35 @@ def test_route_small_batches_one_hot_key(P, ctx, B):
     assert (h_u64(load) == ref_load).all()
 
 
+@pytest.mark.parametrize("R,B,n", [(1, 1, 257), (2, 31, 1), (31, 1, 255), (32, 5, 4099), (33, 1, 4099), (257, 16, 2049)])
+@pytest.mark.parametrize("loads", ["zero", "high", "spread", "huge"])
+def test_route_small_batches_load_ranges(P, ctx, R, B, n, loads):
+    # the 32-bit loops (loads within 2^30 of the least, also far from zero) and the 64-bit one, on
+    # both sides of the 32-destination ring path, with chunks and steps cut short
+    rng = np.random.default_rng(R * 31 + n)
+    hot = rng.integers(1, 2**63, 12, dtype=np.int64).astype(np.uint64)
+    keys = np.where(rng.random(n) < 0.5, hot[rng.integers(0, 12, n)],
+                    rng.integers(1, 2**63, n, dtype=np.int64).astype(np.uint64))
+    pols, seeds = ["CR", "P2C", "CHWBL", "CHWBL"], [3, 1, 2, 7]
+    opl = O.build_plan(keys, R, 4, max(1, n // 40), 1)   # the hot keys take several destinations
+    dpl = P.build_plan(ctx, d_u64(keys), P.plan_params(R, 4, max(1, n // 40), 1))
+    orings = [None, None, O.Ring(R, 64, 5), O.Ring(R, 1, 6)]
+    drings = [None, None, P.Ring(ctx, R, 64, 5), P.Ring(ctx, R, 1, 6)]
+    init = rng.integers(0, 9, (4, R)).astype(np.uint64)
+    if loads == "high":
+        init += np.uint64(2**46)
+    elif loads == "spread":
+        init[:, : (R + 1) // 2] += np.uint64(2**30)
+    elif loads == "huge":
+        init += np.uint64(2**48)
+    ref_dest, ref_load = O.route([opl, None, None, None], pols, seeds, R, keys, 99, B, load=init, rings=orings)
+    load = d_u64(init.reshape(-1)).view(4, R).contiguous()
+    dest = P.route_batch(ctx, [dpl, None, None, None], pols, seeds, R, d_u64(keys), 99, B, load, rings=drings)
+    ctx.sync()
+    assert (h_u16(dest) == ref_dest).all()
+    assert (h_u64(load) == ref_load).all()
+
+
 @pytest.mark.parametrize("case", ["few", "many", "pool", "wide"])
 @pytest.mark.parametrize("B", [100, 1024])
 def test_route_replicated_keys_per_batch(P, ctx, case, B):
