@@ -8,15 +8,18 @@
 //               passes sort every key
 //   per plan    k_b (Eq. 1), inclusive scan of k_b, admission cut, admitted
 //               arrays, cold-tail total and initial loads (small intervals: every
-//               plan in one launch, one CTA each), placement (LPT: one warp per
-//               plan, warp argmin over per-lane minima, runs of equal-count
-//               single-copy keys placed at once; RANDOM: one warp per key,
-//               Fisher-Yates steps in shared memory), then the device hash table
+//               plan in one launch, one CTA each); then every plan's placement in
+//               one launch (LPT: one CTA per plan, warp argmin over per-lane
+//               minima, runs of equal-count single-copy keys placed at once by the
+//               CTA; RANDOM: one thread per single-copy key, one warp per
+//               replicated key) and every plan's device hash table
 //               b -> (offset, k_b, first member) used by dispatch.
 // No host synchronisation: sizes known only on the device (U, S, n_adm) are
 // read by the kernels, and grids are sized from host-side upper bounds.
 #include <stdlib.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "cr_device.cuh"
 #include "cr_internal.cuh"
@@ -932,17 +935,6 @@ __device__ __forceinline__ void lpt32_body(const cr_plan_info_dev *info,
     if (__any_sync(0xffffffffu, overflow) && lane == 0) atomicOr(status, CR_FLAG_OVERFLOW);
 }
 
-__global__ void __launch_bounds__(32) k_plan_lpt32(const cr_plan_info_dev *info,
-                                                   const unsigned long long *__restrict__ adm_cnt,
-                                                   const uint32_t *__restrict__ adm_k,
-                                                   const uint32_t *__restrict__ koff, uint32_t R,
-                                                   unsigned long long *__restrict__ load_g,
-                                                   uint16_t *__restrict__ members,
-                                                   unsigned long long *__restrict__ jobs, uint32_t *status)
-{
-    lpt32_body(info, adm_cnt, adm_k, koff, R, load_g, members, jobs, status);
-}
-
 // Placement jobs of several plans in one launch (the block index picks the plan).
 struct place_job {
     const cr_plan_info_dev *info;
@@ -964,32 +956,55 @@ __global__ void __launch_bounds__(32) k_plan_lpt32_multi(const __grid_constant__
     lpt32_body(J.info, J.adm_cnt, J.adm_k, J.koff, J.R, J.load, J.members, J.jobs, status);
 }
 
-// LPT for 32 < R <= 1024, all LPT plans of one build at once (one warp per
-// plan).  Lane l holds the packed keys of destinations l, l+32, ... in NE
-// registers and their minimum; a job is one warp minimum (two redux.sync),
-// then the owner lane updates the chosen register and recomputes its minimum
-// with a tree over registers.  Destinations chosen earlier for the same key
-// are masked out by a per-lane bit set.
-struct lpt_job {
-    const cr_plan_info_dev *info;
-    const unsigned long long *adm_cnt;
-    const uint32_t *adm_k, *koff;
-    unsigned long long *load;
-    uint16_t *members;
-    unsigned long long *jobs;
-    uint32_t R;
+// ---- placement: LPT for R <= 1024 and random placement, every plan of a build in one launch ----
+// One CTA of 512 threads per LPT plan and as many as the admitted keys take per random
+// plan, told apart by the block index, so that the serial LPT chains and the random
+// placements run side by side.
+//
+// LPT (Algorithm 1's placement loop).  Warp 0 walks the jobs one at a time: lane l holds
+// the packed keys (load << shift | r) of destinations l, l + 32, ... in NE registers and
+// their minimum; a job is one warp minimum, then the owner lane updates the chosen
+// register and takes its minimum again.  The keys are 32-bit (loads relative to the
+// least starting load, r in the low bits) when every load the build can reach fits: one
+// redux and one-instruction minima, where 64-bit keys take two redux and four
+// instructions per minimum; they remain for wider loads.
+// A run of >= 32 keys with k_b = 1 and equal λ = q is placed at once by the whole CTA.
+// Each greedy pick is a current minimum (L_r, r) and raising it by q keeps later picks
+// no smaller, so the m picks are the m smallest pairs (L_r + j q, r), j >= 0.  With L_r =
+// q l_r + f_r (0 <= f_r < q) pair (r, j) sorts by (l_r + j, f_r, r): picks come in rounds
+// t = l_r + j, each visiting {r : l_r <= t} in (f_r, r) order, and between two consecutive
+// distinct levels l the visited set is fixed, so that stretch of rounds cycles through
+// it.  The CTA sorts the destinations by (f_r, r) once per run (stable counting passes over
+// the bits of f) and per stretch compacts the visited set (two barriers) and writes its
+// picks, 512 at a time.
+// Bound by the latency of the serial chain and of the runs' barriers.  Measured on a GB300:
+// R = 1024, 262,144 admitted keys (1,221 jobs one at a time, 45 runs of 117 stretches), an
+// LPT plan, a single-copy plan and eight random ones: 507 us in one launch, of which the
+// random plans alone would take 79; one warp per LPT plan with 64-bit keys and one launch
+// per random plan took 1,908 + 360 us.  R = 16, 919 keys, one LPT and three random plans:
+// 33 us (was 60 + 58).
+constexpr int kPlaceBlock = 512;
+constexpr uint32_t kPlaceMaxR = 1024;
+constexpr uint32_t kRunMin = 32;              // shortest run placed at once
+constexpr uint32_t kRunMaxQ = 1u << 20;       // f << 10 | r in 32 bits
+
+struct lpt_smem {
+    uint32_t rel[kPlaceMaxR];     // run: loads relative to an origin, then levels l_r
+    uint32_t add[kPlaceMaxR];     // run: jobs given to r
+    uint32_t srt[kPlaceMaxR];     // run: f_r << 10 | r, sorted
+    uint32_t cnt[64 * (kPlaceBlock / 32)];  // run: (digit, warp) counts of a sorting pass
+    uint16_t cyc[2][kPlaceMaxR];  // run: destinations visited in a stretch, in order (alternating)
+    uint32_t wcnt[2][kPlaceBlock / 32], wnxt[2][kPlaceBlock / 32];
+    uint32_t a, q, base;          // run: first key, λ, first member offset
+    uint32_t done;
 };
 
-struct lpt_jobs {
-    lpt_job j[16];
-};
-
-template <int NE>
-__device__ __forceinline__ unsigned long long reg_min(const unsigned long long (&v)[NE], uint32_t taken)
+template <int NE, typename KT>
+__device__ __forceinline__ KT reg_min(const KT (&v)[NE])
 {
-    unsigned long long t[NE];
+    KT t[NE];
 #pragma unroll
-    for (int j = 0; j < NE; ++j) t[j] = ((taken >> j) & 1u) ? ~0ull : v[j];
+    for (int j = 0; j < NE; ++j) t[j] = v[j];
 #pragma unroll
     for (int w = NE / 2; w > 0; w >>= 1) {
 #pragma unroll
@@ -998,341 +1013,473 @@ __device__ __forceinline__ unsigned long long reg_min(const unsigned long long (
     return t[0];
 }
 
-// Runs of keys with k_b = 1 and equal λ = q (Algorithm 1's loop over such a
-// run, done at once).  Each greedy pick is a current minimum (L_r, r) and
-// raising it by q keeps later picks no smaller, so the m picks are the m
-// smallest pairs (L_r + j q, r), j >= 0.  With L_r = q l_r + f_r (0 <= f_r < q)
-// pair (r, j) sorts by (l_r + j, f_r, r): picks come in rounds t = l_r + j,
-// each visiting {r : l_r <= t} in (f_r, r) order.  Between two consecutive
-// distinct levels l the visited set is fixed, so that stretch of rounds cycles
-// through it.  Cost: one pass over R per distinct level reached, plus the
-// output writes, instead of one warp minimum per key.
-struct lpt_run_smem {
-    uint16_t order[1024];  // destinations by (f_r, r)
-    uint16_t cyc[1024];    // destinations visited in the current stretch, in that order
-    uint32_t lev[1024];    // l_r
-    uint32_t add[1024];    // jobs given to r in this run; first q buckets reused for the sort
-};
-
-template <int NE>
-__device__ __forceinline__ bool lpt_equal_run(unsigned long long (&v)[NE], uint32_t R, unsigned long long q,
-                                              unsigned long long m, uint32_t base, uint16_t *__restrict__ members,
-                                              unsigned long long *__restrict__ jobs, lpt_run_smem &S,
-                                              bool &overflow)
-{
-    const uint32_t lane = cr_lane(), lt = (1u << lane) - 1u;
-    if (q == 0 || q > 1024) return false;
-    unsigned long long lmax = 0;
+// Minima of groups of four registers: a job changes one register (the same one in every
+// lane's numbering, so the branch is uniform), its group's minimum and the minimum of the groups.
+template <int NE, typename KT>
+struct reg_groups {
+    static constexpr int NG = NE >= 4 ? NE / 4 : 1, GS = NE >= 4 ? 4 : NE;
+    KT g[NG];
+    __device__ __forceinline__ void all(const KT (&v)[NE])
+    {
 #pragma unroll
-    for (int j = 0; j < NE; ++j)
-        if (lane + 32u * j < R) lmax = max(lmax, v[j] >> 16);
-    if (~cr_warp_min_u64(~lmax) >= (1ull << 31)) return false;  // levels in 32 bits
-    const uint32_t q32 = (uint32_t)q;
-    // counting sort by phase f_r, stable in r
-    for (uint32_t x = lane; x < q32; x += 32) S.add[x] = 0;
-    __syncwarp();
+        for (int x = 0; x < NG; ++x) {
+            KT t = v[x * GS];
 #pragma unroll
-    for (int j = 0; j < NE; ++j) {
-        const uint32_t r = lane + 32u * j;
-        if (r < R) {
-            const uint32_t L = (uint32_t)(v[j] >> 16);
-            S.lev[r] = L / q32;
-            atomicAdd(&S.add[L % q32], 1u);
+            for (int y = 1; y < GS; ++y) t = v[x * GS + y] < t ? v[x * GS + y] : t;
+            g[x] = t;
         }
     }
-    __syncwarp();
+    __device__ __forceinline__ KT least() const { return reg_min<NG, KT>(g); }
+    template <int J>
+    __device__ __forceinline__ void one(KT (&v)[NE], KT grow)
     {
-        const uint32_t per = (q32 + 31) / 32, x0 = lane * per;
-        uint32_t run = 0;
-        for (uint32_t x = x0; x < x0 + per && x < q32; ++x) run += S.add[x];
-        uint32_t inc = run;
+        if constexpr (J < NE) {
+            v[J] += grow;
+            constexpr int x = J / GS;
+            KT t = v[x * GS];
+#pragma unroll
+            for (int y = 1; y < GS; ++y) t = v[x * GS + y] < t ? v[x * GS + y] : t;
+            g[x] = t;
+        }
+    }
+    // v[jj] += grow, jj uniform over the warp
+    __device__ __forceinline__ void grow(KT (&v)[NE], uint32_t jj, KT by)
+    {
+#define CR_GROW(J) case J: one<J>(v, by); break;
+#define CR_GROW4(J) CR_GROW(J) CR_GROW(J + 1) CR_GROW(J + 2) CR_GROW(J + 3)
+        switch (jj) {
+            CR_GROW4(0) CR_GROW4(4) CR_GROW4(8) CR_GROW4(12) CR_GROW4(16) CR_GROW4(20) CR_GROW4(24) CR_GROW4(28)
+        }
+#undef CR_GROW4
+#undef CR_GROW
+    }
+};
+
+template <int NE, typename KT>
+__device__ __forceinline__ KT reg_min_untaken(const KT (&v)[NE], uint32_t taken)
+{
+    KT t[NE];
+#pragma unroll
+    for (int j = 0; j < NE; ++j) t[j] = ((taken >> j) & 1u) ? (KT)~(KT)0 : v[j];
+    return reg_min<NE, KT>(t);
+}
+
+__device__ __forceinline__ uint32_t warp_min_key(uint32_t v) { return __reduce_min_sync(0xffffffffu, v); }
+__device__ __forceinline__ unsigned long long warp_min_key(unsigned long long v) { return warp_min_u64(v); }
+
+// One run, by the whole CTA: S.a, S.q, S.base, S.rel set; returns the first key after it.
+// S.add[r] = jobs given to r.
+__device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, uint32_t R, uint32_t na,
+                                            const unsigned long long *__restrict__ adm_cnt,
+                                            uint16_t *__restrict__ members, unsigned long long *__restrict__ jobs)
+{
+    const uint32_t tid = threadIdx.x, lane = cr_lane(), warp = tid >> 5, lt = (1u << lane) - 1u;
+    const uint32_t a = S.a, q = S.q, base = S.base;
+    // end of the run: λ is non-increasing, so the keys equal to q are a prefix of [a, na)
+    uint32_t lo = a, hi = na;  // adm_cnt[lo] == q; answer in (lo, hi]
+    while (hi - lo > 1) {
+        const uint32_t step = (hi - lo - 1 + kPlaceBlock - 1) / kPlaceBlock;  // probes lo + step, lo + 2 step, ...
+        const unsigned long long pr = lo + (unsigned long long)(tid + 1) * step;
+        const bool same = pr < hi && adm_cnt[pr] == q;
+        const uint32_t c = (uint32_t)__syncthreads_count(same);
+        lo += c * step;
+        const unsigned long long nh = (unsigned long long)lo + step;
+        hi = nh < hi ? (uint32_t)nh : hi;
+    }
+    // levels and phases; thread's two places of the order: 64 warp + lane and 32 above
+    uint32_t key[2], fmax = 0;
+    bool have[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const uint32_t r = 64u * warp + 32u * x + lane;
+        have[x] = r < R;
+        key[x] = r;
+        if (have[x]) {
+            const uint32_t L = S.rel[r], l = L / q;
+            key[x] = ((L - l * q) << 10) | r;
+            S.rel[r] = l;
+        }
+    }
+    // sorted by (f_r, r): r is the starting order, so stable counting passes over f, 6 bits each.
+    // Lane l counts its warp's entries of digits l and l + 32 from the ballots of the digit bits;
+    // one scan of the 64 x 16 (digit, warp) counts gives every warp's offsets.
+    fmax = q - 1u;
+    for (uint32_t sh = 10; sh == 10 || (fmax >> (sh - 10u)) != 0u; sh += 6) {
+        const uint32_t v0 = __ballot_sync(0xffffffffu, have[0]), v1 = __ballot_sync(0xffffffffu, have[1]);
+        const uint32_t d0 = (key[0] >> sh) & 63u, d1 = (key[1] >> sh) & 63u;
+        uint32_t c00 = v0, c01 = v1, c10 = v0, c11 = v1;  // entries (of places 0, 1) of digits lane, lane + 32
+        uint32_t s0 = v0, s1 = v1, s10 = v0;              // entries with this lane's digits: 0 in 0, 1 in 1, 1 in 0
+#pragma unroll
+        for (int bt = 0; bt < 6; ++bt) {
+            const uint32_t B0 = __ballot_sync(0xffffffffu, (d0 >> bt) & 1u);
+            const uint32_t B1 = __ballot_sync(0xffffffffu, (d1 >> bt) & 1u);
+            const uint32_t lb = bt < 5 ? 0u - ((lane >> bt) & 1u) : 0u, hb = bt < 5 ? lb : 0xffffffffu;
+            c00 &= ~(B0 ^ lb);
+            c01 &= ~(B1 ^ lb);
+            c10 &= ~(B0 ^ hb);
+            c11 &= ~(B1 ^ hb);
+            const uint32_t m0 = 0u - ((d0 >> bt) & 1u), m1 = 0u - ((d1 >> bt) & 1u);
+            s0 &= ~(B0 ^ m0);
+            s1 &= ~(B1 ^ m1);
+            s10 &= ~(B0 ^ m1);
+        }
+        constexpr uint32_t kW = kPlaceBlock / 32;
+        S.cnt[lane * kW + warp] = (uint32_t)(__popc(c00) + __popc(c01));
+        S.cnt[(lane + 32u) * kW + warp] = (uint32_t)(__popc(c10) + __popc(c11));
+        __syncthreads();
+        // exclusive scan of the 1024 counts, two per thread
+        const uint32_t x0 = S.cnt[2 * tid], x1 = S.cnt[2 * tid + 1];
+        uint32_t inc = x0 + x1;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= (uint32_t)o) inc += y;
         }
-        uint32_t off = inc - run;
-        __syncwarp();
-        for (uint32_t x = x0; x < x0 + per && x < q32; ++x) {
-            const uint32_t c = S.add[x];
-            S.add[x] = off;
-            off += c;
+        if (lane == 31) S.wcnt[0][warp] = inc;
+        __syncthreads();
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? S.wcnt[0][lane & (kW - 1)] : 0u);
+        S.cnt[2 * tid] = before + inc - x0 - x1;
+        S.cnt[2 * tid + 1] = before + inc - x1;
+        __syncthreads();
+        if (have[0]) S.srt[S.cnt[d0 * kW + warp] + (uint32_t)__popc(s0 & lt)] = key[0];
+        if (have[1]) S.srt[S.cnt[d1 * kW + warp] + (uint32_t)__popc(s10) + (uint32_t)__popc(s1 & lt)] = key[1];
+        __syncthreads();
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+            if (have[x]) key[x] = S.srt[64u * warp + 32u * x + lane];
+    }
+    uint32_t r[2], lev[2], add[2] = {0, 0};
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        r[x] = key[x] & 1023u;
+        lev[x] = have[x] ? S.rel[r[x]] : 0xffffffffu;
+    }
+    // first level: minimum over the CTA
+    uint32_t T;
+    {
+        const uint32_t w = __reduce_min_sync(0xffffffffu, lev[0] < lev[1] ? lev[0] : lev[1]);
+        if (lane == 0) S.wnxt[1][warp] = w;
+        __syncthreads();
+        T = __reduce_min_sync(0xffffffffu, S.wnxt[1][lane & (kPlaceBlock / 32 - 1)]);
+    }
+    uint32_t left = hi - a, done = 0, par = 0;
+    while (left) {  // each stretch serves at least one job
+        const bool in0 = have[0] && lev[0] <= T, in1 = have[1] && lev[1] <= T;
+        const uint32_t b0 = __ballot_sync(0xffffffffu, in0), b1 = __ballot_sync(0xffffffffu, in1);
+        uint32_t nx = 0xffffffffu;
+        if (have[0] && !in0) nx = lev[0];
+        if (have[1] && !in1) nx = lev[1] < nx ? lev[1] : nx;
+        nx = __reduce_min_sync(0xffffffffu, nx);
+        if (lane == 0) {
+            S.wcnt[par][warp] = (uint32_t)(__popc(b0) + __popc(b1));
+            S.wnxt[par][warp] = nx;
+        }
+        __syncthreads();
+        constexpr uint32_t kW = kPlaceBlock / 32;
+        const uint32_t c = lane < kW ? S.wcnt[par][lane] : 0u;
+        const uint32_t nxt = __reduce_min_sync(0xffffffffu, lane < kW ? S.wnxt[par][lane] : 0xffffffffu);
+        const uint32_t n_in = __reduce_add_sync(0xffffffffu, c);
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? c : 0u);
+        uint32_t cnt = left;
+        if (nxt != 0xffffffffu && (unsigned long long)n_in * (nxt - T) < left) cnt = n_in * (nxt - T);
+        const uint32_t full = cnt / n_in, part = cnt - full * n_in;
+        if (in0) {
+            const uint32_t k = before + (uint32_t)__popc(b0 & lt);
+            S.cyc[par][k] = (uint16_t)r[0];
+            add[0] += full + (k < part ? 1u : 0u);
+        }
+        if (in1) {
+            const uint32_t k = before + (uint32_t)__popc(b0) + (uint32_t)__popc(b1 & lt);
+            S.cyc[par][k] = (uint16_t)r[1];
+            add[1] += full + (k < part ? 1u : 0u);
+        }
+        __syncthreads();
+        uint32_t ci = tid % n_in;
+        const uint32_t cstep = kPlaceBlock % n_in;
+        for (uint32_t i = tid; i < cnt; i += kPlaceBlock) {
+            members[(size_t)base + done + i] = S.cyc[par][ci];
+            jobs[(size_t)base + done + i] = q;
+            ci += cstep;
+            if (ci >= n_in) ci -= n_in;
+        }
+        done += cnt;
+        left -= cnt;
+        T = nxt;
+        par ^= 1u;
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+        if (have[x]) S.add[r[x]] = add[x];
+    return hi;
+}
+
+// One LPT plan on one CTA.  KT: packed keys; u32 keys hold loads relative to `origin`.
+template <int NE, typename KT>
+__device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, int shift, unsigned long long origin,
+                                         uint32_t *status)
+{
+    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5, R = J.R;
+    const KT rmask = (KT)(((KT)1 << shift) - 1);
+    const uint32_t na = (uint32_t)J.info->n_adm;
+    KT v[NE], m = (KT)~(KT)0;
+    uint32_t a = 0;
+    if (warp == 0) {
+#pragma unroll
+        for (int j = 0; j < NE; ++j) {
+            const uint32_t r = lane + 32u * j;
+            v[j] = r < R ? (KT)(((KT)(J.load[r] - origin) << shift) | (KT)r) : (KT)~(KT)0;
+        }
+        m = reg_min<NE, KT>(v);
+    }
+    for (;;) {
+        if (warp == 0) {
+            bool run = false;
+            unsigned long long rorg = 0;
+            while (a < na) {
+                // 32 keys, one per lane
+                const uint32_t cnt = na - a < 32u ? na - a : 32u;
+                unsigned long long st_lam = 0;
+                uint32_t st_k = 0, st_off = 0;
+                if (lane < cnt) {
+                    st_lam = J.adm_cnt[a + lane];
+                    st_k = J.adm_k[a + lane];
+                    st_off = J.koff[a + lane];
+                }
+                const uint32_t k0 = __shfl_sync(0xffffffffu, st_k, 0);
+                const unsigned long long l0 = __shfl_sync(0xffffffffu, st_lam, 0);
+                const unsigned long long l31 = __shfl_sync(0xffffffffu, st_lam, 31);
+                if (k0 == 1 && cnt == kRunMin && l31 == l0 && l0 <= kRunMaxQ) {
+                    // a run of >= 32 keys with k = 1 and equal λ starts here; it works on
+                    // loads relative to the least one, in 31 bits
+                    KT mx = 0;
+#pragma unroll
+                    for (int j = 0; j < NE; ++j)
+                        if (lane + 32u * j < R && v[j] > mx) mx = v[j];
+                    const KT mn = warp_min_key(m);
+                    const KT far = (KT)~warp_min_key((KT)~mx);
+                    if (((far >> shift) - (mn >> shift)) < (KT)0x7fffffffu) {
+                        run = true;
+                        rorg = (unsigned long long)(mn >> shift);
+                        if (lane == 0) {
+                            S.a = a;
+                            S.q = (uint32_t)l0;
+                            S.base = st_off;
+                        }
+                        break;
+                    }
+                }
+                // keys with several replicas come first (k_b is non-increasing)
+                const uint32_t nm = (uint32_t)__popc(__ballot_sync(0xffffffffu, lane < cnt && st_k != 1u));
+                for (uint32_t slot = 0; slot < nm; ++slot) {
+                    const uint32_t k = __shfl_sync(0xffffffffu, st_k, slot);
+                    const uint32_t base = __shfl_sync(0xffffffffu, st_off, slot);
+                    const uint32_t lam = (uint32_t)__shfl_sync(0xffffffffu, st_lam, slot);  // <= n < 2^32
+                    const uint32_t q = lam / k, rem = lam - q * k;
+                    uint32_t taken = 0;
+                    for (uint32_t s = 0; s < k; ++s) {
+                        const KT best = warp_min_key(m);
+                        const uint32_t br = (uint32_t)(best & rmask);
+                        const uint32_t job = q + (s < rem ? 1u : 0u);
+                        if (lane == 0) {
+                            J.members[base + s] = (uint16_t)br;
+                            J.jobs[base + s] = job;
+                        }
+                        if ((br & 31u) == lane) {
+                            const uint32_t jj = br >> 5;
+#pragma unroll
+                            for (int j = 0; j < NE; ++j)
+                                if (j == (int)jj) v[j] += (KT)job << shift;
+                            taken |= 1u << jj;  // not eligible again for this key
+                            m = reg_min_untaken<NE, KT>(v, taken);
+                        }
+                    }
+                    m = reg_min<NE, KT>(v);
+                }
+                // single copies: lane `slot` keeps its key's destination, written once for all
+                uint32_t mine = 0;
+                reg_groups<NE, KT> G;
+                G.all(v);
+                for (uint32_t slot = nm; slot < cnt; ++slot) {
+                    const KT grow = (KT)__shfl_sync(0xffffffffu, st_lam, slot) << shift;
+                    const KT best = warp_min_key(m);
+                    const uint32_t br = (uint32_t)(best & rmask);
+                    if (lane == slot) mine = br;
+                    G.grow(v, br >> 5, (br & 31u) == lane ? grow : (KT)0);
+                    m = G.least();
+                }
+                if (lane >= nm && lane < cnt) {
+                    J.members[st_off] = (uint16_t)mine;
+                    J.jobs[st_off] = st_lam;
+                }
+                a += cnt;
+            }
+            if (run) {
+#pragma unroll
+                for (int j = 0; j < NE; ++j) {
+                    const uint32_t r = lane + 32u * j;
+                    if (r < R) S.rel[r] = (uint32_t)((unsigned long long)(v[j] >> shift) - rorg);
+                }
+            }
+            if (lane == 0) S.done = run ? 0u : 1u;
+        }
+        __syncthreads();
+        if (S.done) break;
+        const unsigned long long q = S.q;
+        const uint32_t hi = lpt_run(S, R, na, J.adm_cnt, J.members, J.jobs);
+        __syncthreads();
+        if (warp == 0) {
+            a = hi;
+#pragma unroll
+            for (int j = 0; j < NE; ++j) {
+                const uint32_t r = lane + 32u * j;
+                if (r < R) v[j] += (KT)((unsigned long long)S.add[r] * q) << shift;
+            }
+            m = reg_min<NE, KT>(v);
         }
     }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < NE; ++j) {
-        const uint32_t r = lane + 32u * j;
-        const uint32_t f = r < R ? (uint32_t)(v[j] >> 16) % q32 : 0xffffffffu;
-        const uint32_t peers = __match_any_sync(0xffffffffu, f);
-        const uint32_t at = r < R ? S.add[f] : 0u;
-        __syncwarp();
-        if (r < R) {
-            S.order[at + __popc(peers & lt)] = (uint16_t)r;
-            if ((peers & lt) == 0) S.add[f] = at + __popc(peers);
-        }
-        __syncwarp();
-    }
-    for (uint32_t x = lane; x < R; x += 32) S.add[x] = 0;
-    __syncwarp();
-    // stretches of rounds between consecutive distinct levels
-    uint32_t T = 0xffffffffu;
-#pragma unroll
-    for (int j = 0; j < NE; ++j)
-        if (lane + 32u * j < R) T = min(T, S.lev[lane + 32u * j]);
-    T = __reduce_min_sync(0xffffffffu, T);
-    unsigned long long left = m, done = 0;
-    while (left) {
-        uint32_t n_in = 0, nxt = 0xffffffffu;
+    if (warp == 0) {
+        bool overflow = false;
 #pragma unroll
         for (int j = 0; j < NE; ++j) {
             const uint32_t r = lane + 32u * j;
             if (r < R) {
-                const uint32_t l = S.lev[r];
-                n_in += l <= T ? 1u : 0u;
-                if (l > T) nxt = min(nxt, l);
+                const unsigned long long L = origin + (unsigned long long)(v[j] >> shift);
+                overflow |= L >= kLoadLimit;  // loads only grow: the final ones tell
+                J.load[r] = L;
             }
         }
-        n_in = __reduce_add_sync(0xffffffffu, n_in);
-        nxt = __reduce_min_sync(0xffffffffu, nxt);
-        unsigned long long cnt = left;
-        if (nxt != 0xffffffffu && (unsigned long long)n_in * (nxt - T) < left)
-            cnt = (unsigned long long)n_in * (nxt - T);
-        const unsigned long long full = cnt / n_in;
-        const uint32_t part = (uint32_t)(cnt % n_in);
-        uint32_t seen = 0;
-        for (uint32_t p0 = 0; p0 < R; p0 += 32) {
-            const uint32_t p = p0 + lane;
-            const uint32_t r = p < R ? S.order[p] : 0u;
-            const bool in = p < R && S.lev[r] <= T;
-            const uint32_t bal = __ballot_sync(0xffffffffu, in);
-            if (in) {
-                const uint32_t k = seen + __popc(bal & lt);
-                S.cyc[k] = (uint16_t)r;
-                S.add[r] += (uint32_t)full + (k < part ? 1u : 0u);
+        if (__any_sync(0xffffffffu, overflow) && lane == 0) atomicOr(status, CR_FLAG_OVERFLOW);
+    }
+}
+
+// RANDOM placement: T(b) = the first k_b entries of a Fisher-Yates shuffle of
+// 0..R-1 (step s swaps position s with s + floor(u R_s / 2^64), R_s = R - s).
+// A key with k_b = 1 needs no array: its member is the first draw itself, so
+// every lane of a warp places one such key.  The keys with k_b > 1 (k_b is
+// non-increasing in admission order, so they come first) are dealt to warps one
+// by one; a warp draws 32 of a key's steps at once, one per lane, and lane 0
+// does the swaps over a shared-memory array that is never reset: an entry counts
+// only when its stamp equals the key being placed, otherwise position x holds x.
+// Every key therefore costs O(k_b), not O(R).
+constexpr int kRandWarps = 4;  // warps of a CTA that hold such an array
+
+__host__ __device__ inline size_t random_smem(uint32_t R)
+{
+    return (size_t)kRandWarps * ((R + 1u) & ~1u) * 3 * sizeof(uint16_t);
+}
+
+__device__ __forceinline__ void random_plan(const place_job &J, uint32_t block, uint32_t nblocks, uint32_t *status,
+                                            uint16_t *perm_all)
+{
+    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5, R = J.R;
+    const uint32_t na = (uint32_t)J.info->n_adm;
+    if (warp < (uint32_t)kRandWarps) {
+        const uint32_t Rp = (R + 1u) & ~1u;                          // keeps the stamps 4-byte aligned
+        uint16_t *val = perm_all + (size_t)warp * Rp * 3;           // [R] values of touched positions
+        uint32_t *stamp = reinterpret_cast<uint32_t *>(val + Rp);    // [R] key (+1) that touched each
+        bool clear = true;
+        for (uint32_t b = block * kRandWarps + warp; b < na; b += nblocks * kRandWarps) {
+            const uint32_t kb = J.adm_k[b];
+            if (kb <= 1) break;
+            if (clear) {
+                for (uint32_t r = lane; r < R; r += 32) stamp[r] = 0;
+                __syncwarp();
+                clear = false;
             }
-            seen += __popc(bal);
+            const uint32_t base = J.koff[b], tag = b + 1u;
+            const unsigned long long lam = J.adm_cnt[b];
+            const unsigned long long q = lam / kb, rem = lam % kb;
+            for (uint32_t s0 = 0; s0 < kb; s0 += 32) {
+                uint32_t t = 0;
+                if (s0 + lane < kb) {
+                    const uint32_t s = s0 + lane;
+                    const cr_u64x4 u = cr_philox4x64_10(b, s, 1ull, J.epoch, J.seed,
+                                                        (unsigned long long)CR_POLICY_CR_NOLPT);
+                    t = s + cr_scale(u.x, (unsigned long long)(R - s));
+                }
+                const uint32_t cnt = kb - s0 < 32u ? kb - s0 : 32u;
+                for (uint32_t x = 0; x < cnt; ++x) {
+                    const uint32_t tx = __shfl_sync(0xffffffffu, t, x), s = s0 + x;
+                    if (lane == 0) {
+                        const uint32_t vs = stamp[s] == tag ? val[s] : s;
+                        const uint32_t vt = stamp[tx] == tag ? val[tx] : tx;
+                        val[tx] = (uint16_t)vs;
+                        stamp[tx] = tag;
+                        val[s] = (uint16_t)vt;  // later steps only swap positions above s
+                        stamp[s] = tag;
+                    }
+                }
+            }
+            __syncwarp();
+            for (uint32_t s = lane; s < kb; s += 32) {
+                const unsigned long long job = q + (s < rem ? 1ull : 0ull);
+                const uint32_t m = val[s];
+                J.members[base + s] = (uint16_t)m;
+                J.jobs[base + s] = job;
+                const unsigned long long old = atomicAdd(&J.load[m], job);
+                if (old + job >= kLoadLimit) atomicOr(status, CR_FLAG_OVERFLOW);
+            }
+            __syncwarp();
         }
-        __syncwarp();
-        unsigned long long i = lane, ci = lane % n_in;
-        const uint32_t step = 32u % n_in;
-        for (; i < cnt; i += 32) {
-            members[base + done + i] = S.cyc[ci];
-            jobs[base + done + i] = q;
-            ci += step;
-            if (ci >= n_in) ci -= n_in;
-        }
-        __syncwarp();
-        done += cnt;
-        left -= cnt;
-        T = nxt;
     }
-#pragma unroll
-    for (int j = 0; j < NE; ++j) {
-        const uint32_t r = lane + 32u * j;
-        if (r < R) {
-            v[j] += ((unsigned long long)S.add[r] * q) << 16;
-            if ((v[j] >> 16) >= kLoadLimit) overflow = true;
+    for (uint32_t a = block * kPlaceBlock + threadIdx.x; a < na; a += nblocks * kPlaceBlock) {
+        if (J.adm_k[a] != 1) continue;
+        const cr_u64x4 u = cr_philox4x64_10(a, 0ull, 1ull, J.epoch, J.seed, (unsigned long long)CR_POLICY_CR_NOLPT);
+        const uint32_t m = cr_scale(u.x, (unsigned long long)R);
+        const unsigned long long lam = J.adm_cnt[a];
+        const uint32_t o = J.koff[a];
+        J.members[o] = (uint16_t)m;
+        J.jobs[o] = lam;
+        const unsigned long long old = atomicAdd(&J.load[m], lam);
+        if (old + lam >= kLoadLimit) atomicOr(status, CR_FLAG_OVERFLOW);
+    }
+}
+
+// Blocks 0 .. n_lpt-1: the LPT plans pj.j[0 .. n_lpt); then rblocks blocks for each random plan after them.
+template <int NE>
+__global__ void __launch_bounds__(kPlaceBlock) k_plan_place(const __grid_constant__ place_jobs pj, uint32_t n_lpt,
+                                                            uint32_t rblocks, uint32_t *status)
+{
+    extern __shared__ uint4 place_sm[];
+    if (blockIdx.x >= n_lpt) {
+        const uint32_t x = blockIdx.x - n_lpt;
+        random_plan(pj.j[n_lpt + x / rblocks], x % rblocks, rblocks, status, reinterpret_cast<uint16_t *>(place_sm));
+        return;
+    }
+    const place_job &J = pj.j[blockIdx.x];
+    lpt_smem &S = *reinterpret_cast<lpt_smem *>(place_sm);
+    // 32-bit keys when every load the plan can reach, relative to the least starting load, leaves room for r
+    __shared__ unsigned long long s_min, s_max;
+    if (threadIdx.x == 0) {
+        s_min = ~0ull;
+        s_max = 0;
+    }
+    __syncthreads();
+    {
+        unsigned long long mn = ~0ull, mx = 0;
+        for (uint32_t r = threadIdx.x; r < J.R; r += kPlaceBlock) {
+            const unsigned long long L = J.load[r];
+            mn = L < mn ? L : mn;
+            mx = L > mx ? L : mx;
+        }
+        if (threadIdx.x < J.R) {
+            atomicMin(&s_min, mn);
+            atomicMax(&s_max, mx);
         }
     }
-    __syncwarp();
-    return true;
+    __syncthreads();
+    const unsigned long long span = s_max - s_min;
+    const int rb = J.R > 1 ? 32 - __clz(J.R - 1u) : 1;
+    if (span < (1ull << 31) && span + J.info->adm_lam < (1ull << (32 - rb)) - 1ull)
+        lpt_plan<NE, uint32_t>(J, S, rb, s_min, status);
+    else
+        lpt_plan<NE, unsigned long long>(J, S, 16, 0ull, status);
 }
 
 // LPT for R <= 32 uses the sorted-lane kernel (fastest per key) unless the slot
 // budget admits this many keys or more: long admission lists reach the long
 // runs of equal counts in the tail, which the register kernel places at once.
 constexpr uint64_t kLptRunsFrom = 512;
-
-template <int NE>
-__global__ void __launch_bounds__(32) k_plan_lpt_reg(const __grid_constant__ lpt_jobs jobs_in, uint32_t *status)
-{
-    const lpt_job J = jobs_in.j[blockIdx.x];
-    const uint32_t lane = cr_lane(), R = J.R;
-    unsigned long long v[NE];
-#pragma unroll
-    for (int j = 0; j < NE; ++j) {
-        const uint32_t r = lane + 32u * j;
-        v[j] = r < R ? ((J.load[r] << 16) | r) : ~0ull;
-    }
-    uint32_t taken = 0;
-    unsigned long long m = reg_min<NE>(v, 0u);
-    const unsigned long long na = J.info->n_adm;
-    bool overflow = false;
-    unsigned long long st_lam = 0;
-    uint32_t st_k = 0, st_off = 0;
-    __shared__ lpt_run_smem S;
-    unsigned long long stage = 0;  // first key of the 32 staged in st_*
-    for (unsigned long long a = 0; a < na; ++a) {
-        if (a == 0 || a - stage >= 32) {
-            stage = a;
-            const unsigned long long ia = a + lane;
-            if (ia < na) {
-                st_lam = J.adm_cnt[ia];
-                st_k = J.adm_k[ia];
-                st_off = J.koff[ia];
-            }
-            // a run of >= 32 keys with k = 1 and equal λ starts here: place it at once
-            const uint32_t k0 = __shfl_sync(0xffffffffu, st_k, 0);
-            const unsigned long long l0 = __shfl_sync(0xffffffffu, st_lam, 0);
-            const unsigned long long l31 = __shfl_sync(0xffffffffu, st_lam, 31);
-            if (k0 == 1 && a + 31 < na && l31 == l0) {
-                // end of the run: first index after a whose λ differs (λ is non-increasing)
-                unsigned long long lo = a + 31, hi = na;  // adm_cnt[lo] == l0; answer in (lo, hi]
-                while (hi - lo > 1) {
-                    const unsigned long long span = hi - lo;
-                    const unsigned long long pr = lo + 1 + (span - 1) * lane / 32;  // 32 probes in (lo, hi)
-                    const bool differs = J.adm_cnt[pr] != l0;
-                    const uint32_t bl = __ballot_sync(0xffffffffu, differs);
-                    if (!bl) {
-                        lo = __shfl_sync(0xffffffffu, pr, 31);
-                    } else {
-                        const uint32_t f = __ffs(bl) - 1;
-                        hi = __shfl_sync(0xffffffffu, pr, f);
-                        if (f > 0) lo = __shfl_sync(0xffffffffu, pr, f - 1);
-                    }
-                }
-                const unsigned long long runm = hi - a;
-                const uint32_t base0 = __shfl_sync(0xffffffffu, st_off, 0);
-                if (lpt_equal_run<NE>(v, R, l0, runm, base0, J.members, J.jobs, S, overflow)) {
-                    a = hi - 1;      // the loop's ++a moves to the first key after the run
-                    stage = a + 1 - 32;  // forces a restage at hi
-                    m = reg_min<NE>(v, 0u);
-                    continue;
-                }
-            }
-        }
-        const uint32_t slot = (uint32_t)(a - stage);
-        const uint32_t k = __shfl_sync(0xffffffffu, st_k, slot);
-        const uint32_t base = __shfl_sync(0xffffffffu, st_off, slot);
-        const unsigned long long lam = __shfl_sync(0xffffffffu, st_lam, slot);
-        const unsigned long long q = k == 1 ? lam : lam / k, rem = k == 1 ? 0ull : lam % k;
-        for (uint32_t s = 0; s < k; ++s) {
-            const unsigned long long best = warp_min_u64(m);
-            const uint32_t br = (uint32_t)(best & 0xffffu);
-            const unsigned long long job = q + (s < rem ? 1ull : 0ull);
-            if (lane == 0) {
-                J.members[base + s] = (uint16_t)br;
-                J.jobs[base + s] = job;
-            }
-            if ((br & 31u) == lane) {
-                const uint32_t jj = br >> 5;
-#pragma unroll
-                for (int j = 0; j < NE; ++j)
-                    if (j == (int)jj) v[j] += job << 16;
-                if (((best >> 16) + job) >= kLoadLimit) overflow = true;
-                if (k > 1) taken |= 1u << jj;
-                m = reg_min<NE>(v, taken);
-            }
-        }
-        if (k > 1) {  // release this key's destinations for the next key
-            taken = 0;
-            m = reg_min<NE>(v, 0u);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < NE; ++j) {
-        const uint32_t r = lane + 32u * j;
-        if (r < R) J.load[r] = v[j] >> 16;
-    }
-    if (__any_sync(0xffffffffu, overflow) && lane == 0) atomicOr(status, CR_FLAG_OVERFLOW);
-}
-
-// RANDOM placement: T(b) = the first k_b entries of a Fisher-Yates shuffle of
-// 0..R-1 (step s swaps position s with s + floor(u R_s / 2^64), R_s = R - s).
-// A key with k_b = 1 needs no array: its member is the first draw itself, so
-// every lane of a warp places one such key.  Keys with k_b > 1 are shuffled by
-// the warp's lane 0 over a shared-memory array that is never reset: an entry
-// counts only when its stamp equals the key being placed, otherwise position x
-// holds x.  Every key therefore costs O(k_b), not O(R).
-constexpr int kRandWarps = 4;
-
-__device__ __forceinline__ void random_body(const cr_plan_info_dev *info,
-                                                                 const unsigned long long *__restrict__ adm_cnt,
-                                                                 const uint32_t *__restrict__ adm_k,
-                                                                 const uint32_t *__restrict__ koff, uint32_t R,
-                                                                 unsigned long long seed, unsigned long long epoch,
-                                                                 unsigned long long *__restrict__ load_g,
-                                                                 uint16_t *__restrict__ members,
-                                                                 unsigned long long *__restrict__ jobs,
-                                                                 uint32_t *status, uint16_t *perm_all)
-{
-    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5;
-    const uint32_t Rp = (R + 1u) & ~1u;                                  // keeps the stamps 4-byte aligned
-    uint16_t *val = perm_all + (size_t)warp * Rp * 3;                  // [R] values of touched positions
-    uint32_t *stamp = reinterpret_cast<uint32_t *>(val + Rp);           // [R] key (+1) that touched each
-    for (uint32_t r = lane; r < R; r += 32) stamp[r] = 0;
-    __syncwarp();
-    const unsigned long long na = info->n_adm;
-    const unsigned long long nw = (unsigned long long)gridDim.x * kRandWarps;
-    for (unsigned long long a0 = ((unsigned long long)blockIdx.x * kRandWarps + warp) * 32; a0 < na; a0 += nw * 32) {
-        const unsigned long long a = a0 + lane;
-        const bool live = a < na;
-        const uint32_t k = live ? adm_k[a] : 0u;
-        if (live && k == 1) {
-            const cr_u64x4 u = cr_philox4x64_10(a, 0ull, 1ull, epoch, seed, (unsigned long long)CR_POLICY_CR_NOLPT);
-            const uint32_t m = cr_scale(u.x, (unsigned long long)R);
-            const unsigned long long lam = adm_cnt[a];
-            members[koff[a]] = (uint16_t)m;
-            jobs[koff[a]] = lam;
-            const unsigned long long old = atomicAdd(&load_g[m], lam);
-            if (old + lam >= kLoadLimit) atomicOr(status, CR_FLAG_OVERFLOW);
-        }
-        for (unsigned mk = __ballot_sync(0xffffffffu, live && k > 1); mk; mk &= mk - 1) {  // uniform
-            const uint32_t src = (uint32_t)__ffs(mk) - 1u;
-            const unsigned long long b = a0 + src;
-            const uint32_t kb = __shfl_sync(0xffffffffu, k, src), base = koff[b];
-            const unsigned long long lam = adm_cnt[b];
-            const unsigned long long q = lam / kb, rem = lam % kb;
-            const uint32_t tag = (uint32_t)b + 1u;
-            if (lane == 0) {
-                for (uint32_t s2 = 0; s2 < kb; ++s2) {
-                    const cr_u64x4 u = cr_philox4x64_10(b, s2, 1ull, epoch, seed, (unsigned long long)CR_POLICY_CR_NOLPT);
-                    const uint32_t t = s2 + cr_scale(u.x, (unsigned long long)(R - s2));
-                    const uint32_t vs = stamp[s2] == tag ? val[s2] : s2;
-                    const uint32_t vt = stamp[t] == tag ? val[t] : t;
-                    val[t] = (uint16_t)vs;
-                    stamp[t] = tag;
-                    val[s2] = (uint16_t)vt;
-                    stamp[s2] = tag;
-                    members[base + s2] = (uint16_t)vt;  // later steps only swap positions above s2
-                }
-            }
-            __syncwarp();
-            for (uint32_t s2 = lane; s2 < kb; s2 += 32) {
-                const unsigned long long job = q + (s2 < rem ? 1ull : 0ull);
-                const uint32_t m = val[s2];
-                jobs[base + s2] = job;
-                const unsigned long long old = atomicAdd(&load_g[m], job);
-                if (old + job >= kLoadLimit) atomicOr(status, CR_FLAG_OVERFLOW);
-            }
-            __syncwarp();
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kRandWarps * 32) k_plan_random(const cr_plan_info_dev *info,
-                                                                 const unsigned long long *__restrict__ adm_cnt,
-                                                                 const uint32_t *__restrict__ adm_k,
-                                                                 const uint32_t *__restrict__ koff, uint32_t R,
-                                                                 unsigned long long seed, unsigned long long epoch,
-                                                                 unsigned long long *__restrict__ load_g,
-                                                                 uint16_t *__restrict__ members,
-                                                                 unsigned long long *__restrict__ jobs,
-                                                                 uint32_t *status)
-{
-    extern __shared__ uint16_t perm_all[];
-    random_body(info, adm_cnt, adm_k, koff, R, seed, epoch, load_g, members, jobs, status, perm_all);
-}
-
-__global__ void __launch_bounds__(kRandWarps * 32) k_plan_random_multi(const __grid_constant__ place_jobs pj,
-                                                                       uint32_t *status)
-{
-    extern __shared__ uint16_t perm_all[];
-    const place_job &J = pj.j[blockIdx.y];
-    random_body(J.info, J.adm_cnt, J.adm_k, J.koff, J.R, J.seed, J.epoch, J.load, J.members, J.jobs, status,
-                perm_all);
-}
 
 __device__ __forceinline__ void table_body(const cr_plan_info_dev *info, const unsigned long long *__restrict__ adm_key,
                                const uint32_t *__restrict__ adm_k, const uint32_t *__restrict__ koff,
@@ -1602,41 +1749,112 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
     }
 
     // ---- per plan -------------------------------------------------------------
-    // LPT placements with 32 < R <= 1024 are collected and run together, one
-    // warp per plan, followed by their tables.
-    lpt_jobs lj;
-    uint32_t n_lj = 0, lj_maxR = 0, deferred[16];
-    const bool fused = n > 0 && n <= kPlanSortOneCta;  // small intervals: batched launches throughout
-    const bool tables_later = fused;
-    auto table_insert = [&](uint32_t j) -> int {
-        cr_plan *p = plans[j];
-        const uint64_t C = (uint64_t)params[j].R * params[j].W;
-        const int bits = bits_for(p->table_slots - 1);
-        const uint64_t adm = n < C ? n : C;
-        CR_LAUNCH(ctx, k_table_insert, cr_blocks(adm, 256, gcap), 256, 0, (const cr_plan_info_dev *)p->d_info,
-                  (const unsigned long long *)p->d_adm_key, (const uint32_t *)p->d_adm_k,
-                  (const uint32_t *)p->d_koff, (const uint16_t *)p->d_members, p->d_table, bits);
+    // placements are collected and launched together, then every plan's table
+    const bool fused = n > 0 && n <= kPlanSortOneCta;  // small intervals: admission in one launch as well
+    place_jobs lj, rj, l32;                            // LPT (R <= 1024), random, short LPT lists
+    uint32_t n_lj = 0, n_rj = 0, n32 = 0, lj_maxR = 0, rj_maxR = 0;
+    uint64_t rj_adm = 0;
+    auto flush_place = [&]() -> int {
+        if (!n_lj && !n_rj) return CR_OK;
+        for (uint32_t x = 0; x < n_rj; ++x) lj.j[n_lj + x] = rj.j[x];
+        const uint32_t rblocks = cr_blocks(rj_adm, kPlaceBlock, gcap);
+        const size_t smem = std::max(n_lj ? sizeof(lpt_smem) : (size_t)0, n_rj ? random_smem(rj_maxR) : (size_t)0);
+        const uint32_t grid = n_lj + n_rj * rblocks, ne = (lj_maxR + 31) / 32;
+        auto launch = [&](auto kern) -> int {
+            if (smem > 48 * 1024)
+                CR_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            CR_LAUNCH(ctx, kern, grid, kPlaceBlock, smem, lj, n_lj, rblocks, ctx->d_status);
+            return CR_OK;
+        };
+        if (ne <= 1)
+            CR_TRY(launch(k_plan_place<1>));
+        else if (ne <= 2)
+            CR_TRY(launch(k_plan_place<2>));
+        else if (ne <= 4)
+            CR_TRY(launch(k_plan_place<4>));
+        else if (ne <= 8)
+            CR_TRY(launch(k_plan_place<8>));
+        else if (ne <= 16)
+            CR_TRY(launch(k_plan_place<16>));
+        else
+            CR_TRY(launch(k_plan_place<32>));
+        n_lj = n_rj = 0;
+        lj_maxR = rj_maxR = 0;
+        rj_adm = 0;
         return CR_OK;
     };
-    auto flush_lpt = [&]() -> int {
-        if (!n_lj) return CR_OK;
-        const uint32_t ne = (lj_maxR + 31) / 32;
-        if (ne <= 1)
-            CR_LAUNCH(ctx, k_plan_lpt_reg<1>, n_lj, 32, 0, lj, ctx->d_status);
-        else if (ne <= 2)
-            CR_LAUNCH(ctx, k_plan_lpt_reg<2>, n_lj, 32, 0, lj, ctx->d_status);
-        else if (ne <= 4)
-            CR_LAUNCH(ctx, k_plan_lpt_reg<4>, n_lj, 32, 0, lj, ctx->d_status);
-        else if (ne <= 8)
-            CR_LAUNCH(ctx, k_plan_lpt_reg<8>, n_lj, 32, 0, lj, ctx->d_status);
-        else if (ne <= 16)
-            CR_LAUNCH(ctx, k_plan_lpt_reg<16>, n_lj, 32, 0, lj, ctx->d_status);
-        else
-            CR_LAUNCH(ctx, k_plan_lpt_reg<32>, n_lj, 32, 0, lj, ctx->d_status);
-        if (!tables_later)
-            for (uint32_t x = 0; x < n_lj; ++x) CR_TRY(table_insert(deferred[x]));
-        n_lj = 0;
-        lj_maxR = 0;
+    auto flush_l32 = [&]() -> int {
+        if (!n32) return CR_OK;
+        CR_LAUNCH(ctx, k_plan_lpt32_multi, n32, 32, 0, l32, ctx->d_status);
+        n32 = 0;
+        return CR_OK;
+    };
+    auto place = [&](uint32_t j) -> int {
+        cr_plan *p = plans[j];
+        const cr_plan_params &pp = params[j];
+        const uint64_t C = (uint64_t)pp.R * pp.W;
+        place_job J;
+        J.info = p->d_info;
+        J.adm_cnt = p->d_adm_cnt;
+        J.adm_k = p->d_adm_k;
+        J.koff = p->d_koff;
+        J.load = p->d_load;
+        J.jobs = p->d_jobs;
+        J.members = p->d_members;
+        J.seed = pp.seed;
+        J.epoch = pp.epoch;
+        J.R = pp.R;
+        if (pp.variant == CR_VARIANT_SLOTCAP) {
+            const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + sizeof(uint32_t) + 1) + 16;
+            if (smem > 48 * 1024)
+                CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt_capped, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem));
+            CR_LAUNCH(ctx, k_plan_lpt_capped, 1, 32, smem, p->d_info, (const unsigned long long *)p->d_adm_cnt,
+                      p->d_adm_k, p->d_koff, pp.R, pp.W, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
+        } else if (pp.variant == CR_VARIANT_RANDOM) {
+            rj.j[n_rj++] = J;
+            rj_maxR = std::max(rj_maxR, pp.R);
+            rj_adm = std::max(rj_adm, n < C ? n : C);
+        } else if (pp.R <= 32 && C < kLptRunsFrom) {
+            l32.j[n32++] = J;
+            if (n32 == 16) CR_TRY(flush_l32());
+        } else if (pp.R <= kPlaceMaxR) {
+            lj.j[n_lj++] = J;
+            lj_maxR = std::max(lj_maxR, pp.R);
+        } else {
+            const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + 1) + 16;
+            if (smem > 48 * 1024)
+                CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem));
+            CR_LAUNCH(ctx, k_plan_lpt, 1, 32, smem, (const cr_plan_info_dev *)p->d_info,
+                      (const unsigned long long *)p->d_adm_cnt, (const uint32_t *)p->d_adm_k,
+                      (const uint32_t *)p->d_koff, pp.R, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
+        }
+        if (n_lj + n_rj == 16) CR_TRY(flush_place());
+        return CR_OK;
+    };
+    auto finish = [&]() -> int {  // the collected placements, then the tables of every plan
+        CR_TRY(flush_place());
+        CR_TRY(flush_l32());
+        for (uint32_t j0 = 0; j0 < n_plans; j0 += 16) {
+            table_jobs tj;
+            const uint32_t nj = n_plans - j0 < 16 ? n_plans - j0 : 16;
+            uint64_t adm = 0;
+            for (uint32_t x = 0; x < nj; ++x) {
+                cr_plan *p = plans[j0 + x];
+                const uint64_t C = (uint64_t)params[j0 + x].R * params[j0 + x].W;
+                adm = std::max(adm, n < C ? n : C);
+                table_job &T = tj.j[x];
+                T.info = p->d_info;
+                T.adm_key = p->d_adm_key;
+                T.adm_k = p->d_adm_k;
+                T.koff = p->d_koff;
+                T.members = p->d_members;
+                T.table = p->d_table;
+                T.bits = bits_for(p->table_slots - 1);
+            }
+            CR_LAUNCH(ctx, k_table_insert_multi, dim3(cr_blocks(adm, 256, gcap), nj), 256, 0, tj);
+        }
         return CR_OK;
     };
     // small intervals: admission of every plan in one launch, one CTA per plan
@@ -1669,106 +1887,8 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
                       (const unsigned long long *)p0->d_ukey, (const unsigned long long *)p0->d_ucnt,
                       (unsigned long long)n, ctx->d_status);
         }
-        // placements: random and single-warp LPT plans batched per launch
-        place_jobs rj, l32;
-        uint32_t nr = 0, n32 = 0, rmaxR = 0;
-        uint64_t radm = 0;
-        auto flush_random = [&]() -> int {
-            if (!nr) return CR_OK;
-            const size_t smem = (size_t)kRandWarps * (rmaxR + 1) * 3 * sizeof(uint16_t);
-            if (smem > 48 * 1024)
-                CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_random_multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem));
-            CR_LAUNCH(ctx, k_plan_random_multi, dim3(cr_blocks(radm, kRandWarps * 32, gcap), nr), kRandWarps * 32, smem,
-                      rj, ctx->d_status);
-            nr = 0;
-            rmaxR = 0;
-            radm = 0;
-            return CR_OK;
-        };
-        auto flush_l32 = [&]() -> int {
-            if (!n32) return CR_OK;
-            CR_LAUNCH(ctx, k_plan_lpt32_multi, n32, 32, 0, l32, ctx->d_status);
-            n32 = 0;
-            return CR_OK;
-        };
-        for (uint32_t j = 0; j < n_plans; ++j) {
-            cr_plan *p = plans[j];
-            const cr_plan_params &pp = params[j];
-            const uint64_t C = (uint64_t)pp.R * pp.W;
-            place_job J;
-            J.info = p->d_info;
-            J.adm_cnt = p->d_adm_cnt;
-            J.adm_k = p->d_adm_k;
-            J.koff = p->d_koff;
-            J.load = p->d_load;
-            J.jobs = p->d_jobs;
-            J.members = p->d_members;
-            J.seed = pp.seed;
-            J.epoch = pp.epoch;
-            J.R = pp.R;
-            if (pp.variant == CR_VARIANT_SLOTCAP) {
-                const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + sizeof(uint32_t) + 1) + 16;
-                if (smem > 48 * 1024)
-                    CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt_capped, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)smem));
-                CR_LAUNCH(ctx, k_plan_lpt_capped, 1, 32, smem, p->d_info, (const unsigned long long *)p->d_adm_cnt,
-                          p->d_adm_k, p->d_koff, pp.R, pp.W, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
-            } else if (pp.variant == CR_VARIANT_RANDOM) {
-                rj.j[nr++] = J;
-                rmaxR = pp.R > rmaxR ? pp.R : rmaxR;
-                radm = (n < C ? n : C) > radm ? (n < C ? n : C) : radm;
-                if (nr == 16) CR_TRY(flush_random());
-            } else if (pp.R <= 32 && C < kLptRunsFrom) {
-                l32.j[n32++] = J;
-                if (n32 == 16) CR_TRY(flush_l32());
-            } else if (pp.R <= 1024) {
-                lpt_job &jb = lj.j[n_lj++];
-                jb.info = p->d_info;
-                jb.adm_cnt = p->d_adm_cnt;
-                jb.adm_k = p->d_adm_k;
-                jb.koff = p->d_koff;
-                jb.load = p->d_load;
-                jb.members = p->d_members;
-                jb.jobs = p->d_jobs;
-                jb.R = pp.R;
-                lj_maxR = pp.R > lj_maxR ? pp.R : lj_maxR;
-                deferred[n_lj - 1] = j;
-                if (n_lj == 16) CR_TRY(flush_lpt());
-            } else {
-                const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + 1) + 16;
-                if (smem > 48 * 1024)
-                    CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)smem));
-                CR_LAUNCH(ctx, k_plan_lpt, 1, 32, smem, (const cr_plan_info_dev *)p->d_info,
-                          (const unsigned long long *)p->d_adm_cnt, (const uint32_t *)p->d_adm_k,
-                          (const uint32_t *)p->d_koff, pp.R, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
-            }
-        }
-        CR_TRY(flush_random());
-        CR_TRY(flush_l32());
-        CR_TRY(flush_lpt());
-        // tables of every plan, batched per launch
-        for (uint32_t j0 = 0; j0 < n_plans; j0 += 16) {
-            table_jobs tj;
-            const uint32_t nj = n_plans - j0 < 16 ? n_plans - j0 : 16;
-            uint64_t adm = 0;
-            for (uint32_t x = 0; x < nj; ++x) {
-                cr_plan *p = plans[j0 + x];
-                const uint64_t C = (uint64_t)params[j0 + x].R * params[j0 + x].W;
-                adm = (n < C ? n : C) > adm ? (n < C ? n : C) : adm;
-                table_job &T = tj.j[x];
-                T.info = p->d_info;
-                T.adm_key = p->d_adm_key;
-                T.adm_k = p->d_adm_k;
-                T.koff = p->d_koff;
-                T.members = p->d_members;
-                T.table = p->d_table;
-                T.bits = bits_for(p->table_slots - 1);
-            }
-            CR_LAUNCH(ctx, k_table_insert_multi, dim3(cr_blocks(adm, 256, gcap), nj), 256, 0, tj);
-        }
-        return CR_OK;
+        for (uint32_t j = 0; j < n_plans; ++j) CR_TRY(place(j));
+        return finish();
     }
     // large intervals (and empty ones): plan by plan.  Eq. 1 and the admission depend only
     // on (R, W, q_cap, single copy or not): a plan equal in those to an earlier one of the
@@ -1824,58 +1944,9 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         }
         CR_LAUNCH(ctx, k_plan_init_load, cr_blocks(pp.R, 256, gcap), 256, 0, p->d_info,
                   (const unsigned long long *)pp.d_init_load, pp.R, p->d_load, ctx->d_status);
-        if (n > 0) {
-            if (pp.variant == CR_VARIANT_SLOTCAP) {
-                const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + sizeof(uint32_t) + 1) + 16;
-                if (smem > 48 * 1024)
-                    CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt_capped, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)smem));
-                CR_LAUNCH(ctx, k_plan_lpt_capped, 1, 32, smem, p->d_info, (const unsigned long long *)p->d_adm_cnt,
-                          p->d_adm_k, p->d_koff, pp.R, pp.W, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
-            } else if (pp.variant == CR_VARIANT_RANDOM) {
-                size_t smem = (size_t)kRandWarps * (pp.R + 1) * 3 * sizeof(uint16_t);
-                if (smem > 48 * 1024)
-                    CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_random, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)smem));
-                uint64_t adm = n < C ? n : C;
-                CR_LAUNCH(ctx, k_plan_random, cr_blocks(adm, kRandWarps * 32, gcap), kRandWarps * 32, smem,
-                          (const cr_plan_info_dev *)p->d_info, (const unsigned long long *)p->d_adm_cnt,
-                          (const uint32_t *)p->d_adm_k, (const uint32_t *)p->d_koff, pp.R,
-                          (unsigned long long)pp.seed, (unsigned long long)pp.epoch, p->d_load, p->d_members,
-                          p->d_jobs, ctx->d_status);
-            } else {
-                size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + 1) + 16;
-                if (smem > 48 * 1024)
-                    CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)smem));
-                if (pp.R <= 32 && C < kLptRunsFrom)
-                    CR_LAUNCH(ctx, k_plan_lpt32, 1, 32, 0, (const cr_plan_info_dev *)p->d_info,
-                              (const unsigned long long *)p->d_adm_cnt, (const uint32_t *)p->d_adm_k,
-                              (const uint32_t *)p->d_koff, pp.R, p->d_load, p->d_members, p->d_jobs,
-                              ctx->d_status);
-                else if (pp.R <= 1024) {
-                    lpt_job &jb = lj.j[n_lj++];
-                    jb.info = p->d_info;
-                    jb.adm_cnt = p->d_adm_cnt;
-                    jb.adm_k = p->d_adm_k;
-                    jb.koff = p->d_koff;
-                    jb.load = p->d_load;
-                    jb.members = p->d_members;
-                    jb.jobs = p->d_jobs;
-                    jb.R = pp.R;
-                    lj_maxR = pp.R > lj_maxR ? pp.R : lj_maxR;
-                    deferred[n_lj - 1] = j;
-                    if (n_lj == 16) CR_TRY(flush_lpt());
-                    continue;
-                } else
-                CR_LAUNCH(ctx, k_plan_lpt, 1, 32, smem, (const cr_plan_info_dev *)p->d_info,
-                          (const unsigned long long *)p->d_adm_cnt, (const uint32_t *)p->d_adm_k,
-                          (const uint32_t *)p->d_koff, pp.R, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
-            }
-            CR_TRY(table_insert(j));
-        }
+        if (n > 0) CR_TRY(place(j));
     }
-    return flush_lpt();
+    return n > 0 ? finish() : CR_OK;
 }
 
 extern "C" int cr_build_plan(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_plan_params *params,

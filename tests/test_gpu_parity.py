@@ -228,6 +228,37 @@ def test_plan_hand_example_and_init_load(P, ctx):
     _cmp_plan(pl2.export(), O.build_plan(keys, 3, 2, 1000, 1, init_load=init))
 
 
+@pytest.mark.parametrize("R", [1, 33, 1023, 1024])
+@pytest.mark.parametrize("spread", [0, 3000, 2**23, 2**33])
+def test_plan_lpt_runs_at_digit_edges(P, ctx, R, spread):
+    # runs of equal counts on both sides of the run sort's digit (64, 4096) and of the shortest
+    # run (31, 32, 33 keys), from even, uneven (32-bit packed loads) and wide starting loads
+    # (64-bit packed loads; above 2^31 no run is placed at once)
+    rng = np.random.default_rng(R + spread % 97)
+    runs = [(4097, 33), (4096, 32), (4095, 31), (65, 40), (64, 700), (63, 33), (2, 1500), (1, 3000)]
+    ids = rng.integers(1, 2**63, sum(m for _, m in runs), dtype=np.int64).astype(np.uint64)
+    keys = np.repeat(ids, np.repeat([q for q, _ in runs], [m for _, m in runs]))
+    rng.shuffle(keys)
+    init = rng.integers(0, spread + 1, R).astype(np.uint64)
+    W = max(1, 5000 // R)
+    pl = P.build_plan(ctx, d_u64(keys), P.plan_params(R, W, keys.size, 1, init_load=d_u64(init)))
+    _cmp_plan(pl.export(), O.build_plan(keys, R, W, keys.size, 1, init_load=init))
+
+
+@pytest.mark.parametrize("variants", [["RANDOM"] * 17, ["LPT", "RANDOM", "NOREPL", "SLOTCAP"] * 5])
+def test_plan_placements_in_one_launch(P, ctx, variants):
+    # more plans than one placement launch takes, of mixed kinds and fleet sizes (the LPT of
+    # R > 1024 and short LPT lists have launches of their own), replicated keys dealt to warps
+    rng = np.random.default_rng(len(variants))
+    keys = _rates_keys(rng, 3000, 60000)
+    Rs = [(1 + 37 * j) % 300 + 2 if j != 4 else 1500 for j in range(len(variants))]
+    params = [P.plan_params(R, 8, 300, 1, v, seed=j, epoch=3) for j, (R, v) in enumerate(zip(Rs, variants))]
+    plans = [P.Plan(ctx) for _ in variants]
+    P.build_plans(ctx, d_u64(keys), params, plans)
+    for j, (R, v) in enumerate(zip(Rs, variants)):
+        _cmp_plan(plans[j].export(), O.build_plan(keys, R, 8, 300, 1, variant=v, seed=j, epoch=3))
+
+
 @pytest.mark.parametrize("extra", [[2**64 - 1], [0], [2**64 - 1, 0, 2**64 - 1, 2**64 - 2]])
 def test_plan_extreme_keys(P, ctx, extra):
     # the all-ones key doubles as the device table's empty marker and is counted apart
