@@ -259,6 +259,24 @@ def test_plan_placements_in_one_launch(P, ctx, variants):
         _cmp_plan(plans[j].export(), O.build_plan(keys, R, 8, 300, 1, variant=v, seed=j, epoch=3))
 
 
+@pytest.mark.parametrize("U,C", [(63, 1000), (65, 3), (4095, 10**5), (4096, 50), (4097, 4000), (4097, 10**5),
+                                 (9000, 4096), (9000, 4097), (9000, 6000)])
+def test_plan_order_at_sort_edges(P, ctx, U, C):
+    # distinct keys and admission candidates on both sides of the shared-memory sort's size, with
+    # many equal counts (ties broken by key) and keys that differ only in their low or high bits
+    rng = np.random.default_rng(U + C)
+    ids = np.unique(np.concatenate([np.arange(U // 3, dtype=np.uint64), np.arange(U // 3, dtype=np.uint64) << np.uint64(50),
+                                    rng.integers(1, 2**63, U, dtype=np.int64).astype(np.uint64)]))
+    ids = rng.permutation(ids)[:U]
+    keys = np.repeat(ids, rng.integers(1, 6, U))
+    rng.shuffle(keys)
+    pl = P.build_plan(ctx, d_u64(keys), P.plan_params(1, C, keys.size, 1))
+    got = pl.export()
+    uk, uc = O.histogram(keys)
+    assert (got["ukey"] == uk).all() and (got["ucnt"] == uc).all()
+    _cmp_plan(got, O.build_plan(keys, 1, C, keys.size, 1))
+
+
 @pytest.mark.parametrize("extra", [[2**64 - 1], [0], [2**64 - 1, 0, 2**64 - 1, 2**64 - 2]])
 def test_plan_extreme_keys(P, ctx, extra):
     # the all-ones key doubles as the device table's empty marker and is counted apart
