@@ -5,9 +5,10 @@
 // words over lanes gives the same result.  One warp hashes one request: lanes
 // stride over the span with 16-byte streaming loads (four tokens = two words
 // per load, up to eight loads in flight per lane: the next group of four is
-// fetched while the current one is mixed), then the warp reduces its partial
-// sums; the next request's span descriptor is fetched a request ahead.  The path is an HBM stream of 4*P bytes per request; the per-word mix
-// (about two dozen integer instructions) keeps the ALU just under that stream
+// fetched while the current one is mixed; words that straddle two vectors take
+// their first token from the neighbouring lane), then the warp reduces its partial
+// sums; the next request's span descriptor is fetched a request ahead.  The path is an HBM stream of 4*P bytes per request; the
+// per-word mix (about two dozen integer instructions) keeps the ALU just under that stream
 // rate on sm_103a.
 #include "cr_device.cuh"
 #include "cr_internal.cuh"
@@ -22,35 +23,99 @@ __device__ __forceinline__ unsigned long long word_term(uint32_t lo, uint32_t hi
     return cr_fmix64(w ^ k);
 }
 
-// Words [first, nw) of a span starting at `base`, one per lane, scalar loads;
-// used for unaligned spans and for the last words of aligned ones.
-__device__ __forceinline__ unsigned long long scalar_words(const int32_t *__restrict__ base, uint32_t P,
-                                                           uint32_t first, uint32_t nw,
-                                                           unsigned long long salt, uint32_t lane)
+// Word i of a span (tokens 2i, 2i + 1; past the end reads as 0) by scalar loads, mixed.
+__device__ __forceinline__ unsigned long long scalar_word(const int32_t *__restrict__ base, uint32_t P, uint32_t i,
+                                                          unsigned long long salt)
 {
-    unsigned long long acc = 0;
-    for (uint32_t i = first + lane; i < nw; i += 32) {
-        uint32_t lo = (uint32_t)__ldcs(base + 2 * i);
-        uint32_t hi = (2 * i + 1 < P) ? (uint32_t)__ldcs(base + 2 * i + 1) : 0u;
-        acc += word_term(lo, hi, salt + (unsigned long long)(i + 1) * CR_GAMMA);
-    }
-    return acc;
+    const uint32_t lo = (uint32_t)__ldcs(base + 2 * i);
+    const uint32_t hi = (2 * i + 1 < P) ? (uint32_t)__ldcs(base + 2 * i + 1) : 0u;
+    return word_term(lo, hi, salt + (unsigned long long)(i + 1) * CR_GAMMA);
 }
 
-__device__ __forceinline__ void load4(int4 (&x)[4], const int4 *__restrict__ b4, uint32_t v, uint32_t nvec)
+// Four rows of 32 aligned 16-byte vectors, one per lane; vectors from v1 on are not read.
+template <bool FULL>
+__device__ __forceinline__ void load4(int4 (&x)[4], const int4 *__restrict__ b4, uint32_t v, uint32_t v1)
 {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const uint32_t i = v + 32u * q;
-        if (i < nvec)
+        if (FULL || i < v1)
             x[q] = __ldcs(b4 + i);
         else
             x[q] = make_int4(0, 0, 0, 0);
     }
 }
 
+// Mix one group.  k: key of the word whose tokens are (x, y) of this lane's first vector when
+// the span starts on an even token of its vector, or (y, z) when it starts on an odd one.
+// An odd start puts every second word across two vectors: (w of the vector before, x); the
+// vector before is the previous lane's, or the previous row's last (`carry`, lane 0 only).
+// Vectors in [v, v1) count; `head` marks the lane and row whose straddling word lies outside.
+template <bool ODD, bool FULL>
+__device__ __forceinline__ unsigned long long mix4(const int4 (&x)[4], unsigned long long k, uint32_t v, uint32_t v1,
+                                                   uint32_t lane, bool head, uint32_t &carry)
+{
+    const unsigned long long G64 = 64ull * CR_GAMMA;
+    unsigned long long acc = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const unsigned long long kq = k + (unsigned long long)q * G64;
+        const bool in = FULL || v + 32u * q < v1;
+        if (!ODD) {
+            if (in) acc += word_term(x[q].x, x[q].y, kq) + word_term(x[q].z, x[q].w, kq + CR_GAMMA);
+        } else {
+            const uint32_t r = __shfl_sync(0xffffffffu, (uint32_t)x[q].w, (lane + 31u) & 31u);
+            const uint32_t before = lane ? r : carry;
+            carry = r;  // lane 0: this row's last w
+            if (in) {
+                acc += word_term(x[q].y, x[q].z, kq);
+                if (q > 0 || !head) acc += word_term(before, x[q].x, kq - CR_GAMMA);
+            }
+        }
+    }
+    return acc;
+}
+
+// The words of a span that lie inside its aligned vectors [v0, v1), two groups in flight: the next
+// group loads while the current one is mixed.
+template <bool ODD>
+__device__ __forceinline__ unsigned long long vector_words(const int4 *__restrict__ b4, uint32_t v0, uint32_t v1,
+                                                           unsigned long long k, uint32_t lane)
+{
+    const unsigned long long G256 = 256ull * CR_GAMMA;
+    unsigned long long acc = 0;
+    uint32_t carry = 0;
+    int4 cur[4];
+    uint32_t vb = v0;  // first vector of the group (uniform over the warp)
+    const uint32_t groups = (v1 - v0) >> 7;
+    if (groups)
+        load4<true>(cur, b4, vb + lane, v1);
+    else
+        load4<false>(cur, b4, vb + lane, v1);
+    for (uint32_t g = 0; g < groups; ++g) {
+        int4 nxt[4];
+        if (g + 1 < groups)
+            load4<true>(nxt, b4, vb + 128u + lane, v1);
+        else
+            load4<false>(nxt, b4, vb + 128u + lane, v1);
+        acc += mix4<ODD, true>(cur, k, vb + lane, v1, lane, g == 0 && lane == 0, carry);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cur[q] = nxt[q];
+        vb += 128u;
+        k += G256;
+    }
+    if (vb < v1) acc += mix4<ODD, false>(cur, k, vb + lane, v1, lane, groups == 0 && lane == 0, carry);
+    return acc;
+}
+
 // 64 registers per thread: 32 warps per SM, which measured faster than larger
 // unrolls at lower occupancy.
+// A span may start on any token of a 16-byte vector (sh = start address / 4 mod 4): the
+// aligned vectors that lie inside it are read whole, and the words at its ends that they
+// do not hold (at most two before, three after) one per lane with scalar loads, so nothing
+// outside the span is read.  5,000 spans of 1,024-4,096 tokens packed back to back (any start):
+// 28.6 -> 18.4 us against 4- and 8-byte loads; aligned spans (166,667 of ~2,300 tokens) 286 us
+// either way.
 __global__ void __launch_bounds__(kHashBlock, 4)
 k_hash_prefixes(const int32_t *__restrict__ tok, const unsigned long long *__restrict__ off,
                 const uint32_t *__restrict__ plen, unsigned long long n, unsigned long long salt,
@@ -58,7 +123,6 @@ k_hash_prefixes(const int32_t *__restrict__ tok, const unsigned long long *__res
 {
     const uint32_t lane = cr_lane();
     const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-    const unsigned long long G64 = 64ull * CR_GAMMA, G256 = 256ull * CR_GAMMA;
     unsigned long long r = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     unsigned long long o_next = 0;
     uint32_t P_next = 0;
@@ -73,54 +137,31 @@ k_hash_prefixes(const int32_t *__restrict__ tok, const unsigned long long *__res
             o_next = off[r + nwarps];
             P_next = plen[r + nwarps];
         }
-        const uint32_t nw = (P + 1) >> 1;
+        const uint32_t nw = P / 2u + (P & 1u);
         const int32_t *base = tok + o;
         unsigned long long acc = 0;
-        if ((o & 3ull) == 0) {
-            // 16-byte aligned: vector v holds words 2v and 2v+1.  Two groups of
-            // four vectors per lane are in flight: the next group loads while
-            // the current one is mixed.
-            const uint32_t nvec = P >> 2;
-            const int4 *b4 = reinterpret_cast<const int4 *>(base);
-            uint32_t v = lane;
-            unsigned long long k = salt + (unsigned long long)(2 * lane + 1) * CR_GAMMA;  // key of word 2v
-            int4 cur[4];
-            load4(cur, b4, v, nvec);
-            while (v < nvec) {
-                int4 nxt[4];
-                load4(nxt, b4, v + 128u, nvec);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (v + 32u * q < nvec) {
-                        const unsigned long long kq = k + (unsigned long long)q * G64;
-                        acc += word_term(cur[q].x, cur[q].y, kq) + word_term(cur[q].z, cur[q].w, kq + CR_GAMMA);
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) cur[q] = nxt[q];
-                v += 128u;
-                k += G256;
+        // vector v holds tokens 4v - sh .. 4v - sh + 3 of the span; [v0, v1) lie inside it
+        const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(base) >> 2) & 3u;
+        const uint32_t v0 = sh ? 1u : 0u, v1 = (uint32_t)(((unsigned long long)P + sh) >> 2);
+        uint32_t head = nw, tail = nw;  // words [0, head) and [tail, nw) are left to the scalar loads
+        if (v1 > v0) {
+            const int4 *b4 = reinterpret_cast<const int4 *>(base - (int)sh);
+            const uint32_t w0 = 2u * v0 - (sh >> 1);  // first word that vector v0 holds whole
+            // key of this lane's first word: word 2 (v0 + lane) - sh / 2
+            const unsigned long long k = salt + (unsigned long long)(w0 + 2u * lane + 1u) * CR_GAMMA;
+            head = w0;
+            if (sh & 1u) {
+                acc = vector_words<true>(b4, v0, v1, k, lane);
+                tail = 2u * (v1 - 1u) - (sh >> 1) + 1u;
+            } else {
+                acc = vector_words<false>(b4, v0, v1, k, lane);
+                tail = 2u * v1 - (sh >> 1);
             }
-            acc += scalar_words(base, P, 2 * nvec, nw, salt, lane);
-        } else if ((o & 1ull) == 0) {
-            // 8-byte aligned: one word per load
-            const uint32_t nfull = P >> 1;
-            const uint2 *b2 = reinterpret_cast<const uint2 *>(base);
-            uint32_t i = lane;
-            unsigned long long k = salt + (unsigned long long)(lane + 1) * CR_GAMMA;
-            const unsigned long long G32 = 32ull * CR_GAMMA;
-            for (; i + 32 < nfull; i += 64, k += G64) {
-                uint2 a = __ldcs(b2 + i), b = __ldcs(b2 + i + 32);
-                acc += word_term(a.x, a.y, k) + word_term(b.x, b.y, k + G32);
-            }
-            for (; i < nfull; i += 32, k += G32) {
-                uint2 a = __ldcs(b2 + i);
-                acc += word_term(a.x, a.y, k);
-            }
-            acc += scalar_words(base, P, nfull, nw, salt, lane);
-        } else {
-            acc = scalar_words(base, P, 0, nw, salt, lane);
         }
+        // the words left: lanes 0 .. head-1, then the tail's
+        const uint32_t rest = head + (nw - tail);
+        for (uint32_t i = lane; i < rest; i += 32)
+            acc += scalar_word(base, P, i < head ? i : tail + (i - head), salt);
         acc = cr_warp_sum_u64(acc);
         if (lane == 0) out[r] = cr_fmix64(salt ^ (unsigned long long)P) + acc;
     }

@@ -87,6 +87,28 @@ def test_hash_edge_lengths_and_offsets(P, ctx):
     assert (h_u64(got) == ref).all()
 
 
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_hash_every_start_and_remainder(P, ctx, shift):
+    # every start within a 16-byte vector (the arena itself starting `shift` tokens into one) with
+    # lengths around none, one and several groups of 128 vectors, and every remainder
+    plens = np.concatenate([np.arange(0, 24), np.arange(508, 528), np.arange(1020, 1040), np.arange(4090, 4104)])
+    plens = np.repeat(plens, 4).astype(np.uint32)
+    starts = np.tile(np.arange(4), plens.size // 4)
+    pos, offs = 0, []
+    for s, p in zip(starts, plens):  # each span at its start within a vector, right after the last
+        pos = (pos + 3) // 4 * 4 + int(s)
+        offs.append(pos)
+        pos += int(p)
+    offs = np.array(offs, np.uint64)
+    tok = np.random.default_rng(shift).integers(-2**31, 2**31, pos + 1, dtype=np.int64).astype(np.int32)
+    ref = O.hash_prefixes(tok, offs, plens, salt=99)
+    dev = torch.zeros(tok.size + 3, dtype=torch.int32, device=DEV)[shift:shift + tok.size]
+    dev.copy_(torch.from_numpy(tok))
+    got = P.hash_prefixes(ctx, dev, d_u64(offs), d_u32(plens), salt=99)
+    ctx.sync()
+    assert (h_u64(got) == ref).all()
+
+
 def test_hash_empty(P, ctx):
     t = torch.zeros(4, dtype=torch.int32, device=DEV)
     out = P.hash_prefixes(ctx, t, torch.zeros(0, dtype=torch.int64, device=DEV),
