@@ -4,10 +4,10 @@
 //              (replica, destination) stream's request indices in arrival
 //              order; the replay gathers each request's (key, prefix, suffix)
 //              record, packed once per call, through them
-//   replay     one warp per (stream, chunk); the stream's LRU at the LARGEST
-//              capacity lives in shared memory as keys with recency stamps, a
-//              bitmap of live stamps and a hash index, and 32 requests are
-//              simulated per step, one per lane.  A request's depth (its LRU stack distance) decides the
+//   replay     one warp per (stream, chunk); the stream's recent keys live in
+//              shared memory by access time, with a bitmap of last accesses and a
+//              hash index from key to time, and 32 requests are simulated per
+//              step, one per lane.  A request's depth (its LRU stack distance) decides the
 //              hit at every smaller capacity at once, because LRU caches are
 //              nested (Mattson et al. 1970): the cache of capacity c is the c
 //              most recent entries of any larger one.
@@ -288,19 +288,30 @@ struct replay_state {
     uint32_t *fill_out;
 };
 
-// ---- replay: batched stack distances over recency stamps -----------------------
-// One warp per (stream, chunk) holds the LRU of the LARGEST capacity in shared
-// memory.  Each resident key has a slot holding the key and its STAMP, the
-// time of its last access, and an entry in an open-addressing index
-// key -> slot.  Time advances by one 32-bit word per step of 32 requests (the
-// request on lane l of the step at word w has time 32 w + l), and a bitmap
-// over the times of a window marks the live stamps: bit t is set iff t is the
-// stamp of a resident key.  The recency position of a resident key (0 = most
-// recent) is the number of live bits above its stamp, which one warp-wide scan
-// of the words' popcounts gives for every lane of a step at once.  Nothing
-// moves when a key is accessed: its old bit is cleared and its bit in the new
-// word set.  When the window's words are used up, the stamps are renumbered
-// 0 .. fill-1 in recency order (compaction).
+// ---- replay: batched stack distances over access times -------------------------
+// One warp per (stream, chunk) holds the LRU stack in shared memory, indexed by
+// TIME.  Times 0 .. 32 nw - 1 form a window: the carried-in keys take the first
+// ones in recency order, then every step of 32 requests takes one 32-bit word of
+// times (the request on lane l of the step at word w has time 32 w + l).  KT holds
+// the key accessed at each time, a bitmap marks the times that are some key's
+// LAST access, and an index maps each key of the window to that time.  The recency
+// position of a key (0 = most recent) is the number of live bits above its time,
+// which one warp-wide scan of the words' popcounts gives for every lane of a step
+// at once.  An access clears the key's old bit, sets its bit in the new word and
+// writes the new time into its index entry; nothing else moves.  A key that falls
+// below the largest capacity is left where it is: its position is past every
+// capacity, so it counts as a miss, and it goes when the window is used up and the
+// cmax most recent keys are renumbered 0 .. fill-1 (compaction).
+//
+// Bound: the latency of a step's dependence chain (match, index probe, popcount scan,
+// insert) at the warps per SM that the window allows (14 at cmax 1024), 15.3 warp
+// instructions per (request, replica) pair.  Keys indexed by slot, with an eviction per
+// new key (search for the oldest live bits, index erase, slot hand-over), took 16.6 and a
+// chain about a third longer: 48 replicas x 1,066,667 requests over 1,024 destinations
+// at capacities 64 / 256 / 1024, partition included, 2.78 -> 2.23 ms; 30 replicas x
+// 133,333 over 64 destinations at capacity 128, 270 -> 237 us.  Indexing only the
+// requests' keys and streaming the carried-in ones past them fits 24 warps, but costs 18
+// instructions per pair and measured 2.88 ms.
 //
 // A step is 32 consecutive requests of the stream, one per lane.  The depth of
 // request i (its LRU stack distance, Mattson et al. 1970) follows from the
@@ -311,222 +322,151 @@ struct replay_state {
 //     number of distinct keys among lanes < i that were deeper than d0 or
 //     absent;
 //   - absent before the step: a miss at every capacity.
-// A request hits capacity c iff its depth <= c.  The state after the step is
-// the step's distinct keys by last access, then the untouched old keys in
-// their old order, cut at cmax: when the step brings m new keys and the cache
-// would exceed cmax, the oldest untouched keys (the lowest live bits) leave
-// and the new keys take their slots.
+// A request hits capacity c iff its depth <= c.
 constexpr uint32_t kNone = 0xffffffffu;
-constexpr uint32_t kAbsent = 2047u;    // depth code of a key not resident (above every position < 1024)
-
 constexpr uint32_t kStash = 32;              // index entries that found both buckets full
-constexpr uint32_t kDegraded = 0x80000000u;  // stash overflowed: lookups scan the keys
-constexpr uint16_t kInStash = 0xffffu;       // TS of a slot whose entry is in the stash
+constexpr uint32_t kDegraded = 0x80000000u;  // stash overflowed: lookups scan the window
 
-struct stamp_lru {
-    unsigned long long *K;    // [cmax] key of each slot
-    uint32_t *BM;             // [nw] live-stamp bits, word w = times 32 w .. 32 w + 31
+// Index: buckets of four 16-bit entries (tag above, time in the low `tb` bits; 0 =
+// empty, so a tag is never 0), two candidate buckets per key.  A new key goes into
+// the emptier one (the first when equal); a key whose buckets are both full goes to
+// a small stash; if even the stash is full the index is marked degraded and lookups
+// scan the window.  An entry stays where it is until the next compaction.
+struct window_lru {
+    unsigned long long *KT;   // [32 nw] key accessed at each time
+    unsigned long long *bkt;  // [nb] index buckets
+    uint16_t *E;              // the buckets as entries [4 nb], then the stash [kStash]
+    uint32_t *BM;             // [nw] bit t of word w: time 32 w + t is a key's last access
     uint32_t *stash_n;        // stash entries claimed (| kDegraded once it overflowed)
-    unsigned long long *bkt;  // [2^nbb] index buckets of four 16-bit entries (0 = empty)
-    uint16_t *ST;             // [cmax] stamp of each slot
-    uint16_t *T2S;            // [32 nw] slot whose stamp is each time (where the bit is set)
-    uint16_t *EV;             // [32] slots the step's evictions freed
-    uint16_t *stash;          // [kStash] slot + 1 of keys indexed outside their buckets (0 = free)
-    uint16_t *TS;             // [cmax] where each slot's index entry is: bucket << 2 | entry, or kInStash
-    uint32_t nbb;             // log2 of the bucket count
+    uint16_t *PX;             // [nw] compaction: live bits below each word
+    uint32_t nw, nb, tmask;   // words, buckets, (1 << tb) - 1
 };
 
-// Per-warp layout: K at 0 (8-byte entries), BM and the stash count after it, the
-// buckets at the next 16-byte boundary (cleared with 16-byte stores), then ST,
-// T2S, EV and the stash.
-__host__ __device__ inline size_t stamp_bkt_offset(uint32_t cmax, uint32_t nw)
+__host__ __device__ inline size_t window_lru_bytes(uint32_t nw, uint32_t nb)
 {
-    return ((size_t)cmax * 8 + (size_t)(nw + 1) * 4 + 15) & ~(size_t)15;
+    return ((size_t)nw * 256 + (size_t)nb * 8 + kStash * 2 + (size_t)(nw + 1) * 4 + (size_t)nw * 2 + 15) & ~(size_t)15;
 }
 
-__host__ __device__ inline size_t stamp_lru_bytes(uint32_t cmax, uint32_t nw, uint32_t nbb)
+__device__ __forceinline__ window_lru window_lru_at(unsigned char *base, uint32_t nw, uint32_t nb)
 {
-    return (stamp_bkt_offset(cmax, nw) + ((size_t)8 << nbb) + (size_t)cmax * 4 + (size_t)nw * 64 + 64 +
-            (size_t)kStash * 2 + 15) &
-           ~(size_t)15;
-}
-
-__device__ __forceinline__ stamp_lru stamp_lru_at(unsigned char *base, uint32_t cmax, uint32_t nw, uint32_t nbb)
-{
-    stamp_lru X;
-    X.K = reinterpret_cast<unsigned long long *>(base);
-    X.BM = reinterpret_cast<uint32_t *>(base + (size_t)cmax * 8);
+    window_lru X;
+    X.KT = reinterpret_cast<unsigned long long *>(base);
+    X.bkt = X.KT + (size_t)nw * 32;
+    X.E = reinterpret_cast<uint16_t *>(X.bkt);
+    X.BM = reinterpret_cast<uint32_t *>(X.E + (size_t)nb * 4 + kStash);
     X.stash_n = X.BM + nw;
-    X.bkt = reinterpret_cast<unsigned long long *>(base + stamp_bkt_offset(cmax, nw));
-    X.ST = reinterpret_cast<uint16_t *>(X.bkt + (1u << nbb));
-    X.T2S = X.ST + cmax;
-    X.EV = X.T2S + (size_t)nw * 32;
-    X.stash = X.EV + 32;
-    X.TS = X.stash + kStash;
-    X.nbb = nbb;
+    X.PX = reinterpret_cast<uint16_t *>(X.stash_n + 1);
+    X.nw = nw;
+    X.nb = nb;
+    X.tmask = (1u << (32 - __clz(32u * nw - 1u))) - 1u;
     return X;
 }
 
-// Index: two candidate buckets of four 16-bit entries per key, each entry
-// (5-bit tag << 11) | (slot + 1).  A key goes into the emptier of its buckets
-// (the first when equal); a key whose buckets are both full goes to a small
-// stash (with at most a quarter of the entries live that is rare); if even the
-// stash is full the index is marked degraded and lookups scan every key.
-// Entries never move, so concurrent lanes only need compare-and-swap on the
-// 64-bit bucket words, and a deleted entry becomes empty (no tombstones).
-struct bkt_hash {
-    uint32_t b1, b2, tag;
+struct key_hash {
+    uint32_t b1, b2, tag;  // buckets; tag in place, i.e. above the time bits
 };
 
-__device__ __forceinline__ bkt_hash sl_hash(unsigned long long key, uint32_t nbb)
+__device__ __forceinline__ key_hash sl_hash(const window_lru &X, unsigned long long key)
 {
     const unsigned long long h = key * 0x9e3779b97f4a7c15ull;  // an odd multiplier spreads every key bit upwards
-    bkt_hash r;
-    r.b1 = (uint32_t)(h >> (64 - nbb));
-    r.b2 = (uint32_t)(h >> (64 - 2 * nbb)) & ((1u << nbb) - 1u);
-    r.tag = (uint32_t)(h >> (59 - 2 * nbb)) & 31u;
+    key_hash r;
+    r.b1 = __umulhi((uint32_t)(h >> 32), X.nb);
+    r.b2 = __umulhi((uint32_t)(h >> 22), X.nb);
+    r.tag = max((uint32_t)(h >> 28) & (0xffffu & ~X.tmask), X.tmask + 1u);
     return r;
 }
 
-__device__ __forceinline__ uint32_t bkt_entry(unsigned long long w, int p) { return (uint32_t)(w >> (16 * p)) & 0xffffu; }
-
-// Slot of `key`, or kNone (fill: resident keys, scanned only when the index is degraded).
-__device__ __forceinline__ uint32_t sl_lookup(const stamp_lru &X, unsigned long long key, uint32_t fill, uint32_t cmax)
+// Is `key` in the index?  `time` receives its last access, `loc` its entry (kNone when
+// a degraded index does not hold it).  The eight entries' tags are compared as
+// halfwords, four words at once; only tag matches read their key.
+__device__ __forceinline__ bool sl_lookup(const window_lru &X, const key_hash &H, unsigned long long key,
+                                          uint32_t wnow, uint32_t &time, uint32_t &loc)
 {
-    const bkt_hash H = sl_hash(key, X.nbb);
-    const unsigned long long w1 = X.bkt[H.b1], w2 = X.bkt[H.b2];
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-        const uint32_t e = bkt_entry(p < 4 ? w1 : w2, p & 3);
-        if (e != 0 && (e >> 11) == H.tag) {
-            const uint32_t q = (e & 0x7ffu) - 1u;
-            if (q < cmax && X.K[q] == key) return q;
+    const uint32_t T2 = H.tag * 0x10001u, lm = (0x7fffu & ~X.tmask) * 0x10001u;
+    auto match = [&](uint32_t x) {  // bit 15 / 31: that half's tag equals the key's
+        const uint32_t y = x ^ T2;
+        return ~(((y & lm) + lm) | y) & 0x80008000u;
+    };
+    const unsigned long long v1 = X.bkt[H.b1], v2 = X.bkt[H.b2];
+    // bits 12 .. 15: low halves of words 0 .. 3, bits 28 .. 31: their high halves
+    uint32_t M = (match((uint32_t)v1) >> 3) | (match((uint32_t)(v1 >> 32)) >> 2) | (match((uint32_t)v2) >> 1) |
+                 match((uint32_t)(v2 >> 32));
+    time = 0;
+    loc = kNone;
+    while (M) {
+        const uint32_t p = (uint32_t)__ffs(M) - 1u;
+        M &= M - 1u;
+        const uint32_t at = ((p & 2u) ? H.b2 : H.b1) * 4u + ((p & 1u) << 1) + (p >> 4);
+        const uint32_t t = X.E[at] & X.tmask;
+        if (X.KT[t] == key) {
+            time = t;
+            loc = at;
+            return true;
         }
     }
     const uint32_t sn = *X.stash_n;
     if (sn) {
-        if (sn & kDegraded) {
-            for (uint32_t q = 0; q < fill; ++q)
-                if (X.K[q] == key) return q;
-            return kNone;
+        for (uint32_t i = 0; i < (sn & ~kDegraded) && i < kStash; ++i) {
+            const uint32_t e = X.E[4u * X.nb + i];
+            if (e != 0 && X.KT[e & X.tmask] == key) {
+                time = e & X.tmask;
+                loc = 4u * X.nb + i;
+                return true;
+            }
         }
-        for (uint32_t i = 0; i < sn && i < kStash; ++i) {
-            const uint32_t e = X.stash[i];
-            if (e != 0 && e <= cmax && X.K[e - 1] == key) return e - 1;
-        }
+        if (sn & kDegraded)
+            for (uint32_t t = 0; t < 32u * wnow; ++t)
+                if (((X.BM[t >> 5] >> (t & 31u)) & 1u) && X.KT[t] == key) {
+                    time = t;
+                    return true;
+                }
     }
-    return kNone;
+    return false;
 }
 
-// Index an absent key held in slot q.  A lost compare-and-swap means another lane
-// changed the bucket, so the next look sees it; the bound only guards the loop.
-__device__ __forceinline__ void sl_insert(const stamp_lru &X, unsigned long long key, uint32_t q)
+// Index an absent key last accessed at `time`.  A lost compare-and-swap means another
+// lane changed the bucket, so the next look sees it; the bound only guards the loop.
+__device__ __forceinline__ void sl_insert(const window_lru &X, const key_hash &H, uint32_t time)
 {
-    const bkt_hash H = sl_hash(key, X.nbb);
-    const unsigned long long ent = (unsigned long long)((H.tag << 11) | (q + 1u));
+    const unsigned long long ent = H.tag | time;
+    auto empty = [](uint32_t x) { return ~(((x & 0x7fff7fffu) + 0x7fff7fffu) | x | 0x7fff7fffu); };
     for (int it = 0; it < 64; ++it) {
-        const unsigned long long w1 = X.bkt[H.b1], w2 = X.bkt[H.b2];
-        int f1 = -1, f2 = -1, n1 = 0, n2 = 0;
-#pragma unroll
-        for (int p = 3; p >= 0; --p) {
-            if (bkt_entry(w1, p) == 0) {
-                f1 = p;
-                ++n1;
-            }
-            if (bkt_entry(w2, p) == 0) {
-                f2 = p;
-                ++n2;
-            }
-        }
-        uint32_t b;
-        unsigned long long w;
-        int p;
-        if (f1 >= 0 && (n1 >= n2 || f2 < 0)) {
-            b = H.b1;
-            w = w1;
-            p = f1;
-        } else if (f2 >= 0) {
-            b = H.b2;
-            w = w2;
-            p = f2;
-        } else {
-            break;  // both buckets full
-        }
-        if (atomicCAS(&X.bkt[b], w, w | (ent << (16 * p))) == w) {
-            X.TS[q] = (uint16_t)((b << 2) | (uint32_t)p);
-            return;
-        }
+        const unsigned long long v1 = X.bkt[H.b1], v2 = X.bkt[H.b2];
+        // bits 14, 30, 15, 31: entries 0 .. 3 are empty
+        const uint32_t z1 = (empty((uint32_t)v1) >> 1) | empty((uint32_t)(v1 >> 32));
+        const uint32_t z2 = (empty((uint32_t)v2) >> 1) | empty((uint32_t)(v2 >> 32));
+        if (!(z1 | z2)) break;  // both buckets full
+        const bool one = __popc(z1) >= __popc(z2);
+        const uint32_t b = one ? H.b1 : H.b2, p = (uint32_t)__ffs(one ? z1 : z2) - 1u;
+        const unsigned long long v = one ? v1 : v2;
+        if (atomicCAS(&X.bkt[b], v, v | (ent << (((p & 1u) << 5) | (p & 16u)))) == v) return;
     }
-    X.TS[q] = kInStash;
-    const uint32_t i = atomicAdd(X.stash_n, 1u);
+    const uint32_t i = atomicAdd(X.stash_n, 1u) & ~kDegraded;
     if (i < kStash)
-        X.stash[i] = (uint16_t)(q + 1u);
+        X.E[4u * X.nb + i] = (uint16_t)ent;
     else
         atomicOr(X.stash_n, kDegraded);
 }
 
-// Remove the index entry of slot q: its place is recorded in TS[q].
-__device__ __forceinline__ void sl_erase(const stamp_lru &X, uint32_t q)
+// An empty index (warp-cooperative).
+__device__ __forceinline__ void sl_clear_index(const window_lru &X, uint32_t lane)
 {
-    const uint32_t loc = X.TS[q];
-    if (loc != kInStash) {
-        atomicAnd(&X.bkt[loc >> 2], ~(0xffffull << (16 * (loc & 3u))));
-        return;
-    }
-    const uint32_t sn = *X.stash_n & ~kDegraded;
-    for (uint32_t i = 0; i < sn && i < kStash; ++i)
-        if (X.stash[i] == q + 1u) {
-            X.stash[i] = 0;
-            return;
-        }
-}
-
-// Index of slots 0 .. fill-1 from scratch (warp-cooperative).
-__device__ __forceinline__ void sl_reindex(const stamp_lru &X, uint32_t fill, uint32_t lane)
-{
-    uint4 *t4 = reinterpret_cast<uint4 *>(X.bkt);
-    for (uint32_t x = lane; x < (1u << X.nbb) / 2; x += 32) t4[x] = make_uint4(0, 0, 0, 0);
+    for (uint32_t x = lane; x < X.nb; x += 32) X.bkt[x] = 0;
+    X.E[4u * X.nb + lane] = 0;
     if (lane == 0) *X.stash_n = 0;
     __syncwarp();
-    for (uint32_t q = lane; q < fill; q += 32) sl_insert(X, X.K[q], q);
-    __syncwarp();
 }
 
-// Stamps for keys K[0 .. fill) held in recency order (K[0] most recent): times
-// fill-1 .. 0, bits 0 .. fill-1 set, the next step at the first word above them.
-__device__ __forceinline__ void sl_stamps_in_order(const stamp_lru &X, uint32_t fill, uint32_t nw, uint32_t lane,
-                                                   uint32_t &wnow, uint32_t &lo)
+// Live times [a, a + fill); the next step takes the first word above them.
+__device__ __forceinline__ void sl_live_range(const window_lru &X, uint32_t a, uint32_t fill, uint32_t lane)
 {
-    for (uint32_t q = lane; q < fill; q += 32) {
-        const uint32_t t = fill - 1u - q;
-        X.ST[q] = (uint16_t)t;
-        X.T2S[t] = (uint16_t)q;
+    for (uint32_t w = lane; w < X.nw; w += 32) {
+        const uint32_t lo = max(32u * w, a), hi = min(32u * w + 32u, a + fill);
+        X.BM[w] = lo < hi ? (0xffffffffu >> (32u - (hi - lo))) << (lo & 31u) : 0u;
     }
-    for (uint32_t w = lane; w < nw; w += 32)
-        X.BM[w] = 32u * w + 32u <= fill ? 0xffffffffu : (32u * w < fill ? (1u << (fill - 32u * w)) - 1u : 0u);
-    wnow = (fill + 31u) / 32u;
-    lo = 0;
-    __syncwarp();
 }
 
-
-// Position of the k-th (from 0) set bit of w, which has more than k set bits.
-__device__ __forceinline__ uint32_t nth_set_bit(uint32_t w, uint32_t k)
-{
-    uint32_t pos = 0;
-#pragma unroll
-    for (int sh = 16; sh >= 1; sh >>= 1) {
-        const uint32_t lowc = (uint32_t)__popc(w & ((1u << sh) - 1u));
-        if (k >= lowc) {
-            k -= lowc;
-            w >>= sh;
-            pos += (uint32_t)sh;
-        }
-    }
-    return pos;
-}
-
-// Live stamps below any time of the window: lane l keeps word 32 g + l of every
+// Live times below any time of the window: lane l keeps word 32 g + l of every
 // group g of 32 words and the number of live bits in the words before it.
 template <int NG>
 struct live_prefix {
@@ -547,7 +487,7 @@ struct live_prefix {
         ex[0] = ex2 & 0xffffu;
         if (NG > 1) ex[NG - 1] = (ex2 >> 16) + (__shfl_sync(0xffffffffu, incl, 31) & 0xffffu);
     }
-    // live stamps < s; every lane of the warp must call it
+    // live times < s; every lane of the warp must call it
     __device__ __forceinline__ uint32_t below(uint32_t s) const
     {
         const uint32_t src = (s >> 5) & 31u, g = s >> 10;
@@ -564,40 +504,60 @@ struct live_prefix {
     }
 };
 
-// Renumber the stamps of slots 0 .. fill-1 to 0 .. fill-1 keeping their order.
+// Keep the `fill` most recent of the window's `live` keys, renumbered 0 .. fill-1 in
+// order: every index entry takes its new time (or is emptied), then the keys move down.
 template <int NG>
-__device__ __forceinline__ void sl_compact(const stamp_lru &X, uint32_t fill, uint32_t nw, uint32_t lane,
-                                           uint32_t &wnow, uint32_t &lo)
+__device__ __forceinline__ void sl_compact(const window_lru &X, uint32_t live, uint32_t fill, uint32_t lane)
 {
     live_prefix<NG> LP;
-    LP.load(X.BM, nw, lane);
-    for (uint32_t q0 = 0; q0 < fill; q0 += 32) {
-        const uint32_t q = q0 + lane;
-        const uint32_t nb = LP.below(q < fill ? (uint32_t)X.ST[q] : 0u);
-        if (q < fill) {
-            X.ST[q] = (uint16_t)nb;
-            X.T2S[nb] = (uint16_t)q;
-        }
-    }
-    for (uint32_t w = lane; w < nw; w += 32)
-        X.BM[w] = 32u * w + 32u <= fill ? 0xffffffffu : (32u * w < fill ? (1u << (fill - 32u * w)) - 1u : 0u);
-    wnow = (fill + 31u) / 32u;
-    lo = 0;
+    LP.load(X.BM, X.nw, lane);
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+        if (32u * g + lane < X.nw) X.PX[32u * g + lane] = (uint16_t)LP.ex[g];
     __syncwarp();
+    const uint32_t drop = live - fill;
+    const bool rebuild = *X.stash_n != 0;  // a stash in use: index the kept keys afresh below
+    for (uint32_t b = lane; b < X.nb && !rebuild; b += 32) {
+        const unsigned long long v = X.bkt[b];
+        unsigned long long nv = 0;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const uint32_t e = (uint32_t)(v >> (16 * p)) & 0xffffu;
+            const uint32_t t = e & X.tmask, wd = t >> 5;
+            const uint32_t rank = X.PX[wd] + (uint32_t)__popc(X.BM[wd] & ((1u << (t & 31u)) - 1u));
+            if (e != 0 && rank >= drop) nv |= (unsigned long long)((e - t) | (rank - drop)) << (16 * p);
+        }
+        X.bkt[b] = nv;
+    }
+    // keys move to lower times, words in order: a word is read whole before anything above
+    // its first live key's new time is written
+    for (uint32_t w = 0; w < X.nw; ++w) {
+        const uint32_t bits = X.BM[w], rank = X.PX[w] + (uint32_t)__popc(bits & ((1u << lane) - 1u));
+        const unsigned long long k = X.KT[32u * w + lane];
+        __syncwarp();
+        if (((bits >> lane) & 1u) && rank >= drop) X.KT[rank - drop] = k;
+        __syncwarp();
+    }
+    sl_live_range(X, 0, fill, lane);
+    __syncwarp();
+    if (rebuild) {
+        sl_clear_index(X, lane);
+        for (uint32_t t = lane; t < fill; t += 32) sl_insert(X, sl_hash(X, X.KT[t]), t);
+        __syncwarp();
+    }
 }
 
 template <int NC, int NG, bool SMALL>
-__global__ void __launch_bounds__(128)
-k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint32_t ns, uint32_t CL, uint32_t nbb,
-            const uint32_t *__restrict__ start, const uint32_t *__restrict__ coff, const uint32_t *__restrict__ total,
-            const uint32_t *__restrict__ idx, const rec16 *__restrict__ recs, uint32_t nrec,
-            const replay_state st, unsigned long long *__restrict__ ctr,
-            uint32_t *status)
+__global__ void __launch_bounds__(128, 5)
+k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t nb, uint32_t R,
+             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ coff,
+             const uint32_t *__restrict__ total, const uint32_t *__restrict__ idx, const rec16 *__restrict__ recs,
+             uint32_t nrec, const replay_state st, unsigned long long *__restrict__ ctr, uint32_t *status)
 {
     extern __shared__ uint4 smb[];
     const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const size_t per_warp = stamp_lru_bytes(cmax, nw, nbb);
-    const stamp_lru X = stamp_lru_at(reinterpret_cast<unsigned char *>(smb) + per_warp * warp, cmax, nw, nbb);
+    const window_lru X =
+        window_lru_at(reinterpret_cast<unsigned char *>(smb) + window_lru_bytes(nw, nb) * warp, nw, nb);
 
     const uint32_t w = blockIdx.x * wpb + warp;
     if (w >= *total) return;
@@ -606,7 +566,7 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
     const uint32_t p0 = b + ci * CL;
     const uint32_t p1 = (e - p0) < CL ? e : p0 + CL;
     const uint32_t rep = s / R, r = s % R;
-    const uint32_t fill_in = st.fill_in[s];
+    const uint32_t fill_in = min(st.fill_in[s], cmax);
     const unsigned long long *kin = st.keys_in + (unsigned long long)s * cmax;
     const uint32_t lt = (1u << lane) - 1u, gt = ~(lt | (1u << lane));
 
@@ -617,11 +577,12 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
         return;
     }
 
-    // ---- state at p0, in recency order in K[0 .. fill) ------------------------------
-    uint32_t fill = 0;
-    sl_reindex(X, 0, lane);
+    // ---- state at p0: the most recent keys at the highest times below `top` ----------
+    uint32_t live = 0, top = cmax;  // live keys of the window
+    sl_clear_index(X, lane);
     if (ci == 0) {
         // the carried-in keys, eight loads in flight per lane
+        top = live = fill_in;
         for (uint32_t q0 = 0; q0 < fill_in; q0 += 256) {
             unsigned long long kk[8];
 #pragma unroll
@@ -633,43 +594,48 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
             for (uint32_t x = 0; x < 8; ++x) {
                 const uint32_t q = q0 + 32u * x + lane;
                 if (q < fill_in) {
-                    X.K[q] = kk[x];
-                    sl_insert(X, kk[x], q);
+                    X.KT[top - 1u - q] = kk[x];
+                    sl_insert(X, sl_hash(X, kk[x]), top - 1u - q);
                 }
             }
         }
-        fill = fill_in;
     } else {
         // walk backwards collecting distinct keys, most recent first
+        for (uint32_t x = lane; x < nw; x += 32) X.BM[x] = 0;
+        __syncwarp();
         const uint32_t back = p0 - b;
         const uint32_t vtot = back + fill_in;
-        for (uint32_t v0 = 0; v0 < vtot && fill < cmax; v0 += 32) {
+        for (uint32_t v0 = 0; v0 < vtot && live < cmax; v0 += 32) {
             const uint32_t v = v0 + lane;
             const bool valid = v < vtot;
             unsigned long long key = 0;
             if (valid) key = v < back ? recs[min(idx[p0 - 1 - v], nrec - 1u)].key : kin[v - back];
             const uint32_t vm = __ballot_sync(0xffffffffu, valid);
             const uint32_t peers = __match_any_sync(0xffffffffu, key) & vm;
-            const bool fresh = valid && (peers & lt) == 0 && sl_lookup(X, key, fill, cmax) == kNone;
+            const key_hash H = sl_hash(X, key);
+            uint32_t at, loc;
+            const bool fresh = valid && (peers & lt) == 0 && !sl_lookup(X, H, key, (cmax + 31u) / 32u, at, loc);
             const uint32_t bal = __ballot_sync(0xffffffffu, fresh);
-            const uint32_t pos = fill + __popc(bal & lt);
+            const uint32_t pos = live + __popc(bal & lt);
             __syncwarp();
             if (fresh && pos < cmax) {
-                X.K[pos] = key;
-                sl_insert(X, key, pos);
+                const uint32_t t = top - 1u - pos;
+                X.KT[t] = key;
+                atomicOr(&X.BM[t >> 5], 1u << (t & 31u));  // (a degraded index is searched through the bitmap)
+                sl_insert(X, H, t);
             }
-            fill = min(cmax, fill + (uint32_t)__popc(bal));
+            live = min(cmax, live + (uint32_t)__popc(bal));
             __syncwarp();
         }
     }
+    sl_live_range(X, top - live, live, lane);
+    uint32_t wnow = (top + 31u) / 32u;
     __syncwarp();
-    uint32_t wnow, lo;
-    sl_stamps_in_order(X, fill, nw, lane, wnow, lo);
 
-    unsigned long long my_req = 0, my_prompt = 0;
-    unsigned long long my_hit[NC], my_tok[NC];
+    unsigned long long my_prompt = 0, my_tok[NC];
+    uint32_t my_hit[NC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) my_hit[c] = my_tok[c] = 0;
+    for (int c = 0; c < NC; ++c) my_hit[c] = 0, my_tok[c] = 0;
 
     // the next step's records are gathered one step early, through request
     // indices read two steps early
@@ -681,6 +647,12 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
     }
     uint32_t ix_next = p0 + 32u + lane < p1 ? idx[p0 + 32u + lane] : 0u;
     for (uint32_t t0 = p0; t0 < p1; t0 += 32) {
+        if (wnow == nw) {
+            const uint32_t keep = min(live, cmax);
+            sl_compact<NG>(X, live, keep, lane);
+            live = keep;
+            wnow = (live + 31u) / 32u;
+        }
         const uint32_t cnt = (p1 - t0) < 32u ? (p1 - t0) : 32u;
         const bool valid = lane < cnt;
         const rec16 mine = ahead;
@@ -689,35 +661,31 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
             ahead = recs[min(ix_next, nrec - 1u)];
         }
         ix_next = t0 + 64u + lane < p1 ? idx[t0 + 64u + lane] : 0u;
-        if (valid) {
-            my_req += 1;
-            my_prompt += (unsigned long long)mine.P + mine.S;
-        }
+        if (valid) my_prompt += (unsigned long long)mine.P + mine.S;
+        const uint32_t now = 32u * wnow + lane;
+        X.KT[now] = mine.key;
         const uint32_t vm = cnt == 32 ? 0xffffffffu : (1u << cnt) - 1u;
         const uint32_t grp = __match_any_sync(0xffffffffu, mine.key) & vm;
         const uint32_t below = grp & lt, above = grp & gt;
         const bool first = valid && below == 0;
         const bool last = valid && above == 0;
-        uint32_t slot = first ? sl_lookup(X, mine.key, fill, cmax) : kNone;
-        const bool res = slot != kNone;  // first occurrence of a resident key
-        uint32_t s_old = res ? (uint32_t)X.ST[slot] : 0u;
-        if (s_old >= 32u * nw) {  // never: stamps stay inside the window (guards the bitmap)
-            atomicOr(status, CR_FLAG_INTERNAL);
-            s_old = 0;
-        }
+        const key_hash H = sl_hash(X, mine.key);
+        uint32_t s_old = 0, loc = kNone;
+        const bool found = valid && sl_lookup(X, H, mine.key, wnow, s_old, loc);
+        const bool res = first && found;  // first occurrence of a key of the window
+        (void)CR_DCHECK(s_old < 32u * wnow + 32u, status);
 
-        // recency position at the step's start: live stamps above the key's
+        // recency position at the step's start: live times above the key's
         live_prefix<NG> LP;
         LP.load(X.BM, nw, lane);
-        const uint32_t bl = LP.below(s_old);
-        const uint32_t D = res ? fill - 1u - bl : kAbsent;
+        const uint32_t D = live - 1u - LP.below(s_old);
         // a first occurrence at old position D is pushed deeper by the step's earlier
         // first occurrences that were deeper or absent: between the absent ones
         // (jlo) and all of them (jhi).  Where that range straddles a capacity the
         // exact count decides the hit: those lanes (a few per step) are counted one
         // at a time against every lane; any count in the range decides the others.
         const uint32_t firstm = __ballot_sync(0xffffffffu, first);
-        const uint32_t absm = __ballot_sync(0xffffffffu, first && !res);
+        const uint32_t absm = __ballot_sync(0xffffffffu, first && !found);
         const uint32_t jlo = (uint32_t)__popc(absm & lt), jhi = (uint32_t)__popc(firstm & lt);
         bool amb = false;
 #pragma unroll
@@ -727,7 +695,7 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
         for (uint32_t am = __ballot_sync(0xffffffffu, res && amb); am; am &= am - 1u) {  // uniform
             const uint32_t a = (uint32_t)__ffs(am) - 1u;
             const uint32_t Da = __shfl_sync(0xffffffffu, D, a);
-            const uint32_t deeper = __ballot_sync(0xffffffffu, first && (!res || D > Da));
+            const uint32_t deeper = __ballot_sync(0xffffffffu, first && (!found || D > Da));
             if (lane == a) jx = (uint32_t)__popc(deeper & lt);
         }
         uint32_t dep_rep = 1u;
@@ -748,8 +716,7 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
             const uint32_t win = lt & ~((2u << (31u - (uint32_t)__clz(below | 1u))) - 1u);
             dep_rep = 1u + (uint32_t)__popc(gN & win);
         }
-        const uint32_t dep_first = res ? D + 1u + jx : kNone;
-        const uint32_t depth = !valid ? kNone : (first ? dep_first : dep_rep);
+        const uint32_t depth = res ? D + 1u + jx : (valid && !first ? dep_rep : kNone);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             if (c < (int)caps.n_caps && depth <= caps.cap[c]) {
@@ -758,100 +725,20 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
             }
         }
 
-        // ---- state after the step ------------------------------------------------------
+        // ---- state after the step: every key of the step takes its last access's time ----
+        __syncwarp();  // (the bitmap and the index have been read)
+        if (res) atomicAnd(&X.BM[s_old >> 5], ~(1u << (s_old & 31u)));
+        if (last && loc != kNone) X.E[loc] = (uint16_t)(H.tag | now);
         const uint32_t lastm = __ballot_sync(0xffffffffu, last);
-        const uint32_t u = (uint32_t)__popc(lastm);
-        const uint32_t mnew = (uint32_t)__popc(absm);
-        if (SMALL && u > cmax) {
-            // more distinct keys than the capacity: every old key leaves and the
-            // cmax most recently used keys of the step form the cache
-            __syncwarp();
-            sl_reindex(X, 0, lane);
-            for (uint32_t x = lane; x < nw; x += 32) X.BM[x] = 0;
-            __syncwarp();
-            const uint32_t rk = (uint32_t)__popc(lastm & gt);  // 0 = most recent
-            const bool keep = last && rk < cmax;
-            const uint32_t keepm = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const uint32_t t = wnow * 32u + lane;
-                X.K[rk] = mine.key;
-                sl_insert(X, mine.key, rk);
-                X.ST[rk] = (uint16_t)t;
-                X.T2S[t] = (uint16_t)rk;
-            }
-            if (lane == 0) X.BM[wnow] = keepm;
-            fill = cmax;
-            lo = wnow;
-            ++wnow;
-        } else {
-            // touched keys leave their old time
-            if (res) atomicAnd(&X.BM[s_old >> 5], ~(1u << (s_old & 31u)));
-            __syncwarp();
-            // the oldest untouched keys leave until the cache fits: the lowest live
-            // bits, found 32 words at a time from the lowest word that has any
-            uint32_t need = fill + mnew > cmax ? fill + mnew - cmax : 0u;
-            uint32_t done = 0;
-            while (need && lo < wnow) {  // each pass ends the loop or moves lo up
-                const uint32_t wd = lo + lane;
-                const uint32_t word = wd < wnow ? X.BM[wd] : 0u;
-                const uint32_t pc = (uint32_t)__popc(word);
-                const uint32_t incl = warp_incl_scan(pc, lane);
-                const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-                const uint32_t take = min(need, tot);
-                uint32_t o = 0;  // the word holding this lane's bit: first lane whose prefix exceeds lane
-#pragma unroll
-                for (uint32_t stp = 16; stp >= 1; stp >>= 1) {
-                    const uint32_t v = __shfl_sync(0xffffffffu, incl, o + stp - 1u);
-                    if (v <= lane) o += stp;
-                }
-                const uint32_t exo = __shfl_sync(0xffffffffu, incl - pc, o & 31u);
-                const uint32_t wo = __shfl_sync(0xffffffffu, word, o & 31u);
-                const uint32_t olast = __shfl_sync(0xffffffffu, o, (take + 31u) & 31u);
-                __syncwarp();
-                if (lane < take) {
-                    const uint32_t bit = nth_set_bit(wo, lane - exo);
-                    uint32_t q = X.T2S[(lo + o) * 32u + bit];
-                    atomicAnd(&X.BM[lo + o], ~(1u << bit));
-                    if (q < cmax) {
-                        sl_erase(X, q);
-                    } else {  // never: a live time always maps to a slot (guards the arrays)
-                        atomicOr(status, CR_FLAG_INTERNAL);
-                        q = 0;
-                    }
-                    X.EV[done + lane] = (uint16_t)q;
-                }
-                lo = take == tot ? min(lo + 32u, wnow) : lo + olast;
-                need -= take;
-                done += take;
-                __syncwarp();
-            }
-            // new keys take the never-used slots, then the freed ones
-            if (first && !res) {
-                const uint32_t a = (uint32_t)__popc(absm & lt);
-                const uint32_t freecnt = cmax - fill;
-                const uint32_t q = a < freecnt ? fill + a : (uint32_t)X.EV[a - freecnt];
-                X.K[q] = mine.key;
-                sl_insert(X, mine.key, q);
-                slot = q;
-            }
-            // every key of the step takes the time of its last access
-            const uint32_t fl = (uint32_t)__ffs(grp ? grp : 1u) - 1u;
-            const uint32_t ks = __shfl_sync(0xffffffffu, slot, fl);
-            if (last) {
-                const uint32_t t = wnow * 32u + lane;
-                X.ST[ks] = (uint16_t)t;
-                X.T2S[t] = (uint16_t)ks;
-            }
-            if (lane == 0) X.BM[wnow] = lastm;
-            fill = min(cmax, fill + mnew);
-            ++wnow;
-        }
         __syncwarp();
-        if (wnow == nw) sl_compact<NG>(X, fill, nw, lane, wnow, lo);
+        if (last && !found) sl_insert(X, H, now);
+        if (lane == 0) X.BM[wnow] = lastm;
+        live += (uint32_t)__popc(absm);
+        ++wnow;
+        __syncwarp();
     }
 
     // ---- counters -------------------------------------------------------------
-    my_req = cr_warp_sum_u64(my_req);
     my_prompt = cr_warp_sum_u64(my_prompt);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -860,7 +747,7 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
             const unsigned long long tk = cr_warp_sum_u64(my_tok[c]);
             if (lane == 0) {
                 unsigned long long *C = ctr + (((unsigned long long)rep * caps.n_caps + c) * R + r) * CR_CTR_FIELDS;
-                atomicAdd(&C[0], my_req);
+                atomicAdd(&C[0], (unsigned long long)(p1 - p0));
                 if (h) atomicAdd(&C[1], h);
                 if (tk) atomicAdd(&C[2], tk);
                 atomicAdd(&C[3], my_prompt);
@@ -871,68 +758,65 @@ k_lru_stamp(const replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t R, uint
     // ---- the stream's last chunk hands the state to the next call, most recent first
     if (p1 == e) {
         unsigned long long *kout = st.keys_out + (unsigned long long)s * cmax;
-        live_prefix<NG> LP;
-        LP.load(X.BM, nw, lane);
-        for (uint32_t q0 = 0; q0 < fill; q0 += 32) {
-            const uint32_t q = q0 + lane;
-            const uint32_t nb = LP.below(q < fill ? (uint32_t)X.ST[q] : 0u);
-            if (q < fill && nb < fill) kout[fill - 1u - nb] = X.K[q];
+        const uint32_t keep = min(live, cmax);
+        uint32_t above = live;  // live keys from word x on
+        for (uint32_t x = 0; x < wnow; ++x) {
+            const uint32_t bits = X.BM[x];
+            const uint32_t q = above - 1u - (uint32_t)__popc(bits & lt);
+            if (((bits >> lane) & 1u) && q < keep) kout[q] = X.KT[32u * x + lane];
+            above -= (uint32_t)__popc(bits);
         }
-        if (lane == 0) st.fill_out[s] = fill;
+        if (lane == 0) st.fill_out[s] = keep;
     }
 }
 
-// Words of the stamp window: the cmax stamps a compaction leaves plus at least
-// as many steps (and at least 8) before the next one.
-inline uint32_t stamp_words(uint32_t cmax)
+// Words of the window: the cmax keys that a compaction leaves plus twelve steps before the
+// next one.  More steps cost warps per SM, fewer cost compactions: at cmax 1024, 8 / 12 / 16 /
+// 24 / 32 steps measured 2.24 / 2.23 / 2.33 / 2.42 / 2.49 ms, at cmax 128 237 / 233 / 234 /
+// 227 / 262 us (the shapes above).
+inline uint32_t window_words(uint32_t cmax)
 {
-    const uint32_t w0 = (cmax + 31) / 32;
-    return w0 + (w0 > 8 ? w0 : 8);
+    return (cmax + 31) / 32 + 12;
+}
+
+// Index buckets of a window: 1.5 entries per time, so that two full buckets are rare even
+// when every request of the window has a key of its own.
+inline uint32_t window_buckets(uint32_t nw) { return 12u * nw; }
+
+// Registers and shared memory decide the warps per block (the most warps per SM; at most
+// 32 blocks and 64 warps per SM).
+uint32_t window_warps(size_t per_warp, uint32_t regs, uint32_t *per_sm)
+{
+    const uint32_t warps_regs = 65536u / (((regs * 32u + 255u) / 256u) * 256u);
+    uint32_t best = 0, wpb = 1;
+    for (uint32_t x = 4; x >= 1; --x) {
+        uint32_t nb = (uint32_t)((size_t)(227 * 1024) / (per_warp * x + 1024));
+        nb = nb < 32u ? nb : 32u;
+        nb = nb < warps_regs / x ? nb : warps_regs / x;
+        const uint32_t wps = nb * x < 64u ? nb * x : 64u;
+        if (wps > best) {
+            best = wps;
+            wpb = x;
+        }
+    }
+    *per_sm = best;
+    return wpb;
 }
 
 template <int NC, int NG, bool SMALL>
 int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t CL, const uint32_t *start,
-                 const uint32_t *coff, const uint32_t *total, uint64_t m, const uint32_t *idx,
-                 const rec16 *recs, uint64_t *d_ctr)
+                  const uint32_t *coff, const uint32_t *total, uint64_t m, const uint32_t *idx,
+                  const rec16 *recs, uint64_t *d_ctr)
 {
-    const uint32_t cmax = rp->cmax, nw = stamp_words(cmax);
-    // warps per block: the most warps per SM that shared memory allows (at most 32
-    // blocks and 64 warps per SM, and what the registers allow)
-    const size_t sm_bytes = 227 * 1024;
+    const uint32_t cmax = rp->cmax, nw = window_words(cmax), nb = window_buckets(nw);
     cudaFuncAttributes fa;
-    uint32_t warps_regs = 64;
+    uint32_t regs = 64, per_sm = 0;
     if (cudaFuncGetAttributes(&fa, k_lru_stamp<NC, NG, SMALL>) == cudaSuccess && fa.numRegs > 0)
-        warps_regs = 65536u / ((((uint32_t)fa.numRegs * 32u + 255u) / 256u) * 256u);
+        regs = (uint32_t)fa.numRegs;
     else
         cudaGetLastError();
-    auto fit = [&](uint32_t nb_bits, uint32_t *wpb_out) {
-        const size_t pw = stamp_lru_bytes(cmax, nw, nb_bits);
-        uint32_t best = 0;
-        for (uint32_t x = 4; x >= 1; --x) {
-            const size_t blk = pw * x + 1024;
-            uint32_t nb = blk <= sm_bytes ? (uint32_t)(sm_bytes / blk) : 0u;
-            nb = nb < 32u ? nb : 32u;
-            nb = nb < warps_regs / x ? nb : warps_regs / x;
-            const uint32_t wps = nb * x < 64u ? nb * x : 64u;
-            if (wps > best) {
-                best = wps;
-                *wpb_out = x;
-            }
-        }
-        return best;
-    };
-    // index buckets: one per resident key at most (a quarter of the entries live); half
-    // as many (half the entries live: a few more probes and inserts) when that fits more
-    // warps on an SM, i.e. when the state of the largest capacities bounds the occupancy
-    uint32_t nbb = 4;
-    while ((1u << nbb) < cmax) ++nbb;
-    uint32_t wpb = 1, wpb_half = 1;
-    const uint32_t w_full = fit(nbb, &wpb);
-    if (nbb > 4 && fit(nbb - 1, &wpb_half) * 10u >= w_full * 11u) {  // at least 10% more warps
-        --nbb;
-        wpb = wpb_half;
-    }
-    const size_t per_warp = stamp_lru_bytes(cmax, nw, nbb);
+    const size_t per_warp = window_lru_bytes(nw, nb);
+    const uint32_t wpb = window_warps(per_warp, regs, &per_sm);
     const size_t smem = per_warp * wpb;
     if (smem > 48 * 1024)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_lru_stamp<NC, NG, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -946,7 +830,7 @@ int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t C
     st.fill_out = rp->d_fill[rp->cur ^ 1];
     const int pr = cr_prof_begin(ctx, ctx->stream, CR_PROF_REPLAY);
     CR_LAUNCH(ctx, (k_lru_stamp<NC, NG, SMALL>), (unsigned int)((items + wpb - 1) / wpb), wpb * 32, smem, caps, cmax,
-              nw, rp->R, ns, CL, nbb, start, coff, total, idx, recs, (uint32_t)(m / rp->n_rep), st,
+              nw, nb, rp->R, ns, CL, start, coff, total, idx, recs, (uint32_t)(m / rp->n_rep), st,
               (unsigned long long *)d_ctr,
               ctx->d_status);
     cr_prof_end(ctx, ctx->stream, pr);
@@ -962,7 +846,7 @@ int launch_stamp_nc(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_
     uint32_t cmin = 0xffffffffu;
     for (uint32_t c = 0; c < caps.n_caps; ++c) cmin = caps.cap[c] < cmin ? caps.cap[c] : cmin;
     const bool small = cmin < 32;  // a repeat within a step can miss only below capacity 32
-    if (stamp_words(rp->cmax) <= 32)
+    if (window_words(rp->cmax) <= 32)
         return small ? launch_stamp<NC, 1, true>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr)
                      : launch_stamp<NC, 1, false>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr);
     return small ? launch_stamp<NC, 2, true>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr)

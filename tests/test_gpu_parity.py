@@ -1142,6 +1142,41 @@ def test_plan_import_routes_like_the_built_plan(P, ctx):
             P.Plan(ctx).load(R, W, **args)
 
 
+@pytest.mark.parametrize("caps", [[16], [64, 300], [1024]])
+@pytest.mark.parametrize("ncoll", [9, 30, 60, 400])
+def test_replay_parity_colliding_keys(P, ctx, caps, ncoll):
+    # keys that share both index buckets and the tag (their products with the index's odd
+    # multiplier differ in the low 22 bits only): past 8 of them the index's stash holds
+    # them, past 40 it is degraded; mixed with ordinary keys, over several renumberings of
+    # the window and two calls
+    rng = np.random.default_rng(ncoll + sum(caps))
+    inv = np.uint64(pow(0x9E3779B97F4A7C15, -1, 1 << 64))
+    with np.errstate(over="ignore"):
+        coll = (np.uint64(0xABCDEF0123 << 24) + rng.permutation(1 << 22)[:ncoll].astype(np.uint64)) * inv
+    n_rep, R, n = 2, 2, 6000
+    pool = np.concatenate([coll, _rates_keys(rng, 300, 300)])
+    keys = pool[rng.integers(0, pool.size, size=n)]
+    plen = rng.integers(16, 5000, size=n).astype(np.uint32)
+    slen = np.full(n, 64, np.uint32)
+    dest = tg.random_dest(n_rep, n, R, 7)
+    orp = O.Replay(n_rep, R, caps)
+    rp = P.Replay(ctx, n_rep, R, caps)
+    ctr = torch.zeros((n_rep, len(caps), R, 5), dtype=torch.int64, device=DEV)
+    dk, dp, ds, dd = d_u64(keys), d_u32(plen), d_u32(slen), d_u16(dest)
+    cut = n // 2
+    for a, b in ((0, cut), (cut, n)):
+        orp.step(keys[a:b], plen[a:b], slen[a:b], dest[:, a:b])
+        P.shadow_replay(ctx, rp, dk[a:b].contiguous(), dp[a:b].contiguous(), ds[a:b].contiguous(),
+                        dd[:, a:b].contiguous(), ctr)
+        ctx.sync()
+        assert (h_u64(ctr) == orp.ctr).all()
+    for rep in range(n_rep):
+        for r in range(R):
+            st = rp.state(rep, r)
+            for c_i, c in enumerate(caps):
+                assert (st[:c] == orp.state(rep, c_i, r)).all()
+
+
 def test_replay_state_import_resumes(P, ctx):
     # replay two calls in one simulator set; export every state after the first, import
     # it into a fresh set, and the second call's counters match
