@@ -100,6 +100,9 @@ __device__ __forceinline__ unsigned long long chwbl_cap(unsigned long long m, ui
     return (5ull * (m + 1ull) + den - 1ull) / den;
 }
 
+// Entries of a replica's row of candidates: rows start on 16-byte boundaries.
+__host__ __device__ inline unsigned long long cand_row(unsigned long long n) { return (n + 3ull) & ~3ull; }
+
 // Everything that does not depend on the live load, for every (replica, request).
 // A warp takes 32 consecutive requests, reads their keys once and computes the
 // candidates of the replicas of its group for them (blockIdx.y = group g of
@@ -127,7 +130,7 @@ __global__ void __launch_bounds__(256) k_route_cand(const __grid_constant__ rout
         for (uint32_t x = blockIdx.y; x < n_rep; x += gridDim.y) {  // uniform
             const uint32_t rep = args.cand[x];
             const route_desc &rd = args.d[rep];
-            const unsigned long long o = (unsigned long long)rep * n + i;
+            const unsigned long long o = (unsigned long long)rep * n + i, oc = (unsigned long long)rep * cand_row(n) + i;
             switch (rd.policy) {
             case CR_POLICY_RR:
                 // (g0 + i + seed) mod 2^64 mod R: before the sum wraps, (b0 + i mod R) mod R
@@ -146,10 +149,10 @@ __global__ void __launch_bounds__(256) k_route_cand(const __grid_constant__ rout
                 if (valid) dest[o] = (uint16_t)cr_jump_hash(cr_fmix64(key ^ rd.seed), R);
                 break;
             case CR_POLICY_P2C:
-                if (valid) cand[o] = p2c_pair(rd.seed, rd.policy, g0 + i, R);
+                if (valid) cand[oc] = p2c_pair(rd.seed, rd.policy, g0 + i, R);
                 break;
             case CR_POLICY_CHWBL:
-                if (valid) cand[o] = kRing | ring_start(rd, cr_fmix64(key ^ rd.seed));
+                if (valid) cand[oc] = kRing | ring_start(rd, cr_fmix64(key ^ rd.seed));
                 break;
             default: {
                 uint32_t c = 0xffffffffu;
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(256) k_route_cand(const __grid_constant__ rout
                         }
                         sl = (sl + 1) & mask;
                     }
-                    if (c != 0xffffffffu) cand[o] = c;
+                    if (c != 0xffffffffu) cand[oc] = c;
                 }
                 const bool miss = valid && c == 0xffffffffu;
                 const uint32_t mm = __ballot_sync(0xffffffffu, miss);
@@ -176,7 +179,7 @@ __global__ void __launch_bounds__(256) k_route_cand(const __grid_constant__ rout
                     const unsigned long long e = Q[qn - 32u + lane];
                     const uint32_t er = (uint32_t)(e >> 40);
                     const unsigned long long j = e & ((1ull << 40) - 1ull);
-                    cand[(unsigned long long)er * n + j] = p2c_pair(args.d[er].seed, args.d[er].policy, g0 + j, R);
+                    cand[(unsigned long long)er * cand_row(n) + j] = p2c_pair(args.d[er].seed, args.d[er].policy, g0 + j, R);
                     qn -= 32u;
                     __syncwarp();
                 }
@@ -188,7 +191,7 @@ __global__ void __launch_bounds__(256) k_route_cand(const __grid_constant__ rout
         const unsigned long long e = Q[lane];
         const uint32_t er = (uint32_t)(e >> 40);
         const unsigned long long j = e & ((1ull << 40) - 1ull);
-        cand[(unsigned long long)er * n + j] = p2c_pair(args.d[er].seed, args.d[er].policy, g0 + j, R);
+        cand[(unsigned long long)er * cand_row(n) + j] = p2c_pair(args.d[er].seed, args.d[er].policy, g0 + j, R);
     }
 }
 
@@ -314,19 +317,30 @@ __device__ __forceinline__ uint32_t resolve(uint32_t c, const route_desc &rd, co
 // buffer, chunk c+1's loads are in flight into registers and land in the other.
 constexpr uint32_t kStage = 16384;
 
-// 4-byte asynchronous global -> shared copies (the next chunk lands while this
-// one is resolved, without holding registers)
+// Asynchronous global -> shared copies (the next chunk lands while this one is resolved,
+// without holding registers).
 __device__ __forceinline__ void cp_async4(void *smem, const void *gmem)
 {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+{
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Start copying chunk [c1, c1 + CH) of the candidates into buffer nb.
+// Start copying chunk [c1, c1 + CH) of the candidates into buffer nb.  Rows of candidates
+// start and end on 16-byte boundaries, as the buffers do: a chunk of whole quadruples is
+// copied 16 bytes at a time (up to three of the row's padding entries with it).
 __device__ __forceinline__ void stage_next(uint32_t *nb, const uint32_t *__restrict__ Cd, unsigned long long c1,
                                            unsigned long long n, uint32_t CH)
 {
+    if ((CH & 3u) == 0) {
+        for (uint32_t q = threadIdx.x * 4u; q < CH && c1 + q < n; q += blockDim.x * 4u) cp_async16(&nb[q], &Cd[c1 + q]);
+        return;
+    }
     for (uint32_t q = threadIdx.x; q < CH && c1 + q < n; q += blockDim.x) cp_async4(&nb[q], &Cd[c1 + q]);
 }
 
@@ -371,7 +385,7 @@ __device__ __forceinline__ void resolve_batches(const route_desc &rd, const uint
         }
         return;
     }
-    for (uint32_t x = tid; x < CH && x < n; x += blockDim.x) cbuf[x] = Cd[x];
+    cp_async_wait_all();  // the caller has started the first chunk's copy
     __syncthreads();
     int cur = 0;
     for (unsigned long long c0 = 0; c0 < n; c0 += CH) {
@@ -401,238 +415,335 @@ __device__ __forceinline__ void resolve_batches(const route_desc &rd, const uint
     }
 }
 
-// ---- plan replicas: keys with several members decided once per batch ---------
-// Inside a batch every request of a key with k_b > 1 goes to the same member:
-// the least loaded of T(b) at the batch start (ties to the earlier member).  So
-// the CTA keeps the member lists of those keys in shared memory, collected as
-// the staging meets them, and finds each key's member once per batch, at the
-// boundary; a request then reads its key's answer.  Loads and batch counts are
-// double-buffered so that the answers for batch b + 1 (loads of batch b plus
-// its counts) are computed while the loads are being updated, behind the same
-// two barriers per batch.
+// ---- batches on 32-bit relative loads ----------------------------------------
+// The live loads are held as differences from their minimum (the caller checks that
+// every load stays below 2^32 above it) in two buffers.  In batch b the decisions read
+// one of them, A = the loads at the start of the batch, while W still holds those of the
+// batch before; every thread adds its requests of this batch AND its requests of batch
+// b - 1 to W, so that W = the loads at the start of batch b + 1 when the batch's barrier
+// is passed and the two swap.  No pass over the destinations, no counts to clear.
+//
+// Plan replicas: inside a batch every request of a key with k_b > 1 goes to the same
+// member, the least loaded of T(b) at the batch start (ties to the earlier member).  The
+// CTA keeps those keys' member lists in shared memory, collected when a staged chunk is
+// scanned, and the scan rewrites their candidates to the key's index.  While any are
+// tracked, one warp per key finds its member between the batch's barrier and a second
+// one; warp w holds the members of key w in registers.  Keys past the capacity keep their
+// SET candidate, and each request reads the members from the plan.
+//   RING (not otherwise used by plan replicas)  index of a tracked key
+// Bound: issue slots of the replica's SM (about 2.5 of 4 per cycle).  24 plan replicas of
+// 1,066,667 requests, R = 1024, batches of 1,024: the plan-and-route turn around it 3.23 ->
+// 2.80 ms against 64-bit loads with a pass over the destinations per batch and a map lookup
+// per request; 20 replicas of 166,667 requests at R = 30: 158 -> 125 us.
 constexpr uint32_t kSetCap = 256;      // keys with k_b > 1 tracked per replica
 constexpr uint32_t kSetMapCap = 512;   // open-addressing map: table slot -> key index
 constexpr uint32_t kSetPool = 4096;    // member entries of the tracked keys
+constexpr uint16_t kSetNone = 0xffffu;
 
 struct set_cache {
     uint32_t map_slot[kSetMapCap];  // table slot of each map entry, kEmpty when free
-    uint16_t map_j[kSetMapCap];     // key index of each map entry
+    uint16_t map_j[kSetMapCap];     // key index of each map entry, kSetNone until its list is there
     uint32_t off[kSetCap];          // first member of key j in the pool
-    uint16_t k[kSetCap];
-    uint16_t res[2][kSetCap];       // least-loaded member of each key, per batch parity
+    uint16_t k[kSetCap];            // its members (0: they did not fit)
+    uint16_t res[kSetCap];          // least-loaded member of each key
     uint16_t pool[kSetPool];
-    uint32_t n, used, ready, overflow;
+    uint32_t n, used;
 };
 
-__host__ __device__ inline size_t set_cache_bytes() { return (sizeof(set_cache) + 15) & ~(size_t)15; }
-
-// Shared-memory layout of k_route_resolve: loads [R] u64, counts [R] u32, two
-// staging buffers [CH] u32, member lists / ring owners [MC] u16, then (plan
-// replicas) the second loads and counts and the key cache, 16-byte aligned.
-__host__ __device__ inline size_t resolve_plan_extra_at(uint32_t R, uint32_t CH, unsigned long long MC)
+// Shared-memory layout of k_route_resolve: loads [R] u64 and counts [R] u32 (or the two
+// relative load buffers), at the next 16-byte boundary two staging buffers [CH] u32, member
+// lists / ring owners [MC] u16, then (plan replicas) the key cache, 16-byte aligned.
+__host__ __device__ inline size_t resolve_stage_at(uint32_t R) { return ((size_t)R * 12 + 15) & ~(size_t)15; }
+__host__ __device__ inline size_t resolve_cache_at(uint32_t R, uint32_t CH, unsigned long long MC)
 {
-    return ((size_t)R * 12 + (size_t)CH * 8 + (size_t)MC * 2 + 15) & ~(size_t)15;
-}
-__host__ __device__ inline size_t resolve_plan_extra_bytes(uint32_t R)
-{
-    return (((size_t)R * 12 + 15) & ~(size_t)15) + set_cache_bytes();
+    return (resolve_stage_at(R) + (size_t)CH * 8 + (size_t)MC * 2 + 15) & ~(size_t)15;
 }
 
-__device__ __forceinline__ uint32_t set_hash(uint32_t slot) { return (slot * 0x9E3779B1u) >> 23; }  // 9 bits
-
-// Record the key of table slot `slot` (a SET candidate) unless it is known.
-__device__ void set_discover(set_cache &S, const route_desc &rd, const uint16_t *mem, uint32_t slot)
+// Index of the key of table slot `slot` (a SET candidate), tracked from now on if it is new
+// and fits; kSetNone while another thread is still adding it, or when it does not fit.
+__device__ uint32_t set_index(set_cache &S, const route_desc &rd, const uint16_t *mem, uint32_t slot)
 {
-    uint32_t h = set_hash(slot);
+    uint32_t h = (slot * 0x9E3779B1u) >> 23;  // 9 bits
     for (uint32_t it = 0; it < kSetMapCap; ++it, h = (h + 1) & (kSetMapCap - 1)) {
-        const uint32_t cur = *(volatile uint32_t *)&S.map_slot[h];
-        if (cur == slot) return;
-        if (cur != kEmpty) continue;
-        const uint32_t prev = atomicCAS(&S.map_slot[h], kEmpty, slot);
-        if (prev == slot) return;
-        if (prev != kEmpty) continue;
-        const uint32_t j = atomicAdd(&S.n, 1u);
-        const cr_table_slot ts = rd.table[slot];
-        const uint32_t off = atomicAdd(&S.used, (uint32_t)ts.k);
-        if (j >= kSetCap || off + ts.k > kSetPool) {
-            S.overflow = 1u;
-            return;
+        uint32_t cur = *(volatile uint32_t *)&S.map_slot[h];
+        if (cur == kEmpty) {
+            if (*(volatile uint32_t *)&S.n >= kSetCap) return kSetNone;
+            cur = atomicCAS(&S.map_slot[h], kEmpty, slot);
+            if (cur == kEmpty) {
+                const uint32_t j = atomicAdd(&S.n, 1u);
+                const cr_table_slot ts = rd.table[slot];
+                const uint32_t off = atomicAdd(&S.used, (uint32_t)ts.k);
+                const bool fits = off + ts.k <= kSetPool;
+                if (j >= kSetCap) return kSetNone;
+                for (uint32_t m = 0; fits && m < ts.k; ++m) S.pool[off + m] = mem[(size_t)ts.koff + m];
+                S.off[j] = off;
+                S.k[j] = fits ? ts.k : (uint16_t)0;
+                if (!fits) return kSetNone;
+                *(volatile uint16_t *)&S.map_j[h] = (uint16_t)j;
+                return j;
+            }
         }
-        for (uint32_t m = 0; m < ts.k; ++m) S.pool[off + m] = mem[(size_t)ts.koff + m];
-        S.off[j] = off;
-        S.k[j] = ts.k;
-        S.map_j[h] = (uint16_t)j;
-        return;
+        if (cur == slot) return *(volatile uint16_t *)&S.map_j[h];
     }
-    S.overflow = 1u;
+    return kSetNone;
 }
 
-// Key index of a discovered slot, or kEmpty.
-__device__ __forceinline__ uint32_t set_find(const set_cache &S, uint32_t slot)
+// The staged chunk's SET candidates to key indices, four candidates per thread at a time.
+__device__ __forceinline__ void set_scan(set_cache &S, const route_desc &rd, const uint16_t *mem, uint32_t *cb,
+                                         uint32_t len, uint32_t CH)
 {
-    uint32_t h = set_hash(slot);
-    for (uint32_t it = 0; it < kSetMapCap; ++it, h = (h + 1) & (kSetMapCap - 1)) {
-        const uint32_t cur = S.map_slot[h];
-        if (cur == slot) return S.map_j[h];
-        if (cur == kEmpty) return kEmpty;
+    for (uint32_t q = threadIdx.x * 4u; q < len; q += blockDim.x * 4u) {
+        uint32_t c[4];
+        if ((CH & 3u) == 0) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(&cb[q]);
+            c[0] = v.x, c[1] = v.y, c[2] = v.z, c[3] = v.w;
+        } else {
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) c[u] = q + u < len ? cb[q + u] : 0u;
+        }
+        uint32_t sets = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) sets |= (c[u] & kKindMask) == kSet && q + u < len ? 1u << u : 0u;
+        for (; sets; sets &= sets - 1u) {
+            const uint32_t u = (uint32_t)__ffs(sets) - 1u;
+            const uint32_t j = set_index(S, rd, mem, cb[q + u] & kLow30);
+            if (j != kSetNone) cb[q + u] = kRing | j;
+        }
     }
-    return kEmpty;
 }
 
-// res[j] for keys j0 .. j1-1: the first member with the least load Lb[m] (+ db[m]),
-// one warp per key.
-__device__ __forceinline__ void set_results(set_cache &S, uint16_t *res, const unsigned long long *Lb,
-                                            const uint32_t *db, uint32_t j0, uint32_t j1)
+// res[j] of tracked keys j0, j0 + step, .. < n (one warp): the first member with the least load.
+__device__ __forceinline__ void set_results(set_cache &S, const uint32_t *A, uint32_t j0, uint32_t step, uint32_t n)
 {
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (uint32_t j = j0 + warp; j < j1; j += nw) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t j = j0; j < n; j += step) {
         const uint32_t off = S.off[j], k = S.k[j];
-        unsigned long long bl = ~0ull;
-        uint32_t bp = 0xffffffffu;
+        if (k == 0) continue;
+        uint32_t bl = 0xffffffffu, bp = 0xffffffffu;
         for (uint32_t p = lane; p < k; p += 32) {
-            const uint32_t m = S.pool[off + p];
-            const unsigned long long l = Lb[m] + (db ? db[m] : 0u);
-            if (l < bl) {  // positions rise within a lane: the first minimum stays
+            const uint32_t l = A[S.pool[off + p]];
+            if (l < bl || bp == 0xffffffffu) {  // positions rise within a lane: the first minimum stays
                 bl = l;
                 bp = p;
             }
         }
-        // the lexicographic minimum of (load, position) over the warp, by three 32-bit
-        // warp reductions: high word of the load, low word among those, position among those
-        const uint32_t hi = (uint32_t)(bl >> 32), lo = (uint32_t)bl;
-        const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
-        const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
-        const uint32_t mp = __reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? bp : 0xffffffffu);
-        if (lane == 0) res[j] = S.pool[off + mp];
+        const uint32_t ml = __reduce_min_sync(0xffffffffu, bl);
+        const uint32_t mp = __reduce_min_sync(0xffffffffu, bl == ml ? bp : 0xffffffffu);
+        if (lane == 0) S.res[j] = S.pool[off + mp];
     }
 }
 
-// The batch loop of a plan replica with staging (CH > 0).  L0/dl0 hold the loads
-// and zero counts on entry; returns the buffer (0 or 1) that holds the loads at
-// the end.  Falls back to per-request member scans once the cache overflows.
-__device__ int resolve_batches_plan(const route_desc &rd, const uint16_t *mem, unsigned long long *L0,
-                                    unsigned long long *L1, uint32_t *dl0, uint32_t *dl1, set_cache &S,
-                                    uint32_t *cbuf, const uint32_t *__restrict__ Cd, uint16_t *__restrict__ D,
-                                    unsigned long long n, uint32_t B, uint32_t CH, uint32_t R, uint32_t *status)
+// ONE: a batch has at most one request per thread, which keeps its last destination and
+// its next candidate in registers; otherwise a resolved candidate is replaced by its
+// destination in the stage and read back in the next batch.  Returns the buffer that
+// holds the loads at the end.
+template <bool ONE, bool PLAN>
+__device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, const uint16_t *mem, uint32_t *A,
+                                                      uint32_t *W, set_cache &S, uint32_t *cbuf,
+                                                      const uint32_t *__restrict__ Cd, uint16_t *__restrict__ D,
+                                                      unsigned long long n, uint32_t B, uint32_t CH, uint32_t R,
+                                                      uint32_t *status)
 {
-    const uint32_t tid = threadIdx.x;
-    for (uint32_t x = tid; x < kSetMapCap; x += blockDim.x) S.map_slot[x] = kEmpty;
-    if (tid == 0) {
-        S.n = 0;
-        S.used = 0;
-        S.ready = 0;
-        S.overflow = 0;
+    const uint32_t tid = threadIdx.x, T = blockDim.x, lane = tid & 31u, warp = tid >> 5;
+    auto decide = [&](uint32_t c) -> uint32_t {
+        if (!PLAN) {
+            const uint32_t d1 = c & 0x1fffu, d2 = (c >> 13) & 0x1fffu;
+            return A[d1] <= A[d2] ? d1 : d2;
+        }
+        // FIXED and PAIR without a branch: for FIXED the two fields read are the
+        // destination (< R <= 8192) and 0, in range as well; others read entry 0
+        const uint32_t kind = c & kKindMask;
+        const bool two = kind < kSet;
+        const uint32_t d1 = two ? (c & 0x1fffu) : 0u, d2 = two ? ((c >> 13) & 0x1fffu) : 0u;
+        const bool p1 = A[d1] <= A[d2];
+        if (two) return kind == kFixed ? (c & 0xffffu) : (p1 ? d1 : d2);
+        if (kind == kRing) return S.res[c & (kSetCap - 1u)];
+        const cr_table_slot slot = rd.table[c & kLow30];
+        if (!CR_DCHECK(rd.n_members == nullptr || (unsigned long long)slot.koff + slot.k <= *rd.n_members, status))
+            return 0u;
+        auto load_of = [&](uint32_t r) { return (unsigned long long)A[r]; };
+        return set_min(mem, slot.koff, slot.k, slot.m0, load_of);
+    };
+    if (PLAN) {
+        for (uint32_t x = tid; x < kSetMapCap; x += T) {
+            S.map_slot[x] = kEmpty;
+            S.map_j[x] = kSetNone;
+        }
+        if (tid == 0) S.n = S.used = 0;
     }
-    for (uint32_t r = tid; r < R; r += blockDim.x) dl1[r] = 0;
+    cp_async_wait_all();  // the caller has started the first chunk's copy
     __syncthreads();
-    for (uint32_t x = tid; x < CH && x < n; x += blockDim.x) {
-        const uint32_t c = Cd[x];
-        cbuf[x] = c;
-        if ((c & kKindMask) == kSet) set_discover(S, rd, mem, c & kLow30);
-    }
-    __syncthreads();
-    if (!S.overflow) set_results(S, S.res[0], L0, nullptr, 0, min(S.n, kSetCap));
-    if (tid == 0) S.ready = min(S.n, kSetCap);  // read by nobody before the barrier
-    __syncthreads();
-    int par = 0, cur = 0;
+    // a scan that met new keys is repeated, for the candidates whose key another thread was
+    // just adding (uniform: keys are added only while scanning)
+    uint32_t known = 0;
+    auto scan = [&](uint32_t *buf, uint32_t len) {
+        set_scan(S, rd, mem, buf, len, CH);
+        __syncthreads();
+        if (S.n != known) {
+            known = S.n;
+            set_scan(S, rd, mem, buf, len, CH);
+            __syncthreads();
+        }
+    };
+    if (PLAN) scan(cbuf, n < CH ? (uint32_t)n : CH);
+    uint32_t pd = kEmpty;  // ONE: this thread's destination of the batch before
+    int cur = 0;
     for (unsigned long long c0 = 0; c0 < n; c0 += CH) {
         const unsigned long long c1 = (c0 + CH < n) ? c0 + CH : n;
         uint32_t *nb = cbuf + (size_t)(cur ^ 1) * CH;
-        stage_next(nb, Cd, c1, n, CH);
-        const uint32_t *cb = cbuf + (size_t)cur * CH;
+        uint32_t *cb = cbuf + (size_t)cur * CH;
         uint16_t *Dc = D + c0;
         const uint32_t len = (uint32_t)(c1 - c0);
-        const bool ovf = S.overflow != 0u;  // uniform: written only while staging
+        uint32_t keys = 0;            // tracked
+        uint32_t my_k = 0, my_m = 0;  // this warp's first key, when its members fit the lanes
+        if (PLAN) {
+            keys = min(known, kSetCap);
+            if (warp < keys && S.k[warp] <= 32u) {
+                my_k = S.k[warp];
+                my_m = my_k ? S.pool[S.off[warp] + min(lane, my_k - 1u)] : 0u;
+            }
+            set_results(S, A, warp, T >> 5, keys);
+            __syncthreads();
+        }
+        stage_next(nb, Cd, c1, n, CH);
+        uint32_t cn = ONE && tid < min(B, len) ? cb[tid] : 0u;  // ONE: the next batch's candidate
+        uint32_t p0 = 0, p1 = 0;                                // otherwise: the batch before, of this chunk
         for (uint32_t o0 = 0; o0 < len; o0 += B) {
             const uint32_t o1 = (o0 + B < len) ? o0 + B : len;
-            unsigned long long *Lc = par ? L1 : L0, *Ln = par ? L0 : L1;
-            uint32_t *dc = par ? dl1 : dl0, *dn = par ? dl0 : dl1;
-            const uint16_t *res = S.res[par];
-            for (uint32_t o = o0 + tid; o < o1; o += blockDim.x) {
-                const uint32_t c = cb[o], kind = c & kKindMask;
-                // FIXED and PAIR without a branch: for FIXED the two fields read are the
-                // destination (< R <= 8192) and 0, in range as well; a SET reads entry 0
-                const bool two = kind < kSet;
-                const uint32_t d1 = two ? (c & 0x1fffu) : 0u, d2 = two ? ((c >> 13) & 0x1fffu) : 0u;
-                const bool p1 = Lc[d1] <= Lc[d2];
-                uint32_t d = kind == kFixed ? (c & 0xffffu) : (p1 ? d1 : d2);
-                if (!two) {
-                    const uint32_t j = ovf ? kEmpty : set_find(S, c & kLow30);
-                    if (j < kSetCap) {
-                        d = res[j];
-                    } else {
-                        const cr_table_slot slot = rd.table[c & kLow30];
-                        auto load_of = [&](uint32_t x) { return Lc[x]; };
-                        d = set_min(mem, slot.koff, slot.k, slot.m0, load_of);
+            if (ONE) {
+                const uint32_t o = o0 + tid, c = cn;
+                cn = o1 + tid < len ? cb[o1 + tid] : 0u;
+                if (pd != kEmpty) atomicAdd(&W[pd], 1u);
+                pd = kEmpty;
+                if (o < o1) {
+                    const uint32_t d = decide(c);
+                    if (CR_DCHECK(d < R, status)) {
+                        Dc[o] = (uint16_t)d;
+                        atomicAdd(&W[d], 1u);
+                        pd = d;
                     }
                 }
-                if (!CR_DCHECK(d < R, status)) continue;
-                Dc[o] = (uint16_t)d;
-                atomicAdd(&dc[d], 1u);
+            } else {
+                for (uint32_t o = p0 + tid; o < p1; o += T) atomicAdd(&W[cb[o]], 1u);
+                for (uint32_t o = o0 + tid; o < o1; o += T) {
+                    uint32_t d = decide(cb[o]);
+                    if (!CR_DCHECK(d < R, status)) d = 0;
+                    Dc[o] = (uint16_t)d;
+                    atomicAdd(&W[d], 1u);
+                    cb[o] = d;  // (candidate o is this thread's in both batches)
+                }
+                p0 = o0;
+                p1 = o1;
             }
             __syncthreads();
-            for (uint32_t r = tid; r < R; r += blockDim.x) {
-                Ln[r] = Lc[r] + dc[r];
-                dn[r] = 0;
+            uint32_t *t = A;
+            A = W;
+            W = t;
+            if (PLAN && keys) {
+                uint32_t j0 = warp;
+                if (my_k) {  // of equal loads, the lowest lane's
+                    const uint32_t l = lane < my_k ? A[my_m] : 0xffffffffu;
+                    const uint32_t least = __ballot_sync(0xffffffffu, l == __reduce_min_sync(0xffffffffu, l));
+                    if (lane == (uint32_t)__ffs(least) - 1u) S.res[warp] = (uint16_t)my_m;
+                    j0 += T >> 5;
+                }
+                set_results(S, A, j0, T >> 5, keys);
+                __syncthreads();
             }
-            if (!ovf) set_results(S, S.res[par ^ 1], Lc, dc, 0, min(S.ready, kSetCap));
-            __syncthreads();
-            par ^= 1;
         }
+        if (!ONE)  // W catches up before the chunk's stage is overwritten
+            for (uint32_t o = p0 + tid; o < p1; o += T) atomicAdd(&W[cb[o]], 1u);
         cp_async_wait_all();
         __syncthreads();
-        for (uint32_t q = tid; q < CH && c1 + q < n; q += blockDim.x)
-            if ((nb[q] & kKindMask) == kSet) set_discover(S, rd, mem, nb[q] & kLow30);
-        __syncthreads();
-        // keys met for the first time: their answers for the next batch, from its loads
-        const uint32_t nn = min(S.n, kSetCap), rd0 = S.ready;
-        if (nn > rd0 && !S.overflow) set_results(S, S.res[par], par ? L1 : L0, nullptr, rd0, nn);  // uniform
-        __syncthreads();  // every thread has read S.ready
-        if (tid == 0) S.ready = S.overflow ? rd0 : nn;
-        __syncthreads();
+        if (PLAN) scan(nb, n - c1 < CH ? (uint32_t)(n - c1) : CH);
         cur ^= 1;
     }
-    return par;
+    return A;
 }
 
-__global__ void __launch_bounds__(kRouteBlock) k_route_resolve(const __grid_constant__ route_args args,
+// The replica's loads as differences from their minimum in A and W (= A + R), and the
+// minimum; false (neither is then meaningful) when a load could pass 2^32 - 1 above it.
+__device__ __forceinline__ bool loads_relative(const unsigned long long *Lg, uint32_t R, unsigned long long n,
+                                               uint32_t *A, uint32_t *W, unsigned long long &base)
+{
+    __shared__ unsigned long long s_lo, s_hi;
+    if (threadIdx.x == 0) {
+        s_lo = ~0ull;
+        s_hi = 0;
+    }
+    __syncthreads();
+    unsigned long long lo = ~0ull, hi = 0;
+    for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) {
+        const unsigned long long v = Lg[r];
+        lo = v < lo ? v : lo;
+        hi = v > hi ? v : hi;
+        A[r] = (uint32_t)v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
+        lo = a < lo ? a : lo;
+        hi = b > hi ? b : hi;
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(&s_lo, lo);
+        atomicMax(&s_hi, hi);
+    }
+    __syncthreads();
+    base = s_lo;
+    if (n >= 0xffffffffull || s_hi - s_lo >= 0xffffffffull - n) return false;
+    for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) A[r] = W[r] = A[r] - (uint32_t)base;  // mod 2^32
+    __syncthreads();
+    return true;
+}
+
+__global__ void __launch_bounds__(kRouteBlock, 1) k_route_resolve(const __grid_constant__ route_args args,
                                                                const uint32_t *__restrict__ cand,
                                                                unsigned long long n, uint32_t B, uint32_t CH,
                                                                uint32_t R, unsigned long long *__restrict__ load,
                                                                uint16_t *__restrict__ dest, uint32_t *status,
                                                                unsigned long long MC, int plan_x)
 {
-    extern __shared__ unsigned long long sh[];
+    extern __shared__ __align__(16) unsigned long long sh[];
+    unsigned char *shb = reinterpret_cast<unsigned char *>(sh);
     unsigned long long *L = sh;                              // [R] live load
     uint32_t *delta = reinterpret_cast<uint32_t *>(sh + R);  // [R] this batch
-    uint32_t *cbuf = delta + R;                              // [2][CH] staged candidates
+    uint32_t *cbuf = reinterpret_cast<uint32_t *>(shb + resolve_stage_at(R));  // [2][CH] staged candidates
     uint16_t *smem_aux = reinterpret_cast<uint16_t *>(cbuf + 2 * (size_t)CH);  // [MC] members or ring owners
-    // plan replicas (when the launch reserved it): the second load and count buffers and the key cache
-    unsigned char *px = reinterpret_cast<unsigned char *>(sh) + resolve_plan_extra_at(R, CH, MC);
     const uint32_t rep = args.dep[blockIdx.x];
     const route_desc rd = args.d[rep];
     unsigned long long *Lg = load + (unsigned long long)rep * R;
-    const uint32_t *Cd = cand + (unsigned long long)rep * n;
+    const uint32_t *Cd = cand + (unsigned long long)rep * cand_row(n);
     uint16_t *D = dest + (unsigned long long)rep * n;
+    const bool plan = rd.policy != CR_POLICY_CHWBL && rd.policy != CR_POLICY_P2C;
+    if (CH > 0) stage_next(cbuf, Cd, 0, n, CH);
+    const uint16_t *mem = stage_aux(rd, smem_aux, MC);
+    if (CH > 0 && rd.policy != CR_POLICY_CHWBL && (plan_x || !plan)) {
+        uint32_t *A = reinterpret_cast<uint32_t *>(sh), *W = A + R, *F;  // in place of the 64-bit loads
+        set_cache &S = *reinterpret_cast<set_cache *>(shb + resolve_cache_at(R, CH, MC));
+        unsigned long long base;
+        if (loads_relative(Lg, R, n, A, W, base)) {  // uniform over the block
+            if (plan)
+                F = B <= blockDim.x ? resolve_relative<true, true>(rd, mem, A, W, S, cbuf, Cd, D, n, B, CH, R, status)
+                                    : resolve_relative<false, true>(rd, mem, A, W, S, cbuf, Cd, D, n, B, CH, R, status);
+            else
+                F = B <= blockDim.x ? resolve_relative<true, false>(rd, mem, A, W, S, cbuf, Cd, D, n, B, CH, R, status)
+                                    : resolve_relative<false, false>(rd, mem, A, W, S, cbuf, Cd, D, n, B, CH, R, status);
+            for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) Lg[r] = base + F[r];
+            return;
+        }
+    }
+    // loads 2^32 - n or more apart, batches longer than the stage, bounded loads: 64-bit
+    // loads and counts, every request of a key scanning its members
     for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) {
         L[r] = Lg[r];
         delta[r] = 0;
     }
-    const uint16_t *mem = stage_aux(rd, smem_aux, MC);
     if (rd.policy == CR_POLICY_CHWBL) {  // uniform over the block
         const unsigned long long tot0 = block_load_sum(L, R);
         resolve_batches<kResolveRing>(rd, mem, L, delta, cbuf, Cd, D, n, B, CH, R, tot0, status);
     } else if (rd.policy == CR_POLICY_P2C) {
         __syncthreads();  // orders the copies above
         resolve_batches<kResolvePair>(rd, mem, L, delta, cbuf, Cd, D, n, B, CH, R, 0ull, status);
-    } else if (plan_x && CH > 0) {
-        __syncthreads();
-        unsigned long long *L1 = reinterpret_cast<unsigned long long *>(px);
-        uint32_t *dl1 = reinterpret_cast<uint32_t *>(L1 + R);
-        set_cache &S = *reinterpret_cast<set_cache *>(px + (((size_t)R * 12 + 15) & ~(size_t)15));
-        if (resolve_batches_plan(rd, mem, L, L1, delta, dl1, S, cbuf, Cd, D, n, B, CH, R, status))
-            for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) L[r] = L1[r];
-        __syncthreads();
     } else {
         __syncthreads();
         resolve_batches<kResolvePlan>(rd, mem, L, delta, cbuf, Cd, D, n, B, CH, R, 0ull, status);
@@ -1354,7 +1465,7 @@ extern "C" int cr_route_batch(cr_ctx *ctx, const cr_plan *const *plans, const cr
     const uint64_t *key_dep = d_key;
     if (!warp_path) {
         void *pc;
-        CR_TRY(cr_scratch(ctx, SCR_ROUTE_DESC, (size_t)n * n_rep * sizeof(uint32_t), &pc));
+        CR_TRY(cr_scratch(ctx, SCR_ROUTE_DESC, (size_t)cand_row(n) * n_rep * sizeof(uint32_t), &pc));
         cand = (uint32_t *)pc;
     } else if (split && n_dep) {
         // the resolution reads the keys on its own stream: from a copy, so that the caller's
@@ -1429,12 +1540,12 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     }
     // staging chunk: a whole number of batches, at most kStage requests
     uint32_t CH = batch_B <= kStage ? (kStage / batch_B) * batch_B : 0u;  // 0: no staging
-    const size_t loads = (size_t)R * (sizeof(unsigned long long) + sizeof(uint32_t));
-    // plan replicas take the second load and count buffers and the key cache when they
-    // fit beside a stage of at least one batch (the stage shrinks by whole batches)
+    const size_t loads = resolve_stage_at(R);
+    // plan replicas take the key cache when it fits beside a stage of at least one batch
+    // (the stage shrinks by whole batches)
     bool any_plan = false;
     for (uint32_t i = 0; i < n_dep; ++i) any_plan |= args.d[args.dep[i]].policy <= CR_POLICY_CR_NOREPL;
-    const size_t px = resolve_plan_extra_bytes(R);
+    const size_t px = sizeof(set_cache);
     int plan_x = 0;
     if (any_plan && CH) {
         uint32_t ch = CH;
@@ -1448,13 +1559,17 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     if (plan_x) {
         const size_t fixed = loads + (size_t)CH * 8 + 16 + px;
         MC = (mc && fixed + mc * sizeof(uint16_t) <= kSmemBudget) ? mc : 0;
-        smem = resolve_plan_extra_at(R, CH, MC) + px;
+        smem = resolve_cache_at(R, CH, MC) + px;
     } else {
         smem = with_members(loads + 2ull * CH * sizeof(uint32_t), &MC);
     }
     if (smem > 48 * 1024)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_route_resolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CR_LAUNCH_ON(ctx, rs, k_route_resolve, n_dep, kRouteBlock, smem, args, (const uint32_t *)cand, (unsigned long long)n,
+    // no more threads than a batch has requests (a barrier of idle warps costs time), but
+    // enough to stage candidates
+    const uint32_t threads = batch_B >= (uint32_t)kRouteBlock ? (uint32_t)kRouteBlock
+                                                              : std::max(256u, (batch_B + 31u) / 32u * 32u);
+    CR_LAUNCH_ON(ctx, rs, k_route_resolve, n_dep, threads, smem, args, (const uint32_t *)cand, (unsigned long long)n,
               batch_B, CH, R, (unsigned long long *)d_load, d_dest, ctx->d_status, (unsigned long long)MC, plan_x);
     return CR_OK;
 }

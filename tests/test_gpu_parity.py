@@ -480,6 +480,45 @@ def test_route_small_batches_load_ranges(P, ctx, R, B, n, loads):
     assert (h_u64(load) == ref_load).all()
 
 
+@pytest.mark.parametrize("R", [31, 700])
+@pytest.mark.parametrize("B", [33, 700, 1024, 1025, 4096, 4097])
+@pytest.mark.parametrize("loads", ["zero", "high", "limit", "spread"])
+def test_route_batches_load_ranges(P, ctx, R, B, loads):
+    # batches of more than 32: the loop on 32-bit relative loads (one request per thread and
+    # batch up to 1024, up to four above) and the 64-bit one that larger batches and loads
+    # 2^32 - n or more apart take; keys with short and long member lists, some of them met
+    # only in a later staging chunk
+    rng = np.random.default_rng(R + B)
+    n = 37000
+    hot = rng.integers(1, 2**63, 14, dtype=np.int64).astype(np.uint64)
+    planned = np.concatenate([np.repeat(hot, 40 * (1 + np.arange(14) * 2)),
+                              rng.integers(1, 2**63, 900, dtype=np.int64).astype(np.uint64)])
+    opl = O.build_plan(planned, R, 4, 12, 1)   # k_b = ceil(lambda / 12): 4 .. 90, at most R
+    dpl = P.build_plan(ctx, d_u64(planned), P.plan_params(R, 4, 12, 1))
+    assert 1 < np.asarray(opl.adm_k).max() <= R
+    keys = planned[rng.integers(0, planned.size, n)]
+    keys[:20000] = np.where(np.isin(keys[:20000], hot[8:]), hot[0], keys[:20000])
+    fresh = rng.random(n) < 0.3
+    keys[fresh] = rng.integers(1, 2**63, int(fresh.sum()), dtype=np.int64).astype(np.uint64)
+    pols, seeds = ["CR", "P2C", "CHWBL", "CR"], [3, 1, 2, 7]
+    init = rng.integers(0, 9, (4, R)).astype(np.uint64)
+    if loads == "high":
+        init += np.uint64(2**47)
+    elif loads == "limit":
+        init[:, 0] = np.uint64(2**32 - 2 - n)  # the largest difference of the 32-bit loop
+        init[:, 1] = 0
+    elif loads == "spread":
+        init[:, : (R + 1) // 2] += np.uint64(2**32)
+    orings = [None, None, O.Ring(R, 16, 5), None]
+    drings = [None, None, P.Ring(ctx, R, 16, 5), None]
+    ref_dest, ref_load = O.route([opl, None, None, opl], pols, seeds, R, keys, 99, B, load=init, rings=orings)
+    load = d_u64(init.reshape(-1)).view(4, R).contiguous()
+    dest = P.route_batch(ctx, [dpl, None, None, dpl], pols, seeds, R, d_u64(keys), 99, B, load, rings=drings)
+    ctx.sync()
+    assert (h_u16(dest) == ref_dest).all()
+    assert (h_u64(load) == ref_load).all()
+
+
 @pytest.mark.parametrize("case", ["few", "many", "pool", "wide"])
 @pytest.mark.parametrize("B", [100, 1024])
 def test_route_replicated_keys_per_batch(P, ctx, case, B):
