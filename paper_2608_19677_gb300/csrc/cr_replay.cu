@@ -113,8 +113,9 @@ __global__ void __launch_bounds__(kPartBlock) k_part_count(const uint16_t *__res
 
 // start[s] = first record of stream s = (replica, r); start[ns] = number of records.
 __global__ void k_part_starts(const uint32_t *__restrict__ off, uint32_t ns, uint32_t ntiles,
-                              const uint32_t *__restrict__ total, uint32_t *__restrict__ start)
+                              const uint32_t *__restrict__ total, uint32_t *__restrict__ start, uint32_t *next)
 {
+    if (blockIdx.x == 0 && threadIdx.x < 3) next[threadIdx.x] = 0;  // the work items' counters
     for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s <= ns; s += gridDim.x * blockDim.x)
         start[s] = s < ns ? off[(unsigned long long)s * ntiles] : *total;
 }
@@ -263,21 +264,58 @@ __global__ void k_part_records(const unsigned long long *__restrict__ keys, cons
     }
 }
 
-// The stream of every work item: items coff[s] .. coff[s + 1] - 1 belong to stream s
-// (coff[ns] is the total), written at wmap[item].
-__global__ void k_item_streams(const uint32_t *__restrict__ coff, uint32_t ns, uint32_t *__restrict__ wmap,
-                               uint64_t items_max)
+// Work items: every stream's chunks (an empty stream gets one that carries its state
+// over); all but a stream's last have CL requests.  Items longer than `longer` requests come
+// first, so that the launch does not end with a few SMs on a hot key's stream (sticky-hash
+// replicas have streams 13 times the mean: SMs were busy 78% of the launch; 48 replicas x
+// 1,066,667 requests, 2.23 -> 1.90 ms a call).
+__device__ __forceinline__ uint32_t long_chunks(uint32_t len, uint32_t nch, uint32_t CL, uint32_t longer)
 {
-    for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += gridDim.x * blockDim.x)
-        for (uint32_t w = coff[s]; w < coff[s + 1] && w < items_max; ++w) wmap[w] = s;
+    return (CL > longer ? nch - 1u : 0u) + (len - (nch - 1u) * CL > longer ? 1u : 0u);
 }
 
-// Chunks per stream (an empty stream still gets one work item that carries its state over).
-__global__ void k_chunk_counts(const uint32_t *__restrict__ start, uint32_t ns, uint32_t CL, uint32_t *__restrict__ nch)
+// nch[s] = chunks of stream s; next[2] += the long ones.
+__global__ void k_chunk_counts(const uint32_t *__restrict__ start, uint32_t ns, uint32_t CL, uint32_t longer,
+                               uint32_t *__restrict__ nch, uint32_t *next)
 {
+    uint32_t nf = 0;
     for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += gridDim.x * blockDim.x) {
         const uint32_t len = start[s + 1] - start[s];
-        nch[s] = len ? (len + CL - 1) / CL : 1u;
+        const uint32_t c = len ? (len + CL - 1) / CL : 1u;
+        nch[s] = c;
+        nf += long_chunks(len, c, CL, longer);
+    }
+    nf = __reduce_add_sync(0xffffffffu, nf);
+    if ((threadIdx.x & 31u) == 0 && nf) atomicAdd(&next[2], nf);
+}
+
+// map[x] and map[items_max + x]: item x's stream and chunk.  coff[s]: chunks of the streams
+// before s; next[0], next[1]: long and other items placed so far.
+__global__ void k_item_map(const uint32_t *__restrict__ start, const uint32_t *__restrict__ coff, uint32_t ns,
+                           uint32_t CL, uint32_t longer, uint32_t *next, uint32_t *__restrict__ map,
+                           uint64_t items_max)
+{
+    const uint32_t lane = threadIdx.x & 31u, first = next[2];
+    for (uint32_t s0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; s0 < ns; s0 += gridDim.x * blockDim.x) {
+        const uint32_t s = s0 + lane;
+        const bool in = s < ns;
+        const uint32_t len = in ? start[s + 1] - start[s] : 0u, nch = in ? coff[s + 1] - coff[s] : 0u;
+        const uint32_t nf = nch ? long_chunks(len, nch, CL, longer) : 0u;
+        const uint32_t fi = warp_incl_scan(nf, lane), bi = warp_incl_scan(nch - nf, lane);
+        uint32_t f0 = 0, b0 = 0;
+        if (lane == 31) {
+            if (fi) f0 = atomicAdd(&next[0], fi);
+            if (bi) b0 = atomicAdd(&next[1], bi);
+        }
+        f0 = __shfl_sync(0xffffffffu, f0, 31) + fi - nf;
+        b0 = __shfl_sync(0xffffffffu, b0, 31) + first + bi - (nch - nf);
+        for (uint32_t c = 0; c < nch; ++c) {
+            const uint32_t x = min(len - c * CL, CL) > longer ? f0++ : b0++;
+            if (x < items_max) {
+                map[x] = s;
+                map[items_max + x] = c;
+            }
+        }
     }
 }
 
@@ -550,7 +588,7 @@ __device__ __forceinline__ void sl_compact(const window_lru &X, uint32_t live, u
 template <int NC, int NG, bool SMALL>
 __global__ void __launch_bounds__(128, 5)
 k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t nb, uint32_t R,
-             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ coff,
+             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ map, uint32_t items_max,
              const uint32_t *__restrict__ total, const uint32_t *__restrict__ idx, const rec16 *__restrict__ recs,
              uint32_t nrec, const replay_state st, unsigned long long *__restrict__ ctr, uint32_t *status)
 {
@@ -561,7 +599,7 @@ k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw
 
     const uint32_t w = blockIdx.x * wpb + warp;
     if (w >= *total) return;
-    const uint32_t s = min(coff[ns + 2 + w], ns - 1u), ci = w - coff[s];  // the item's stream and chunk
+    const uint32_t s = min(map[w], ns - 1u), ci = map[items_max + w];  // the item's stream and chunk
     const uint32_t b = start[s], e = start[s + 1];
     const uint32_t p0 = b + ci * CL;
     const uint32_t p1 = (e - p0) < CL ? e : p0 + CL;
@@ -600,16 +638,27 @@ k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw
             }
         }
     } else {
-        // walk backwards collecting distinct keys, most recent first
+        // walk backwards collecting distinct keys, most recent first; keys are loaded two
+        // steps early, through request indices read four steps early (in a hot key's stream
+        // the walk is long, and nothing else hides the two dependent loads)
         for (uint32_t x = lane; x < nw; x += 32) X.BM[x] = 0;
         __syncwarp();
         const uint32_t back = p0 - b;
         const uint32_t vtot = back + fill_in;
+        auto index_at = [&](uint32_t v) { return v < back ? min(idx[p0 - 1u - v], nrec - 1u) : 0u; };
+        auto key_at = [&](uint32_t v, uint32_t ix) {
+            return v < back ? recs[ix].key : (v < vtot ? kin[v - back] : 0ull);
+        };
+        uint32_t ix2 = index_at(lane + 64u), ix3 = index_at(lane + 96u);
+        unsigned long long k0 = key_at(lane, index_at(lane)), k1 = key_at(lane + 32u, index_at(lane + 32u));
         for (uint32_t v0 = 0; v0 < vtot && live < cmax; v0 += 32) {
             const uint32_t v = v0 + lane;
             const bool valid = v < vtot;
-            unsigned long long key = 0;
-            if (valid) key = v < back ? recs[min(idx[p0 - 1 - v], nrec - 1u)].key : kin[v - back];
+            const unsigned long long key = k0;
+            k0 = k1;
+            k1 = key_at(v + 64u, ix2);
+            ix2 = ix3;
+            ix3 = index_at(v + 128u);
             const uint32_t vm = __ballot_sync(0xffffffffu, valid);
             const uint32_t peers = __match_any_sync(0xffffffffu, key) & vm;
             const key_hash H = sl_hash(X, key);
@@ -805,7 +854,7 @@ uint32_t window_warps(size_t per_warp, uint32_t regs, uint32_t *per_sm)
 
 template <int NC, int NG, bool SMALL>
 int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t CL, const uint32_t *start,
-                  const uint32_t *coff, const uint32_t *total, uint64_t m, const uint32_t *idx,
+                  const uint32_t *map, uint32_t items_max, const uint32_t *total, uint64_t m, const uint32_t *idx,
                   const rec16 *recs, uint64_t *d_ctr)
 {
     const uint32_t cmax = rp->cmax, nw = window_words(cmax), nb = window_buckets(nw);
@@ -830,7 +879,7 @@ int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t C
     st.fill_out = rp->d_fill[rp->cur ^ 1];
     const int pr = cr_prof_begin(ctx, ctx->stream, CR_PROF_REPLAY);
     CR_LAUNCH(ctx, (k_lru_stamp<NC, NG, SMALL>), (unsigned int)((items + wpb - 1) / wpb), wpb * 32, smem, caps, cmax,
-              nw, nb, rp->R, ns, CL, start, coff, total, idx, recs, (uint32_t)(m / rp->n_rep), st,
+              nw, nb, rp->R, ns, CL, start, map, items_max, total, idx, recs, (uint32_t)(m / rp->n_rep), st,
               (unsigned long long *)d_ctr,
               ctx->d_status);
     cr_prof_end(ctx, ctx->stream, pr);
@@ -840,26 +889,26 @@ int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t C
 
 template <int NC>
 int launch_stamp_nc(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t CL, const uint32_t *start,
-                    const uint32_t *coff, const uint32_t *total, uint64_t m, const uint32_t *idx,
+                    const uint32_t *map, uint32_t items_max, const uint32_t *total, uint64_t m, const uint32_t *idx,
                  const rec16 *recs, uint64_t *d_ctr)
 {
     uint32_t cmin = 0xffffffffu;
     for (uint32_t c = 0; c < caps.n_caps; ++c) cmin = caps.cap[c] < cmin ? caps.cap[c] : cmin;
     const bool small = cmin < 32;  // a repeat within a step can miss only below capacity 32
     if (window_words(rp->cmax) <= 32)
-        return small ? launch_stamp<NC, 1, true>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr)
-                     : launch_stamp<NC, 1, false>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr);
-    return small ? launch_stamp<NC, 2, true>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr)
-                 : launch_stamp<NC, 2, false>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr);
+        return small ? launch_stamp<NC, 1, true>(ctx, rp, caps, CL, start, map, items_max, total, m, idx, recs, d_ctr)
+                     : launch_stamp<NC, 1, false>(ctx, rp, caps, CL, start, map, items_max, total, m, idx, recs, d_ctr);
+    return small ? launch_stamp<NC, 2, true>(ctx, rp, caps, CL, start, map, items_max, total, m, idx, recs, d_ctr)
+                 : launch_stamp<NC, 2, false>(ctx, rp, caps, CL, start, map, items_max, total, m, idx, recs, d_ctr);
 }
 
 int launch_batch(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t CL, const uint32_t *start,
-                 const uint32_t *coff, const uint32_t *total, uint64_t m, const uint32_t *idx,
+                 const uint32_t *map, uint32_t items_max, const uint32_t *total, uint64_t m, const uint32_t *idx,
                  const rec16 *recs, uint64_t *d_ctr)
 {
-    if (caps.n_caps == 1) return launch_stamp_nc<1>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr);
-    if (caps.n_caps <= 3) return launch_stamp_nc<3>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr);
-    return launch_stamp_nc<CR_MAX_CAPS>(ctx, rp, caps, CL, start, coff, total, m, idx, recs, d_ctr);
+    if (caps.n_caps == 1) return launch_stamp_nc<1>(ctx, rp, caps, CL, start, map, items_max, total, m, idx, recs, d_ctr);
+    if (caps.n_caps <= 3) return launch_stamp_nc<3>(ctx, rp, caps, CL, start, map, items_max, total, m, idx, recs, d_ctr);
+    return launch_stamp_nc<CR_MAX_CAPS>(ctx, rp, caps, CL, start, map, items_max, total, m, idx, recs, d_ctr);
 }
 
 // ---- token-weighted variant ---------------------------------------------------
@@ -897,7 +946,7 @@ struct token_state {
 
 __global__ void __launch_bounds__(kTokWarps * 32) k_lru_tokens(const __grid_constant__ replay_caps caps, uint32_t ns,
                                                                uint32_t R, uint32_t CL, const uint32_t *__restrict__ start,
-                                                               const uint32_t *__restrict__ coff,
+                                                               const uint32_t *__restrict__ map, uint32_t items_max,
                                                                const uint32_t *__restrict__ total,
                                                                const uint32_t *__restrict__ idx,
                                                                const rec16 *__restrict__ recs, uint32_t nrec,
@@ -908,8 +957,7 @@ __global__ void __launch_bounds__(kTokWarps * 32) k_lru_tokens(const __grid_cons
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t wi = blockIdx.x * kTokWarps + w;
     if (wi >= *total) return;  // whole warps only; the kernel has no block-wide barrier
-    // work item -> (stream, chunk)
-    const uint32_t s = min(coff[ns + 2 + wi], ns - 1u), ci = wi - coff[s];
+    const uint32_t s = min(map[wi], ns - 1u), ci = map[items_max + wi];  // the item's stream and chunk
     const uint32_t b = start[s], e = start[s + 1];
     unsigned long long *K = tok_sh + (size_t)w * kTokMax;
     uint32_t *Cm = reinterpret_cast<uint32_t *>(tok_sh + (size_t)kTokWarps * kTokMax) + (size_t)w * kTokMax;
@@ -1235,7 +1283,8 @@ struct cr_replay_input {
     rec16 *d_recs;               // [n]
     uint32_t *d_cnt;             // [ns * ntiles + 2]: tile counts -> offsets, and their total
     uint32_t *d_start;           // [ns + 1]
-    uint32_t *d_coff;            // [ns + 2 + items]: work-item offsets, their total, then each item's stream
+    uint32_t *d_coff;            // [ns + 4]: work-item offsets, their total, k_item_map's counters; then its map
+    uint32_t items_max;          // upper bound on the work items; the map is [2 items_max]
     uint64_t cap_m, cap_n, cap_cnt, cap_ns, cap_coff;
 };
 
@@ -1306,8 +1355,17 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
         // chunks long against the rebuild walk, which reaches back until the largest capacity fills
         in->CL = capmax <= (1u << 16) ? 1024u : (capmax <= (1u << 17) ? 4096u : 16384u);
     } else {
-        // long enough that rebuilding an LRU state of cmax entries is amortised
-        in->CL = rp->cmax * 16u > 256u ? rp->cmax * 16u : 256u;
+        // about one chunk per warp that the GPU holds at once, but long enough that
+        // rebuilding an LRU state of cmax entries is amortised, and not so long that one hot
+        // stream outlasts the rest.  Against 16 cmax whatever the call's size: 30 replicas x
+        // 133,333 over 64 destinations at cmax 128 230 -> 214 us; two streams of 100,000 at cmax
+        // 1024 1.7-5.3 -> 0.36 ms; 160 streams of 62,500 6.2 -> 0.91 ms
+        const uint32_t nw = window_words(rp->cmax);
+        uint32_t per_sm = 1;
+        window_warps(window_lru_bytes(nw, window_buckets(nw)), 96, &per_sm);
+        const uint64_t fill = m / ((uint64_t)ctx->num_sms * per_sm);
+        const uint32_t lo = rp->cmax * 4u > 256u ? rp->cmax * 4u : 256u, hi = rp->cmax * 32u > 256u ? rp->cmax * 32u : 256u;
+        in->CL = fill < lo ? lo : (fill > hi ? hi : (uint32_t)fill);
     }
     if (n == 0) return CR_OK;
     CR_TRY(grow_u32(ctx, &in->d_idx, &in->cap_m, m));
@@ -1315,9 +1373,11 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     CR_TRY(grow_u32(ctx, &in->d_cnt, &in->cap_cnt, ncnt + 2));
     CR_TRY(grow_u32(ctx, &in->d_start, &in->cap_ns, (uint64_t)ns + 2));
     const uint64_t items_max = (uint64_t)ns + m / in->CL + 1;  // every stream's chunks, at least one each
-    CR_TRY(grow_u32(ctx, &in->d_coff, &in->cap_coff, (uint64_t)ns + 2 + items_max));
+    in->items_max = (uint32_t)items_max;
+    CR_TRY(grow_u32(ctx, &in->d_coff, &in->cap_coff, (uint64_t)ns + 4 + 2 * items_max));
     uint32_t *cnt = in->d_cnt, *nrec = cnt + ncnt, *start = in->d_start;
-    uint32_t *coff = in->d_coff, *total = coff + ns;
+    uint32_t *coff = in->d_coff, *total = coff + ns, *next = coff + ns + 1;
+    const uint32_t longer = (uint32_t)(2u * (n / R + 1u));  // twice the mean stream
     const unsigned int gcap = (unsigned int)ctx->num_sms * 8u;
     const dim3 pgrid(ntiles, rp->n_rep);
     const size_t csmem = (size_t)R * sizeof(uint32_t), ssmem = part_scatter_smem(R);
@@ -1332,13 +1392,14 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
               ctx->d_status);
     CR_TRY(cr_scan_u32(ctx, cnt, cnt, ncnt, nrec));
     CR_LAUNCH(ctx, k_part_starts, cr_blocks((uint64_t)ns + 1, 256, gcap), 256, 0, (const uint32_t *)cnt, ns, ntiles,
-              (const uint32_t *)nrec, start);
+              (const uint32_t *)nrec, start, next);
     CR_LAUNCH(ctx, k_part_scatter, pgrid, kPartBlock, ssmem, d_dest, (unsigned long long)n, R, ntiles,
               (const uint32_t *)cnt, in->d_idx, (unsigned long long)m);
-    CR_LAUNCH(ctx, k_chunk_counts, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, ns, in->CL, coff);
+    CR_LAUNCH(ctx, k_chunk_counts, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, ns, in->CL, longer, coff,
+              next);
     CR_TRY(cr_scan_u32(ctx, coff, coff, ns, total));
-    CR_LAUNCH(ctx, k_item_streams, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)coff, ns, coff + ns + 2,
-              items_max);
+    CR_LAUNCH(ctx, k_item_map, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, (const uint32_t *)coff, ns,
+              in->CL, longer, next, coff + ns + 4, items_max);
     cr_prof_end(ctx, ctx->stream, pp);
     return CR_OK;
 }
@@ -1353,7 +1414,7 @@ extern "C" int cr_replay_simulate(cr_ctx *ctx, cr_replay *rp, const cr_replay_in
     if (!d_ctr) return cr_fail(ctx, CR_EINVAL, "cr_replay_simulate: d_ctr is NULL");
     const uint32_t R = rp->R, ns = in->ns;
     const uint64_t m = in->m, n = in->n;
-    const uint32_t *start = in->d_start, *coff = in->d_coff, *total = in->d_coff + ns;
+    const uint32_t *start = in->d_start, *map = in->d_coff + ns + 4, *total = in->d_coff + ns;
     replay_caps caps;
     caps.n_caps = rp->n_caps;
     for (uint32_t c = 0; c < CR_MAX_CAPS; ++c) caps.cap[c] = c < rp->n_caps ? rp->caps[c] : 0;
@@ -1373,13 +1434,13 @@ extern "C" int cr_replay_simulate(cr_ctx *ctx, cr_replay *rp, const cr_replay_in
         const uint64_t items = (uint64_t)ns + (m + TCL - 1) / TCL;  // upper bound on work items
         const int pt = cr_prof_begin(ctx, ctx->stream, CR_PROF_REPLAY);
         CR_LAUNCH(ctx, k_lru_tokens, (unsigned int)((items + kTokWarps - 1) / kTokWarps), kTokWarps * 32, tsmem,
-                  caps, ns, R, TCL, start, coff, total, (const uint32_t *)in->d_idx, (const rec16 *)in->d_recs,
+                  caps, ns, R, TCL, start, map, in->items_max, total, (const uint32_t *)in->d_idx, (const rec16 *)in->d_recs,
                   (uint32_t)n, tst, (unsigned long long *)d_ctr, ctx->d_status);
         cr_prof_end(ctx, ctx->stream, pt);
         rp->cur ^= 1;
         return CR_OK;
     }
-    return launch_batch(ctx, rp, caps, in->CL, start, coff, total, m, in->d_idx, in->d_recs, d_ctr);
+    return launch_batch(ctx, rp, caps, in->CL, start, map, in->items_max, total, m, in->d_idx, in->d_recs, d_ctr);
 }
 
 extern "C" int cr_shadow_replay(cr_ctx *ctx, cr_replay *rp, const uint64_t *d_key, const uint32_t *d_plen,

@@ -1216,6 +1216,36 @@ def test_replay_parity_colliding_keys(P, ctx, caps, ncoll):
                 assert (st[:c] == orp.state(rep, c_i, r)).all()
 
 
+@pytest.mark.parametrize("tokens", [False, True])
+@pytest.mark.parametrize("R,hot", [(40, [7]), (700, [3, 200, 699]), (700, list(range(0, 700, 9))), (33, [])])
+def test_replay_items_of_long_streams(P, ctx, tokens, R, hot):
+    # streams longer than twice the mean take the first work items: none, a few, and one in
+    # nine of them, in whole chunks and in one, with empty streams between
+    rng = np.random.default_rng(R + len(hot))
+    n_rep, n = 3, 24000
+    caps = [400000] if tokens else [16, 1000]
+    keys = _rates_keys(rng, 4000, n)[:n]
+    n = keys.size
+    plen = (16 + keys % np.uint64(3000)).astype(np.uint32)
+    slen = np.full(n, 64, np.uint32)
+    dest = rng.integers(0, R, size=(n_rep, n)).astype(np.uint16)
+    if hot:
+        to = rng.random((n_rep, n)) < 0.8
+        dest[to] = rng.choice(np.array(hot, np.uint16), size=int(to.sum()))
+    dest[dest == 5] = 4
+    orp = O.Replay(n_rep, R, caps, tokens=tokens)
+    rp = P.Replay(ctx, n_rep, R, caps, tokens=tokens)
+    ctr = torch.zeros((n_rep, len(caps), R, 5), dtype=torch.int64, device=DEV)
+    dk, dp, ds, dd = d_u64(keys), d_u32(plen), d_u32(slen), d_u16(dest)
+    cut = n // 3
+    for a, b in ((0, cut), (cut, n)):
+        orp.step(keys[a:b], plen[a:b], slen[a:b], dest[:, a:b])
+        P.shadow_replay(ctx, rp, dk[a:b].contiguous(), dp[a:b].contiguous(), ds[a:b].contiguous(),
+                        dd[:, a:b].contiguous(), ctr)
+        ctx.sync()
+        assert (h_u64(ctr) == orp.ctr).all()
+
+
 def test_replay_state_import_resumes(P, ctx):
     # replay two calls in one simulator set; export every state after the first, import
     # it into a fresh set, and the second call's counters match
