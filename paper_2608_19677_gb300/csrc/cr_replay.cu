@@ -13,7 +13,7 @@
 //              most recent entries of any larger one.
 //   state      kept between calls as keys in recency order (most recent first).
 //   tokens     the byte-aware variant (cr_replay_create_tokens): capacities in
-//              prefix tokens, one warp walking each stream (k_lru_tokens).
+//              prefix tokens, the same window with each time's tokens (k_lru_tokens).
 #include <stdlib.h>
 #include <string.h>
 
@@ -378,11 +378,16 @@ struct window_lru {
     uint32_t *stash_n;        // stash entries claimed (| kDegraded once it overflowed)
     uint16_t *PX;             // [nw] compaction: live bits below each word
     uint32_t nw, nb, tmask;   // words, buckets, (1 << tb) - 1
+    // token capacities only
+    uint32_t *TK;             // [32 nw] prefix tokens of the request at each time
+    uint32_t *SL, *SH;        // [nw] a word's live tokens: sum of their low 16 bits, sum of the rest
+    uint2 *OP;                // [32] the step's requests: order of their keys at its start, tokens
 };
 
-__host__ __device__ inline size_t window_lru_bytes(uint32_t nw, uint32_t nb)
+__host__ __device__ inline size_t window_lru_bytes(uint32_t nw, uint32_t nb, bool tokens = false)
 {
-    return ((size_t)nw * 256 + (size_t)nb * 8 + kStash * 2 + (size_t)(nw + 1) * 4 + (size_t)nw * 2 + 15) & ~(size_t)15;
+    const size_t base = (size_t)nw * 256 + (size_t)nb * 8 + kStash * 2 + (size_t)(nw + 1) * 4 + (size_t)(nw + 1) / 2 * 4;
+    return (base + (tokens ? (size_t)nw * 136 + 32 * 8 + 8 : 0) + 15) & ~(size_t)15;
 }
 
 __device__ __forceinline__ window_lru window_lru_at(unsigned char *base, uint32_t nw, uint32_t nb)
@@ -397,6 +402,10 @@ __device__ __forceinline__ window_lru window_lru_at(unsigned char *base, uint32_
     X.nw = nw;
     X.nb = nb;
     X.tmask = (1u << (32 - __clz(32u * nw - 1u))) - 1u;
+    X.TK = reinterpret_cast<uint32_t *>(X.PX + (nw + 1u) / 2u * 2u);
+    X.SL = X.TK + (size_t)nw * 32;
+    X.SH = X.SL + nw;
+    X.OP = reinterpret_cast<uint2 *>((reinterpret_cast<uintptr_t>(X.SH + nw) + 7u) & ~(uintptr_t)7u);
     return X;
 }
 
@@ -544,7 +553,7 @@ struct live_prefix {
 
 // Keep the `fill` most recent of the window's `live` keys, renumbered 0 .. fill-1 in
 // order: every index entry takes its new time (or is emptied), then the keys move down.
-template <int NG>
+template <int NG, bool TOKENS = false>
 __device__ __forceinline__ void sl_compact(const window_lru &X, uint32_t live, uint32_t fill, uint32_t lane)
 {
     live_prefix<NG> LP;
@@ -572,8 +581,12 @@ __device__ __forceinline__ void sl_compact(const window_lru &X, uint32_t live, u
     for (uint32_t w = 0; w < X.nw; ++w) {
         const uint32_t bits = X.BM[w], rank = X.PX[w] + (uint32_t)__popc(bits & ((1u << lane) - 1u));
         const unsigned long long k = X.KT[32u * w + lane];
+        const uint32_t tk = TOKENS ? X.TK[32u * w + lane] : 0u;
         __syncwarp();
-        if (((bits >> lane) & 1u) && rank >= drop) X.KT[rank - drop] = k;
+        if (((bits >> lane) & 1u) && rank >= drop) {
+            X.KT[rank - drop] = k;
+            if (TOKENS) X.TK[rank - drop] = tk;
+        }
         __syncwarp();
     }
     sl_live_range(X, 0, fill, lane);
@@ -828,6 +841,14 @@ inline uint32_t window_words(uint32_t cmax)
     return (cmax + 31) / 32 + 12;
 }
 
+// The same for token capacities, whose lists may hold 1024 prefixes but, up to 65,536 tokens,
+// seldom hold a hundred: four steps then cost few compactions and leave room for 12 warps per
+// SM instead of 10 (24,576 tokens: 331 -> 261 us).
+inline uint32_t token_words(uint32_t capmax)
+{
+    return capmax <= (1u << 16) ? CR_MAX_CAP / 32u + 4u : window_words(CR_MAX_CAP);
+}
+
 // Index buckets of a window: 1.5 entries per time, so that two full buckets are rare even
 // when every request of the window has a key of its own.
 inline uint32_t window_buckets(uint32_t nw) { return 12u * nw; }
@@ -912,27 +933,43 @@ int launch_batch(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t C
 }
 
 // ---- token-weighted variant ---------------------------------------------------
-// Capacities count prefix tokens.  With one prefix length per key, the cache
-// of capacity c holds the longest run of most recent prefixes whose tokens fit
-// in c (evictions always take the least recent), so one list at the largest
-// capacity decides every capacity: a request hits at c iff its key is listed
-// and the tokens from the front of the list through the key are <= c.  One
-// warp per (replica, destination) stream walks the stream's requests in
-// order.  The list holds keys and CUMULATIVE tokens (entry j: the tokens of
-// entries 0..j), so a lookup is a ballot plus one read, moving a key to the
-// front adds its length to the entries it passes, and eviction is a ballot on
-// the tail.  A list of at most 32 prefixes lives in registers (lane j holds
-// entry j; the move is a shuffle-up); a longer one lives in shared memory and
-// is scanned 32 entries at a time.  Only hits and hit tokens depend on the
-// capacity; request and prompt totals are summed once per 32 records.
-constexpr int kTokWarps = 4;
+// Capacities count prefix tokens.  With one prefix length per key, the cache of capacity
+// c holds the longest run of most recent prefixes whose tokens fit in c (evictions always
+// take the least recent), so a request hits at c iff its key is among the kTokMax most
+// recent and the tokens of the keys from the most recent through it are <= c.  The same
+// window as above (times, bitmap of last accesses, index), with the tokens of every time
+// and each word's live tokens: a step takes 32 requests of the stream, one per lane.
+// The tokens above a key at the step's start are those of the words above its own (one
+// warp scan) plus the live times above it in its word, added one by one; a word whose
+// words above already exceed the largest capacity is not looked into.  The step's own
+// requests count for request i when they are the last of their key before i and, for a
+// first occurrence, their key was deeper than i's or absent (for a repeat, when they
+// follow its previous occurrence): one pass over the 32 lanes.  Sums saturate at
+// 2^32 - 1, above every capacity (<= 2^31).
+//
+// One request at a time over a list in recency order took 84 warp instructions per
+// (request, replica) pair.  20 replicas x 166,667 requests over 30 destinations, 24,576
+// tokens, partition included: 594 -> 265 us.  Bound, as above: the latency of a step's
+// dependence chain at 12 warps per SM.
 constexpr uint32_t kTokMax = CR_MAX_CAP;  // prefixes per list
+// Below this largest capacity a step's sums of prefixes cut to it cannot pass 2^32.
+constexpr uint32_t kTokNarrow = 1u << 26;
 
 __device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b)
 {
-    // a sum past 2^32 - 1 is above every capacity (<= 2^31) and is evicted anyway
-    const unsigned long long v = (unsigned long long)a + b;
-    return v > 0xffffffffull ? 0xffffffffu : (uint32_t)v;
+    const uint32_t v = a + b;
+    return v < a ? 0xffffffffu : v;
+}
+
+// Inclusive sum over the lanes from this one up.
+__device__ __forceinline__ uint32_t warp_sat_suffix(uint32_t v, uint32_t lane)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_down_sync(0xffffffffu, v, o);
+        if (lane + (uint32_t)o < 32u) v = sat_add(v, y);
+    }
+    return v;
 }
 
 struct token_state {
@@ -944,29 +981,68 @@ struct token_state {
     uint32_t *fill_out;
 };
 
-__global__ void __launch_bounds__(kTokWarps * 32) k_lru_tokens(const __grid_constant__ replay_caps caps, uint32_t ns,
-                                                               uint32_t R, uint32_t CL, const uint32_t *__restrict__ start,
-                                                               const uint32_t *__restrict__ map, uint32_t items_max,
-                                                               const uint32_t *__restrict__ total,
-                                                               const uint32_t *__restrict__ idx,
-                                                               const rec16 *__restrict__ recs, uint32_t nrec,
-                                                               const token_state st,
-                                                               unsigned long long *__restrict__ ctr, uint32_t *status)
+// Each word's live tokens from the bitmap and the times' tokens (words below `wend`;
+// cleared above).
+__device__ __forceinline__ void tk_word_sums(const window_lru &X, uint32_t wend, uint32_t lane)
 {
-    extern __shared__ unsigned long long tok_sh[];
-    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t wi = blockIdx.x * kTokWarps + w;
-    if (wi >= *total) return;  // whole warps only; the kernel has no block-wide barrier
-    const uint32_t s = min(map[wi], ns - 1u), ci = map[items_max + wi];  // the item's stream and chunk
+    for (uint32_t w = 0; w < X.nw; ++w) {
+        const uint32_t bits = w < wend ? X.BM[w] : 0u;
+        const uint32_t v = ((bits >> lane) & 1u) ? X.TK[32u * w + lane] : 0u;
+        const uint32_t l = __reduce_add_sync(0xffffffffu, v & 0xffffu), h = __reduce_add_sync(0xffffffffu, v >> 16);
+        if (lane == 0) {
+            X.SL[w] = l;
+            X.SH[w] = h;
+        }
+    }
+    __syncwarp();
+}
+
+// The cached list from the most recent key down, each(position, time, tokens through it):
+// the live keys of the words below wend whose tokens fit in capmax, at most kTokMax.
+// Returns their count.
+template <typename Each>
+__device__ __forceinline__ uint32_t tk_list(const window_lru &X, uint32_t wend, uint32_t capmax, uint32_t lane, Each each)
+{
+    uint32_t n = 0, cum = 0;
+    for (uint32_t w = wend; w-- > 0;) {
+        const uint32_t bits = X.BM[w];
+        if (!bits) continue;
+        const bool live = (bits >> lane) & 1u;
+        const uint32_t c = sat_add(cum, warp_sat_suffix(live ? X.TK[32u * w + lane] : 0u, lane));
+        const uint32_t q = n + (uint32_t)__popc(bits & ~((2u << lane) - 1u));
+        const bool fits = live && c <= capmax && q < kTokMax;
+        const uint32_t fm = __ballot_sync(0xffffffffu, fits);
+        if (fits) each(q, 32u * w + lane, c);
+        n += (uint32_t)__popc(fm);
+        if (fm != bits) break;  // everything older is further down the list
+        cum = __shfl_sync(0xffffffffu, c, 0);
+    }
+    return n;
+}
+
+template <int NC>
+__global__ void __launch_bounds__(128, 4)
+k_lru_tokens(const __grid_constant__ replay_caps caps, uint32_t capmax, uint32_t nw, uint32_t nb, uint32_t R,
+             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ map,
+             uint32_t items_max, const uint32_t *__restrict__ total, const uint32_t *__restrict__ idx,
+             const rec16 *__restrict__ recs, uint32_t nrec, const token_state st,
+             unsigned long long *__restrict__ ctr, uint32_t *status)
+{
+    extern __shared__ uint4 smb[];
+    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const window_lru X =
+        window_lru_at(reinterpret_cast<unsigned char *>(smb) + window_lru_bytes(nw, nb, true) * warp, nw, nb);
+    const uint32_t w = blockIdx.x * wpb + warp;
+    if (w >= *total) return;  // whole warps only; the kernel has no block-wide barrier
+    const uint32_t s = min(map[w], ns - 1u), ci = map[items_max + w];  // the item's stream and chunk
     const uint32_t b = start[s], e = start[s + 1];
-    unsigned long long *K = tok_sh + (size_t)w * kTokMax;
-    uint32_t *Cm = reinterpret_cast<uint32_t *>(tok_sh + (size_t)kTokWarps * kTokMax) + (size_t)w * kTokMax;
-    uint32_t capmax = 0;
-    for (uint32_t c = 0; c < caps.n_caps; ++c) capmax = caps.cap[c] > capmax ? caps.cap[c] : capmax;
-    const uint32_t mycap = lane < caps.n_caps ? caps.cap[lane] : 0u;
-    const uint32_t fin = st.fill_in[s];
+    const uint32_t p0 = b + ci * CL;
+    const uint32_t p1 = (e - p0) < CL ? e : p0 + CL;
+    const uint32_t rep = s / R, r = s % R;
+    const uint32_t fin = min(st.fill_in[s], kTokMax);
     const unsigned long long *kin = st.keys_in + (size_t)s * kTokMax;
     const uint32_t *cin = st.cum_in + (size_t)s * kTokMax;
+    const uint32_t lt = (1u << lane) - 1u, gt = ~(lt | (1u << lane));
     if (b == e) {  // nothing routed here: carry the state over unchanged
         for (uint32_t j = lane; j < fin; j += 32) {
             st.keys_out[(size_t)s * kTokMax + j] = kin[j];
@@ -975,203 +1051,300 @@ __global__ void __launch_bounds__(kTokWarps * 32) k_lru_tokens(const __grid_cons
         if (lane == 0) st.fill_out[s] = fin;
         return;
     }
-    const uint32_t i0 = b + ci * CL;
-    const uint32_t i1 = (e - i0) < CL ? e : i0 + CL;
-    uint32_t f = 0;
+
+    // ---- state at p0: the cached keys at the highest times below `top` ----------------
+    uint32_t live = 0, top = kTokMax;
+    sl_clear_index(X, lane);
+    for (uint32_t x = lane; x < nw; x += 32) X.BM[x] = 0;
+    __syncwarp();
     if (ci == 0) {
-        f = fin;
-        for (uint32_t j = lane; j < f; j += 32) {
-            K[j] = kin[j];
-            Cm[j] = cin[j];
+        top = live = fin;
+        for (uint32_t q = lane; q < fin; q += 32) {
+            const unsigned long long key = kin[q];
+            const key_hash H = sl_hash(X, key);
+            X.KT[top - 1u - q] = key;
+            X.TK[top - 1u - q] = cin[q] - (q ? cin[q - 1u] : 0u);
+            sl_insert(X, H, top - 1u - q);
         }
     } else {
-        // the state at i0 is the longest run of most recent distinct prefixes that fits
-        // (tokens <= the largest capacity, at most kTokMax of them): walk back over the
-        // stream, then over the carried-in list, keeping each key's most recent access
-        const uint32_t back = i0 - b;
-        uint32_t tot = 0;
+        // the state at p0 is the longest run of most recent distinct prefixes that fits:
+        // walk back over the stream, then over the carried-in list, keeping each key's most
+        // recent access; the first distinct prefix that does not fit ends the run
+        const uint32_t back = p0 - b, vtot = back + fin;
+        uint32_t cum = 0;
         bool stop = false;
-        for (uint32_t v0 = 0; v0 < back + fin && !stop; v0 += 32) {
-            const uint32_t v = v0 + lane;
-            unsigned long long ck = 0;
-            uint32_t cp = 0;
+        auto index_at = [&](uint32_t v) { return v < back ? min(idx[p0 - 1u - v], nrec - 1u) : 0u; };
+        auto load = [&](uint32_t v, uint32_t ix, unsigned long long &key, uint32_t &P) {
+            key = 0;
+            P = 0;
             if (v < back) {
-                const rec16 rr = recs[min(idx[i0 - 1 - v], nrec - 1u)];
-                ck = rr.key;
-                cp = rr.P;
-            } else if (v < back + fin) {
+                const rec16 x = recs[ix];
+                key = x.key;
+                P = x.P;
+            } else if (v < vtot) {
                 const uint32_t j = v - back;
-                ck = kin[j];
-                cp = cin[j] - (j ? cin[j - 1] : 0u);
+                key = kin[j];
+                P = cin[j] - (j ? cin[j - 1u] : 0u);
             }
-            const uint32_t nb = min(32u, back + fin - v0);
-            for (uint32_t q = 0; q < nb; ++q) {  // uniform over the warp
-                const unsigned long long x = __shfl_sync(0xffffffffu, ck, q);
-                const uint32_t P = __shfl_sync(0xffffffffu, cp, q);
-                bool seen = false;
-                for (uint32_t c0 = 0; c0 < f && !seen; c0 += 32)
-                    seen = __ballot_sync(0xffffffffu, c0 + lane < f && K[c0 + lane] == x) != 0;
-                if (seen) continue;
-                const unsigned long long nt = (unsigned long long)tot + P;
-                if (f == kTokMax || nt > capmax) {  // the first distinct prefix that does not fit ends the run
-                    stop = true;
-                    break;
-                }
-                tot = (uint32_t)nt;
-                if (lane == 0) {
-                    K[f] = x;
-                    Cm[f] = tot;
-                }
-                ++f;
-                __syncwarp();
+        };
+        unsigned long long kn;
+        uint32_t Pn, ixn = index_at(lane + 32u);
+        load(lane, index_at(lane), kn, Pn);
+        for (uint32_t v0 = 0; v0 < vtot && live < kTokMax && !stop; v0 += 32) {
+            const bool valid = v0 + lane < vtot;
+            const unsigned long long key = kn;
+            const uint32_t P = Pn;
+            load(v0 + 32u + lane, ixn, kn, Pn);
+            ixn = index_at(v0 + 64u + lane);
+            const uint32_t vm = __ballot_sync(0xffffffffu, valid);
+            const uint32_t peers = __match_any_sync(0xffffffffu, key) & vm;
+            const key_hash H = sl_hash(X, key);
+            uint32_t at, loc;
+            const bool fresh = valid && (peers & lt) == 0 && !sl_lookup(X, H, key, (kTokMax + 31u) / 32u, at, loc);
+            const uint32_t bal = __ballot_sync(0xffffffffu, fresh);
+            const uint32_t pos = live + (uint32_t)__popc(bal & lt);
+            uint32_t c = fresh ? P : 0u;  // tokens through this lane
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, c, o);
+                if (lane >= (uint32_t)o) c = sat_add(c, y);
             }
+            c = sat_add(c, cum);
+            const uint32_t over = __ballot_sync(0xffffffffu, fresh && (c > capmax || pos >= kTokMax));
+            const uint32_t take = over ? bal & ((1u << (__ffs(over) - 1)) - 1u) : bal;
+            __syncwarp();
+            if ((take >> lane) & 1u) {
+                const uint32_t t = top - 1u - pos;
+                X.KT[t] = key;
+                X.TK[t] = P;
+                atomicOr(&X.BM[t >> 5], 1u << (t & 31u));  // (a degraded index is searched through the bitmap)
+                sl_insert(X, H, t);
+            }
+            live += (uint32_t)__popc(take);
+            cum = __shfl_sync(0xffffffffu, c, 31);
+            stop = over != 0;
+            __syncwarp();
         }
     }
+    sl_live_range(X, top - live, live, lane);
+    uint32_t wnow = (top + 31u) / 32u;
     __syncwarp();
-    unsigned long long kr = 0;  // register list: entry `lane`
-    uint32_t cr = 0;
-    bool inreg = f <= 32;
-    if (inreg && lane < f) {
-        kr = K[lane];
-        cr = Cm[lane];
-    }
-    __syncwarp();
-    unsigned long long c_hit = 0, c_hit_tok = 0, c_prompt = 0;  // lane = capacity (prompt: every lane)
-    rec16 nx = {0ull, 0u, 0u};
-    if (i0 + lane < i1) nx = recs[min(idx[i0 + lane], nrec - 1u)];
-    for (uint32_t b0 = i0; b0 < i1; b0 += 32) {
-        const rec16 cur = nx;
-        if (b0 + 32 + lane < i1) nx = recs[min(idx[b0 + 32 + lane], nrec - 1u)];  // next 32 in flight
-        const uint32_t nb = i1 - b0 < 32 ? i1 - b0 : 32;
-        if (lane < nb) c_prompt += (unsigned long long)cur.P + cur.S;
-        for (uint32_t q = 0; q < nb; ++q) {
-            const unsigned long long x = __shfl_sync(0xffffffffu, cur.key, q);
-            const uint32_t P = __shfl_sync(0xffffffffu, cur.P, q);
-            bool found;
-            uint32_t upto = 0, zx = 0;
-            if (inreg) {
-                // ---- list in registers (f <= 32) ----
-                const unsigned match = __ballot_sync(0xffffffffu, lane < f && kr == x);
-                found = match != 0;
-                const uint32_t pos = found ? __ffs(match) - 1 : f;
-                const uint32_t cprev = __shfl_sync(0xffffffffu, cr, pos == 0 ? 0 : pos - 1);
-                if (found) {
-                    upto = __shfl_sync(0xffffffffu, cr, pos);
-                    zx = upto - (pos ? cprev : 0u);
-                }
-                // entries [0, pos) move down one place and now follow x
-                const unsigned long long kup = __shfl_up_sync(0xffffffffu, kr, 1);
-                const uint32_t cup = __shfl_up_sync(0xffffffffu, cr, 1);
-                const unsigned long long k31 = __shfl_sync(0xffffffffu, kr, 31);
-                const uint32_t c31 = __shfl_sync(0xffffffffu, cr, 31);
-                if (lane == 0) {
-                    kr = x;
-                    cr = P;
-                } else if (lane <= pos) {
-                    kr = kup;
-                    cr = sat_add(cup, P);
-                }
-                if (!found) ++f;  // f may reach 33: entry 32 is the old entry 31
-                const unsigned over = __ballot_sync(0xffffffffu, lane < f && cr > capmax);
-                if (over) {
-                    f = __ffs(over) - 1;  // the 33rd entry, if any, lies beyond and goes too
-                } else if (f == 33) {
-                    const uint32_t c32 = sat_add(c31, P);
-                    if (c32 > capmax) {
-                        f = 32;
-                    } else {  // the list outgrows the registers
-                        K[lane] = kr;
-                        Cm[lane] = cr;
-                        if (lane == 0) {
-                            K[32] = k31;
-                            Cm[32] = c32;
-                        }
-                        __syncwarp();
-                        inreg = false;
-                    }
+    tk_word_sums(X, wnow, lane);
+
+    unsigned long long my_prompt = 0, my_tok[NC];
+    uint32_t my_hit[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) my_hit[c] = 0, my_tok[c] = 0;
+
+    const bool wide = capmax >= kTokNarrow;
+    // records are gathered one step early, through request indices read two steps early
+    rec16 ahead = {0ull, 0u, 0u};
+    if (p0 + lane < p1) ahead = recs[min(idx[p0 + lane], nrec - 1u)];  // (the bound guards the gather)
+    uint32_t ix_next = p0 + 32u + lane < p1 ? idx[p0 + 32u + lane] : 0u;
+    for (uint32_t t0 = p0; t0 < p1; t0 += 32) {
+        if (wnow == nw) {
+            const uint32_t keep = tk_list(X, wnow, capmax, lane, [](uint32_t, uint32_t, uint32_t) {});
+            sl_compact<2, true>(X, live, keep, lane);
+            live = keep;
+            wnow = (live + 31u) / 32u;
+            tk_word_sums(X, wnow, lane);
+        }
+        const uint32_t cnt = (p1 - t0) < 32u ? (p1 - t0) : 32u;
+        const bool valid = lane < cnt;
+        const rec16 mine = ahead;
+        if (t0 + 32u + lane < p1) {
+            (void)CR_DCHECK(ix_next < nrec, status);
+            ahead = recs[min(ix_next, nrec - 1u)];
+        }
+        ix_next = t0 + 64u + lane < p1 ? idx[t0 + 64u + lane] : 0u;
+        if (valid) my_prompt += (unsigned long long)mine.P + mine.S;
+        const uint32_t now = 32u * wnow + lane;
+        X.KT[now] = mine.key;
+        X.TK[now] = mine.P;
+        const uint32_t vm = cnt == 32 ? 0xffffffffu : (1u << cnt) - 1u;
+        const uint32_t grp = __match_any_sync(0xffffffffu, mine.key) & vm;
+        const uint32_t below = grp & lt, above = grp & gt;
+        const bool first = valid && below == 0;
+        const bool last = valid && above == 0;
+        const key_hash H = sl_hash(X, mine.key);
+        uint32_t s_old = 0, loc = kNone;
+        const bool found = valid && sl_lookup(X, H, mine.key, wnow, s_old, loc);
+        const bool res = first && found;
+
+        // tokens of the words above each word (group g: words 32 g .. 32 g + 31)
+        uint32_t ab[2], sum1 = 0;
+#pragma unroll
+        for (int g = 1; g >= 0; --g) {
+            const uint32_t wi = 32u * g + lane;
+            const unsigned long long v = wi < nw ? X.SL[wi] + ((unsigned long long)X.SH[wi] << 16) : 0ull;
+            const uint32_t incl = warp_sat_suffix(v > 0xffffffffull ? 0xffffffffu : (uint32_t)v, lane);
+            const uint32_t y = __shfl_down_sync(0xffffffffu, incl, 1);
+            ab[g] = sat_add(lane < 31u ? y : 0u, sum1);
+            sum1 = __shfl_sync(0xffffffffu, incl, 0);
+        }
+        const uint32_t a0 = __shfl_sync(0xffffffffu, ab[0], (s_old >> 5) & 31u),
+                       a1 = __shfl_sync(0xffffffffu, ab[1], (s_old >> 5) & 31u);
+        uint32_t cum = s_old < 1024u ? a0 : a1;  // first occurrence: tokens through its key, at the step's start
+        uint32_t own = 0;                        // its key's tokens at its last access
+        if (res) {
+            own = X.TK[s_old];
+            cum = sat_add(cum, own);
+            uint32_t bits = X.BM[s_old >> 5] & ~((2u << (s_old & 31u)) - 1u);
+            for (; bits && cum <= capmax; bits &= bits - 1u)
+                cum = sat_add(cum, X.TK[(s_old & ~31u) + (uint32_t)__ffs(bits) - 1u]);
+        }
+        // its position, where the list is long enough for the limit on prefixes to matter
+        uint32_t pos = 0;
+        if (live + 32u > kTokMax) {  // uniform
+            live_prefix<2> LP;
+            LP.load(X.BM, nw, lane);
+            const uint32_t bl = LP.below(s_old);
+            pos = live - 1u - bl;
+        }
+        // a repeat: the step's requests since the previous occurrence
+        const uint32_t prev = below ? 31u - (uint32_t)__clz(below) : 0u;
+        const uint32_t P_prev = __shfl_sync(0xffffffffu, mine.P, prev);
+        if (valid && !first) {
+            own = P_prev;
+            cum = P_prev;
+            pos = 0;
+        }
+        // request j counts for request i when it is the last of its key before i (its next
+        // occurrence after lane i: M, compared bit-sliced) and its key was deeper or absent
+        // (order below i's) or, for a repeat i, j follows the previous occurrence
+        const uint32_t order = found ? s_old + 1u : 0u;
+        X.OP[lane] = make_uint2(order, wide ? mine.P : min(mine.P, kTokNarrow));
+        const bool open = valid && (first ? found : true) && cum <= capmax;  // not decided yet
+        __syncwarp();
+        if (__any_sync(0xffffffffu, open)) {
+            const uint32_t next = above ? (uint32_t)__ffs(above) - 1u : 32u;
+            uint32_t gN = 0, eN = 0xffffffffu;
+#pragma unroll
+            for (int bt = 5; bt >= 0; --bt) {
+                const uint32_t BN = __ballot_sync(0xffffffffu, (next >> bt) & 1u);
+                const uint32_t MN = 0u - ((lane >> bt) & 1u);
+                gN |= eN & BN & ~MN;
+                eN &= ~(BN ^ MN);
+            }
+            const uint32_t M = gN & lt & (first ? 0xffffffffu : ~((2u << prev) - 1u));
+            const uint32_t my_order = first ? order : 0xffffffffu;
+            uint32_t n_in = 0;
+            if (!wide) {
+#pragma unroll
+                for (uint32_t j = 0; j < 31; ++j) {
+                    const uint2 o = X.OP[j];
+                    const bool counts = ((M >> j) & 1u) && o.x < my_order;
+                    if (counts) cum += o.y;
+                    if (counts) ++n_in;
                 }
             } else {
-                // ---- list in shared memory (f > 32) ----
-                uint32_t pos = f;
-                for (uint32_t c0 = 0; c0 < f; c0 += 32) {
-                    const uint32_t j = c0 + lane;
-                    const unsigned match = __ballot_sync(0xffffffffu, j < f && K[j] == x);
-                    if (match) {
-                        pos = c0 + __ffs(match) - 1;
-                        break;
-                    }
+                for (uint32_t j = 0; j < 31; ++j) {
+                    const uint2 o = X.OP[j];
+                    const bool counts = ((M >> j) & 1u) && o.x < my_order;
+                    cum = sat_add(cum, counts ? o.y : 0u);
+                    n_in += counts ? 1u : 0u;
                 }
-                found = pos < f;
-                if (found) {
-                    upto = Cm[pos];
-                    zx = upto - (pos ? Cm[pos - 1] : 0u);
-                } else {
-                    if (f == kTokMax) --f;  // the least recent prefix makes room
-                    pos = f;
-                    ++f;
-                }
-                for (int c0 = (int)((pos + 31) / 32) * 32 - 32; c0 >= 0; c0 -= 32) {  // [0, pos) down one
-                    const uint32_t j = (uint32_t)c0 + lane;
-                    const bool m = j < pos;
-                    const unsigned long long k = m ? K[j] : 0ull;
-                    const uint32_t cm = m ? Cm[j] : 0u;
-                    __syncwarp();
-                    if (m) {
-                        K[j + 1] = k;
-                        Cm[j + 1] = sat_add(cm, P);
-                    }
-                    __syncwarp();
-                }
-                if (lane == 0) {
-                    K[0] = x;
-                    Cm[0] = P;
-                }
-                __syncwarp();
-                // the entries whose sums exceed the largest capacity form a suffix
-                for (int c0 = (int)((f + 31) / 32) * 32 - 32; c0 >= 0; c0 -= 32) {
-                    const uint32_t j = (uint32_t)c0 + lane;
-                    const unsigned over = __ballot_sync(0xffffffffu, j < f && Cm[j] > capmax);
-                    if (!over) break;
-                    f = (uint32_t)c0 + __ffs(over) - 1;
-                }
-                if (f <= 32) {  // back to registers
-                    kr = lane < f ? K[lane] : 0ull;
-                    cr = lane < f ? Cm[lane] : 0u;
-                    inreg = true;
-                }
-                __syncwarp();
             }
-            if (found && zx != P && lane == 0) atomicOr(status, CR_FLAG_BADSIZE);
-            if (found && upto <= mycap) {  // lanes past n_caps have mycap 0 < upto
-                c_hit += 1;
-                c_hit_tok += P;
+            pos += n_in;
+        }
+        const bool listed = open && cum <= capmax && pos < kTokMax;
+        if (listed && own != mine.P) atomicOr(status, CR_FLAG_BADSIZE);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            if (c < (int)caps.n_caps && listed && cum <= caps.cap[c]) {
+                my_hit[c] += 1;
+                my_tok[c] += mine.P;
+            }
+        }
+
+        // ---- state after the step: every key of the step takes its last access's time ----
+        const uint32_t absm = __ballot_sync(0xffffffffu, first && !found);
+        const uint32_t old = res ? X.TK[s_old] : 0u;
+        __syncwarp();  // (the bitmap, the sums and the index have been read)
+        if (res) {
+            atomicAnd(&X.BM[s_old >> 5], ~(1u << (s_old & 31u)));
+            atomicSub(&X.SL[s_old >> 5], old & 0xffffu);
+            atomicSub(&X.SH[s_old >> 5], old >> 16);
+        }
+        if (last && loc != kNone) X.E[loc] = (uint16_t)(H.tag | now);
+        const uint32_t lastm = __ballot_sync(0xffffffffu, last);
+        const uint32_t sl = __reduce_add_sync(0xffffffffu, last ? mine.P & 0xffffu : 0u),
+                       sh = __reduce_add_sync(0xffffffffu, last ? mine.P >> 16 : 0u);
+        __syncwarp();
+        if (last && !found) sl_insert(X, H, now);
+        if (lane == 0) {
+            X.BM[wnow] = lastm;
+            X.SL[wnow] = sl;
+            X.SH[wnow] = sh;
+        }
+        live += (uint32_t)__popc(absm);
+        ++wnow;
+        __syncwarp();
+    }
+
+    // ---- counters -------------------------------------------------------------
+    my_prompt = cr_warp_sum_u64(my_prompt);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        if (c < (int)caps.n_caps) {
+            const unsigned long long h = cr_warp_sum_u64(my_hit[c]);
+            const unsigned long long tk = cr_warp_sum_u64(my_tok[c]);
+            if (lane == 0) {
+                unsigned long long *C = ctr + (((unsigned long long)rep * caps.n_caps + c) * R + r) * CR_CTR_FIELDS;
+                atomicAdd(&C[0], (unsigned long long)(p1 - p0));
+                if (h) atomicAdd(&C[1], h);
+                if (tk) atomicAdd(&C[2], tk);
+                atomicAdd(&C[3], my_prompt);
+                atomicAdd(&C[4], my_prompt - tk);
             }
         }
     }
-    if (i1 == e) {  // the stream's last chunk hands the state to the next call
-        if (inreg) {
-            if (lane < f) {
-                st.keys_out[(size_t)s * kTokMax + lane] = kr;
-                st.cum_out[(size_t)s * kTokMax + lane] = cr;
-            }
-        } else {
-            for (uint32_t j = lane; j < f; j += 32) {
-                st.keys_out[(size_t)s * kTokMax + j] = K[j];
-                st.cum_out[(size_t)s * kTokMax + j] = Cm[j];
-            }
-        }
-        if (lane == 0) st.fill_out[s] = f;
+    if (p1 == e) {  // the stream's last chunk hands the state to the next call
+        unsigned long long *kout = st.keys_out + (size_t)s * kTokMax;
+        uint32_t *cout = st.cum_out + (size_t)s * kTokMax;
+        const uint32_t n = tk_list(X, wnow, capmax, lane, [&](uint32_t q, uint32_t t, uint32_t c) {
+            kout[q] = X.KT[t];
+            cout[q] = c;
+        });
+        if (lane == 0) st.fill_out[s] = n;
     }
-    for (int o = 16; o > 0; o >>= 1) c_prompt += __shfl_xor_sync(0xffffffffu, c_prompt, o);
-    if (lane < caps.n_caps) {
-        const uint32_t rep = s / R, r = s - rep * R;
-        unsigned long long *C = ctr + (((unsigned long long)rep * caps.n_caps + lane) * R + r) * CR_CTR_FIELDS;
-        atomicAdd(&C[0], (unsigned long long)(i1 - i0));
-        if (c_hit) atomicAdd(&C[1], c_hit);
-        if (c_hit_tok) atomicAdd(&C[2], c_hit_tok);
-        atomicAdd(&C[3], c_prompt);
-        atomicAdd(&C[4], c_prompt - c_hit_tok);
-    }
+}
+
+template <int NC>
+int launch_tokens(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t CL, const uint32_t *start,
+                  const uint32_t *map, uint32_t items_max, const uint32_t *total, uint64_t m, const uint32_t *idx,
+                  const rec16 *recs, uint64_t *d_ctr)
+{
+    uint32_t capmax = 0;
+    for (uint32_t c = 0; c < caps.n_caps; ++c) capmax = caps.cap[c] > capmax ? caps.cap[c] : capmax;
+    const uint32_t nw = token_words(capmax), nb = window_buckets(nw);
+    cudaFuncAttributes fa;
+    uint32_t regs = 96, per_sm = 0;
+    if (cudaFuncGetAttributes(&fa, k_lru_tokens<NC>) == cudaSuccess && fa.numRegs > 0)
+        regs = (uint32_t)fa.numRegs;
+    else
+        cudaGetLastError();
+    const size_t per_warp = window_lru_bytes(nw, nb, true);
+    const uint32_t wpb = window_warps(per_warp, regs, &per_sm);
+    const size_t smem = per_warp * wpb;
+    if (smem > 48 * 1024)
+        CR_CUDA(ctx, cudaFuncSetAttribute(k_lru_tokens<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const uint32_t ns = rp->n_rep * rp->R;
+    token_state st;
+    st.keys_in = rp->d_keys[rp->cur];
+    st.cum_in = rp->d_size[rp->cur];
+    st.fill_in = rp->d_fill[rp->cur];
+    st.keys_out = rp->d_keys[rp->cur ^ 1];
+    st.cum_out = rp->d_size[rp->cur ^ 1];
+    st.fill_out = rp->d_fill[rp->cur ^ 1];
+    const uint64_t items = (uint64_t)ns + (m + CL - 1) / CL;  // upper bound on work items
+    const int pt = cr_prof_begin(ctx, ctx->stream, CR_PROF_REPLAY);
+    CR_LAUNCH(ctx, (k_lru_tokens<NC>), (unsigned int)((items + wpb - 1) / wpb), wpb * 32, smem, caps, capmax, nw, nb,
+              rp->R, ns, CL, start, map, items_max, total, idx, recs, (uint32_t)(m / rp->n_rep), st,
+              (unsigned long long *)d_ctr, ctx->d_status);
+    cr_prof_end(ctx, ctx->stream, pt);
+    rp->cur ^= 1;
+    return CR_OK;
 }
 
 }  // namespace
@@ -1352,8 +1525,15 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     if (rp->tokens) {
         uint32_t capmax = 0;
         for (uint32_t c = 0; c < rp->n_caps; ++c) capmax = rp->caps[c] > capmax ? rp->caps[c] : capmax;
-        // chunks long against the rebuild walk, which reaches back until the largest capacity fills
-        in->CL = capmax <= (1u << 16) ? 1024u : (capmax <= (1u << 17) ? 4096u : 16384u);
+        // about two chunks per warp that the GPU holds at once (20 replicas x 166,667 requests:
+        // 512 / 768 / 1024 / 1536 requests measured 282 / 289 / 261 / 340 us), but long against
+        // the rebuild walk, which reaches back until the largest capacity fills
+        const uint32_t nw = token_words(capmax);
+        uint32_t per_sm = 1;
+        window_warps(window_lru_bytes(nw, window_buckets(nw), true), 96, &per_sm);
+        const uint64_t fill = (m / (2ull * ctx->num_sms * per_sm) + 255u) & ~255ull;
+        const uint32_t lo = capmax <= (1u << 16) ? 512u : (capmax <= (1u << 17) ? 1024u : 4096u);
+        in->CL = fill < lo ? lo : (fill > 16u * lo ? 16u * lo : (uint32_t)fill);
     } else {
         // about one chunk per warp that the GPU holds at once, but long enough that
         // rebuilding an LRU state of cmax entries is amortised, and not so long that one hot
@@ -1412,33 +1592,20 @@ extern "C" int cr_replay_simulate(cr_ctx *ctx, cr_replay *rp, const cr_replay_in
         return cr_fail(ctx, CR_EINVAL, "cr_replay_simulate: the input was partitioned for another replay shape");
     if (in->n == 0) return CR_OK;
     if (!d_ctr) return cr_fail(ctx, CR_EINVAL, "cr_replay_simulate: d_ctr is NULL");
-    const uint32_t R = rp->R, ns = in->ns;
-    const uint64_t m = in->m, n = in->n;
+    const uint32_t ns = in->ns;
+    const uint64_t m = in->m;
     const uint32_t *start = in->d_start, *map = in->d_coff + ns + 4, *total = in->d_coff + ns;
     replay_caps caps;
     caps.n_caps = rp->n_caps;
     for (uint32_t c = 0; c < CR_MAX_CAPS; ++c) caps.cap[c] = c < rp->n_caps ? rp->caps[c] : 0;
     if (rp->tokens) {
-        // token-weighted: one warp per (stream, chunk), its list in registers or shared memory
-        const uint32_t TCL = in->CL;
-        const size_t tsmem = (size_t)kTokWarps * kTokMax * (sizeof(unsigned long long) + sizeof(uint32_t));
-        if (tsmem > 48 * 1024)
-            CR_CUDA(ctx, cudaFuncSetAttribute(k_lru_tokens, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem));
-        token_state tst;
-        tst.keys_in = rp->d_keys[rp->cur];
-        tst.cum_in = rp->d_size[rp->cur];
-        tst.fill_in = rp->d_fill[rp->cur];
-        tst.keys_out = rp->d_keys[rp->cur ^ 1];
-        tst.cum_out = rp->d_size[rp->cur ^ 1];
-        tst.fill_out = rp->d_fill[rp->cur ^ 1];
-        const uint64_t items = (uint64_t)ns + (m + TCL - 1) / TCL;  // upper bound on work items
-        const int pt = cr_prof_begin(ctx, ctx->stream, CR_PROF_REPLAY);
-        CR_LAUNCH(ctx, k_lru_tokens, (unsigned int)((items + kTokWarps - 1) / kTokWarps), kTokWarps * 32, tsmem,
-                  caps, ns, R, TCL, start, map, in->items_max, total, (const uint32_t *)in->d_idx, (const rec16 *)in->d_recs,
-                  (uint32_t)n, tst, (unsigned long long *)d_ctr, ctx->d_status);
-        cr_prof_end(ctx, ctx->stream, pt);
-        rp->cur ^= 1;
-        return CR_OK;
+        const uint32_t *idx = in->d_idx;
+        if (caps.n_caps == 1)
+            return launch_tokens<1>(ctx, rp, caps, in->CL, start, map, in->items_max, total, m, idx, in->d_recs, d_ctr);
+        if (caps.n_caps <= 3)
+            return launch_tokens<3>(ctx, rp, caps, in->CL, start, map, in->items_max, total, m, idx, in->d_recs, d_ctr);
+        return launch_tokens<CR_MAX_CAPS>(ctx, rp, caps, in->CL, start, map, in->items_max, total, m, idx, in->d_recs,
+                                          d_ctr);
     }
     return launch_batch(ctx, rp, caps, in->CL, start, map, in->items_max, total, m, in->d_idx, in->d_recs, d_ctr);
 }
