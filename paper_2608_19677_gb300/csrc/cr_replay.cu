@@ -58,51 +58,36 @@ constexpr int kPartPer = 32;                      // requests per thread
 constexpr int kPartTile = kPartBlock * kPartPer;  // 8192
 constexpr uint32_t kNoDest = 0xffffu;
 
-// Counts of one tile in u32 bins [R], one shared-memory atomic add per item:
-// counting needs no order, so lane l of warp w takes the 32 consecutive items
-// 1024 w + 32 l .. + 31, read up front with four 16-byte loads.
+// Counts of one tile in u32 bins [R], one shared-memory atomic add per item.  A warp's
+// lanes take consecutive items, 16 loads of two bytes in flight each: a replica's row may
+// start on any even address (n is often odd), and round-robin destinations, consecutive in
+// memory, fall into different banks.  51 M destinations, R = 1024, n odd: 144 -> 53 us
+// against 32 consecutive items per lane.
 __global__ void __launch_bounds__(kPartBlock) k_part_count(const uint16_t *__restrict__ dest, unsigned long long n,
                                                            uint32_t R, uint32_t ntiles, uint32_t *__restrict__ cnt,
                                                            uint32_t *status)
 {
     extern __shared__ uint32_t pcb[];  // [R]
-    const uint32_t rep = blockIdx.y, tile = blockIdx.x, lane = cr_lane(), warp = threadIdx.x >> 5;
+    const uint32_t rep = blockIdx.y, tile = blockIdx.x, lane = cr_lane();
     for (uint32_t r = threadIdx.x; r < R; r += kPartBlock) pcb[r] = 0;
     __syncthreads();
     const uint16_t *D = dest + (unsigned long long)rep * n;
     const unsigned long long base = (unsigned long long)tile * kPartTile;
     const uint32_t cnt_t = (uint32_t)min((unsigned long long)kPartTile, n - base);
-    constexpr uint32_t kPerWarp = kPartTile / kPartWarps;
-    const uint32_t first = warp * kPerWarp + lane * 32u;
-    uint32_t dv[16];  // two destinations per word
-    const bool whole = base + first + 32u <= n && ((base + first) & 7u) == 0 &&
-                       ((reinterpret_cast<uintptr_t>(D) & 15u) == 0);
-    if (whole) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(D + base + first);
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const uint4 v = src[x];
-            dv[4 * x] = v.x;
-            dv[4 * x + 1] = v.y;
-            dv[4 * x + 2] = v.z;
-            dv[4 * x + 3] = v.w;
-        }
-    } else {
-#pragma unroll
-        for (int x = 0; x < 16; ++x) {
-            const uint32_t i0 = first + 2u * x, i1 = i0 + 1u;
-            const uint32_t a = i0 < cnt_t ? D[base + i0] : kNoDest, c = i1 < cnt_t ? D[base + i1] : kNoDest;
-            dv[x] = a | (c << 16);
-        }
-    }
     bool bad = false;
+    constexpr uint32_t kInFlight = 16;
+    for (uint32_t i0 = threadIdx.x; i0 < cnt_t; i0 += kPartBlock * kInFlight) {
+        uint32_t d[kInFlight];
 #pragma unroll
-    for (uint32_t j = 0; j < (uint32_t)kPartPer; ++j) {
-        const uint32_t d = (dv[j >> 1] >> (16 * (j & 1))) & 0xffffu;
-        if (first + j < cnt_t) {
-            if (d < R)
-                atomicAdd(&pcb[d], 1u);
-            else
+        for (uint32_t x = 0; x < kInFlight; ++x) {
+            const uint32_t i = i0 + x * kPartBlock;
+            d[x] = i < cnt_t ? D[base + i] : 0x10000u;
+        }
+#pragma unroll
+        for (uint32_t x = 0; x < kInFlight; ++x) {
+            if (d[x] < R)
+                atomicAdd(&pcb[d[x]], 1u);
+            else if (d[x] != 0x10000u)
                 bad = true;  // skipped: reported through the status word
         }
     }
@@ -120,25 +105,33 @@ __global__ void k_part_starts(const uint32_t *__restrict__ off, uint32_t ns, uin
         start[s] = s < ns ? off[(unsigned long long)s * ntiles] : *total;
 }
 
-// Shared memory of k_part_scatter: per-warp counters wc[8][R] (u16), the
-// tile's destination offsets toff[R] (u32), each item's (destination << 16 |
-// rank among its warp's items of that destination) (u32), and the tile's items
-// in (destination, arrival) order (u16 item numbers).
+// Shared memory of k_part_scatter: per-warp counters wc[8][R] (u16), the tile's
+// destination offsets toff[R] (u32), and the tile's items in (destination, arrival) order
+// (u32: destination << 16 | item number).
 __host__ __device__ inline size_t part_scatter_smem(uint32_t R)
 {
-    return (size_t)R * kPartWarps * 2 + (size_t)R * 4 + (size_t)kPartTile * 6;
+    return (size_t)R * kPartWarps * 2 + (size_t)R * 4 + (size_t)kPartTile * 4;
 }
 
-__global__ void __launch_bounds__(kPartBlock) k_part_scatter(const uint16_t *__restrict__ dest, unsigned long long n,
-                                                             uint32_t R, uint32_t ntiles,
-                                                             const uint32_t *__restrict__ off,
-                                                             uint32_t *__restrict__ out, unsigned long long m)
+// From this R on, a round's equal destinations are found by writing lane numbers to the
+// counters (BALLOTS false): few of 32 requests then share one.  Below, one ballot per bit
+// of the destination.
+constexpr uint32_t kPartSparse = 192;
+
+// Bound: instructions (ranking about half).  51 M destinations, R = 1024: 345 -> 239 us;
+// ranks are kept in registers instead of shared memory (a pass less; 80 registers, three
+// blocks per SM: four with 64 spill and take 315 us), and the lane numbers take about 20
+// instructions per 32 requests where a ballot per destination bit takes 50.
+template <bool BALLOTS>
+__global__ void __launch_bounds__(kPartBlock, 3) k_part_scatter(const uint16_t *__restrict__ dest, unsigned long long n,
+                                                                uint32_t R, uint32_t ntiles,
+                                                                const uint32_t *__restrict__ off,
+                                                                uint32_t *__restrict__ out, unsigned long long m)
 {
     extern __shared__ uint4 psm[];
     uint16_t *wc = reinterpret_cast<uint16_t *>(psm);                            // [8][R]
     uint32_t *toff = reinterpret_cast<uint32_t *>(wc + (size_t)R * kPartWarps);  // [R]
-    uint32_t *spk = toff + R;                                                    // [kPartTile]
-    uint16_t *sitem = reinterpret_cast<uint16_t *>(spk + kPartTile);            // [kPartTile]
+    uint32_t *sitem = toff + R;                                                  // [kPartTile]
     __shared__ uint32_t part[kPartBlock];
     __shared__ uint32_t s_valid;
     const uint32_t rep = blockIdx.y, tile = blockIdx.x, lane = cr_lane(), warp = threadIdx.x >> 5;
@@ -151,34 +144,51 @@ __global__ void __launch_bounds__(kPartBlock) k_part_scatter(const uint16_t *__r
     const uint32_t cnt = (uint32_t)min((unsigned long long)kPartTile, n - base);
     // ranks: warp w takes items [1024 w, 1024 w + 1024) of the tile, 32 at a time
     // (lane order is arrival order); all 32 rounds' destinations are read up front.
-    // The lanes of a round with equal destinations are found from one ballot per
-    // bit of the destination (R stands for "no item").
     constexpr uint32_t kPerWarp = kPartTile / kPartWarps;
     const uint32_t nb = 32u - (uint32_t)__clz(R);
-    uint16_t *wcw = wc + (size_t)warp * R;
-    uint32_t dv[kPartPer / 2];
+    volatile uint16_t *wcw = wc + (size_t)warp * R;
+    uint32_t dv[kPartPer / 2];  // two rounds' destinations per word (kNoDest: no item)
+    uint32_t rk[kPartPer / 2];  // and ranks among the warp's items of the destination
 #pragma unroll
     for (int x = 0; x < kPartPer / 2; ++x) {
         const uint32_t i0 = warp * kPerWarp + (2u * x) * 32u + lane, i1 = i0 + 32u;
         const uint32_t a = i0 < cnt ? D[base + i0] : kNoDest, c = i1 < cnt ? D[base + i1] : kNoDest;
-        dv[x] = a | (c << 16);
+        dv[x] = (a < R ? a : kNoDest) | ((c < R ? c : kNoDest) << 16);
+        rk[x] = 0;
     }
 #pragma unroll
     for (uint32_t j = 0; j < (uint32_t)kPartPer; ++j) {
-        const uint32_t it = warp * kPerWarp + j * 32u + lane;
-        uint32_t d = (dv[j >> 1] >> (16 * (j & 1))) & 0xffffu;
-        const uint32_t dd = d < R ? d : R;
-        if (d >= R) d = kNoDest;
-        uint32_t peers = 0xffffffffu;
-        for (uint32_t bt = 0; bt < nb; ++bt) {
-            const uint32_t bit = (dd >> bt) & 1u;
-            const uint32_t B = __ballot_sync(0xffffffffu, bit);
-            peers &= bit ? B : ~B;
+        const uint32_t d = (dv[j >> 1] >> (16 * (j & 1))) & 0xffffu;
+        const bool in = d != kNoDest;
+        const uint32_t before = in ? wcw[d] : 0u;
+        uint32_t peers = 1u << lane;  // the round's lanes with this destination
+        if (BALLOTS) {
+            // one ballot per bit of the destination (R stands for "no item")
+            const uint32_t dd = in ? d : R;
+            peers = 0xffffffffu;
+            for (uint32_t bt = 0; bt < nb; ++bt) {
+                const uint32_t bit = (dd >> bt) & 1u;
+                const uint32_t B = __ballot_sync(0xffffffffu, bit);
+                peers &= bit ? B : ~B;
+            }
+            __syncwarp();
+        } else {
+            // every lane writes its number to its counter: a lane that does not read it back
+            // shares its destination, and those lanes' destinations are settled one by one
+            __syncwarp();
+            if (in) wcw[d] = (uint16_t)lane;
+            __syncwarp();
+            uint32_t lost = __ballot_sync(0xffffffffu, in && wcw[d] != lane);
+            while (lost) {  // uniform; every pass settles at least one lane
+                const uint32_t dl = __shfl_sync(0xffffffffu, d, __ffs(lost) - 1);
+                const uint32_t same = __ballot_sync(0xffffffffu, d == dl);
+                if (d == dl) peers = same;
+                lost &= ~same;
+            }
+            __syncwarp();
         }
-        const uint32_t before = d != kNoDest ? wcw[d] : 0u;
-        spk[it] = (d << 16) | (before + (uint32_t)__popc(peers & lt));
-        __syncwarp();
-        if (d != kNoDest && (peers & lt) == 0) wcw[d] = (uint16_t)(before + __popc(peers));
+        rk[j >> 1] |= (before + (uint32_t)__popc(peers & lt)) << (16 * (j & 1));
+        if (in && (peers & lt) == 0) wcw[d] = (uint16_t)(before + __popc(peers));
         __syncwarp();
     }
     __syncthreads();
@@ -225,12 +235,12 @@ __global__ void __launch_bounds__(kPartBlock) k_part_scatter(const uint16_t *__r
     }
     __syncthreads();
     // staging: every valid item at its place in (destination, arrival) order
-    for (uint32_t it = threadIdx.x; it < cnt; it += kPartBlock) {
-        const uint32_t pk = spk[it];
-        const uint32_t d = pk >> 16;
+#pragma unroll
+    for (uint32_t j = 0; j < (uint32_t)kPartPer; ++j) {
+        const uint32_t d = (dv[j >> 1] >> (16 * (j & 1))) & 0xffffu;
         if (d == kNoDest) continue;
-        const uint32_t pos = toff[d] + wc[(size_t)(it / kPerWarp) * R + d] + (pk & 0xffffu);
-        sitem[pos] = (uint16_t)it;
+        const uint32_t pos = toff[d] + wc[(size_t)warp * R + d] + ((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu);
+        sitem[pos] = (d << 16) | (warp * kPerWarp + j * 32u + lane);
     }
     // each destination's output position minus its staging position (mod 2^32), in
     // the counters' space, which the staging no longer needs
@@ -242,11 +252,10 @@ __global__ void __launch_bounds__(kPartBlock) k_part_scatter(const uint16_t *__r
     // output: consecutive threads write consecutive positions of each destination's run
     const uint32_t valid = s_valid;
     for (uint32_t j = threadIdx.x; j < valid; j += kPartBlock) {
-        const uint32_t it = sitem[j];
-        const uint32_t d = spk[it] >> 16;
+        const uint32_t it = sitem[j], d = it >> 16;
         if (d >= R) continue;  // never: every staged item is valid (guards the writes)
         const uint32_t o = gb[d] + j;
-        if (o < m) out[o] = (uint32_t)(base + it);
+        if (o < m) out[o] = (uint32_t)base + (it & 0xffffu);
     }
 }
 
@@ -1563,8 +1572,9 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     const size_t csmem = (size_t)R * sizeof(uint32_t), ssmem = part_scatter_smem(R);
     if (csmem > 48 * 1024)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_part_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
+    auto *scatter = R >= kPartSparse ? k_part_scatter<false> : k_part_scatter<true>;
     if (ssmem > 48 * 1024)
-        CR_CUDA(ctx, cudaFuncSetAttribute(k_part_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
+        CR_CUDA(ctx, cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
     const int pp = cr_prof_begin(ctx, ctx->stream, CR_PROF_PARTITION);
     CR_LAUNCH(ctx, k_part_records, cr_blocks(n, 256, gcap), 256, 0, (const unsigned long long *)d_key, d_plen, d_slen,
               (unsigned long long)n, in->d_recs);
@@ -1573,7 +1583,7 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     CR_TRY(cr_scan_u32(ctx, cnt, cnt, ncnt, nrec));
     CR_LAUNCH(ctx, k_part_starts, cr_blocks((uint64_t)ns + 1, 256, gcap), 256, 0, (const uint32_t *)cnt, ns, ntiles,
               (const uint32_t *)nrec, start, next);
-    CR_LAUNCH(ctx, k_part_scatter, pgrid, kPartBlock, ssmem, d_dest, (unsigned long long)n, R, ntiles,
+    CR_LAUNCH(ctx, scatter, pgrid, kPartBlock, ssmem, d_dest, (unsigned long long)n, R, ntiles,
               (const uint32_t *)cnt, in->d_idx, (unsigned long long)m);
     CR_LAUNCH(ctx, k_chunk_counts, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, ns, in->CL, longer, coff,
               next);

@@ -1216,6 +1216,29 @@ def test_replay_parity_colliding_keys(P, ctx, caps, ncoll):
                 assert (st[:c] == orp.state(rep, c_i, r)).all()
 
 
+@pytest.mark.parametrize("R", [2, 191, 192, 193, 1024, 8192])
+@pytest.mark.parametrize("n", [1, 33, 8191, 8192, 8193, 24577])
+def test_replay_partition_edges(P, ctx, R, n):
+    # every stream in arrival order (capacity 1 counts exactly the immediate repeats): both
+    # ways of ranking equal destinations, tiles cut short, rows at odd addresses, and
+    # destinations that are random, round robin, equal, or shared by pairs and runs of lanes
+    rng = np.random.default_rng(R * 31 + n)
+    rows = [rng.integers(0, R, n), np.arange(n) % R, np.full(n, R - 1), (np.arange(n) // 2 * 7) % R,
+            np.where(rng.random(n) < 0.5, R // 2, rng.integers(0, R, n)), (np.arange(n) // 16) % R]
+    dest = np.stack(rows).astype(np.uint16)
+    keys = rng.integers(1, 6, n).astype(np.uint64)
+    plen = rng.integers(1, 5000, n).astype(np.uint32)
+    slen = np.full(n, 64, np.uint32)
+    caps = [1, 3]
+    orp = O.Replay(len(rows), R, caps)
+    rp = P.Replay(ctx, len(rows), R, caps)
+    ctr = torch.zeros((len(rows), len(caps), R, 5), dtype=torch.int64, device=DEV)
+    orp.step(keys, plen, slen, dest)
+    P.shadow_replay(ctx, rp, d_u64(keys), d_u32(plen), d_u32(slen), d_u16(dest), ctr)
+    ctx.sync()
+    assert (h_u64(ctr) == orp.ctr).all()
+
+
 @pytest.mark.parametrize("tokens", [False, True])
 @pytest.mark.parametrize("R,hot", [(40, [7]), (700, [3, 200, 699]), (700, list(range(0, 700, 9))), (33, [])])
 def test_replay_items_of_long_streams(P, ctx, tokens, R, hot):
