@@ -63,12 +63,29 @@ constexpr uint32_t kNoDest = 0xffffu;
 // start on any even address (n is often odd), and round-robin destinations, consecutive in
 // memory, fall into different banks.  51 M destinations, R = 1024, n odd: 144 -> 53 us
 // against 32 consecutive items per lane.
+// One more row of blocks packs a (key, prefix, suffix) record per request, read by the
+// replay through the indices.
 __global__ void __launch_bounds__(kPartBlock) k_part_count(const uint16_t *__restrict__ dest, unsigned long long n,
-                                                           uint32_t R, uint32_t ntiles, uint32_t *__restrict__ cnt,
-                                                           uint32_t *status)
+                                                           uint32_t R, uint32_t ntiles, uint32_t n_rep,
+                                                           uint32_t *__restrict__ cnt,
+                                                           const unsigned long long *__restrict__ keys,
+                                                           const uint32_t *__restrict__ plen,
+                                                           const uint32_t *__restrict__ slen,
+                                                           rec16 *__restrict__ recs, uint32_t *status)
 {
     extern __shared__ uint32_t pcb[];  // [R]
     const uint32_t rep = blockIdx.y, tile = blockIdx.x, lane = cr_lane();
+    if (rep == n_rep) {
+        const unsigned long long i0 = (unsigned long long)tile * kPartTile;
+        for (unsigned long long i = i0 + threadIdx.x; i < n && i < i0 + kPartTile; i += kPartBlock) {
+            rec16 r;
+            r.key = keys[i];
+            r.P = plen[i];
+            r.S = slen[i];
+            recs[i] = r;
+        }
+        return;
+    }
     for (uint32_t r = threadIdx.x; r < R; r += kPartBlock) pcb[r] = 0;
     __syncthreads();
     const uint16_t *D = dest + (unsigned long long)rep * n;
@@ -259,20 +276,6 @@ __global__ void __launch_bounds__(kPartBlock, 3) k_part_scatter(const uint16_t *
     }
 }
 
-// One (key, prefix, suffix) record per request, read by the replay through the indices.
-__global__ void k_part_records(const unsigned long long *__restrict__ keys, const uint32_t *__restrict__ plen,
-                               const uint32_t *__restrict__ slen, unsigned long long n, rec16 *__restrict__ recs)
-{
-    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (unsigned long long)gridDim.x * blockDim.x) {
-        rec16 r;
-        r.key = keys[i];
-        r.P = plen[i];
-        r.S = slen[i];
-        recs[i] = r;
-    }
-}
-
 // Work items: every stream's chunks (an empty stream gets one that carries its state
 // over); all but a stream's last have CL requests.  Items longer than `longer` requests come
 // first, so that the launch does not end with a few SMs on a hot key's stream (sticky-hash
@@ -318,6 +321,64 @@ __global__ void k_item_map(const uint32_t *__restrict__ start, const uint32_t *_
         }
         f0 = __shfl_sync(0xffffffffu, f0, 31) + fi - nf;
         b0 = __shfl_sync(0xffffffffu, b0, 31) + first + bi - (nch - nf);
+        for (uint32_t c = 0; c < nch; ++c) {
+            const uint32_t x = min(len - c * CL, CL) > longer ? f0++ : b0++;
+            if (x < items_max) {
+                map[x] = s;
+                map[items_max + x] = c;
+            }
+        }
+    }
+}
+
+// The same for up to kItemsCta streams by one CTA, stream starts included: one launch in
+// place of k_part_starts, k_chunk_counts, a scan and k_item_map.  Thread t takes `per`
+// consecutive streams.  30 replicas x 133,333 requests, 64 destinations,
+// with the records packed in the count launch: 212 -> 192 us a call; one interval of 20,000
+// requests, two replicas 154 -> 142 us.
+constexpr uint32_t kItemsCta = 8192;
+__global__ void __launch_bounds__(1024) k_items_cta(const uint32_t *__restrict__ off, uint32_t ns, uint32_t ntiles,
+                                                    const uint32_t *__restrict__ total_in,
+                                                    uint32_t *__restrict__ start, uint32_t CL, uint32_t longer,
+                                                    uint32_t *__restrict__ total, uint32_t *__restrict__ map,
+                                                    uint64_t items_max)
+{
+    __shared__ uint32_t wf[32], wb[32];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t per = (ns + 1023u) / 1024u, s0 = threadIdx.x * per, s1 = min(s0 + per, ns);
+    uint32_t st[kItemsCta / 1024 + 1];
+#pragma unroll
+    for (uint32_t k = 0; k <= kItemsCta / 1024; ++k) {
+        const uint32_t s = s0 + k;
+        st[k] = k > per || s > ns ? 0u : (s < ns ? off[(unsigned long long)s * ntiles] : *total_in);
+        if (k < per && s < ns) start[s] = st[k];
+    }
+    if (threadIdx.x == 0) start[ns] = *total_in;
+    uint32_t nf = 0, nb = 0;  // long and other chunks of this thread's streams
+#pragma unroll
+    for (uint32_t k = 0; k < kItemsCta / 1024; ++k) {
+        if (s0 + k >= s1) continue;
+        const uint32_t len = st[k + 1] - st[k], nch = len ? (len + CL - 1u) / CL : 1u;
+        const uint32_t f = long_chunks(len, nch, CL, longer);
+        nf += f;
+        nb += nch - f;
+    }
+    const uint32_t fi = warp_incl_scan(nf, lane), bi = warp_incl_scan(nb, lane);
+    if (lane == 31) {
+        wf[warp] = fi;
+        wb[warp] = bi;
+    }
+    __syncthreads();
+    const uint32_t fw = warp_incl_scan(wf[lane], lane), bw = warp_incl_scan(wb[lane], lane);  // over the 32 warps
+    const uint32_t first = __shfl_sync(0xffffffffu, fw, 31);
+    const uint32_t fp = __shfl_sync(0xffffffffu, fw, (warp + 31u) & 31u), bp = __shfl_sync(0xffffffffu, bw, (warp + 31u) & 31u);
+    uint32_t f0 = fi - nf + (warp ? fp : 0u), b0 = first + bi - nb + (warp ? bp : 0u);
+    if (threadIdx.x == 1023) *total = b0 + nb;
+#pragma unroll
+    for (uint32_t k = 0; k < kItemsCta / 1024; ++k) {
+        const uint32_t s = s0 + k;
+        if (s >= s1) continue;
+        const uint32_t len = st[k + 1] - st[k], nch = len ? (len + CL - 1u) / CL : 1u;
         for (uint32_t c = 0; c < nch; ++c) {
             const uint32_t x = min(len - c * CL, CL) > longer ? f0++ : b0++;
             if (x < items_max) {
@@ -1568,7 +1629,6 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     uint32_t *coff = in->d_coff, *total = coff + ns, *next = coff + ns + 1;
     const uint32_t longer = (uint32_t)(2u * (n / R + 1u));  // twice the mean stream
     const unsigned int gcap = (unsigned int)ctx->num_sms * 8u;
-    const dim3 pgrid(ntiles, rp->n_rep);
     const size_t csmem = (size_t)R * sizeof(uint32_t), ssmem = part_scatter_smem(R);
     if (csmem > 48 * 1024)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_part_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
@@ -1576,20 +1636,23 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     if (ssmem > 48 * 1024)
         CR_CUDA(ctx, cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
     const int pp = cr_prof_begin(ctx, ctx->stream, CR_PROF_PARTITION);
-    CR_LAUNCH(ctx, k_part_records, cr_blocks(n, 256, gcap), 256, 0, (const unsigned long long *)d_key, d_plen, d_slen,
-              (unsigned long long)n, in->d_recs);
-    CR_LAUNCH(ctx, k_part_count, pgrid, kPartBlock, csmem, d_dest, (unsigned long long)n, R, ntiles, cnt,
-              ctx->d_status);
+    CR_LAUNCH(ctx, k_part_count, dim3(ntiles, rp->n_rep + 1), kPartBlock, csmem, d_dest, (unsigned long long)n, R, ntiles,
+              rp->n_rep, cnt, (const unsigned long long *)d_key, d_plen, d_slen, in->d_recs, ctx->d_status);
     CR_TRY(cr_scan_u32(ctx, cnt, cnt, ncnt, nrec));
-    CR_LAUNCH(ctx, k_part_starts, cr_blocks((uint64_t)ns + 1, 256, gcap), 256, 0, (const uint32_t *)cnt, ns, ntiles,
-              (const uint32_t *)nrec, start, next);
-    CR_LAUNCH(ctx, scatter, pgrid, kPartBlock, ssmem, d_dest, (unsigned long long)n, R, ntiles,
+    CR_LAUNCH(ctx, scatter, dim3(ntiles, rp->n_rep), kPartBlock, ssmem, d_dest, (unsigned long long)n, R, ntiles,
               (const uint32_t *)cnt, in->d_idx, (unsigned long long)m);
-    CR_LAUNCH(ctx, k_chunk_counts, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, ns, in->CL, longer, coff,
-              next);
-    CR_TRY(cr_scan_u32(ctx, coff, coff, ns, total));
-    CR_LAUNCH(ctx, k_item_map, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, (const uint32_t *)coff, ns,
-              in->CL, longer, next, coff + ns + 4, items_max);
+    if (ns <= kItemsCta) {
+        CR_LAUNCH(ctx, k_items_cta, 1, 1024, 0, (const uint32_t *)cnt, ns, ntiles, (const uint32_t *)nrec, start, in->CL,
+                  longer, total, coff + ns + 4, items_max);
+    } else {
+        CR_LAUNCH(ctx, k_part_starts, cr_blocks((uint64_t)ns + 1, 256, gcap), 256, 0, (const uint32_t *)cnt, ns, ntiles,
+                  (const uint32_t *)nrec, start, next);
+        CR_LAUNCH(ctx, k_chunk_counts, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, ns, in->CL, longer,
+                  coff, next);
+        CR_TRY(cr_scan_u32(ctx, coff, coff, ns, total));
+        CR_LAUNCH(ctx, k_item_map, cr_blocks(ns, 256, gcap), 256, 0, (const uint32_t *)start, (const uint32_t *)coff, ns,
+                  in->CL, longer, next, coff + ns + 4, items_max);
+    }
     cr_prof_end(ctx, ctx->stream, pp);
     return CR_OK;
 }
