@@ -87,6 +87,7 @@ struct cr_plan_info_dev {
     unsigned long long n_adm, sum_k, cold, max_k, special;
     unsigned long long adm_lam;  // requests of the admitted keys
     unsigned long long by_rate;  // the candidates stand in admission order in ukey/ucnt, not in key order
+    unsigned long long trimmed;  // slot-capped: k_plan_place met a key that must get fewer replicas
 };
 
 struct cr_table_slot {               // 16 bytes: one sector-aligned probe

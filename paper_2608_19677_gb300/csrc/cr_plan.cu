@@ -28,6 +28,7 @@ namespace {
 
 constexpr uint32_t kEmpty = 0xffffffffu;
 constexpr unsigned long long kLoadLimit = 1ull << 47;
+constexpr uint32_t kPlaceMaxR = 1024;  // destinations of an LPT plan that k_plan_place takes
 
 __global__ void k_plan_reset(cr_plan_info_dev *info, unsigned long long n)
 {
@@ -41,6 +42,7 @@ __global__ void k_plan_reset(cr_plan_info_dev *info, unsigned long long n)
     info->max_k = 0;
     info->special = 0;
     info->by_rate = 0;
+    info->trimmed = 0;
 }
 
 // ---- histogram: counts in an L2-resident open-addressing table ----------
@@ -858,6 +860,7 @@ __global__ void __launch_bounds__(32) k_plan_lpt_capped(cr_plan_info_dev *info,
                                                         uint16_t *__restrict__ members,
                                                         unsigned long long *__restrict__ jobs, uint32_t *status)
 {
+    if (R <= kPlaceMaxR && !info->trimmed) return;  // k_plan_place has placed it
     extern __shared__ unsigned long long smem_u64[];
     unsigned long long *L = smem_u64;                                      // [R]
     uint32_t *slots = reinterpret_cast<uint32_t *>(L + R);                 // [R] replicas held
@@ -1017,6 +1020,8 @@ struct place_job {
     uint16_t *members;
     unsigned long long seed, epoch;
     uint32_t R;
+    uint32_t W;                 // slot-capped LPT: replicas a destination may hold (0: any number)
+    cr_plan_info_dev *info_w;   // and where `trimmed` is reported
 };
 
 struct place_jobs {
@@ -1057,7 +1062,6 @@ __global__ void __launch_bounds__(32) k_plan_lpt32_multi(const __grid_constant__
 // per random plan took 1,908 + 360 us.  R = 16, 919 keys, one LPT and three random plans:
 // 33 us (was 60 + 58).
 constexpr int kPlaceBlock = 512;
-constexpr uint32_t kPlaceMaxR = 1024;
 constexpr uint32_t kRunMin = 32;              // shortest run placed at once
 constexpr uint32_t kRunMaxQ = 1u << 20;       // f << 10 | r in 32 bits
 
@@ -1070,6 +1074,14 @@ struct lpt_smem {
     uint32_t wcnt[2][kPlaceBlock / 32], wnxt[2][kPlaceBlock / 32];
     uint32_t a, q, base;          // run: first key, λ, first member offset
     uint32_t done;
+};
+
+// Slot-capped plans: replicas each destination holds, the final loads of the full ones, and
+// a run's least free-slot count per warp.
+struct cap_smem {
+    unsigned long long fin[kPlaceMaxR];
+    uint32_t slots[kPlaceMaxR];
+    uint32_t wrem[2][kPlaceBlock / 32];
 };
 
 template <int NE, typename KT>
@@ -1142,7 +1154,10 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long v)
 
 // One run, by the whole CTA: S.a, S.q, S.base, S.rel set; returns the first key after it.
 // S.add[r] = jobs given to r.
-__device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, uint32_t R, uint32_t na,
+// CAP: a destination leaves the cycle when its W slots are used, so a stretch also ends
+// after as many rounds as its members have free slots.
+template <bool CAP>
+__device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, cap_smem &Q, uint32_t W, uint32_t R, uint32_t na,
                                             const unsigned long long *__restrict__ adm_cnt,
                                             uint16_t *__restrict__ members, unsigned long long *__restrict__ jobs)
 {
@@ -1165,7 +1180,7 @@ __device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, uint32_t R, uint32_t na
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
         const uint32_t r = 64u * warp + 32u * x + lane;
-        have[x] = r < R;
+        have[x] = r < R && (!CAP || Q.slots[r] < W);
         key[x] = r;
         if (have[x]) {
             const uint32_t L = S.rel[r], l = L / q;
@@ -1216,16 +1231,22 @@ __device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, uint32_t R, uint32_t na
         __syncthreads();
         if (have[0]) S.srt[S.cnt[d0 * kW + warp] + (uint32_t)__popc(s0 & lt)] = key[0];
         if (have[1]) S.srt[S.cnt[d1 * kW + warp] + (uint32_t)__popc(s10) + (uint32_t)__popc(s1 & lt)] = key[1];
+        if (CAP && sh == 10) {  // the sorted ones stand without gaps from here on
+            const uint32_t n = (uint32_t)__syncthreads_count(have[0]) + (uint32_t)__syncthreads_count(have[1]);
+            have[0] = 64u * warp + lane < n;
+            have[1] = 64u * warp + 32u + lane < n;
+        }
         __syncthreads();
 #pragma unroll
         for (int x = 0; x < 2; ++x)
             if (have[x]) key[x] = S.srt[64u * warp + 32u * x + lane];
     }
-    uint32_t r[2], lev[2], add[2] = {0, 0};
+    uint32_t r[2], lev[2], add[2] = {0, 0}, rem[2] = {0, 0};
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
         r[x] = key[x] & 1023u;
         lev[x] = have[x] ? S.rel[r[x]] : 0xffffffffu;
+        if (CAP && have[x]) rem[x] = W - Q.slots[r[x]];
     }
     // first level: minimum over the CTA
     uint32_t T;
@@ -1236,13 +1257,22 @@ __device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, uint32_t R, uint32_t na
         T = __reduce_min_sync(0xffffffffu, S.wnxt[1][lane & (kPlaceBlock / 32 - 1)]);
     }
     uint32_t left = hi - a, done = 0, par = 0;
-    while (left) {  // each stretch serves at least one job
+    while (left) {  // each stretch serves at least one job (CAP: or moves T up to a level)
+        if (CAP) {
+            have[0] = have[0] && rem[0] != 0;
+            have[1] = have[1] && rem[1] != 0;
+        }
         const bool in0 = have[0] && lev[0] <= T, in1 = have[1] && lev[1] <= T;
         const uint32_t b0 = __ballot_sync(0xffffffffu, in0), b1 = __ballot_sync(0xffffffffu, in1);
         uint32_t nx = 0xffffffffu;
         if (have[0] && !in0) nx = lev[0];
         if (have[1] && !in1) nx = lev[1] < nx ? lev[1] : nx;
         nx = __reduce_min_sync(0xffffffffu, nx);
+        if (CAP) {
+            const uint32_t f0 = in0 ? rem[0] : 0xffffffffu, f1 = in1 ? rem[1] : 0xffffffffu;
+            const uint32_t f = __reduce_min_sync(0xffffffffu, f0 < f1 ? f0 : f1);
+            if (lane == 0) Q.wrem[par][warp] = f;
+        }
         if (lane == 0) {
             S.wcnt[par][warp] = (uint32_t)(__popc(b0) + __popc(b1));
             S.wnxt[par][warp] = nx;
@@ -1253,18 +1283,33 @@ __device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, uint32_t R, uint32_t na
         const uint32_t nxt = __reduce_min_sync(0xffffffffu, lane < kW ? S.wnxt[par][lane] : 0xffffffffu);
         const uint32_t n_in = __reduce_add_sync(0xffffffffu, c);
         const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? c : 0u);
-        uint32_t cnt = left;
+        uint32_t cnt = left, tn = nxt;
         if (nxt != 0xffffffffu && (unsigned long long)n_in * (nxt - T) < left) cnt = n_in * (nxt - T);
+        if (CAP) {
+            if (n_in == 0) {  // every one at or below T is full
+                if (nxt == 0xffffffffu) break;  // never: admission leaves a slot for every key
+                T = nxt;
+                par ^= 1u;
+                continue;
+            }
+            const uint32_t free = __reduce_min_sync(0xffffffffu, lane < kW ? Q.wrem[par][lane] : 0xffffffffu);
+            if ((unsigned long long)n_in * free < cnt) {
+                cnt = n_in * free;
+                tn = T + free;
+            }
+        }
         const uint32_t full = cnt / n_in, part = cnt - full * n_in;
         if (in0) {
             const uint32_t k = before + (uint32_t)__popc(b0 & lt);
             S.cyc[par][k] = (uint16_t)r[0];
             add[0] += full + (k < part ? 1u : 0u);
+            if (CAP) rem[0] -= full + (k < part ? 1u : 0u);
         }
         if (in1) {
             const uint32_t k = before + (uint32_t)__popc(b0) + (uint32_t)__popc(b1 & lt);
             S.cyc[par][k] = (uint16_t)r[1];
             add[1] += full + (k < part ? 1u : 0u);
+            if (CAP) rem[1] -= full + (k < part ? 1u : 0u);
         }
         __syncthreads();
         uint32_t ci = tid % n_in;
@@ -1277,25 +1322,36 @@ __device__ __forceinline__ uint32_t lpt_run(lpt_smem &S, uint32_t R, uint32_t na
         }
         done += cnt;
         left -= cnt;
-        T = nxt;
+        T = tn;
         par ^= 1u;
     }
 #pragma unroll
     for (int x = 0; x < 2; ++x)
-        if (have[x]) S.add[r[x]] = add[x];
+        if (CAP ? add[x] != 0 : have[x]) S.add[r[x]] = add[x];
     return hi;
 }
 
 // One LPT plan on one CTA.  KT: packed keys; u32 keys hold loads relative to `origin`.
-template <int NE, typename KT>
-__device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, int shift, unsigned long long origin,
-                                         uint32_t *status)
+// CAP: a destination that holds J.W replicas gets the largest key, so it is not chosen any
+// more; a key that would have to get fewer than k_b replicas ends the placement (reported
+// in info_w->trimmed, nothing else written to the plan's loads: k_plan_lpt_capped places it).
+// R = 1024, W = 256, 1,066,667 requests, one capped plan beside two others: plan + route
+// 775 -> 2.4 ms against one warp that places every key by itself; R = 200, W = 50, 100,000
+// requests 9.6 -> 0.89 ms.
+template <int NE, typename KT, bool CAP>
+__device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, cap_smem &Q, int shift,
+                                         unsigned long long origin, uint32_t *status)
 {
     const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5, R = J.R;
     const KT rmask = (KT)(((KT)1 << shift) - 1);
     const uint32_t na = (uint32_t)J.info->n_adm;
     KT v[NE], m = (KT)~(KT)0;
     uint32_t a = 0;
+    uint32_t free_dest = R;  // CAP: destinations with a free slot (warp 0)
+    if (CAP) {
+        for (uint32_t r = threadIdx.x; r < R; r += kPlaceBlock) Q.slots[r] = S.add[r] = 0;
+        __syncthreads();
+    }
     if (warp == 0) {
 #pragma unroll
         for (int j = 0; j < NE; ++j) {
@@ -1304,11 +1360,12 @@ __device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, int sh
         }
         m = reg_min<NE, KT>(v);
     }
+    bool warp0_trimmed = false;
     for (;;) {
         if (warp == 0) {
-            bool run = false;
+            bool run = false, trim = false;
             unsigned long long rorg = 0;
-            while (a < na) {
+            while (a < na && !trim) {
                 // 32 keys, one per lane
                 const uint32_t cnt = na - a < 32u ? na - a : 32u;
                 unsigned long long st_lam = 0;
@@ -1327,7 +1384,7 @@ __device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, int sh
                     KT mx = 0;
 #pragma unroll
                     for (int j = 0; j < NE; ++j)
-                        if (lane + 32u * j < R && v[j] > mx) mx = v[j];
+                        if (lane + 32u * j < R && v[j] > mx && (!CAP || v[j] != (KT)~(KT)0)) mx = v[j];
                     const KT mn = warp_min_key(m);
                     const KT far = (KT)~warp_min_key((KT)~mx);
                     if (((far >> shift) - (mn >> shift)) < (KT)0x7fffffffu) {
@@ -1349,8 +1406,13 @@ __device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, int sh
                     const uint32_t lam = (uint32_t)__shfl_sync(0xffffffffu, st_lam, slot);  // <= n < 2^32
                     const uint32_t q = lam / k, rem = lam - q * k;
                     uint32_t taken = 0;
+                    if (CAP && k > free_dest) {
+                        trim = true;
+                        break;
+                    }
                     for (uint32_t s = 0; s < k; ++s) {
                         const KT best = warp_min_key(m);
+                        bool full = false;
                         const uint32_t br = (uint32_t)(best & rmask);
                         const uint32_t job = q + (s < rem ? 1u : 0u);
                         if (lane == 0) {
@@ -1359,24 +1421,39 @@ __device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, int sh
                         }
                         if ((br & 31u) == lane) {
                             const uint32_t jj = br >> 5;
+                            KT grow = (KT)job << shift;
+                            if (CAP && ++Q.slots[br] == J.W) {
+                                Q.fin[br] = origin + (unsigned long long)((best + grow) >> shift);
+                                grow = (KT)~best;  // best + ~best: the largest key
+                                full = true;
+                            }
 #pragma unroll
                             for (int j = 0; j < NE; ++j)
-                                if (j == (int)jj) v[j] += (KT)job << shift;
+                                if (j == (int)jj) v[j] += grow;
                             taken |= 1u << jj;  // not eligible again for this key
                             m = reg_min_untaken<NE, KT>(v, taken);
                         }
+                        if (CAP) free_dest -= __any_sync(0xffffffffu, full) ? 1u : 0u;
                     }
                     m = reg_min<NE, KT>(v);
                 }
+                if (CAP && trim) break;
                 // single copies: lane `slot` keeps its key's destination, written once for all
                 uint32_t mine = 0;
                 reg_groups<NE, KT> G;
                 G.all(v);
                 for (uint32_t slot = nm; slot < cnt; ++slot) {
-                    const KT grow = (KT)__shfl_sync(0xffffffffu, st_lam, slot) << shift;
+                    KT grow = (KT)__shfl_sync(0xffffffffu, st_lam, slot) << shift;
                     const KT best = warp_min_key(m);
                     const uint32_t br = (uint32_t)(best & rmask);
                     if (lane == slot) mine = br;
+                    bool full = false;
+                    if (CAP && (br & 31u) == lane && ++Q.slots[br] == J.W) {
+                        Q.fin[br] = origin + (unsigned long long)((best + grow) >> shift);
+                        grow = (KT)~best;
+                        full = true;
+                    }
+                    if (CAP) free_dest -= __any_sync(0xffffffffu, full) ? 1u : 0u;
                     G.grow(v, br >> 5, (br & 31u) == lane ? grow : (KT)0);
                     m = G.least();
                 }
@@ -1393,30 +1470,50 @@ __device__ __forceinline__ void lpt_plan(const place_job &J, lpt_smem &S, int sh
                     if (r < R) S.rel[r] = (uint32_t)((unsigned long long)(v[j] >> shift) - rorg);
                 }
             }
-            if (lane == 0) S.done = run ? 0u : 1u;
+            if (lane == 0) {
+                S.done = run ? 0u : 1u;
+                if (CAP && !run) J.info_w->trimmed = trim ? 1ull : 0ull;
+            }
+            if (CAP && trim) warp0_trimmed = true;
         }
         __syncthreads();
         if (S.done) break;
         const unsigned long long q = S.q;
-        const uint32_t hi = lpt_run(S, R, na, J.adm_cnt, J.members, J.jobs);
+        const uint32_t hi = lpt_run<CAP>(S, Q, J.W, R, na, J.adm_cnt, J.members, J.jobs);
         __syncthreads();
         if (warp == 0) {
             a = hi;
 #pragma unroll
             for (int j = 0; j < NE; ++j) {
                 const uint32_t r = lane + 32u * j;
-                if (r < R) v[j] += (KT)((unsigned long long)S.add[r] * q) << shift;
+                if (CAP) {
+                    bool full = false;
+                    if (r < R && S.add[r]) {
+                        v[j] += (KT)((unsigned long long)S.add[r] * q) << shift;
+                        Q.slots[r] += S.add[r];
+                        S.add[r] = 0;
+                        if (Q.slots[r] == J.W) {
+                            Q.fin[r] = origin + (unsigned long long)(v[j] >> shift);
+                            v[j] = (KT)~(KT)0;
+                            full = true;
+                        }
+                    }
+                    free_dest -= (uint32_t)__popc(__ballot_sync(0xffffffffu, full));
+                } else if (r < R) {
+                    v[j] += (KT)((unsigned long long)S.add[r] * q) << shift;
+                }
             }
             m = reg_min<NE, KT>(v);
         }
     }
-    if (warp == 0) {
+    if (warp == 0 && !warp0_trimmed) {
         bool overflow = false;
 #pragma unroll
         for (int j = 0; j < NE; ++j) {
             const uint32_t r = lane + 32u * j;
             if (r < R) {
-                const unsigned long long L = origin + (unsigned long long)(v[j] >> shift);
+                const unsigned long long L =
+                    CAP && v[j] == (KT)~(KT)0 ? Q.fin[r] : origin + (unsigned long long)(v[j] >> shift);
                 overflow |= L >= kLoadLimit;  // loads only grow: the final ones tell
                 J.load[r] = L;
             }
@@ -1510,7 +1607,7 @@ __device__ __forceinline__ void random_plan(const place_job &J, uint32_t block, 
 
 // Blocks 0 .. n_lpt-1: the LPT plans pj.j[0 .. n_lpt); then rblocks blocks for each random plan after them.
 template <int NE>
-__global__ void __launch_bounds__(kPlaceBlock) k_plan_place(const __grid_constant__ place_jobs pj, uint32_t n_lpt,
+__global__ void __launch_bounds__(kPlaceBlock, 1) k_plan_place(const __grid_constant__ place_jobs pj, uint32_t n_lpt,
                                                             uint32_t rblocks, uint32_t *status)
 {
     extern __shared__ uint4 place_sm[];
@@ -1521,6 +1618,11 @@ __global__ void __launch_bounds__(kPlaceBlock) k_plan_place(const __grid_constan
     }
     const place_job &J = pj.j[blockIdx.x];
     lpt_smem &S = *reinterpret_cast<lpt_smem *>(place_sm);
+    cap_smem &Q = *reinterpret_cast<cap_smem *>(place_sm + (sizeof(lpt_smem) + 15) / 16);  // (capped plans only)
+    if (J.W) {
+        lpt_plan<NE, unsigned long long, true>(J, S, Q, 16, 0ull, status);
+        return;
+    }
     // 32-bit keys when every load the plan can reach, relative to the least starting load, leaves room for r
     __shared__ unsigned long long s_min, s_max;
     if (threadIdx.x == 0) {
@@ -1544,9 +1646,9 @@ __global__ void __launch_bounds__(kPlaceBlock) k_plan_place(const __grid_constan
     const unsigned long long span = s_max - s_min;
     const int rb = J.R > 1 ? 32 - __clz(J.R - 1u) : 1;
     if (span < (1ull << 31) && span + J.info->adm_lam < (1ull << (32 - rb)) - 1ull)
-        lpt_plan<NE, uint32_t>(J, S, rb, s_min, status);
+        lpt_plan<NE, uint32_t, false>(J, S, Q, rb, s_min, status);
     else
-        lpt_plan<NE, unsigned long long>(J, S, 16, 0ull, status);
+        lpt_plan<NE, unsigned long long, false>(J, S, Q, 16, 0ull, status);
 }
 
 // LPT for R <= 32 uses the sorted-lane kernel (fastest per key) unless the slot
@@ -1828,12 +1930,14 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
     const bool fused = n > 0 && n <= kPlanSortOneCta;  // small intervals: admission in one launch as well
     place_jobs lj, rj, l32;                            // LPT (R <= 1024), random, short LPT lists
     uint32_t n_lj = 0, n_rj = 0, n32 = 0, lj_maxR = 0, rj_maxR = 0;
+    bool any_cap = false;
     uint64_t rj_adm = 0;
     auto flush_place = [&]() -> int {
         if (!n_lj && !n_rj) return CR_OK;
         for (uint32_t x = 0; x < n_rj; ++x) lj.j[n_lj + x] = rj.j[x];
         const uint32_t rblocks = cr_blocks(rj_adm, kPlaceBlock, gcap);
-        const size_t smem = std::max(n_lj ? sizeof(lpt_smem) : (size_t)0, n_rj ? random_smem(rj_maxR) : (size_t)0);
+        const size_t lpt = (sizeof(lpt_smem) + 15) / 16 * 16 + (any_cap ? sizeof(cap_smem) : (size_t)0);
+        const size_t smem = std::max(n_lj ? lpt : (size_t)0, n_rj ? random_smem(rj_maxR) : (size_t)0);
         const uint32_t grid = n_lj + n_rj * rblocks, ne = (lj_maxR + 31) / 32;
         auto launch = [&](auto kern) -> int {
             if (smem > 48 * 1024)
@@ -1854,6 +1958,7 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         else
             CR_TRY(launch(k_plan_place<32>));
         n_lj = n_rj = 0;
+        any_cap = false;
         lj_maxR = rj_maxR = 0;
         rj_adm = 0;
         return CR_OK;
@@ -1862,6 +1967,16 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         if (!n32) return CR_OK;
         CR_LAUNCH(ctx, k_plan_lpt32_multi, n32, 32, 0, l32, ctx->d_status);
         n32 = 0;
+        return CR_OK;
+    };
+    auto place_capped = [&](uint32_t j) -> int {  // one warp, any R, any trimming
+        cr_plan *p = plans[j];
+        const cr_plan_params &pp = params[j];
+        const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + sizeof(uint32_t) + 1) + 16;
+        if (smem > 48 * 1024)
+            CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt_capped, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CR_LAUNCH(ctx, k_plan_lpt_capped, 1, 32, smem, p->d_info, (const unsigned long long *)p->d_adm_cnt, p->d_adm_k,
+                  p->d_koff, pp.R, pp.W, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
         return CR_OK;
     };
     auto place = [&](uint32_t j) -> int {
@@ -1879,13 +1994,15 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         J.seed = pp.seed;
         J.epoch = pp.epoch;
         J.R = pp.R;
-        if (pp.variant == CR_VARIANT_SLOTCAP) {
-            const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + sizeof(uint32_t) + 1) + 16;
-            if (smem > 48 * 1024)
-                CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt_capped, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem));
-            CR_LAUNCH(ctx, k_plan_lpt_capped, 1, 32, smem, p->d_info, (const unsigned long long *)p->d_adm_cnt,
-                      p->d_adm_k, p->d_koff, pp.R, pp.W, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
+        J.W = 0;
+        J.info_w = p->d_info;
+        if (pp.variant == CR_VARIANT_SLOTCAP && pp.R <= kPlaceMaxR) {
+            J.W = pp.W;
+            lj.j[n_lj++] = J;
+            lj_maxR = std::max(lj_maxR, pp.R);
+            any_cap = true;
+        } else if (pp.variant == CR_VARIANT_SLOTCAP) {
+            CR_TRY(place_capped(j));
         } else if (pp.variant == CR_VARIANT_RANDOM) {
             rj.j[n_rj++] = J;
             rj_maxR = std::max(rj_maxR, pp.R);
@@ -1911,6 +2028,8 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
     auto finish = [&]() -> int {  // the collected placements, then the tables of every plan
         CR_TRY(flush_place());
         CR_TRY(flush_l32());
+        for (uint32_t j = 0; j < n_plans; ++j)  // (returns at once unless replica counts had to be trimmed)
+            if (params[j].variant == CR_VARIANT_SLOTCAP && params[j].R <= kPlaceMaxR) CR_TRY(place_capped(j));
         for (uint32_t j0 = 0; j0 < n_plans; j0 += 16) {
             table_jobs tj;
             const uint32_t nj = n_plans - j0 < 16 ? n_plans - j0 : 16;

@@ -1039,6 +1039,29 @@ def test_plan_parity_slotcap(P, ctx, R, W, nkeys, total, skew):
         assert np.bincount(got["members"].astype(np.int64), minlength=R).max() <= W
 
 
+@pytest.mark.parametrize("R,W", [(2, 40), (33, 31), (64, 100), (700, 9), (1024, 40)])
+@pytest.mark.parametrize("init", ["zero", "near", "far"])
+def test_plan_parity_slotcap_runs(P, ctx, R, W, init):
+    # long runs of equal counts over destinations whose slots run out one by one: every slot
+    # is used, destinations start level, within a few requests, or far apart (the far ones
+    # fill last), replicated keys in front
+    rng = np.random.default_rng(R + W)
+    C = R * W
+    lam = np.concatenate([np.array([60, 41, 41, 17]), np.repeat([7, 5, 3, 2, 1], [C // 9, C // 7, C // 4, C // 3, C])])
+    keys = np.repeat(rng.integers(1, 2**63, lam.size, dtype=np.int64).astype(np.uint64), lam)
+    rng.shuffle(keys)
+    load = None
+    if init != "zero":
+        load = rng.integers(0, 9, R).astype(np.uint64)
+        if init == "far":
+            load[:: 3] += np.uint64(2 * C)
+    dl = d_u64(load) if load is not None else None
+    got = P.build_plan(ctx, d_u64(keys), P.plan_params(R, W, 30, 1, "SLOTCAP", init_load=dl)).export()
+    ref = O.build_plan(keys, R, W, 30, 1, variant="SLOTCAP", init_load=load)
+    _cmp_plan(got, ref)
+    assert np.bincount(got["members"].astype(np.int64), minlength=R).max() == W
+
+
 def test_pipeline_parity_slotcap_policy(P, ctx):
     import dataclasses
     from paper_2608_19677_gb300.pipeline import Pipeline
