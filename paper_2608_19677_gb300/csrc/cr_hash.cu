@@ -23,15 +23,6 @@ __device__ __forceinline__ unsigned long long word_term(uint32_t lo, uint32_t hi
     return cr_fmix64(w ^ k);
 }
 
-// Word i of a span (tokens 2i, 2i + 1; past the end reads as 0) by scalar loads, mixed.
-__device__ __forceinline__ unsigned long long scalar_word(const int32_t *__restrict__ base, uint32_t P, uint32_t i,
-                                                          unsigned long long salt)
-{
-    const uint32_t lo = (uint32_t)__ldcs(base + 2 * i);
-    const uint32_t hi = (2 * i + 1 < P) ? (uint32_t)__ldcs(base + 2 * i + 1) : 0u;
-    return word_term(lo, hi, salt + (unsigned long long)(i + 1) * CR_GAMMA);
-}
-
 // Four rows of 32 aligned 16-byte vectors, one per lane; vectors from v1 on are not read.
 template <bool FULL>
 __device__ __forceinline__ void load4(int4 (&x)[4], const int4 *__restrict__ b4, uint32_t v, uint32_t v1)
@@ -114,7 +105,7 @@ __device__ __forceinline__ unsigned long long vector_words(const int4 *__restric
 // aligned vectors that lie inside it are read whole, and the words at its ends that they
 // do not hold (at most two before, three after) one per lane with scalar loads, so nothing
 // outside the span is read.  5,000 spans of 1,024-4,096 tokens packed back to back (any start):
-// 28.6 -> 18.4 us against 4- and 8-byte loads; aligned spans (166,667 of ~2,300 tokens) 286 us
+// 28.6 -> 16.5 us against 4- and 8-byte loads; aligned spans (166,667 of ~2,300 tokens) 286 us
 // either way.
 __global__ void __launch_bounds__(kHashBlock, 4)
 k_hash_prefixes(const int32_t *__restrict__ tok, const unsigned long long *__restrict__ off,
@@ -137,31 +128,38 @@ k_hash_prefixes(const int32_t *__restrict__ tok, const unsigned long long *__res
             o_next = off[r + nwarps];
             P_next = plen[r + nwarps];
         }
-        const uint32_t nw = P / 2u + (P & 1u);
         const int32_t *base = tok + o;
         unsigned long long acc = 0;
         // vector v holds tokens 4v - sh .. 4v - sh + 3 of the span; [v0, v1) lie inside it
         const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(base) >> 2) & 3u;
-        const uint32_t v0 = sh ? 1u : 0u, v1 = (uint32_t)(((unsigned long long)P + sh) >> 2);
-        uint32_t head = nw, tail = nw;  // words [0, head) and [tail, nw) are left to the scalar loads
-        if (v1 > v0) {
-            const int4 *b4 = reinterpret_cast<const int4 *>(base - (int)sh);
-            const uint32_t w0 = 2u * v0 - (sh >> 1);  // first word that vector v0 holds whole
-            // key of this lane's first word: word 2 (v0 + lane) - sh / 2
-            const unsigned long long k = salt + (unsigned long long)(w0 + 2u * lane + 1u) * CR_GAMMA;
-            head = w0;
-            if (sh & 1u) {
-                acc = vector_words<true>(b4, v0, v1, k, lane);
-                tail = 2u * (v1 - 1u) - (sh >> 1) + 1u;
-            } else {
-                acc = vector_words<false>(b4, v0, v1, k, lane);
-                tail = 2u * v1 - (sh >> 1);
+        uint32_t v0 = 0, v1 = P >> 2, head = 0, rest = 0, sw = 0;
+        int32_t slo = 0, shi = 0;
+        if (sh | (P & 3u)) {  // uniform; whole vectors only otherwise, as records padded to 16 bytes have
+            const uint32_t nw = P / 2u + (P & 1u);
+            uint32_t tail = nw;  // words [0, head) and [tail, nw) are left to scalar loads
+            v0 = sh ? 1u : 0u;
+            v1 = (uint32_t)(((unsigned long long)P + sh) >> 2);
+            head = nw;
+            if (v1 > v0) {
+                head = 2u * v0 - (sh >> 1);  // first word that vector v0 holds whole
+                tail = 2u * (v1 - 1u) - (sh >> 1) + ((sh & 1u) ? 1u : 2u);
+            }
+            // at most five, one per lane: in flight while the vectors are mixed
+            rest = head + (nw - tail);
+            sw = lane < head ? lane : tail + (lane - head);
+            if (lane < rest) {
+                slo = __ldcs(base + 2 * sw);
+                if (2 * sw + 1 < P) shi = __ldcs(base + 2 * sw + 1);
             }
         }
-        // the words left: lanes 0 .. head-1, then the tail's
-        const uint32_t rest = head + (nw - tail);
-        for (uint32_t i = lane; i < rest; i += 32)
-            acc += scalar_word(base, P, i < head ? i : tail + (i - head), salt);
+        if (v1 > v0) {
+            const int4 *b4 = reinterpret_cast<const int4 *>(base - (int)sh);
+            // key of this lane's first word: word 2 (v0 + lane) - sh / 2
+            const unsigned long long k = salt + (unsigned long long)(head + 2u * lane + 1u) * CR_GAMMA;
+            acc = (sh & 1u) ? vector_words<true>(b4, v0, v1, k, lane) : vector_words<false>(b4, v0, v1, k, lane);
+        }
+        if (lane < rest)
+            acc += word_term((uint32_t)slo, (uint32_t)shi, salt + (unsigned long long)(sw + 1u) * CR_GAMMA);
         acc = cr_warp_sum_u64(acc);
         if (lane == 0) out[r] = cr_fmix64(salt ^ (unsigned long long)P) + acc;
     }

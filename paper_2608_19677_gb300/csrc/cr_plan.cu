@@ -506,10 +506,27 @@ __global__ void __launch_bounds__(kSmallBlock) k_plan_topk(cr_plan_info_dev *inf
 constexpr size_t kTopkSmem = sizeof(small_sort_smem) > sizeof(bitonic_smem) ? sizeof(small_sort_smem)
                                                                             : sizeof(bitonic_smem);
 
-// Intervals of up to this many requests sort their histogram in one CTA (one
-// launch, one SM, so the planner barely touches the SMs the overlapped main
-// stream uses); larger ones in device-wide radix passes.
+// Which sort orders the histogram.  One CTA (one launch, one SM) where it is short: up to
+// kPlanSortAll requests whatever the slot budget C, or where admission can reach at most
+// kBitonicMax keys, up to kPlanSortOneCta requests; device-wide radix passes otherwise
+// (eleven of them, ~15 us each).  Measured, one CTA / device-wide, per build: 6,000 requests
+// 127 / 288 us; 20,000 380 / 421; 30,000 with C = 3,000 292 / 335; 50,000 with C = 10,000
+// 787 / 483; 133,333 with C = 8,192 706 / 514; 500,000 with C = 30,000 3,187 / 1,125.
 constexpr uint64_t kPlanSortOneCta = 524288;
+constexpr uint64_t kPlanSortAll = 24576;
+inline bool plan_sort_one_cta(uint64_t n, uint64_t c_max)
+{
+    return n <= kPlanSortAll || (n <= kPlanSortOneCta && c_max <= kBitonicMax);
+}
+
+// Admission of every plan in one launch, one CTA each (true), or plan by plan in
+// device-wide launches: worth ~40 us a plan once a CTA would walk tens of thousands of keys
+// (200,000 requests, C = 262,144: 928 / 624 us for one plan, 973 / 789 for four).
+inline bool plan_admit_one_cta(uint64_t n, uint64_t c_max, uint32_t n_plans)
+{
+    const uint64_t reach = n < c_max ? n : c_max;
+    return n > 0 && n <= kPlanSortOneCta && (reach <= 65536 || (uint64_t)n_plans * 24576 >= reach);
+}
 
 // Large histograms (multi-CTA passes): after the key sort, the per-key output
 // and the count-descending sort key n - count.
@@ -1857,6 +1874,12 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
             if (plans[i] == plans[j]) return cr_fail(ctx, CR_EINVAL, "cr_build_plans: plan %u repeated", j);
         CR_TRY(check_params(ctx, &params[j]));
     }
+    unsigned long long cmax = 0;  // the largest slot budget of the build
+    for (uint32_t j = 0; j < n_plans; ++j) {
+        const unsigned long long c = (unsigned long long)params[j].R * params[j].W;
+        cmax = c > cmax ? c : cmax;
+    }
+    const bool fused = plan_admit_one_cta(n, cmax, n_plans);
     for (uint32_t j = 0; j < n_plans; ++j) {
         CR_TRY(plan_reserve(ctx, plans[j], n, params[j].R, params[j].W));
         plans[j]->n = n;
@@ -1864,7 +1887,7 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         plans[j]->qden = params[j].qcap_den;
         plans[j]->variant = params[j].variant;
         plans[j]->built = 1;
-        if (j == 0 || n == 0 || n > kPlanSortOneCta)  // small intervals: the admission CTA writes every field
+        if (j == 0 || !fused)  // the admission CTA writes every field
             CR_LAUNCH(ctx, k_plan_reset, 1, 1, 0, plans[j]->d_info, (unsigned long long)n);
     }
     cr_plan *p0 = plans[0];
@@ -1896,13 +1919,8 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         // the (n - count) keys and the order ping-pong through the now idle table memory
         uint32_t *s32A = (uint32_t *)ptk, *s32B = s32A + n, *o32B = (uint32_t *)ptc;
         uint32_t *ord = (uint32_t *)po;
-        if (n <= kPlanSortOneCta) {
+        if (plan_sort_one_cta(n, cmax)) {
             // admission candidates only: the largest slot budget of the build bounds how far it reaches
-            unsigned long long cmax = 0;
-            for (uint32_t j = 0; j < n_plans; ++j) {
-                const unsigned long long c = (unsigned long long)params[j].R * params[j].W;
-                cmax = c > cmax ? c : cmax;
-            }
             CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_topk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)kTopkSmem));  // with the static part above 48 KB
             CR_LAUNCH(ctx, k_plan_topk, 1, kSmallBlock, kTopkSmem, p0->d_info, (unsigned long long)n, bits_for(n), cmax,
@@ -1927,7 +1945,6 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
 
     // ---- per plan -------------------------------------------------------------
     // placements are collected and launched together, then every plan's table
-    const bool fused = n > 0 && n <= kPlanSortOneCta;  // small intervals: admission in one launch as well
     place_jobs lj, rj, l32;                            // LPT (R <= 1024), random, short LPT lists
     uint32_t n_lj = 0, n_rj = 0, n32 = 0, lj_maxR = 0, rj_maxR = 0;
     bool any_cap = false;

@@ -1039,6 +1039,23 @@ def test_plan_parity_slotcap(P, ctx, R, W, nkeys, total, skew):
         assert np.bincount(got["members"].astype(np.int64), minlength=R).max() <= W
 
 
+@pytest.mark.parametrize("n,R,W,n_rand", [(24576, 1024, 200, 1), (24577, 1024, 4, 1), (24577, 1024, 5, 1),
+                                          (70000, 1024, 64, 1), (70000, 1024, 65, 1), (70000, 1024, 65, 3),
+                                          (130000, 1024, 200, 1), (130000, 16, 300, 5)])
+def test_plan_parity_sort_and_admission_rules(P, ctx, n, R, W, n_rand):
+    # both sides of the rules on interval and slot budget: histogram sorted by one CTA or in
+    # device-wide passes, admission of all plans by one CTA each or plan by plan
+    rng = np.random.default_rng(n + R + W)
+    pool = rng.integers(1, 2**63, n, dtype=np.int64).astype(np.uint64)
+    keys = pool[np.minimum((rng.random(n) ** 2 * n).astype(np.int64), n - 1)]
+    kinds = [("LPT", 0), ("NOREPL", 0), ("SLOTCAP", 0)] + [("RANDOM", s) for s in range(n_rand)]
+    params = [P.plan_params(R, W, 5 * n, 4 * R, v, seed=s, epoch=1) for v, s in kinds]
+    plans = [P.Plan(ctx) for _ in kinds]
+    P.build_plans(ctx, d_u64(keys), params, plans)
+    for (v, s), p in zip(kinds, plans):
+        _cmp_plan(p.export(), O.build_plan(keys, R, W, 5 * n, 4 * R, variant=v, seed=s, epoch=1))
+
+
 @pytest.mark.parametrize("R,W", [(2, 40), (33, 31), (64, 100), (700, 9), (1024, 40)])
 @pytest.mark.parametrize("init", ["zero", "near", "far"])
 def test_plan_parity_slotcap_runs(P, ctx, R, W, init):
