@@ -425,17 +425,18 @@ __device__ __forceinline__ void resolve_batches(const route_desc &rd, const uint
 // ---- batches on 32-bit relative loads ----------------------------------------
 // The live loads are held as differences from their minimum (the caller checks that
 // every load stays below 2^32 above it) in two buffers.  In batch b the decisions read
-// one of them, A = the loads at the start of the batch, while W still holds those of the
-// batch before; every thread adds its requests of this batch AND its requests of batch
-// b - 1 to W, so that W = the loads at the start of batch b + 1 when the batch's barrier
-// is passed and the two swap.  No pass over the destinations, no counts to clear.
+// one of them, A = the loads at the start of the batch, and every request adds itself to
+// the other, W, which starts equal; when the batch's barrier is passed the two swap, and
+// the new W catches up by a copy before a second barrier.  (Adding the requests of batch
+// b - 1 to W again instead, without the copy and its barrier, costs a second atomic per
+// request: few destinations then meet in it.)
 //
 // Plan replicas: inside a batch every request of a key with k_b > 1 goes to the same
 // member, the least loaded of T(b) at the batch start (ties to the earlier member).  The
 // CTA keeps those keys' member lists in shared memory, collected when a staged chunk is
-// scanned, and the scan rewrites their candidates to the key's index.  While any are
-// tracked, one warp per key finds its member between the batch's barrier and a second
-// one; warp w holds the members of key w in registers.  Keys past the capacity keep their
+// scanned, and the scan rewrites their candidates to the key's index.  One warp per key
+// finds its member between the two barriers; warp w holds the members of key w in
+// registers.  Keys past the capacity keep their
 // SET candidate, and each request reads the members from the plan.
 //   RING (not otherwise used by plan replicas)  index of a tracked key
 // Bound: issue slots of the replica's SM (about 2.5 of 4 per cycle).  24 plan replicas of
@@ -540,10 +541,8 @@ __device__ __forceinline__ void set_results(set_cache &S, const uint32_t *A, uin
     }
 }
 
-// ONE: a batch has at most one request per thread, which keeps its last destination and
-// its next candidate in registers; otherwise a resolved candidate is replaced by its
-// destination in the stage and read back in the next batch.  Returns the buffer that
-// holds the loads at the end.
+// ONE: a batch has at most one request per thread, whose next candidate is read a batch
+// early.  Returns the buffer that holds the loads at the end.
 template <bool ONE, bool PLAN>
 __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, const uint16_t *mem, uint32_t *A,
                                                       uint32_t *W, set_cache &S, uint32_t *cbuf,
@@ -593,7 +592,6 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
         }
     };
     if (PLAN) scan(cbuf, n < CH ? (uint32_t)n : CH);
-    uint32_t pd = kEmpty;  // ONE: this thread's destination of the batch before
     int cur = 0;
     for (unsigned long long c0 = 0; c0 < n; c0 += CH) {
         const unsigned long long c1 = (c0 + CH < n) ? c0 + CH : n;
@@ -614,38 +612,31 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
         }
         stage_next(nb, Cd, c1, n, CH);
         uint32_t cn = ONE && tid < min(B, len) ? cb[tid] : 0u;  // ONE: the next batch's candidate
-        uint32_t p0 = 0, p1 = 0;                                // otherwise: the batch before, of this chunk
         for (uint32_t o0 = 0; o0 < len; o0 += B) {
             const uint32_t o1 = (o0 + B < len) ? o0 + B : len;
             if (ONE) {
                 const uint32_t o = o0 + tid, c = cn;
                 cn = o1 + tid < len ? cb[o1 + tid] : 0u;
-                if (pd != kEmpty) atomicAdd(&W[pd], 1u);
-                pd = kEmpty;
                 if (o < o1) {
                     const uint32_t d = decide(c);
                     if (CR_DCHECK(d < R, status)) {
                         Dc[o] = (uint16_t)d;
                         atomicAdd(&W[d], 1u);
-                        pd = d;
                     }
                 }
             } else {
-                for (uint32_t o = p0 + tid; o < p1; o += T) atomicAdd(&W[cb[o]], 1u);
                 for (uint32_t o = o0 + tid; o < o1; o += T) {
-                    uint32_t d = decide(cb[o]);
-                    if (!CR_DCHECK(d < R, status)) d = 0;
+                    const uint32_t d = decide(cb[o]);
+                    if (!CR_DCHECK(d < R, status)) continue;
                     Dc[o] = (uint16_t)d;
                     atomicAdd(&W[d], 1u);
-                    cb[o] = d;  // (candidate o is this thread's in both batches)
                 }
-                p0 = o0;
-                p1 = o1;
             }
             __syncthreads();
             uint32_t *t = A;
             A = W;
             W = t;
+            for (uint32_t r = tid; r < R; r += T) W[r] = A[r];
             if (PLAN && keys) {
                 uint32_t j0 = warp;
                 if (my_k) {  // of equal loads, the lowest lane's
@@ -655,11 +646,9 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
                     j0 += T >> 5;
                 }
                 set_results(S, A, j0, T >> 5, keys);
-                __syncthreads();
             }
+            __syncthreads();
         }
-        if (!ONE)  // W catches up before the chunk's stage is overwritten
-            for (uint32_t o = p0 + tid; o < p1; o += T) atomicAdd(&W[cb[o]], 1u);
         cp_async_wait_all();
         __syncthreads();
         if (PLAN) scan(nb, n - c1 < CH ? (uint32_t)(n - c1) : CH);
@@ -673,12 +662,8 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
 __device__ __forceinline__ bool loads_relative(const unsigned long long *Lg, uint32_t R, unsigned long long n,
                                                uint32_t *A, uint32_t *W, unsigned long long &base)
 {
-    __shared__ unsigned long long s_lo, s_hi;
-    if (threadIdx.x == 0) {
-        s_lo = ~0ull;
-        s_hi = 0;
-    }
-    __syncthreads();
+    __shared__ unsigned long long s_lo[32], s_hi[32];
+    const uint32_t lane = threadIdx.x & 31u, warps = min((R + 31u) / 32u, blockDim.x >> 5);  // those with a load
     unsigned long long lo = ~0ull, hi = 0;
     for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) {
         const unsigned long long v = Lg[r];
@@ -686,18 +671,30 @@ __device__ __forceinline__ bool loads_relative(const unsigned long long *Lg, uin
         hi = v > hi ? v : hi;
         A[r] = (uint32_t)v;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
-        lo = a < lo ? a : lo;
-        hi = b > hi ? b : hi;
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMin(&s_lo, lo);
-        atomicMax(&s_hi, hi);
+    auto reduce = [&]() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
+            lo = a < lo ? a : lo;
+            hi = b > hi ? b : hi;
+        }
+    };
+    if ((threadIdx.x >> 5) < warps) {
+        reduce();
+        if (lane == 0) {
+            s_lo[threadIdx.x >> 5] = lo;
+            s_hi[threadIdx.x >> 5] = hi;
+        }
     }
     __syncthreads();
-    base = s_lo;
-    if (n >= 0xffffffffull || s_hi - s_lo >= 0xffffffffull - n) return false;
+    lo = lane < warps ? s_lo[lane] : ~0ull;
+    hi = lane < warps ? s_hi[lane] : 0ull;
+    if (warps > 1)
+        reduce();
+    else
+        lo = s_lo[0], hi = s_hi[0];
+    base = lo;
+    if (n >= 0xffffffffull || hi - lo >= 0xffffffffull - n) return false;
     for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) A[r] = W[r] = A[r] - (uint32_t)base;  // mod 2^32
     __syncthreads();
     return true;
