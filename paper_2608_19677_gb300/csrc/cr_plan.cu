@@ -405,7 +405,9 @@ __device__ __forceinline__ void select_from_top(const uint32_t *hist, uint32_t n
     }
 }
 
-__global__ void __launch_bounds__(kSmallBlock) k_plan_topk(cr_plan_info_dev *info, unsigned long long n, int cbits,
+// Nothing is done when there are more than `most` keys (device-wide passes sort those).
+__global__ void __launch_bounds__(kSmallBlock) k_plan_topk(cr_plan_info_dev *info, unsigned long long most,
+                                                           unsigned long long n, int cbits,
                                                            unsigned long long cmax, unsigned long long *kA,
                                                            uint32_t *vA, unsigned long long *kB, uint32_t *vB,
                                                            unsigned long long *__restrict__ ukey,
@@ -418,6 +420,7 @@ __global__ void __launch_bounds__(kSmallBlock) k_plan_topk(cr_plan_info_dev *inf
     bitonic_smem &bs = *reinterpret_cast<bitonic_smem *>(topk_sm);
     __shared__ uint32_t res[4];
     __shared__ uint32_t wtot[2][kSmallWarps];
+    if (info->U > most) return;
     const uint32_t U = (uint32_t)info->U;
     const uint32_t tid = threadIdx.x, lane = cr_lane(), warp = tid >> 5, lt = (1u << lane) - 1u;
     if (U <= kBitonicMax) {  // few keys: all of them in order, whatever the budget
@@ -508,8 +511,9 @@ constexpr size_t kTopkSmem = sizeof(small_sort_smem) > sizeof(bitonic_smem) ? si
 
 // Which sort orders the histogram.  One CTA (one launch, one SM) where it is short: up to
 // kPlanSortAll requests whatever the slot budget C, or where admission can reach at most
-// kBitonicMax keys, up to kPlanSortOneCta requests; device-wide radix passes otherwise
-// (eleven of them, ~15 us each).  Measured, one CTA / device-wide, per build: 6,000 requests
+// kBitonicMax keys, or where there are no more keys than that (known on the device only: the
+// other passes then return at once), up to kPlanSortOneCta requests; device-wide radix
+// passes otherwise (eleven of them, ~12 us each).  Measured, one CTA / device-wide, per build: 6,000 requests
 // 127 / 288 us; 20,000 380 / 421; 30,000 with C = 3,000 292 / 335; 50,000 with C = 10,000
 // 787 / 483; 133,333 with C = 8,192 706 / 514; 500,000 with C = 30,000 3,187 / 1,125.
 constexpr uint64_t kPlanSortOneCta = 524288;
@@ -530,12 +534,13 @@ inline bool plan_admit_one_cta(uint64_t n, uint64_t c_max, uint32_t n_plans)
 
 // Large histograms (multi-CTA passes): after the key sort, the per-key output
 // and the count-descending sort key n - count.
-__global__ void k_plan_sorted_keys(const cr_plan_info_dev *info, unsigned long long n,
+__global__ void k_plan_sorted_keys(const cr_plan_info_dev *info, unsigned long long skip_le, unsigned long long n,
                                    const unsigned long long *__restrict__ k, const uint32_t *__restrict__ c,
                                    unsigned long long *__restrict__ ukey, unsigned long long *__restrict__ ucnt,
                                    uint32_t *__restrict__ s32)
 {
     const unsigned long long U = info->U;
+    if (U <= skip_le) return;
     for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < U; u += (uint64_t)gridDim.x * blockDim.x) {
         ukey[u] = k[u];
         ucnt[u] = c[u];
@@ -543,10 +548,11 @@ __global__ void k_plan_sorted_keys(const cr_plan_info_dev *info, unsigned long l
     }
 }
 
-__global__ void k_plan_copy_order(cr_plan_info_dev *info, const uint32_t *__restrict__ src,
-                                  uint32_t *__restrict__ order)
+__global__ void k_plan_copy_order(cr_plan_info_dev *info, unsigned long long skip_le,
+                                  const uint32_t *__restrict__ src, uint32_t *__restrict__ order)
 {
     const unsigned long long U = info->U;
+    if (U <= skip_le) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) info->S = U;  // every key ordered
     for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < U; u += (uint64_t)gridDim.x * blockDim.x)
         order[u] = src[u];
@@ -1919,25 +1925,30 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         // the (n - count) keys and the order ping-pong through the now idle table memory
         uint32_t *s32A = (uint32_t *)ptk, *s32B = s32A + n, *o32B = (uint32_t *)ptc;
         uint32_t *ord = (uint32_t *)po;
-        if (plan_sort_one_cta(n, cmax)) {
+        const bool one_cta = plan_sort_one_cta(n, cmax);
+        if (n <= kPlanSortOneCta) {
             // admission candidates only: the largest slot budget of the build bounds how far it reaches
             CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_topk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)kTopkSmem));  // with the static part above 48 KB
-            CR_LAUNCH(ctx, k_plan_topk, 1, kSmallBlock, kTopkSmem, p0->d_info, (unsigned long long)n, bits_for(n), cmax,
+            CR_LAUNCH(ctx, k_plan_topk, 1, kSmallBlock, kTopkSmem, p0->d_info, one_cta ? ~0ull : (unsigned long long)kBitonicMax,
+                      (unsigned long long)n, bits_for(n), cmax,
                       (unsigned long long *)pk0, (uint32_t *)pv0, (unsigned long long *)pk1, (uint32_t *)pv1,
                       p0->d_ukey, p0->d_ucnt, s32A, s32B, ord + n, o32B, ord);
-        } else {
+        }
+        if (!one_cta) {
             // the same two sorts in device-wide passes, the key count read on the device
+            // (no-ops when the one-CTA kernel has sorted the few keys there are)
             const unsigned long long *dU = &p0->d_info->U;
+            const unsigned long long skip = n <= kPlanSortOneCta ? kBitonicMax : 0ull;
             int in1 = 0;
             CR_TRY(cr_radix_pairs_u64_dev(ctx, (unsigned long long *)pk0, (uint32_t *)pv0, (unsigned long long *)pk1,
-                                          (uint32_t *)pv1, n, dU, 0ull, 64, 0, &in1));
-            CR_LAUNCH(ctx, k_plan_sorted_keys, grid_n, 256, 0, (const cr_plan_info_dev *)p0->d_info,
+                                          (uint32_t *)pv1, n, dU, skip, 64, 0, &in1));
+            CR_LAUNCH(ctx, k_plan_sorted_keys, grid_n, 256, 0, (const cr_plan_info_dev *)p0->d_info, skip,
                       (unsigned long long)n, (const unsigned long long *)(in1 ? pk1 : pk0),
                       (const uint32_t *)(in1 ? pv1 : pv0), p0->d_ukey, p0->d_ucnt, s32A);
             uint32_t *o32A = (uint32_t *)pv0;  // free again after the key sort's results were copied out
-            CR_TRY(cr_radix_pairs_u32_dev(ctx, s32A, o32A, s32B, o32B, n, dU, 0ull, bits_for(n), 1, &in1));
-            CR_LAUNCH(ctx, k_plan_copy_order, grid_n, 256, 0, p0->d_info,
+            CR_TRY(cr_radix_pairs_u32_dev(ctx, s32A, o32A, s32B, o32B, n, dU, skip, bits_for(n), 1, &in1));
+            CR_LAUNCH(ctx, k_plan_copy_order, grid_n, 256, 0, p0->d_info, skip,
                       (const uint32_t *)(in1 ? o32B : o32A), ord);
         }
         order = ord;

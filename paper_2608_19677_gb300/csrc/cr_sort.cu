@@ -96,6 +96,38 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_block(const T *__restrict__
     if (total_out && threadIdx.x == kScanBlock - 1 && blockIdx.x == gridDim.x - 1) *total_out = pre;
 }
 
+// Scan of up to kScanOne elements by one CTA, kScanOne / 1024 consecutive elements per
+// thread: one launch instead of three.
+constexpr uint32_t kScanOne = 32768;
+template <typename T>
+__global__ void __launch_bounds__(kScanBlock) k_scan_one(const T *__restrict__ in, T *__restrict__ out, uint64_t n,
+                                                         int inclusive, T *__restrict__ total_out,
+                                                         const unsigned long long *n_dev, unsigned long long skip_le)
+{
+    if (n_dev && *n_dev <= skip_le) return;
+    __shared__ T tot;
+    T carry = 0;
+    for (uint64_t t0 = 0; t0 < n; t0 += 4ull * kScanBlock * 2) {  // 8,192 elements a round
+        const uint64_t base = t0 + (uint64_t)threadIdx.x * 8;
+        T x[8], s = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            x[j] = base + j < n ? in[base + j] : (T)0;
+            s += x[j];
+        }
+        T pre = carry + block_excl_scan<T>(s, &tot);
+        carry += tot;
+        __syncthreads();  // (tot is written again)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const T nx = pre + x[j];
+            if (base + j < n) out[base + j] = inclusive ? nx : pre;
+            pre = nx;
+        }
+    }
+    if (total_out && threadIdx.x == 0) *total_out = carry;
+}
+
 // Elements of partial sums needed below a scan of n elements (all levels).
 static uint64_t scan_partials_size(uint64_t n)
 {
@@ -114,6 +146,11 @@ int scan_rec(cr_ctx *ctx, const T *in, T *out, uint64_t n, int inclusive, T *d_t
     uint64_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb == 1) {
         CR_LAUNCH(ctx, k_scan_block<T>, 1, kScanBlock, 0, in, out, n, (const T *)nullptr, inclusive, d_total);
+        return CR_OK;
+    }
+    if (n <= kScanOne) {
+        CR_LAUNCH(ctx, k_scan_one<T>, 1, kScanBlock, 0, in, out, n, inclusive, d_total,
+                  (const unsigned long long *)nullptr, 0ull);
         return CR_OK;
     }
     T *partial = partials;
@@ -266,8 +303,12 @@ int radix_pairs_dev(cr_ctx *ctx, K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint6
         uint32_t *vd = cur ? v0 : v1;
         CR_LAUNCH(ctx, k_radix_upsweep<K>, ntiles, kSortBlock, 0, (const K *)ks, n_max, shift, ntiles,
                   (uint32_t *)hist, n_dev, skip_le);
-        CR_TRY(scan_impl<uint32_t>(ctx, (const uint32_t *)hist, (uint32_t *)hist, (uint64_t)256 * ntiles, 0,
-                                   (uint32_t *)nullptr));
+        if ((uint64_t)256 * ntiles <= kScanOne)
+            CR_LAUNCH(ctx, k_scan_one<uint32_t>, 1, kScanBlock, 0, (const uint32_t *)hist, (uint32_t *)hist,
+                      (uint64_t)256 * ntiles, 0, (uint32_t *)nullptr, n_dev, skip_le);
+        else
+            CR_TRY(scan_impl<uint32_t>(ctx, (const uint32_t *)hist, (uint32_t *)hist, (uint64_t)256 * ntiles, 0,
+                                       (uint32_t *)nullptr));
         CR_LAUNCH(ctx, k_radix_downsweep<K>, ntiles, kSortBlock, 0, (const K *)ks, vs, kd, vd, n_max, shift, ntiles,
                   (const uint32_t *)hist, n_dev, skip_le);
         cur ^= 1;
