@@ -137,6 +137,10 @@ struct cr_replay {
     int cur;                         // buffer holding the current state
 };
 
+// Dynamic shared memory that a launch may take without raising the kernel's limit: 48 KB
+// hold the static part as well (at most 2 KB in the kernels here).
+constexpr size_t kDefaultSmem = 46 * 1024;
+
 // ---- host helpers (cr_api.cu) ----------------------------------------------
 int cr_fail(cr_ctx *ctx, int code, const char *fmt, ...);
 int cr_scratch(cr_ctx *ctx, int slot, size_t bytes, void **out);

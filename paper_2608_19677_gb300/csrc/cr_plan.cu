@@ -1968,7 +1968,7 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         const size_t smem = std::max(n_lj ? lpt : (size_t)0, n_rj ? random_smem(rj_maxR) : (size_t)0);
         const uint32_t grid = n_lj + n_rj * rblocks, ne = (lj_maxR + 31) / 32;
         auto launch = [&](auto kern) -> int {
-            if (smem > 48 * 1024)
+            if (smem > kDefaultSmem)
                 CR_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             CR_LAUNCH(ctx, kern, grid, kPlaceBlock, smem, lj, n_lj, rblocks, ctx->d_status);
             return CR_OK;
@@ -2001,7 +2001,7 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         cr_plan *p = plans[j];
         const cr_plan_params &pp = params[j];
         const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + sizeof(uint32_t) + 1) + 16;
-        if (smem > 48 * 1024)
+        if (smem > kDefaultSmem)
             CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt_capped, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         CR_LAUNCH(ctx, k_plan_lpt_capped, 1, 32, smem, p->d_info, (const unsigned long long *)p->d_adm_cnt, p->d_adm_k,
                   p->d_koff, pp.R, pp.W, p->d_load, p->d_members, p->d_jobs, ctx->d_status);
@@ -2043,7 +2043,7 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
             lj_maxR = std::max(lj_maxR, pp.R);
         } else {
             const size_t smem = (size_t)pp.R * (sizeof(unsigned long long) + 1) + 16;
-            if (smem > 48 * 1024)
+            if (smem > kDefaultSmem)
                 CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_lpt, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)smem));
             CR_LAUNCH(ctx, k_plan_lpt, 1, 32, smem, (const cr_plan_info_dev *)p->d_info,

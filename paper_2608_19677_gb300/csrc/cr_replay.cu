@@ -958,7 +958,7 @@ int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t C
     const size_t per_warp = window_lru_bytes(nw, nb);
     const uint32_t wpb = window_warps(per_warp, regs, &per_sm);
     const size_t smem = per_warp * wpb;
-    if (smem > 48 * 1024)
+    if (smem > kDefaultSmem)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_lru_stamp<NC, NG, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)smem));
     const uint32_t ns = rp->n_rep * rp->R;
@@ -1397,7 +1397,7 @@ int launch_tokens(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t 
     const size_t per_warp = window_lru_bytes(nw, nb, true);
     const uint32_t wpb = window_warps(per_warp, regs, &per_sm);
     const size_t smem = per_warp * wpb;
-    if (smem > 48 * 1024)
+    if (smem > kDefaultSmem)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_lru_tokens<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const uint32_t ns = rp->n_rep * rp->R;
     token_state st;
@@ -1630,10 +1630,10 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     const uint32_t longer = (uint32_t)(2u * (n / R + 1u));  // twice the mean stream
     const unsigned int gcap = (unsigned int)ctx->num_sms * 8u;
     const size_t csmem = (size_t)R * sizeof(uint32_t), ssmem = part_scatter_smem(R);
-    if (csmem > 48 * 1024)
+    if (csmem > kDefaultSmem)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_part_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
     auto *scatter = R >= kPartSparse ? k_part_scatter<false> : k_part_scatter<true>;
-    if (ssmem > 48 * 1024)
+    if (ssmem > kDefaultSmem)
         CR_CUDA(ctx, cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
     const int pp = cr_prof_begin(ctx, ctx->stream, CR_PROF_PARTITION);
     CR_LAUNCH(ctx, k_part_count, dim3(ntiles, rp->n_rep + 1), kPartBlock, csmem, d_dest, (unsigned long long)n, R, ntiles,

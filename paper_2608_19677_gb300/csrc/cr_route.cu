@@ -1534,7 +1534,7 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     uint64_t MC;
     if (batch_B <= 32) {
         const size_t smem = sizeof(prep_buf) + (size_t)R * (sizeof(unsigned long long) + sizeof(uint32_t));
-        if (smem > 48 * 1024)
+        if (smem > kDefaultSmem)
             CR_CUDA(ctx, cudaFuncSetAttribute(k_route_resolve_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
         CR_LAUNCH_ON(ctx, rs, k_route_resolve_warp, n_dep, 32 * kWarpPathWarps, smem, args,
@@ -1567,7 +1567,7 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     } else {
         smem = with_members(loads + 2ull * CH * sizeof(uint32_t), &MC);
     }
-    if (smem > 48 * 1024)
+    if (smem > kDefaultSmem)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_route_resolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // no more threads than a batch has requests (a barrier of idle warps costs time), but
     // enough to stage candidates

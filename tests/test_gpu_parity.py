@@ -1256,12 +1256,13 @@ def test_replay_parity_colliding_keys(P, ctx, caps, ncoll):
                 assert (st[:c] == orp.state(rep, c_i, r)).all()
 
 
-@pytest.mark.parametrize("R", [2, 191, 192, 193, 1024, 8192])
+@pytest.mark.parametrize("R", [2, 191, 192, 193, 770, 800, 819, 820, 1024, 8192])
 @pytest.mark.parametrize("n", [1, 33, 8191, 8192, 8193, 24577])
 def test_replay_partition_edges(P, ctx, R, n):
     # every stream in arrival order (capacity 1 counts exactly the immediate repeats): both
     # ways of ranking equal destinations, tiles cut short, rows at odd addresses, and
     # destinations that are random, round robin, equal, or shared by pairs and runs of lanes
+    # (from 768 to 819 destinations the dynamic shared memory alone is just below 48 KB)
     rng = np.random.default_rng(R * 31 + n)
     rows = [rng.integers(0, R, n), np.arange(n) % R, np.full(n, R - 1), (np.arange(n) // 2 * 7) % R,
             np.where(rng.random(n) < 0.5, R // 2, rng.integers(0, R, n)), (np.arange(n) // 16) % R]
