@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kDiffWarps * 32) k_plan_diff(diff_keys a, diff
         const unsigned long long key = a.adm_key[e];
         const uint32_t ka = a.adm_k[e], oa = a.koff[e];
         // every lane probes the same slots (one L2 line per probe)
-        unsigned long long sl = key >> (64 - b.tbits);
+        unsigned long long sl = cr_table_home(key, b.tbits);
         uint32_t kb = 0, ob = 0;
         for (;;) {
             const cr_table_slot slot = b.table[sl];

@@ -1689,7 +1689,7 @@ __device__ __forceinline__ void table_body(const cr_plan_info_dev *info, const u
     for (uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; a < na; a += (uint64_t)gridDim.x * blockDim.x) {
         if (adm_k[a] == 0) continue;  // a key placed on no destination has no entry
         const unsigned long long key = adm_key[a];
-        unsigned long long s = key >> (64 - bits);
+        unsigned long long s = cr_table_home(key, bits);
         for (;;) {
             uint32_t prev = atomicCAS(&table[s].koff, kEmpty, koff[a]);
             if (prev == kEmpty) {

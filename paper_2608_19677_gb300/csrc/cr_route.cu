@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256) k_route_cand(const __grid_constant__ rout
                     c = 0xffffffffu;
                     if (valid) {
                         const unsigned long long mask = (1ull << rd.tbits) - 1ull;
-                        unsigned long long sl = key >> (64 - rd.tbits);
+                        unsigned long long sl = cr_table_home(key, rd.tbits);
                         for (;;) {
                             const cr_table_slot slot = rd.table[sl];
                             if (slot.koff == kEmpty) break;
@@ -809,7 +809,7 @@ struct prep_buf {
 __device__ __forceinline__ cr_table_slot plan_probe(const route_desc &rd, unsigned long long key)
 {
     const unsigned long long mask = (1ull << rd.tbits) - 1ull;
-    unsigned long long sl = key >> (64 - rd.tbits);
+    unsigned long long sl = cr_table_home(key, rd.tbits);
     cr_table_slot slot = rd.table[sl];
     while (slot.koff != kEmpty && slot.key != key) {  // at least twice as many slots as keys: an empty one ends it
         sl = (sl + 1) & mask;
