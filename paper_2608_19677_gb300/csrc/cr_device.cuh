@@ -97,7 +97,7 @@ __device__ __forceinline__ uint32_t cr_lane() { return threadIdx.x & 31u; }
 // First slot of a key in a plan's table of 2^bits slots.  The key's own top bits would not
 // do: admission cuts a run of equal counts by key, so the admitted keys crowd at the low end
 // of the key space (R = 18, W = 203, 15,362 requests: probes of hundreds of slots, exact
-// dispatch 7.7 ms; 0.3 ms with the product's top bits).
+// dispatch 7.7 ms; 0.17 ms with the product's top bits).
 __device__ __forceinline__ unsigned long long cr_table_home(unsigned long long key, int bits)
 {
     return (key * CR_GAMMA) >> (64 - bits);

@@ -467,11 +467,13 @@ __host__ __device__ inline size_t resolve_cache_at(uint32_t R, uint32_t CH, unsi
     return (resolve_stage_at(R) + (size_t)CH * 8 + (size_t)MC * 2 + 15) & ~(size_t)15;
 }
 
+__device__ __forceinline__ uint32_t set_hash(uint32_t slot) { return (slot * 0x9E3779B1u) >> 23; }  // 9 bits
+
 // Index of the key of table slot `slot` (a SET candidate), tracked from now on if it is new
 // and fits; kSetNone while another thread is still adding it, or when it does not fit.
 __device__ uint32_t set_index(set_cache &S, const route_desc &rd, const uint16_t *mem, uint32_t slot)
 {
-    uint32_t h = (slot * 0x9E3779B1u) >> 23;  // 9 bits
+    uint32_t h = set_hash(slot);
     for (uint32_t it = 0; it < kSetMapCap; ++it, h = (h + 1) & (kSetMapCap - 1)) {
         uint32_t cur = *(volatile uint32_t *)&S.map_slot[h];
         if (cur == kEmpty) {
@@ -509,11 +511,30 @@ __device__ __forceinline__ void set_scan(set_cache &S, const route_desc &rd, con
 #pragma unroll
             for (uint32_t u = 0; u < 4; ++u) c[u] = q + u < len ? cb[q + u] : 0u;
         }
-        uint32_t sets = 0;
+        // a key that stands in its first map entry needs no walk; the four looks are independent
+        uint32_t sets = 0, left = 0;
 #pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) sets |= (c[u] & kKindMask) == kSet && q + u < len ? 1u << u : 0u;
-        for (; sets; sets &= sets - 1u) {
-            const uint32_t u = (uint32_t)__ffs(sets) - 1u;
+        for (uint32_t u = 0; u < 4; ++u) {
+            if ((c[u] & kKindMask) != kSet || q + u >= len) continue;
+            sets |= 1u << u;
+            const uint32_t slot = c[u] & kLow30, h = set_hash(slot);
+            if (*(volatile uint32_t *)&S.map_slot[h] == slot) {
+                const uint32_t j = *(volatile uint16_t *)&S.map_j[h];
+                if (j != kSetNone) c[u] = kRing | j;
+            } else {
+                left |= 1u << u;
+            }
+        }
+        if (!sets) continue;
+        if ((CH & 3u) == 0) {
+            *reinterpret_cast<uint4 *>(&cb[q]) = make_uint4(c[0], c[1], c[2], c[3]);
+        } else {
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u)
+                if ((sets >> u) & 1u) cb[q + u] = c[u];
+        }
+        for (; left; left &= left - 1u) {
+            const uint32_t u = (uint32_t)__ffs(left) - 1u;
             const uint32_t j = set_index(S, rd, mem, cb[q + u] & kLow30);
             if (j != kSetNone) cb[q + u] = kRing | j;
         }
@@ -625,11 +646,19 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
                     }
                 }
             } else {
-                for (uint32_t o = o0 + tid; o < o1; o += T) {
-                    const uint32_t d = decide(cb[o]);
-                    if (!CR_DCHECK(d < R, status)) continue;
-                    Dc[o] = (uint16_t)d;
-                    atomicAdd(&W[d], 1u);
+                // four requests at a time: every read before the first atomic
+                for (uint32_t o = o0 + tid; o < o1; o += 4u * T) {
+                    uint32_t c[4], d[4];
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u) c[u] = o + u * T < o1 ? cb[o + u * T] : 0u;  // (0: FIXED, entry 0)
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u) d[u] = decide(c[u]);
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u) {
+                        if (o + u * T >= o1 || !CR_DCHECK(d[u] < R, status)) continue;
+                        Dc[o + u * T] = (uint16_t)d[u];
+                        atomicAdd(&W[d[u]], 1u);
+                    }
                 }
             }
             __syncthreads();
@@ -649,6 +678,7 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
             }
             __syncthreads();
         }
+        if (c1 == n) break;
         cp_async_wait_all();
         __syncthreads();
         if (PLAN) scan(nb, n - c1 < CH ? (uint32_t)(n - c1) : CH);
