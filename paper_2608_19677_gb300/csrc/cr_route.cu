@@ -9,9 +9,9 @@
 // every other replica leaves one packed candidate per request.  The
 // load-dependent pass then walks each replica's requests in arrival order:
 //   - batches longer than a warp: k_route_resolve, one CTA per replica that
-//     holds the live load in shared memory; a batch is resolved by all its
-//     threads against the batch-start loads, the batch's counts accumulate in
-//     a second shared vector and are merged at the boundary;
+//     holds the live load in shared memory, twice; a batch is resolved by all its
+//     threads against the batch-start loads while its requests add up in the
+//     other copy, and the two swap at the boundary;
 //   - batches of at most 32 requests (batch_B = 1 is exact sequential
 //     dispatch): k_route_resolve_warp, one CTA per replica whose first warp
 //     takes S = floor(32 / B) * B requests (whole batches) per step, and whose
@@ -514,9 +514,11 @@ __device__ __forceinline__ void set_scan(set_cache &S, const route_desc &rd, con
         // a key that stands in its first map entry needs no walk; the four looks are independent
         uint32_t sets = 0, left = 0;
 #pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) sets |= (c[u] & kKindMask) == kSet && q + u < len ? 1u << u : 0u;
+        if (!sets) continue;
+#pragma unroll
         for (uint32_t u = 0; u < 4; ++u) {
-            if ((c[u] & kKindMask) != kSet || q + u >= len) continue;
-            sets |= 1u << u;
+            if (!((sets >> u) & 1u)) continue;
             const uint32_t slot = c[u] & kLow30, h = set_hash(slot);
             if (*(volatile uint32_t *)&S.map_slot[h] == slot) {
                 const uint32_t j = *(volatile uint16_t *)&S.map_j[h];
@@ -525,7 +527,6 @@ __device__ __forceinline__ void set_scan(set_cache &S, const route_desc &rd, con
                 left |= 1u << u;
             }
         }
-        if (!sets) continue;
         if ((CH & 3u) == 0) {
             *reinterpret_cast<uint4 *>(&cb[q]) = make_uint4(c[0], c[1], c[2], c[3]);
         } else {
@@ -1572,8 +1573,11 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
                      (unsigned long long *)d_load, d_dest, ctx->d_status);
         return CR_OK;
     }
-    // staging chunk: a whole number of batches, at most kStage requests
-    uint32_t CH = batch_B <= kStage ? (kStage / batch_B) * batch_B : 0u;  // 0: no staging
+    // staging chunk: a whole number of batches, at most kStage requests, whole quadruples
+    // (16-byte copies) where four batches fit
+    uint32_t unit = batch_B;
+    while ((unit & 3u) && unit <= kStage / 2u) unit *= 2u;
+    uint32_t CH = unit <= kStage ? (kStage / unit) * unit : 0u;  // 0: no staging
     const size_t loads = resolve_stage_at(R);
     // plan replicas take the key cache when it fits beside a stage of at least one batch
     // (the stage shrinks by whole batches)
@@ -1583,8 +1587,13 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     int plan_x = 0;
     if (any_plan && CH) {
         uint32_t ch = CH;
-        while (ch >= batch_B && loads + (size_t)ch * 8 + 16 + px > kSmemBudget) ch -= batch_B;
-        if (ch >= batch_B) {
+        while (ch >= unit && loads + (size_t)ch * 8 + 16 + px > kSmemBudget) ch -= unit;
+        if (ch < unit && unit > batch_B) {
+            unit = batch_B;
+            ch = CH;
+            while (ch >= unit && loads + (size_t)ch * 8 + 16 + px > kSmemBudget) ch -= unit;
+        }
+        if (ch >= unit) {
             CH = ch;
             plan_x = 1;
         }
@@ -1600,9 +1609,13 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     if (smem > kDefaultSmem)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_route_resolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // no more threads than a batch has requests (a barrier of idle warps costs time), but
-    // enough to stage candidates
+    // enough to stage candidates, and, where a plan's keys can have members by the dozen, warps
+    // to decide those keys at once.  Ten replicas x 535,947 requests, R = 587, batches of 333:
+    // 384 / 512 / 768 / 1,024 threads 2.55 / 2.01 / 1.66 / 1.68 ms; R = 30 without replicated
+    // keys, batches of 256: 256 / 512 / 768 threads 182 / 192 / 211 us
+    const uint32_t least = any_plan && R > 64 ? 768u : 256u;
     const uint32_t threads = batch_B >= (uint32_t)kRouteBlock ? (uint32_t)kRouteBlock
-                                                              : std::max(256u, (batch_B + 31u) / 32u * 32u);
+                                                              : std::max(least, (batch_B + 31u) / 32u * 32u);
     CR_LAUNCH_ON(ctx, rs, k_route_resolve, n_dep, threads, smem, args, (const uint32_t *)cand, (unsigned long long)n,
               batch_B, CH, R, (unsigned long long *)d_load, d_dest, ctx->d_status, (unsigned long long)MC, plan_x);
     return CR_OK;
