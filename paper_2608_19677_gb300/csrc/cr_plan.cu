@@ -510,17 +510,18 @@ constexpr size_t kTopkSmem = sizeof(small_sort_smem) > sizeof(bitonic_smem) ? si
                                                                             : sizeof(bitonic_smem);
 
 // Which sort orders the histogram.  One CTA (one launch, one SM) where it is short: up to
-// kPlanSortAll requests whatever the slot budget C, or where admission can reach at most
-// kBitonicMax keys, or where there are no more keys than that (known on the device only: the
-// other passes then return at once), up to kPlanSortOneCta requests; device-wide radix
-// passes otherwise (eleven of them, ~12 us each).  Measured, one CTA / device-wide, per build: 6,000 requests
+// kPlanSortAll requests whatever the slot budget C, or up to kPlanSortOneCta requests where
+// admission can reach at most kPlanSortReach keys or where there are at most kBitonicMax keys
+// (known on the device only: the other passes then return at once, ~55 us for all of them);
+// device-wide radix passes otherwise (eleven of them, ~12 us each).  Measured, one CTA / device-wide, per build: 6,000 requests
 // 127 / 288 us; 20,000 380 / 421; 30,000 with C = 3,000 292 / 335; 50,000 with C = 10,000
 // 787 / 483; 133,333 with C = 8,192 706 / 514; 500,000 with C = 30,000 3,187 / 1,125.
 constexpr uint64_t kPlanSortOneCta = 524288;
 constexpr uint64_t kPlanSortAll = 24576;
+constexpr uint64_t kPlanSortReach = 8192;
 inline bool plan_sort_one_cta(uint64_t n, uint64_t c_max)
 {
-    return n <= kPlanSortAll || (n <= kPlanSortOneCta && c_max <= kBitonicMax);
+    return n <= kPlanSortAll || (n <= kPlanSortOneCta && c_max <= kPlanSortReach);
 }
 
 // Admission of every plan in one launch, one CTA each (true), or plan by plan in

@@ -336,29 +336,22 @@ __global__ void k_item_map(const uint32_t *__restrict__ start, const uint32_t *_
 // consecutive streams.  30 replicas x 133,333 requests, 64 destinations,
 // with the records packed in the count launch: 212 -> 192 us a call; one interval of 20,000
 // requests, two replicas 154 -> 142 us.
-constexpr uint32_t kItemsCta = 8192;
+constexpr uint32_t kItemsCta = 32768;
 __global__ void __launch_bounds__(1024) k_items_cta(const uint32_t *__restrict__ off, uint32_t ns, uint32_t ntiles,
-                                                    const uint32_t *__restrict__ total_in,
-                                                    uint32_t *__restrict__ start, uint32_t CL, uint32_t longer,
-                                                    uint32_t *__restrict__ total, uint32_t *__restrict__ map,
-                                                    uint64_t items_max)
+                                                    const uint32_t *__restrict__ total_in, uint32_t *start, uint32_t CL,
+                                                    uint32_t longer, uint32_t *__restrict__ total,
+                                                    uint32_t *__restrict__ map, uint64_t items_max)
 {
+    extern __shared__ uint32_t st[];  // [ns + 1] the starts again: the loops below are serial
     __shared__ uint32_t wf[32], wb[32];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t per = (ns + 1023u) / 1024u, s0 = threadIdx.x * per, s1 = min(s0 + per, ns);
-    uint32_t st[kItemsCta / 1024 + 1];
-#pragma unroll
-    for (uint32_t k = 0; k <= kItemsCta / 1024; ++k) {
-        const uint32_t s = s0 + k;
-        st[k] = k > per || s > ns ? 0u : (s < ns ? off[(unsigned long long)s * ntiles] : *total_in);
-        if (k < per && s < ns) start[s] = st[k];
-    }
-    if (threadIdx.x == 0) start[ns] = *total_in;
+    for (uint32_t s = threadIdx.x; s <= ns; s += 1024u)
+        start[s] = st[s] = s < ns ? off[(unsigned long long)s * ntiles] : *total_in;
+    __syncthreads();
+    const uint32_t per = (ns + 1023u) / 1024u, s0 = min(threadIdx.x * per, ns), s1 = min(s0 + per, ns);
     uint32_t nf = 0, nb = 0;  // long and other chunks of this thread's streams
-#pragma unroll
-    for (uint32_t k = 0; k < kItemsCta / 1024; ++k) {
-        if (s0 + k >= s1) continue;
-        const uint32_t len = st[k + 1] - st[k], nch = len ? (len + CL - 1u) / CL : 1u;
+    for (uint32_t s = s0; s < s1; ++s) {
+        const uint32_t len = st[s + 1] - st[s], nch = len ? (len + CL - 1u) / CL : 1u;
         const uint32_t f = long_chunks(len, nch, CL, longer);
         nf += f;
         nb += nch - f;
@@ -374,11 +367,8 @@ __global__ void __launch_bounds__(1024) k_items_cta(const uint32_t *__restrict__
     const uint32_t fp = __shfl_sync(0xffffffffu, fw, (warp + 31u) & 31u), bp = __shfl_sync(0xffffffffu, bw, (warp + 31u) & 31u);
     uint32_t f0 = fi - nf + (warp ? fp : 0u), b0 = first + bi - nb + (warp ? bp : 0u);
     if (threadIdx.x == 1023) *total = b0 + nb;
-#pragma unroll
-    for (uint32_t k = 0; k < kItemsCta / 1024; ++k) {
-        const uint32_t s = s0 + k;
-        if (s >= s1) continue;
-        const uint32_t len = st[k + 1] - st[k], nch = len ? (len + CL - 1u) / CL : 1u;
+    for (uint32_t s = s0; s < s1; ++s) {
+        const uint32_t len = st[s + 1] - st[s], nch = len ? (len + CL - 1u) / CL : 1u;
         for (uint32_t c = 0; c < nch; ++c) {
             const uint32_t x = min(len - c * CL, CL) > longer ? f0++ : b0++;
             if (x < items_max) {
@@ -1055,8 +1045,9 @@ struct token_state {
 // cleared above).
 __device__ __forceinline__ void tk_word_sums(const window_lru &X, uint32_t wend, uint32_t lane)
 {
-    for (uint32_t w = 0; w < X.nw; ++w) {
-        const uint32_t bits = w < wend ? X.BM[w] : 0u;
+    for (uint32_t w = wend + lane; w < X.nw; w += 32) X.SL[w] = X.SH[w] = 0;
+    for (uint32_t w = 0; w < wend; ++w) {
+        const uint32_t bits = X.BM[w];
         const uint32_t v = ((bits >> lane) & 1u) ? X.TK[32u * w + lane] : 0u;
         const uint32_t l = __reduce_add_sync(0xffffffffu, v & 0xffffu), h = __reduce_add_sync(0xffffffffu, v >> 16);
         if (lane == 0) {
@@ -1642,7 +1633,10 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     CR_LAUNCH(ctx, scatter, dim3(ntiles, rp->n_rep), kPartBlock, ssmem, d_dest, (unsigned long long)n, R, ntiles,
               (const uint32_t *)cnt, in->d_idx, (unsigned long long)m);
     if (ns <= kItemsCta) {
-        CR_LAUNCH(ctx, k_items_cta, 1, 1024, 0, (const uint32_t *)cnt, ns, ntiles, (const uint32_t *)nrec, start, in->CL,
+        const size_t ismem = ((size_t)ns + 1) * sizeof(uint32_t);
+        if (ismem > kDefaultSmem)
+            CR_CUDA(ctx, cudaFuncSetAttribute(k_items_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem));
+        CR_LAUNCH(ctx, k_items_cta, 1, 1024, ismem, (const uint32_t *)cnt, ns, ntiles, (const uint32_t *)nrec, start, in->CL,
                   longer, total, coff + ns + 4, items_max);
     } else {
         CR_LAUNCH(ctx, k_part_starts, cr_blocks((uint64_t)ns + 1, 256, gcap), 256, 0, (const uint32_t *)cnt, ns, ntiles,

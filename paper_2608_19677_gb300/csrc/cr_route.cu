@@ -1201,10 +1201,17 @@ k_route_resolve_warp(const __grid_constant__ route_args args, const unsigned lon
             mx = v > mx ? v : mx;
             mi = v < mi ? v : mi;
         }
-        if (threadIdx.x < R) {
-            atomicAdd(&s_tot, tot);
-            atomicMax(&s_max, mx);
-            atomicMin(&s_min, mi);
+        // one 64-bit shared atomic (a compare-and-swap loop) per warp, not per thread: five
+        // requests at R = 520 17.3 -> 9.4 us, 256 at R = 64 17.4 -> 16.5
+        if ((threadIdx.x & ~31u) < R) {
+            tot = cr_warp_sum_u64(tot);
+            mx = ~cr_warp_min_u64(~mx);
+            mi = cr_warp_min_u64(mi);
+            if (lane == 0) {
+                atomicAdd(&s_tot, tot);
+                atomicMax(&s_max, mx);
+                atomicMin(&s_min, mi);
+            }
         }
     }
     __syncthreads();

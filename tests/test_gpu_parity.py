@@ -1039,7 +1039,7 @@ def test_plan_parity_slotcap(P, ctx, R, W, nkeys, total, skew):
         assert np.bincount(got["members"].astype(np.int64), minlength=R).max() <= W
 
 
-@pytest.mark.parametrize("n,R,W,n_rand", [(24576, 1024, 200, 1), (24577, 1024, 4, 1), (24577, 1024, 5, 1),
+@pytest.mark.parametrize("n,R,W,n_rand", [(24576, 1024, 200, 1), (24577, 1024, 8, 1), (24577, 1024, 9, 1),
                                           (70000, 1024, 64, 1), (70000, 1024, 65, 1), (70000, 1024, 65, 3),
                                           (130000, 1024, 200, 1), (130000, 16, 300, 5)])
 def test_plan_parity_sort_and_admission_rules(P, ctx, n, R, W, n_rand):
