@@ -105,8 +105,8 @@ __device__ __forceinline__ unsigned long long vector_words(const int4 *__restric
 // aligned vectors that lie inside it are read whole, and the words at its ends that they
 // do not hold (at most two before, three after) one per lane with scalar loads, so nothing
 // outside the span is read.  5,000 spans of 1,024-4,096 tokens packed back to back (any start):
-// 28.6 -> 16.5 us against 4- and 8-byte loads; aligned spans (166,667 of ~2,300 tokens) 286 us
-// either way.
+// 28 -> 18 us against 4- and 8-byte loads (16.5 with the spans in L2); aligned spans (166,667 of
+// ~2,300 tokens) 286 -> 283 us.
 __global__ void __launch_bounds__(kHashBlock, 4)
 k_hash_prefixes(const int32_t *__restrict__ tok, const unsigned long long *__restrict__ off,
                 const uint32_t *__restrict__ plen, unsigned long long n, unsigned long long salt,

@@ -406,8 +406,9 @@ struct replay_state {
 // instructions per (request, replica) pair.  Keys indexed by slot, with an eviction per
 // new key (search for the oldest live bits, index erase, slot hand-over), took 16.6 and a
 // chain about a third longer: 48 replicas x 1,066,667 requests over 1,024 destinations
-// at capacities 64 / 256 / 1024, partition included, 2.78 -> 2.23 ms; 30 replicas x
-// 133,333 over 64 destinations at capacity 128, 270 -> 237 us.  Indexing only the
+// at capacities 64 / 256 / 1024, partition included, 2.78 -> 2.23 ms (1.72 with the item
+// order and the partition below); 30 replicas x 133,333 over 64 destinations at capacity
+// 128, 270 -> 237 us (207).  Indexing only the
 // requests' keys and streaming the carried-in ones past them fits 24 warps, but costs 18
 // instructions per pair and measured 2.88 ms.
 //
@@ -893,9 +894,9 @@ k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw
 }
 
 // Words of the window: the cmax keys that a compaction leaves plus twelve steps before the
-// next one.  More steps cost warps per SM, fewer cost compactions: at cmax 1024, 8 / 12 / 16 /
-// 24 / 32 steps measured 2.24 / 2.23 / 2.33 / 2.42 / 2.49 ms, at cmax 128 237 / 233 / 234 /
-// 227 / 262 us (the shapes above).
+// next one.  More steps cost warps per SM, fewer cost compactions: at cmax 1024, 4 / 8 / 12 / 17 /
+// 20 / 32 steps measured 1.80 / 1.73 / 1.73 / 1.83 / 1.80 / 2.02 ms, at cmax 128 223 / 217 / 215 /
+// 215 / 219 / 254 us (the shapes above).
 inline uint32_t window_words(uint32_t cmax)
 {
     return (cmax + 31) / 32 + 12;

@@ -1202,7 +1202,7 @@ k_route_resolve_warp(const __grid_constant__ route_args args, const unsigned lon
             mi = v < mi ? v : mi;
         }
         // one 64-bit shared atomic (a compare-and-swap loop) per warp, not per thread: five
-        // requests at R = 520 17.3 -> 9.4 us, 256 at R = 64 17.4 -> 16.5
+        // requests at R = 520 17.3 -> 9.4 us, 256 at R = 64 17.4 -> 13.3
         if ((threadIdx.x & ~31u) < R) {
             tot = cr_warp_sum_u64(tot);
             mx = ~cr_warp_min_u64(~mx);
