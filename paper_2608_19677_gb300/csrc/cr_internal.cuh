@@ -82,11 +82,13 @@ struct cr_ctx {
 
 // Plan: every array lives on the device; capacities are host-side upper bounds.
 struct cr_plan_info_dev {
-    unsigned long long n, U;
+    unsigned long long n;
+    // of the histogram, copied together from a build's first plan to the others
+    unsigned long long U;        // distinct keys
     unsigned long long S;        // admission candidates ordered by (count desc, key asc): order[0..S)
+    unsigned long long by_rate;  // the candidates stand in admission order in ukey/ucnt, not in key order
     unsigned long long n_adm, sum_k, cold, max_k, special;
     unsigned long long adm_lam;  // requests of the admitted keys
-    unsigned long long by_rate;  // the candidates stand in admission order in ukey/ucnt, not in key order
     unsigned long long trimmed;  // slot-capped: k_plan_place met a key that must get fewer replicas
 };
 

@@ -16,6 +16,7 @@
 //               b -> (offset, k_b, first member) used by dispatch.
 // No host synchronisation: sizes known only on the device (U, S, n_adm) are
 // read by the kernels, and grids are sized from host-side upper bounds.
+#include <stddef.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -1760,6 +1761,8 @@ struct plan_caps {
     uint64_t n, adm, mem, load;
 };
 
+static_assert(offsetof(cr_plan_info_dev, by_rate) == offsetof(cr_plan_info_dev, U) + 16, "U, S, by_rate: one copy");
+
 int plan_reserve(cr_ctx *ctx, cr_plan *p, uint64_t n, uint32_t R, uint32_t W)
 {
     const uint64_t C = (uint64_t)R * W;
@@ -2134,8 +2137,8 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
                                          cudaMemcpyDeviceToDevice, ctx->stream));
             CR_CUDA(ctx, cudaMemcpyAsync(p->d_ucnt, p0->d_ucnt, n * sizeof(unsigned long long),
                                          cudaMemcpyDeviceToDevice, ctx->stream));
-            CR_CUDA(ctx, cudaMemcpyAsync(&p->d_info->U, &p0->d_info->U, 2 * sizeof(unsigned long long),
-                                         cudaMemcpyDeviceToDevice, ctx->stream));  // U and S
+            CR_CUDA(ctx, cudaMemcpyAsync(&p->d_info->U, &p0->d_info->U, 3 * sizeof(unsigned long long),
+                                         cudaMemcpyDeviceToDevice, ctx->stream));  // U, S and by_rate
         }
         CR_CUDA(ctx, cudaMemsetAsync(p->d_table, 0xff, p->table_slots * sizeof(cr_table_slot), ctx->stream));
         if (n > 0 && src != j) {

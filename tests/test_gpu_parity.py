@@ -1056,6 +1056,26 @@ def test_plan_parity_sort_and_admission_rules(P, ctx, n, R, W, n_rand):
         _cmp_plan(p.export(), O.build_plan(keys, R, W, 5 * n, 4 * R, variant=v, seed=s, epoch=1))
 
 
+@pytest.mark.parametrize("n,U", [(66000, 1), (130000, 145), (130000, 4095), (130000, 4096), (130000, 4097),
+                                 (524288, 2000), (524289, 2000)])
+def test_every_plan_exports_its_histogram(P, ctx, n, U):
+    # builds whose admission runs plan by plan and whose plans admit differently: every plan's
+    # histogram comes out in key order, whichever kernel sorted it (few keys: by count, one CTA)
+    rng = np.random.default_rng(n + U)
+    pool = rng.choice(2**62, U, replace=False).astype(np.uint64)
+    keys = pool[np.concatenate([np.arange(U), (rng.random(n - U) ** 2 * U).astype(np.int64)])]
+    rng.shuffle(keys)
+    R, W = 1024, 200
+    kinds = [("LPT", R, W, 5 * n, 4 * R), ("NOREPL", R, W, 5 * n, 4 * R), ("LPT", 64, 3, n, 64)][: 2 if n < 10 ** 5 else 3]
+    plans = [P.Plan(ctx) for _ in kinds]
+    P.build_plans(ctx, d_u64(keys), [P.plan_params(r, w, a, b, v) for v, r, w, a, b in kinds], plans)
+    uk, uc = O.histogram(keys)
+    for (v, r, w, a, b), p in zip(kinds, plans):
+        got = p.export()
+        _cmp_plan(got, O.build_plan(keys, r, w, a, b, variant=v))
+        assert (got["ukey"] == uk).all() and (got["ucnt"] == uc).all()
+
+
 @pytest.mark.parametrize("R,W", [(2, 40), (33, 31), (64, 100), (700, 9), (1024, 40)])
 @pytest.mark.parametrize("init", ["zero", "near", "far"])
 def test_plan_parity_slotcap_runs(P, ctx, R, W, init):
