@@ -2034,7 +2034,8 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
             lj_maxR = std::max(lj_maxR, pp.R);
             any_cap = true;
         } else if (pp.variant == CR_VARIANT_SLOTCAP) {
-            CR_TRY(place_capped(j));
+            // with the trims, in finish(): it may rewrite adm_k, koff and sum_k, which a later
+            // plan of equal admission copies
         } else if (pp.variant == CR_VARIANT_RANDOM) {
             rj.j[n_rj++] = J;
             rj_maxR = std::max(rj_maxR, pp.R);
@@ -2060,8 +2061,10 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
     auto finish = [&]() -> int {  // the collected placements, then the tables of every plan
         CR_TRY(flush_place());
         CR_TRY(flush_l32());
-        for (uint32_t j = 0; j < n_plans; ++j)  // (returns at once unless replica counts had to be trimmed)
-            if (params[j].variant == CR_VARIANT_SLOTCAP && params[j].R <= kPlaceMaxR) CR_TRY(place_capped(j));
+        // every admission is filled by now (up to kPlaceMaxR: returns at once unless replica
+        // counts have to be trimmed)
+        for (uint32_t j = 0; j < n_plans; ++j)
+            if (params[j].variant == CR_VARIANT_SLOTCAP) CR_TRY(place_capped(j));
         for (uint32_t j0 = 0; j0 < n_plans; j0 += 16) {
             table_jobs tj;
             const uint32_t nj = n_plans - j0 < 16 ? n_plans - j0 : 16;

@@ -1076,6 +1076,27 @@ def test_every_plan_exports_its_histogram(P, ctx, n, U):
         assert (got["ukey"] == uk).all() and (got["ucnt"] == uc).all()
 
 
+@pytest.mark.parametrize("R,W,kinds", [(1024, 66, ("SLOTCAP", "LPT")), (2048, 33, ("SLOTCAP", "LPT")),
+                                       (2048, 33, ("SLOTCAP", "RANDOM")), (4096, 33, ("SLOTCAP", "SLOTCAP", "LPT", "RANDOM"))])
+def test_plans_beside_a_trimmed_slotcap(P, ctx, R, W, kinds):
+    # plan by plan, the slot-capped plan listed first: its replica counts are trimmed (an eighth
+    # of the destinations starts too loaded to be chosen before the others are full), those of the
+    # plans after it, which share its admission, are not
+    rng = np.random.default_rng(R)
+    lam = np.concatenate([rng.integers(R // 4, R // 3, 300), np.ones(9000, np.int64)])
+    keys = np.repeat(rng.choice(2**62, lam.size, replace=False).astype(np.uint64), lam)
+    rng.shuffle(keys)
+    init = np.zeros(R, np.uint64)
+    init[: R // 8] = 10 ** 6
+    plans = [P.Plan(ctx) for _ in kinds]
+    dl = d_u64(init)
+    P.build_plans(ctx, d_u64(keys), [P.plan_params(R, W, 1, 1, v, seed=3, init_load=dl) for v in kinds], plans)
+    refs = [O.build_plan(keys, R, W, 1, 1, variant=v, seed=3, init_load=init) for v in kinds]
+    assert (refs[0].adm_k != refs[-1].adm_k).any()
+    for p, ref in zip(plans, refs):
+        _cmp_plan(p.export(), ref)
+
+
 @pytest.mark.parametrize("R,W", [(2, 40), (33, 31), (64, 100), (700, 9), (1024, 40)])
 @pytest.mark.parametrize("init", ["zero", "near", "far"])
 def test_plan_parity_slotcap_runs(P, ctx, R, W, init):
