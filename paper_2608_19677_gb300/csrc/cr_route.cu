@@ -689,7 +689,8 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
 }
 
 // The replica's loads as differences from their minimum in A and W (= A + R), and the
-// minimum; false (neither is then meaningful) when a load could pass 2^32 - 1 above it.
+// minimum; false (neither is then meaningful) when a load could pass 2^32 - 1 above it, or
+// 2^64 (loads wrap there, and are compared wrapped).
 __device__ __forceinline__ bool loads_relative(const unsigned long long *Lg, uint32_t R, unsigned long long n,
                                                uint32_t *A, uint32_t *W, unsigned long long &base)
 {
@@ -725,7 +726,7 @@ __device__ __forceinline__ bool loads_relative(const unsigned long long *Lg, uin
     else
         lo = s_lo[0], hi = s_hi[0];
     base = lo;
-    if (n >= 0xffffffffull || hi - lo >= 0xffffffffull - n) return false;
+    if (n >= 0xffffffffull || hi - lo >= 0xffffffffull - n || hi > ~0ull - n) return false;
     for (uint32_t r = threadIdx.x; r < R; r += blockDim.x) A[r] = W[r] = A[r] - (uint32_t)base;  // mod 2^32
     __syncthreads();
     return true;

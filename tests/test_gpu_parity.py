@@ -519,6 +519,31 @@ def test_route_batches_load_ranges(P, ctx, R, B, loads):
     assert (h_u64(load) == ref_load).all()
 
 
+@pytest.mark.parametrize("B", [32, 33, 1024, 4097])
+@pytest.mark.parametrize("room", [9000, 8999, 150])
+def test_route_loads_that_wrap(P, ctx, B, room):
+    # loads at most `room` requests below 2^64 - 1: all 9,000 just fit at one destination, one
+    # more than fits, or most destinations wrap to 0 on the way and are the least loaded after
+    rng = np.random.default_rng(B + room)
+    n, R = 9000, 30
+    hot = rng.choice(2**62, 40, replace=False).astype(np.uint64)
+    keys = np.where(rng.random(n) < 0.6, hot[rng.integers(0, 40, n)], rng.integers(1, 2**63, n).astype(np.uint64))
+    opl = O.build_plan(keys, R, 4, n, 200)
+    dpl = P.build_plan(ctx, d_u64(keys), P.plan_params(R, 4, n, 200))
+    assert opl.adm_k.max() > 1
+    init = np.uint64(2**64 - 1 - room) - rng.integers(0, 50, (2, R)).astype(np.uint64)
+    init[:, 3] = 2**64 - 1 - room
+    if room < 1000:
+        init += rng.integers(0, room, (2, R)).astype(np.uint64)
+    ref_dest, ref_load = O.route([opl, None], ["CR", "P2C"], [3, 1], R, keys, 99, B, load=init)
+    assert (ref_load < np.uint64(2**32)).any() == (room < 1000)
+    load = d_u64(init.reshape(-1)).view(2, R).contiguous()
+    dest = P.route_batch(ctx, [dpl, None], ["CR", "P2C"], [3, 1], R, d_u64(keys), 99, B, load)
+    ctx.sync()
+    assert (h_u16(dest) == ref_dest).all()
+    assert (h_u64(load) == ref_load).all()
+
+
 @pytest.mark.parametrize("case", ["few", "many", "pool", "wide"])
 @pytest.mark.parametrize("B", [100, 1024])
 def test_route_replicated_keys_per_batch(P, ctx, case, B):
