@@ -1510,7 +1510,7 @@ extern "C" int cr_replay_destroy(cr_ctx *ctx, cr_replay *rp)
 // A partitioned input: every (replica, destination) stream's request indices in
 // arrival order, the packed records, the streams' starts and their chunking.
 struct cr_replay_input {
-    uint32_t n_rep, R, tokens;   // shape of the replay it was built for
+    uint32_t n_rep, R, tokens;   // shape of the replay it was built for (n_rep 0: no partition)
     uint32_t CL;                 // chunk length of the work items
     uint64_t n, m;               // requests, (request, replica) pairs
     uint32_t ns, ntiles;
@@ -1577,7 +1577,7 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
     const uint32_t ntiles = (uint32_t)((n + kPartTile - 1) / kPartTile);
     const uint64_t ncnt = (uint64_t)ns * ntiles;
     if (ncnt >= 0xffffffffull) return cr_fail(ctx, CR_EINVAL, "cr_replay_partition: too many (stream, tile) pairs");
-    in->n_rep = rp->n_rep;
+    in->n_rep = 0;  // holds nothing until everything below is enqueued: simulate refuses it
     in->R = R;
     in->tokens = (uint32_t)rp->tokens;
     in->n = n;
@@ -1609,7 +1609,10 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
         const uint32_t lo = rp->cmax * 4u > 256u ? rp->cmax * 4u : 256u, hi = rp->cmax * 32u > 256u ? rp->cmax * 32u : 256u;
         in->CL = fill < lo ? lo : (fill > hi ? hi : (uint32_t)fill);
     }
-    if (n == 0) return CR_OK;
+    if (n == 0) {
+        in->n_rep = rp->n_rep;
+        return CR_OK;
+    }
     CR_TRY(grow_u32(ctx, &in->d_idx, &in->cap_m, m));
     CR_TRY(grow_u32(ctx, (uint32_t **)&in->d_recs, &in->cap_n, n * (sizeof(rec16) / sizeof(uint32_t))));
     CR_TRY(grow_u32(ctx, &in->d_cnt, &in->cap_cnt, ncnt + 2));
@@ -1649,6 +1652,7 @@ extern "C" int cr_replay_partition(cr_ctx *ctx, const cr_replay *rp, const uint6
                   in->CL, longer, next, coff + ns + 4, items_max);
     }
     cr_prof_end(ctx, ctx->stream, pp);
+    in->n_rep = rp->n_rep;
     return CR_OK;
 }
 

@@ -1469,3 +1469,35 @@ def test_replay_partition_then_simulate_equals_shadow_replay(P, ctx):
         P.replay_simulate(ctx, other, inp, torch.zeros((n_rep, len(caps), R + 1, 5), dtype=torch.int64, device=DEV))
     inp.close()
     pctx.close()
+
+
+def test_replay_input_without_memory_is_refused(P, ctx):
+    # a partition whose buffers cannot be had leaves its input without a partition: the simulation
+    # refuses it (its pointers would be of the call before, or none), and works once memory is there
+    n, R = 40_000_000, 16
+    dk = torch.arange(n, dtype=torch.int64, device=DEV) % 1000
+    one = torch.ones(n, dtype=torch.int32, device=DEV)
+    dest = (torch.arange(n, dtype=torch.int32, device=DEV) % R).to(torch.int16)[None].contiguous()
+    small = [x[..., :5000].contiguous() for x in (dk, one, one, dest)]
+    rp = P.Replay(ctx, 1, R, [64])
+    inp = P.ReplayInput(ctx)
+    ctr = torch.zeros((1, 1, R, 5), dtype=torch.int64, device=DEV)
+    P.replay_partition(ctx, rp, *small, inp)
+    ctx.sync()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info(0)[0]
+    hog = torch.empty(free - (500 << 20), dtype=torch.uint8, device=DEV)  # the records alone take 640 MB
+    try:
+        with pytest.raises(P.CacheRouteError, match="allocate"):
+            P.replay_partition(ctx, rp, dk, one, one, dest, inp)
+        with pytest.raises(P.CacheRouteError, match="another replay shape"):
+            P.replay_simulate(ctx, rp, inp, ctr)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    for args in (small, (dk, one, one, dest)):
+        P.replay_partition(ctx, rp, *args, inp)
+        P.replay_simulate(ctx, rp, inp, ctr)
+    ctx.sync()
+    assert int(ctr[..., 0].sum()) == n + 5000
+    inp.close()
