@@ -1769,8 +1769,10 @@ int plan_reserve(cr_ctx *ctx, cr_plan *p, uint64_t n, uint32_t R, uint32_t W)
     const uint64_t adm = n < C ? n : C;
     uint64_t mem = C;
     if (n * (uint64_t)R < mem) mem = n * (uint64_t)R;
+    // (a capacity is 0 while its arrays are replaced: when one cannot be had, the next call starts over)
     if (p->cap_n < n + 1 || !p->d_ukey) {
         uint64_t c0 = 0, c1 = 0;
+        p->cap_n = 0;
         if (p->d_ukey) cudaFree(p->d_ukey), p->d_ukey = nullptr;
         if (p->d_ucnt) cudaFree(p->d_ucnt), p->d_ucnt = nullptr;
         CR_TRY(ensure(ctx, &p->d_ukey, &c0, n + 1));
@@ -1779,6 +1781,7 @@ int plan_reserve(cr_ctx *ctx, cr_plan *p, uint64_t n, uint32_t R, uint32_t W)
     }
     if (p->cap_adm < adm + 1 || !p->d_adm_key) {
         uint64_t c[4] = {0, 0, 0, 0};
+        p->cap_adm = 0;
         if (p->d_adm_key) cudaFree(p->d_adm_key), p->d_adm_key = nullptr;
         if (p->d_adm_cnt) cudaFree(p->d_adm_cnt), p->d_adm_cnt = nullptr;
         if (p->d_adm_k) cudaFree(p->d_adm_k), p->d_adm_k = nullptr;
@@ -1792,6 +1795,7 @@ int plan_reserve(cr_ctx *ctx, cr_plan *p, uint64_t n, uint32_t R, uint32_t W)
     }
     if (p->cap_mem < mem + 1 || !p->d_members) {
         uint64_t c0 = 0, c1 = 0;
+        p->cap_mem = 0;
         if (p->d_members) cudaFree(p->d_members), p->d_members = nullptr;
         if (p->d_jobs) cudaFree(p->d_jobs), p->d_jobs = nullptr;
         CR_TRY(ensure(ctx, &p->d_members, &c0, mem + 1));
@@ -1868,6 +1872,8 @@ extern "C" int cr_build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, co
     const int pi = cr_prof_begin(ctx, ctx->stream, CR_PROF_PLAN);
     const int st = build_plans(ctx, d_key, n, params, n_plans, plans);
     cr_prof_end(ctx, ctx->stream, pi);
+    if (st == CR_OK)
+        for (uint32_t j = 0; j < n_plans; ++j) plans[j]->built = 1;
     return st;
 }
 
@@ -1890,13 +1896,14 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         cmax = c > cmax ? c : cmax;
     }
     const bool fused = plan_admit_one_cta(n, cmax, n_plans);
+    // no plan holds anything until the whole build is enqueued (cr_build_plans sets `built`)
+    for (uint32_t j = 0; j < n_plans; ++j) plans[j]->built = 0;
     for (uint32_t j = 0; j < n_plans; ++j) {
         CR_TRY(plan_reserve(ctx, plans[j], n, params[j].R, params[j].W));
         plans[j]->n = n;
         plans[j]->qnum = params[j].qcap_num;
         plans[j]->qden = params[j].qcap_den;
         plans[j]->variant = params[j].variant;
-        plans[j]->built = 1;
         if (j == 0 || !fused)  // the admission CTA writes every field
             CR_LAUNCH(ctx, k_plan_reset, 1, 1, 0, plans[j]->d_info, (unsigned long long)n);
     }
@@ -2405,7 +2412,10 @@ extern "C" int cr_plan_import(cr_ctx *ctx, cr_plan *p, uint32_t R, uint32_t W, u
     if (bad == 1) st = cr_fail(ctx, CR_ENOMEM, "cr_plan_import: host allocation failed");
     else if (bad == 2) st = cr_fail(ctx, CR_EINVAL, "cr_plan_import: a member is >= R or repeated within a key");
     else if (bad == 3) st = cr_fail(ctx, CR_EINVAL, "cr_plan_import: a key is listed twice");
-    if (st == CR_OK) st = plan_reserve(ctx, p, n_adm, R, W);
+    if (st == CR_OK) {
+        p->built = 0;
+        st = plan_reserve(ctx, p, n_adm, R, W);
+    }
     if (st == CR_OK) {
         cudaStream_t s = ctx->stream;
         // the histogram of an imported plan is its admitted keys, ascending

@@ -1501,3 +1501,35 @@ def test_replay_input_without_memory_is_refused(P, ctx):
     ctx.sync()
     assert int(ctr[..., 0].sum()) == n + 5000
     inp.close()
+
+
+def test_plan_build_without_memory_leaves_no_plan(P, ctx):
+    # a build whose buffers cannot be had leaves none of its plans built (their tables would not
+    # be filled), and the same objects build again once memory is there
+    rng = np.random.default_rng(3)
+    keys = _rates_keys(rng, 2000, 100000)
+    n, R = keys.size, 1024
+    dk = d_u64(keys)
+    small = P.plan_params(R, 4, n, R)
+    plans = [P.Plan(ctx), P.Plan(ctx)]
+    P.build_plans(ctx, dk, [small, small], plans)
+    load = torch.zeros((1, R), dtype=torch.int64, device=DEV)
+    ctx.sync()
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info(0)[0] - (500 << 20), dtype=torch.uint8, device=DEV)
+    try:
+        with pytest.raises(P.CacheRouteError, match="allocate"):  # 102 M slots: 1 GB of jobs
+            P.build_plans(ctx, dk, [small, P.plan_params(R, 100000, n, R)], plans)
+        for p in plans:
+            with pytest.raises(P.CacheRouteError, match="built"):
+                P.route_batch(ctx, [p], ["CR"], [0], R, dk, 0, 64, load)
+            with pytest.raises(P.CacheRouteError, match="never built"):
+                p.info()
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    ctx.sync()
+    P.build_plans(ctx, dk, [small, small], plans)
+    ref = O.build_plan(keys, R, 4, n, R)
+    for p in plans:
+        _cmp_plan(p.export(), ref)
