@@ -51,11 +51,16 @@ struct route_desc {
         const uint16_t *rowner;          // ring: owner of each point
     };
     union {
-        const unsigned long long *n_members;  // plan, device: the sum of k_b
-        const uint32_t *rdir;                 // ring: start directory
+        const cr_plan_info_dev *info;    // plan, device: its counters
+        const uint32_t *rdir;            // ring: start directory
     };
-    uint32_t rM;                      // ring points
-    int32_t rdbits;                   // log2 directory entries
+    union {
+        const uint32_t *adm_k;           // plan: k_b in admission order, NULL when it has no entry kSetCap
+        struct {
+            uint32_t rM;                 // ring points
+            int32_t rdbits;              // log2 directory entries
+        };
+    };
 };
 static_assert(sizeof(route_desc) == 48, "route_desc layout");
 
@@ -70,10 +75,14 @@ struct route_args {
 // Candidate encoding, one u32 per (replica, request):
 //   kind 0 FIXED  bits 0..15  destination (RR, HASH, and keys with k_b = 1)
 //   kind 1 PAIR   bits 0..12  d1, bits 13..25 d2 (power-of-two choices; R <= 8192)
-//   kind 2 SET    bits 0..29  table slot of a key with k_b > 1
+//   kind 2 SET    bits 0..29  table slot of a key with k_b > 1; tables of at most 2^29 slots:
+//                 bits 0..28, and bit 29 set for kLongSet members or more
 //   kind 3 RING   bits 0..29  first ring index at or after the key's position
 constexpr uint32_t kFixed = 0u << 30, kPair = 1u << 30, kSet = 2u << 30, kRing = 3u << 30,
-                   kKindMask = 3u << 30, kLow30 = 0x3fffffffu;
+                   kKindMask = 3u << 30, kLow30 = 0x3fffffffu, kLow29 = 0x1fffffffu, kLongBit = 1u << 29;
+constexpr uint32_t kLongSet = 16;
+
+__device__ __forceinline__ uint32_t set_slot(const route_desc &rd, uint32_t c) { return c & ((1u << rd.tbits) - 1u); }
 
 __device__ __forceinline__ uint32_t p2c_pair(unsigned long long seed, uint32_t policy, unsigned long long g,
                                              uint32_t R)
@@ -169,7 +178,8 @@ __global__ void __launch_bounds__(256) k_route_cand(const __grid_constant__ rout
                             const cr_table_slot slot = rd.table[sl];
                             if (slot.koff == kEmpty) break;
                             if (slot.key == key) {
-                                c = slot.k == 1 ? (kFixed | slot.m0) : (kSet | (uint32_t)sl);
+                                c = slot.k == 1 ? (kFixed | slot.m0)
+                                                : (kSet | (slot.k >= kLongSet && rd.tbits < 30 ? kLongBit : 0u) | (uint32_t)sl);
                                 break;
                             }
                             sl = (sl + 1) & mask;
@@ -278,7 +288,7 @@ __device__ __forceinline__ const uint16_t *stage_aux(const route_desc &rd, uint1
 {
     const uint16_t *src = rd.policy == CR_POLICY_CHWBL ? rd.rowner : rd.members;
     if (cap == 0 || src == nullptr) return src;
-    const unsigned long long nk = rd.policy == CR_POLICY_CHWBL ? rd.rM : (rd.n_members ? *rd.n_members : cap + 1);
+    const unsigned long long nk = rd.policy == CR_POLICY_CHWBL ? rd.rM : (rd.info ? rd.info->sum_k : cap + 1);
     if (nk > cap) return src;
     for (unsigned long long x = threadIdx.x; x < nk; x += blockDim.x) sm[x] = src[x];
     return sm;
@@ -310,10 +320,10 @@ __device__ __forceinline__ uint32_t resolve(uint32_t c, const route_desc &rd, co
         const uint32_t d1 = c & 0x1fffu, d2 = (c >> 13) & 0x1fffu;
         return L[d1] <= L[d2] ? d1 : d2;
     }
-    const cr_table_slot slot = rd.table[c & kLow30];
+    const cr_table_slot slot = rd.table[set_slot(rd, c)];
 #ifdef CR_DEBUG_CHECKS
     // the member list of the slot lies inside the plan's members (sum of k_b)
-    if (!CR_DCHECK(rd.n_members == nullptr || (unsigned long long)slot.koff + slot.k <= *rd.n_members, status))
+    if (!CR_DCHECK(rd.info == nullptr || (unsigned long long)slot.koff + slot.k <= rd.info->sum_k, status))
         return 0;
 #endif
     return set_min(mem, slot.koff, slot.k, slot.m0, load_of);
@@ -439,6 +449,11 @@ __device__ __forceinline__ void resolve_batches(const route_desc &rd, const uint
 // registers.  Keys past the capacity keep their
 // SET candidate, and each request reads the members from the plan.
 //   RING (not otherwise used by plan replicas)  index of a tracked key
+// A plan with more replicated keys than can be tracked has only those of kLongSet members
+// or more tracked: deciding a key costs its warp ~0.1 us a batch, and a list shorter than
+// that is scanned as fast by the request itself.  R = 8192, two replicas of 100,000
+// requests, 2,000 replicated keys of 2 to 145 members, batches of 1,024: 0.41 ms (whichever
+// keys came first tracked, and the map left to fill up: 1.92; none tracked: 1.23).
 // Bound: issue slots of the replica's SM (about 2.5 of 4 per cycle).  24 plan replicas of
 // 1,066,667 requests, R = 1024, batches of 1,024: the plan-and-route turn around it 3.23 ->
 // 2.80 ms against 64-bit loads with a pass over the destinations per batch and a map lookup
@@ -456,6 +471,7 @@ struct set_cache {
     uint16_t res[kSetCap];          // least-loaded member of each key
     uint16_t pool[kSetPool];
     uint32_t n, used;
+    uint32_t only[2];               // both kLongBit: only keys with long member lists are tracked
 };
 
 // Shared-memory layout of k_route_resolve: loads [R] u64 and counts [R] u32 (or the two
@@ -481,10 +497,16 @@ __device__ uint32_t set_index(set_cache &S, const route_desc &rd, const uint16_t
             cur = atomicCAS(&S.map_slot[h], kEmpty, slot);
             if (cur == kEmpty) {
                 const uint32_t j = atomicAdd(&S.n, 1u);
+                if (j >= kSetCap) {
+                    // threads that were here together overran the limit: free the entry again, or
+                    // the map fills up and every key it does not hold walks all of it.  A key that
+                    // has passed over the entry may no longer be found, and keeps its SET candidates.
+                    *(volatile uint32_t *)&S.map_slot[h] = kEmpty;
+                    return kSetNone;
+                }
                 const cr_table_slot ts = rd.table[slot];
                 const uint32_t off = atomicAdd(&S.used, (uint32_t)ts.k);
                 const bool fits = off + ts.k <= kSetPool;
-                if (j >= kSetCap) return kSetNone;
                 for (uint32_t m = 0; fits && m < ts.k; ++m) S.pool[off + m] = mem[(size_t)ts.koff + m];
                 S.off[j] = off;
                 S.k[j] = fits ? ts.k : (uint16_t)0;
@@ -502,6 +524,7 @@ __device__ uint32_t set_index(set_cache &S, const route_desc &rd, const uint16_t
 __device__ __forceinline__ void set_scan(set_cache &S, const route_desc &rd, const uint16_t *mem, uint32_t *cb,
                                          uint32_t len, uint32_t CH)
 {
+    const uint32_t which = kSet | (S.only[0] & S.only[1]), mask = kKindMask | which;
     for (uint32_t q = threadIdx.x * 4u; q < len; q += blockDim.x * 4u) {
         uint32_t c[4];
         if ((CH & 3u) == 0) {
@@ -514,12 +537,12 @@ __device__ __forceinline__ void set_scan(set_cache &S, const route_desc &rd, con
         // a key that stands in its first map entry needs no walk; the four looks are independent
         uint32_t sets = 0, left = 0;
 #pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) sets |= (c[u] & kKindMask) == kSet && q + u < len ? 1u << u : 0u;
+        for (uint32_t u = 0; u < 4; ++u) sets |= (c[u] & mask) == which && q + u < len ? 1u << u : 0u;
         if (!sets) continue;
 #pragma unroll
         for (uint32_t u = 0; u < 4; ++u) {
             if (!((sets >> u) & 1u)) continue;
-            const uint32_t slot = c[u] & kLow30, h = set_hash(slot);
+            const uint32_t slot = c[u] & kLow29, h = set_hash(slot);
             if (*(volatile uint32_t *)&S.map_slot[h] == slot) {
                 const uint32_t j = *(volatile uint16_t *)&S.map_j[h];
                 if (j != kSetNone) c[u] = kRing | j;
@@ -536,7 +559,7 @@ __device__ __forceinline__ void set_scan(set_cache &S, const route_desc &rd, con
         }
         for (; left; left &= left - 1u) {
             const uint32_t u = (uint32_t)__ffs(left) - 1u;
-            const uint32_t j = set_index(S, rd, mem, cb[q + u] & kLow30);
+            const uint32_t j = set_index(S, rd, mem, cb[q + u] & kLow29);
             if (j != kSetNone) cb[q + u] = kRing | j;
         }
     }
@@ -586,8 +609,8 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
         const bool p1 = A[d1] <= A[d2];
         if (two) return kind == kFixed ? (c & 0xffffu) : (p1 ? d1 : d2);
         if (kind == kRing) return S.res[c & (kSetCap - 1u)];
-        const cr_table_slot slot = rd.table[c & kLow30];
-        if (!CR_DCHECK(rd.n_members == nullptr || (unsigned long long)slot.koff + slot.k <= *rd.n_members, status))
+        const cr_table_slot slot = rd.table[c & kLow29];
+        if (!CR_DCHECK(rd.info == nullptr || (unsigned long long)slot.koff + slot.k <= rd.info->sum_k, status))
             return 0u;
         auto load_of = [&](uint32_t r) { return (unsigned long long)A[r]; };
         return set_min(mem, slot.koff, slot.k, slot.m0, load_of);
@@ -597,7 +620,13 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
             S.map_slot[x] = kEmpty;
             S.map_j[x] = kSetNone;
         }
-        if (tid == 0) S.n = S.used = 0;
+        // more replicated keys than can be tracked (k_b is non-increasing in admission order): only
+        // those with long member lists (two warps: the two reads are in flight together)
+        if (tid == 0) {
+            S.n = S.used = 0;
+            S.only[0] = rd.adm_k && rd.info->n_adm > kSetCap ? kLongBit : 0u;
+        }
+        if (tid == 32) S.only[1] = rd.adm_k && rd.adm_k[kSetCap] > 1u ? kLongBit : 0u;
     }
     cp_async_wait_all();  // the caller has started the first chunk's copy
     __syncthreads();
@@ -1461,7 +1490,8 @@ extern "C" int cr_route_batch(cr_ctx *ctx, const cr_plan *const *plans, const cr
             d.tbits = bits;
             d.table = p->d_table;
             d.members = p->d_members;
-            d.n_members = &p->d_info->sum_k;
+            d.info = p->d_info;
+            d.adm_k = p->cap_adm > kSetCap ? p->d_adm_k : nullptr;  // (as many keys as can be tracked: all of them)
             mc = std::max<uint64_t>(mc, (uint64_t)p->R * p->W);  // sum of k_b <= C = R W
         } else if (reps[i].policy == CR_POLICY_CHWBL) {
             const cr_ring *g = reps[i].ring;
@@ -1590,10 +1620,15 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     // plan replicas take the key cache when it fits beside a stage of at least one batch
     // (the stage shrinks by whole batches)
     bool any_plan = false;
-    for (uint32_t i = 0; i < n_dep; ++i) any_plan |= args.d[args.dep[i]].policy <= CR_POLICY_CR_NOREPL;
+    bool slots29 = true;  // slot numbers leave bit 29 of a candidate free
+    for (uint32_t i = 0; i < n_dep; ++i)
+        if (args.d[args.dep[i]].policy <= CR_POLICY_CR_NOREPL) {
+            any_plan = true;
+            slots29 = slots29 && args.d[args.dep[i]].tbits < 30;
+        }
     const size_t px = sizeof(set_cache);
     int plan_x = 0;
-    if (any_plan && CH) {
+    if (any_plan && slots29 && CH) {
         uint32_t ch = CH;
         while (ch >= unit && loads + (size_t)ch * 8 + 16 + px > kSmemBudget) ch -= unit;
         if (ch < unit && unit > batch_B) {

@@ -574,6 +574,29 @@ def test_route_replicated_keys_per_batch(P, ctx, case, B):
     assert (h_u64(load) == ref_load).all()
 
 
+@pytest.mark.parametrize("R,W,counts", [(64, 64, [2] * 256), (64, 64, [2] * 257), (64, 64, [15] * 100 + [16] * 100 + [2] * 57),
+                                        (512, 64, [40] * 300 + [17] * 40 + [16] * 40 + [15] * 40 + [2] * 400),
+                                        (8192, 2, [40] * 200 + [16] * 100 + [3] * 700)])
+@pytest.mark.parametrize("B", [33, 1024, 1030])
+def test_route_more_replicated_keys_than_tracked(P, ctx, R, W, counts, B):
+    # at most 256 keys with k_b > 1: all may be tracked; more: only those with 16 members or more,
+    # as many of them as there is room for.  q_cap = 1, so a key seen c times gets k_b = min(c, R).
+    rng = np.random.default_rng(B + len(counts))
+    ks = rng.choice(2**62, len(counts) + 5000, replace=False).astype(np.uint64)
+    keys = np.concatenate([np.repeat(ks[: len(counts)], counts), ks[len(counts):]])
+    rng.shuffle(keys)
+    opl = O.build_plan(keys, R, W, 1, 1)
+    dpl = P.build_plan(ctx, d_u64(keys), P.plan_params(R, W, 1, 1))
+    assert (np.asarray(opl.adm_k) > 1).sum() == len(counts)
+    init = rng.integers(0, 9, (2, R)).astype(np.uint64)
+    ref_dest, ref_load = O.route([opl, opl], ["CR", "CR"], [0, 3], R, keys, 11, B, load=init)
+    load = d_u64(init.reshape(-1)).view(2, R).contiguous()
+    dest = P.route_batch(ctx, [dpl, dpl], ["CR", "CR"], [0, 3], R, d_u64(keys), 11, B, load)
+    ctx.sync()
+    assert (h_u16(dest) == ref_dest).all()
+    assert (h_u64(load) == ref_load).all()
+
+
 def test_route_rejects_bad_args(P, ctx):
     keys = d_u64(np.array([1, 2, 3], np.uint64))
     load = torch.zeros((1, 4), dtype=torch.int64, device=DEV)
