@@ -27,6 +27,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "cr_device.cuh"
 #include "cr_internal.cuh"
@@ -676,19 +677,31 @@ __device__ __forceinline__ uint32_t *resolve_relative(const route_desc &rd, cons
                     }
                 }
             } else {
-                // four requests at a time: every read before the first atomic
-                for (uint32_t o = o0 + tid; o < o1; o += 4u * T) {
-                    uint32_t c[4], d[4];
+                // up to four requests at a time: every read before the first atomic; as many as the
+                // warp has left (100,000 requests, R = 30, batches of 1,025: 112.6 us with four always,
+                // 77.0 so)
+                auto take = [&](auto num, uint32_t o) {
+                    constexpr uint32_t N = decltype(num)::value;
+                    uint32_t c[N], d[N];
 #pragma unroll
-                    for (uint32_t u = 0; u < 4; ++u) c[u] = o + u * T < o1 ? cb[o + u * T] : 0u;  // (0: FIXED, entry 0)
+                    for (uint32_t u = 0; u < N; ++u) c[u] = o + u * T < o1 ? cb[o + u * T] : 0u;  // (0: FIXED, entry 0)
 #pragma unroll
-                    for (uint32_t u = 0; u < 4; ++u) d[u] = decide(c[u]);
+                    for (uint32_t u = 0; u < N; ++u) d[u] = decide(c[u]);
 #pragma unroll
-                    for (uint32_t u = 0; u < 4; ++u) {
+                    for (uint32_t u = 0; u < N; ++u) {
                         if (o + u * T >= o1 || !CR_DCHECK(d[u] < R, status)) continue;
                         Dc[o + u * T] = (uint16_t)d[u];
                         atomicAdd(&W[d[u]], 1u);
                     }
+                };
+                for (uint32_t ow = o0 + (tid & ~31u); ow < o1; ow += 4u * T) {  // uniform over the warp
+                    const uint32_t left = o1 - ow;
+                    if (left > 2u * T)
+                        take(std::integral_constant<uint32_t, 4>(), ow + lane);
+                    else if (left > T)
+                        take(std::integral_constant<uint32_t, 2>(), ow + lane);
+                    else
+                        take(std::integral_constant<uint32_t, 1>(), ow + lane);
                 }
             }
             __syncthreads();
@@ -1615,6 +1628,7 @@ static int launch_resolve(cr_ctx *ctx, cudaStream_t rs, const route_args &args, 
     // (16-byte copies) where four batches fit
     uint32_t unit = batch_B;
     while ((unit & 3u) && unit <= kStage / 2u) unit *= 2u;
+    if (unit & 3u) unit = batch_B;  // none fit: the largest chunk then
     uint32_t CH = unit <= kStage ? (kStage / unit) * unit : 0u;  // 0: no staging
     const size_t loads = resolve_stage_at(R);
     // plan replicas take the key cache when it fits beside a stage of at least one batch

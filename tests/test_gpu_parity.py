@@ -597,6 +597,25 @@ def test_route_more_replicated_keys_than_tracked(P, ctx, R, W, counts, B):
     assert (h_u64(load) == ref_load).all()
 
 
+@pytest.mark.parametrize("B", [1025, 2047, 2048, 2049, 3073, 4098, 5001, 8200, 16381])
+def test_route_batch_remainders(P, ctx, B):
+    # batches of one to many requests per thread: four, two or one at a time, and staging chunks
+    # of whole quadruples (16-byte copies) or not
+    rng = np.random.default_rng(B)
+    n, R = 20011, 31
+    hot = rng.choice(2**62, 60, replace=False).astype(np.uint64)
+    keys = np.where(rng.random(n) < 0.7, hot[rng.integers(0, 60, n)], rng.integers(1, 2**63, n).astype(np.uint64))
+    opl = O.build_plan(keys, R, 6, n, 100)
+    dpl = P.build_plan(ctx, d_u64(keys), P.plan_params(R, 6, n, 100))
+    init = rng.integers(0, 9, (2, R)).astype(np.uint64)
+    ref_dest, ref_load = O.route([opl, None], ["CR", "P2C"], [0, 3], R, keys, 11, B, load=init)
+    load = d_u64(init.reshape(-1)).view(2, R).contiguous()
+    dest = P.route_batch(ctx, [dpl, None], ["CR", "P2C"], [0, 3], R, d_u64(keys), 11, B, load)
+    ctx.sync()
+    assert (h_u16(dest) == ref_dest).all()
+    assert (h_u64(load) == ref_load).all()
+
+
 def test_route_rejects_bad_args(P, ctx):
     keys = d_u64(np.array([1, 2, 3], np.uint64))
     load = torch.zeros((1, 4), dtype=torch.int64, device=DEV)
