@@ -616,6 +616,26 @@ def test_route_batch_remainders(P, ctx, B):
     assert (h_u64(load) == ref_load).all()
 
 
+@pytest.mark.parametrize("R", [1, 2, 3, 5, 6, 8, 9, 17, 32])
+@pytest.mark.parametrize("B", [1, 5, 32])
+def test_route_bounded_loads_few_destinations(P, ctx, R, B):
+    # steps of at most 32 requests: the list of a walk's owners ends before all are met (rings of
+    # one point per destination or of many), and a few hot keys fill the first ones
+    rng = np.random.default_rng(40 * R + B)
+    keys = rng.choice(2**62, 4, replace=False).astype(np.uint64)[rng.integers(0, 4, 3001)]
+    keys[rng.random(3001) < 0.2] = rng.integers(1, 2**63)
+    V = [1, 3, 100]
+    pols, seeds = ["CHWBL"] * 3, [0, 1, 2]
+    init = np.zeros((3, R), np.uint64)
+    init[:, : R // 2] = 40
+    ref_dest, ref_load = O.route([None] * 3, pols, seeds, R, keys, 11, B, load=init, rings=[O.Ring(R, v, 7) for v in V])
+    load = d_u64(init.reshape(-1)).view(3, R).contiguous()
+    dest = P.route_batch(ctx, [None] * 3, pols, seeds, R, d_u64(keys), 11, B, load, rings=[P.Ring(ctx, R, v, 7) for v in V])
+    ctx.sync()
+    assert (h_u16(dest) == ref_dest).all()
+    assert (h_u64(load) == ref_load).all()
+
+
 def test_route_rejects_bad_args(P, ctx):
     keys = d_u64(np.array([1, 2, 3], np.uint64))
     load = torch.zeros((1, 4), dtype=torch.int64, device=DEV)
