@@ -202,25 +202,21 @@ static inline unsigned int cr_blocks(uint64_t work, unsigned int per_block, unsi
 }
 
 // ---- sort and scan primitives (cr_sort.cu) -----------------------------------
-// Stable LSD radix sort of keys (and optional u32 values) on bits [0, bits).
-// Input in (k_in, v_in); the sorted result is returned through *k_out/*v_out,
-// which point at either the input buffers or the context's ping-pong scratch.
-int cr_radix_sort_u64(cr_ctx *ctx, const unsigned long long *k_in, const uint32_t *v_in, uint64_t n,
-                      int bits, const unsigned long long **k_out, const uint32_t **v_out);
-int cr_radix_sort_u32(cr_ctx *ctx, const uint32_t *k_in, const uint32_t *v_in, uint64_t n, int bits,
-                      const uint32_t **k_out, const uint32_t **v_out);
+// Stable sort of n 64-bit keys: the sorted keys and the positions they had, in the
+// context's ping-pong scratch (k_in itself and no positions when n == 0).
+int cr_radix_sort_u64(cr_ctx *ctx, const unsigned long long *k_in, uint64_t n, const unsigned long long **k_out,
+                      const uint32_t **pos_out);
+// A plan's histogram in order: the info->U (key, count) pairs of (k0, v0) (at most n of them,
+// n their counts' sum) by key ascending into ukey / ucnt, then order[0 .. U) = their places by
+// (count descending, key ascending), and info->S = U.  (k1, v1), sA, sB and oB are scratch of
+// n items each, as k0 and v0 are afterwards.  U <= skip_le: nothing is touched.  The caller
+// has zeroed the counters (cr_sort_counters: `quads` 16-byte words in the context's scratch).
+int cr_sort_counters(cr_ctx *ctx, uint64_t n, uint4 **counters, uint32_t *quads);
+int cr_plan_sort_histogram(cr_ctx *ctx, cr_plan_info_dev *info, uint64_t n, unsigned long long skip_le,
+                           unsigned long long *k0, uint32_t *v0, unsigned long long *k1, uint32_t *v1,
+                           unsigned long long *ukey, unsigned long long *ucnt, uint32_t *sA, uint32_t *sB,
+                           uint32_t *oB, uint32_t *order);
 // Exclusive scan of u32 counts into u32 offsets (in place allowed); total to *d_total if non-null.
-// Radix sort of (key, value) pairs by bits [0, bits), ping-ponging between the
-// caller's buffers 0 and 1; the item count is read from n_dev (grid sized by
-// n_max); a count <= skip_le leaves everything untouched.  With iota the
-// values start as the items' positions.  *in1 tells whether the result ended
-// in buffers 1.
-int cr_radix_pairs_u64_dev(cr_ctx *ctx, unsigned long long *k0, uint32_t *v0, unsigned long long *k1, uint32_t *v1,
-                           uint64_t n_max, const unsigned long long *n_dev, unsigned long long skip_le, int bits,
-                           int iota, int *in1);
-int cr_radix_pairs_u32_dev(cr_ctx *ctx, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, uint64_t n_max,
-                           const unsigned long long *n_dev, unsigned long long skip_le, int bits, int iota,
-                           int *in1);
 int cr_scan_u32(cr_ctx *ctx, const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *d_total);
 // Inclusive scan of u64 values.
 int cr_scan_u64_inclusive(cr_ctx *ctx, const unsigned long long *in, unsigned long long *out, uint64_t n);

@@ -2,10 +2,10 @@
 //
 //   histogram   warp-aggregated counts in an L2-resident open-addressing table,
 //               occupied slots compacted to (b, lambda_b)
-//   order       (lambda desc, key asc): for intervals of up to 524,288 requests
-//               one CTA sorts only the admission candidates (the keys whose count
-//               reaches the C-th largest, C = R*W); above, device-wide radix
-//               passes sort every key
+//   order       (lambda desc, key asc): up to 4,096 keys are sorted by one CTA; of more
+//               keys one CTA sorts only the admission candidates (the keys whose count
+//               reaches the C-th largest, C = R*W) where C is at most 4,096, and a sort by
+//               the whole GPU orders them all otherwise
 //   per plan    k_b (Eq. 1), inclusive scan of k_b, admission cut, admitted
 //               arrays, cold-tail total and initial loads (small intervals: every
 //               plan in one launch, one CTA each); then every plan's placement in
@@ -31,19 +31,25 @@ constexpr uint32_t kEmpty = 0xffffffffu;
 constexpr unsigned long long kLoadLimit = 1ull << 47;
 constexpr uint32_t kPlaceMaxR = 1024;  // destinations of an LPT plan that k_plan_place takes
 
-__global__ void k_plan_reset(cr_plan_info_dev *info, unsigned long long n)
+__device__ __forceinline__ void plan_reset(cr_plan_info_dev *info, unsigned long long n)
 {
+    const cr_plan_info_dev empty = {};
+    *info = empty;
     info->n = n;
-    info->U = 0;
-    info->S = 0;
-    info->adm_lam = 0;
-    info->n_adm = 0;
-    info->sum_k = 0;
-    info->cold = 0;
-    info->max_k = 0;
-    info->special = 0;
-    info->by_rate = 0;
-    info->trimmed = 0;
+}
+
+__global__ void k_plan_reset(cr_plan_info_dev *info, unsigned long long n) { plan_reset(info, n); }
+
+// The same for a build's first plan, with the histogram table's counts and, when a wide sort
+// follows, its counters: one node where two memsets and a launch stood.
+__global__ void k_plan_clear(cr_plan_info_dev *info, unsigned long long n, uint4 *__restrict__ tcnt, uint64_t tq,
+                             uint4 *__restrict__ counters, uint32_t cq)
+{
+    const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (uint64_t)gridDim.x * blockDim.x;
+    if (i0 == 0) plan_reset(info, n);
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    for (uint64_t i = i0; i < cq; i += step) counters[i] = zero;
+    for (uint64_t i = i0; i < tq; i += step) tcnt[i] = zero;
 }
 
 // ---- histogram: counts in an L2-resident open-addressing table ----------
@@ -406,7 +412,8 @@ __device__ __forceinline__ void select_from_top(const uint32_t *hist, uint32_t n
     }
 }
 
-// Nothing is done when there are more than `most` keys (device-wide passes sort those).
+// Nothing is done when there are more than `most` keys (the wide sort takes those); with more
+// than kBitonicMax, cmax is below their number.
 __global__ void __launch_bounds__(kSmallBlock) k_plan_topk(cr_plan_info_dev *info, unsigned long long most,
                                                            unsigned long long n, int cbits,
                                                            unsigned long long cmax, unsigned long long *kA,
@@ -430,11 +437,6 @@ __global__ void __launch_bounds__(kSmallBlock) k_plan_topk(cr_plan_info_dev *inf
             info->S = U;
             info->by_rate = 1;
         }
-        return;
-    }
-    if (U <= cmax) {  // every key is a candidate
-        small_sort(sm, U, n, cbits, kA, vA, kB, vB, ukey, ucnt, s32A, s32B, o32A, o32B, order);
-        if (tid == 0) info->S = U;
         return;
     }
     uint32_t *h1 = &sm.hist[0][0], *h2 = h1 + 1024;
@@ -510,19 +512,17 @@ __global__ void __launch_bounds__(kSmallBlock) k_plan_topk(cr_plan_info_dev *inf
 constexpr size_t kTopkSmem = sizeof(small_sort_smem) > sizeof(bitonic_smem) ? sizeof(small_sort_smem)
                                                                             : sizeof(bitonic_smem);
 
-// Which sort orders the histogram.  One CTA (one launch, one SM) where it is short: up to
-// kPlanSortAll requests whatever the slot budget C, or up to kPlanSortOneCta requests where
-// admission can reach at most kPlanSortReach keys or where there are at most kBitonicMax keys
-// (known on the device only: the other passes then return at once, ~55 us for all of them);
-// device-wide radix passes otherwise (eleven of them, ~12 us each).  Measured, one CTA / device-wide, per build: 6,000 requests
-// 127 / 288 us; 20,000 380 / 421; 30,000 with C = 3,000 292 / 335; 50,000 with C = 10,000
-// 787 / 483; 133,333 with C = 8,192 706 / 514; 500,000 with C = 30,000 3,187 / 1,125.
+// Which sort orders the histogram: one CTA (true) where admission reaches at most kBitonicMax
+// keys, up to kPlanSortOneCta requests; else the wide sort, which returns at once when there
+// turn out to be at most kBitonicMax keys (the CTA has then sorted them; the launch costs
+// 4-8 us).  Measured, one CTA / wide, per build of one LPT plan: 8,000 requests and as many keys
+// 243 / 172 us; 24,000 and 12,000 keys 400 / 203; 130,000 and 65,000 keys with C = 8,192 516 /
+// 235; 500,000 of as many keys 1,111 / 257, with 145 keys 74 / 82.  C = 4,000, 130,000 requests:
+// 4,300 keys 180 / 222, 65,000 keys 397 / 222.
 constexpr uint64_t kPlanSortOneCta = 524288;
-constexpr uint64_t kPlanSortAll = 24576;
-constexpr uint64_t kPlanSortReach = 8192;
 inline bool plan_sort_one_cta(uint64_t n, uint64_t c_max)
 {
-    return n <= kPlanSortAll || (n <= kPlanSortOneCta && c_max <= kPlanSortReach);
+    return n <= kBitonicMax || (n <= kPlanSortOneCta && c_max <= kBitonicMax);
 }
 
 // Admission of every plan in one launch, one CTA each (true), or plan by plan in
@@ -532,32 +532,6 @@ inline bool plan_admit_one_cta(uint64_t n, uint64_t c_max, uint32_t n_plans)
 {
     const uint64_t reach = n < c_max ? n : c_max;
     return n > 0 && n <= kPlanSortOneCta && (reach <= 65536 || (uint64_t)n_plans * 24576 >= reach);
-}
-
-// Large histograms (multi-CTA passes): after the key sort, the per-key output
-// and the count-descending sort key n - count.
-__global__ void k_plan_sorted_keys(const cr_plan_info_dev *info, unsigned long long skip_le, unsigned long long n,
-                                   const unsigned long long *__restrict__ k, const uint32_t *__restrict__ c,
-                                   unsigned long long *__restrict__ ukey, unsigned long long *__restrict__ ucnt,
-                                   uint32_t *__restrict__ s32)
-{
-    const unsigned long long U = info->U;
-    if (U <= skip_le) return;
-    for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < U; u += (uint64_t)gridDim.x * blockDim.x) {
-        ukey[u] = k[u];
-        ucnt[u] = c[u];
-        s32[u] = (uint32_t)(n - c[u]);
-    }
-}
-
-__global__ void k_plan_copy_order(cr_plan_info_dev *info, unsigned long long skip_le,
-                                  const uint32_t *__restrict__ src, uint32_t *__restrict__ order)
-{
-    const unsigned long long U = info->U;
-    if (U <= skip_le) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) info->S = U;  // every key ordered
-    for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < U; u += (uint64_t)gridDim.x * blockDim.x)
-        order[u] = src[u];
 }
 
 // Eq. 1: k_b = min(R, max(1, ceil(lambda * den / num))); NOREPL: 1.
@@ -1904,7 +1878,7 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         plans[j]->qnum = params[j].qcap_num;
         plans[j]->qden = params[j].qcap_den;
         plans[j]->variant = params[j].variant;
-        if (j == 0 || !fused)  // the admission CTA writes every field
+        if ((j == 0 && n == 0) || (j > 0 && !fused))  // (k_plan_clear; the admission CTA writes every field)
             CR_LAUNCH(ctx, k_plan_reset, 1, 1, 0, plans[j]->d_info, (unsigned long long)n);
     }
     cr_plan *p0 = plans[0];
@@ -1927,8 +1901,13 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         CR_TRY(cr_scratch(ctx, SCR_PLAN_C, (2 * n + 1) * sizeof(uint32_t), &po));
         unsigned long long *tkey = (unsigned long long *)ptk;
         uint32_t *tcnt = (uint32_t *)ptc;
+        const bool one_cta = plan_sort_one_cta(n, cmax);
+        uint4 *cnt = nullptr;
+        uint32_t cq = 0;
+        if (!one_cta) CR_TRY(cr_sort_counters(ctx, n, &cnt, &cq));
         CR_CUDA(ctx, cudaMemsetAsync(tkey, 0xff, slots * sizeof(unsigned long long), ctx->stream));
-        CR_CUDA(ctx, cudaMemsetAsync(tcnt, 0, slots * sizeof(uint32_t), ctx->stream));
+        CR_LAUNCH(ctx, k_plan_clear, cr_blocks(slots / 4, 256, gcap), 256, 0, p0->d_info, (unsigned long long)n, (uint4 *)tcnt,
+                  slots / 4, cnt, cq);
         CR_LAUNCH(ctx, k_hist_insert, grid_n, 256, 0, (const unsigned long long *)d_key, n, tkey, tcnt, tbits,
                   p0->d_info);
         CR_LAUNCH(ctx, k_hist_compact, cr_blocks(slots, 256, gcap), 256, 0, (const unsigned long long *)tkey,
@@ -1936,7 +1915,6 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
         // the (n - count) keys and the order ping-pong through the now idle table memory
         uint32_t *s32A = (uint32_t *)ptk, *s32B = s32A + n, *o32B = (uint32_t *)ptc;
         uint32_t *ord = (uint32_t *)po;
-        const bool one_cta = plan_sort_one_cta(n, cmax);
         if (n <= kPlanSortOneCta) {
             // admission candidates only: the largest slot budget of the build bounds how far it reaches
             CR_CUDA(ctx, cudaFuncSetAttribute(k_plan_topk, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1947,20 +1925,11 @@ static int build_plans(cr_ctx *ctx, const uint64_t *d_key, uint64_t n, const cr_
                       p0->d_ukey, p0->d_ucnt, s32A, s32B, ord + n, o32B, ord);
         }
         if (!one_cta) {
-            // the same two sorts in device-wide passes, the key count read on the device
-            // (no-ops when the one-CTA kernel has sorted the few keys there are)
-            const unsigned long long *dU = &p0->d_info->U;
-            const unsigned long long skip = n <= kPlanSortOneCta ? kBitonicMax : 0ull;
-            int in1 = 0;
-            CR_TRY(cr_radix_pairs_u64_dev(ctx, (unsigned long long *)pk0, (uint32_t *)pv0, (unsigned long long *)pk1,
-                                          (uint32_t *)pv1, n, dU, skip, 64, 0, &in1));
-            CR_LAUNCH(ctx, k_plan_sorted_keys, grid_n, 256, 0, (const cr_plan_info_dev *)p0->d_info, skip,
-                      (unsigned long long)n, (const unsigned long long *)(in1 ? pk1 : pk0),
-                      (const uint32_t *)(in1 ? pv1 : pv0), p0->d_ukey, p0->d_ucnt, s32A);
-            uint32_t *o32A = (uint32_t *)pv0;  // free again after the key sort's results were copied out
-            CR_TRY(cr_radix_pairs_u32_dev(ctx, s32A, o32A, s32B, o32B, n, dU, skip, bits_for(n), 1, &in1));
-            CR_LAUNCH(ctx, k_plan_copy_order, grid_n, 256, 0, p0->d_info, skip,
-                      (const uint32_t *)(in1 ? o32B : o32A), ord);
+            // every key, the whole GPU, the key count read on the device (it returns at once when
+            // the one-CTA kernel has sorted the few keys there are)
+            CR_TRY(cr_plan_sort_histogram(ctx, p0->d_info, n, n <= kPlanSortOneCta ? kBitonicMax : 0ull,
+                                          (unsigned long long *)pk0, (uint32_t *)pv0, (unsigned long long *)pk1,
+                                          (uint32_t *)pv1, p0->d_ukey, p0->d_ucnt, s32A, s32B, o32B, ord));
         }
         order = ord;
     }
@@ -2213,7 +2182,7 @@ __global__ void k_gather_u64(const unsigned long long *__restrict__ src, const u
                              unsigned long long n, unsigned long long *__restrict__ out)
 {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-        out[i] = src[idx[i]];
+        out[i] = src[min((unsigned long long)idx[i], n - 1ull)];  // (a sort that gave up leaves places unset)
 }
 
 extern "C" int cr_plan_export(cr_ctx *ctx, const cr_plan *p, uint64_t *ukey, uint64_t *ucnt, uint64_t *adm_key,
@@ -2231,7 +2200,7 @@ extern "C" int cr_plan_export(cr_ctx *ctx, const cr_plan *p, uint64_t *ukey, uin
         // only the admission candidates are in key order, or none: sort the whole histogram by key
         const unsigned long long *ks;
         const uint32_t *pos;
-        CR_TRY(cr_radix_sort_u64(ctx, (const unsigned long long *)p->d_ukey, nullptr, d.U, 64, &ks, &pos));
+        CR_TRY(cr_radix_sort_u64(ctx, (const unsigned long long *)p->d_ukey, d.U, &ks, &pos));
         void *pc;
         CR_TRY(cr_scratch(ctx, SCR_PLAN_A, d.U * sizeof(unsigned long long), &pc));
         CR_LAUNCH(ctx, k_gather_u64, cr_blocks(d.U, 256, (unsigned int)ctx->num_sms * 8u), 256, 0,

@@ -1375,7 +1375,7 @@ __global__ void __launch_bounds__(256) k_ring_finish(const unsigned long long *_
     for (unsigned long long j = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; j < M;
          j += (unsigned long long)gridDim.x * blockDim.x) {
         pt[j] = ks[j];
-        ow[j] = (uint16_t)(pos[j] / V);
+        ow[j] = (uint16_t)(min((unsigned long long)pos[j], M - 1ull) / V);  // (a sort that gave up leaves places unset)
     }
 }
 
@@ -1408,7 +1408,7 @@ static int ring_fill(cr_ctx *ctx, cr_ring *g, uint64_t seed)
     const unsigned long long *ks = nullptr;
     const uint32_t *pos = nullptr;
     CR_LAUNCH(ctx, k_ring_points, cr_blocks(M, 256, gcap), 256, 0, (unsigned long long)seed, M, g->d_point);
-    CR_TRY(cr_radix_sort_u64(ctx, g->d_point, nullptr, M, 64, &ks, &pos));
+    CR_TRY(cr_radix_sort_u64(ctx, g->d_point, M, &ks, &pos));
     CR_LAUNCH(ctx, k_ring_finish, cr_blocks(M, 256, gcap), 256, 0, ks, pos, M, g->V, g->d_point, g->d_owner);
     CR_LAUNCH(ctx, k_ring_dir, cr_blocks(1ull << g->dbits, 256, gcap), 256, 0, (const unsigned long long *)g->d_point,
               M, (int)g->dbits, g->d_dir);

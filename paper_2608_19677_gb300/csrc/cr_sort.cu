@@ -1,10 +1,6 @@
 // Device-wide scan and stable LSD radix sort.
 //
-// Radix sort: 8-bit digits, three launches per pass and no inter-block waits:
-//   upsweep   per-tile digit counts, written digit-major [256][ntiles]
-//   scan      exclusive scan of those counts = each tile's output base per digit
-//   downsweep each tile ranks its items stably (arrival order = round, warp,
-//             lane; warp peers found with __match_any_sync) and scatters them.
+// Radix sort: 8-bit digits, tiles of 2048 items, the whole sort in one launch (k_sort).
 // Scan: reduce-then-scan over 4096-element blocks, recursing on the partials.
 #include "cr_device.cuh"
 #include "cr_internal.cuh"
@@ -101,10 +97,8 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_block(const T *__restrict__
 constexpr uint32_t kScanOne = 32768;
 template <typename T>
 __global__ void __launch_bounds__(kScanBlock) k_scan_one(const T *__restrict__ in, T *__restrict__ out, uint64_t n,
-                                                         int inclusive, T *__restrict__ total_out,
-                                                         const unsigned long long *n_dev, unsigned long long skip_le)
+                                                         int inclusive, T *__restrict__ total_out)
 {
-    if (n_dev && *n_dev <= skip_le) return;
     __shared__ T tot;
     T carry = 0;
     for (uint64_t t0 = 0; t0 < n; t0 += 4ull * kScanBlock * 2) {  // 8,192 elements a round
@@ -149,8 +143,7 @@ int scan_rec(cr_ctx *ctx, const T *in, T *out, uint64_t n, int inclusive, T *d_t
         return CR_OK;
     }
     if (n <= kScanOne) {
-        CR_LAUNCH(ctx, k_scan_one<T>, 1, kScanBlock, 0, in, out, n, inclusive, d_total,
-                  (const unsigned long long *)nullptr, 0ull);
+        CR_LAUNCH(ctx, k_scan_one<T>, 1, kScanBlock, 0, in, out, n, inclusive, d_total);
         return CR_OK;
     }
     T *partial = partials;
@@ -171,167 +164,264 @@ int scan_impl(cr_ctx *ctx, const T *in, T *out, uint64_t n, int inclusive, T *d_
 }
 
 // ---------------------------------------------------------- radix sort ----
-// n_dev (optional): the item count in device memory; n is then an upper bound
-// that sized the grid and the histogram, and tiles past the count stay empty.
-// A count <= skip_le makes the pass a no-op (another path sorts those).
+// The whole sort is one launch.  Its work is a sequence of phases of `tiles` items each: the
+// digit counts of every pass (an LSD sort only reorders the items), a phase per 8-bit digit,
+// and for a plan the histogram's arrays and a second sort by count.  Blocks take items in
+// order by a ticket and wait, before an item, until the phase before is done, so what a
+// block waits for is always held by a block that is running, however few of them are.
+constexpr uint32_t kSortPasses = 12;           // 8 of a 64-bit key, up to 4 of a 32-bit one
+constexpr uint32_t kSortPhases = kSortPasses + 2;
+constexpr uint32_t kSortSpin = 1u << 20;       // looks at a word that does not come, ~0.5 s
+
+// Counters of a sort, zero before it.
+struct sort_counters {
+    uint32_t digits[kSortPasses][256];  // items of each digit value, per pass
+    uint32_t done[kSortPhases];         // items finished, per phase
+    uint32_t ticket, gave_up;
+    uint32_t pad[48];
+};
+static_assert(sizeof(sort_counters) % 256 == 0, "the tile states start aligned");
+
+struct sort_job {
+    const unsigned long long *k_in;  // the keys, and their values (NULL: the positions)
+    const uint32_t *v_in;
+    unsigned long long *k[2];        // pass p of the keys writes k[p & 1], v[p & 1]
+    uint32_t *v[2];
+    // a plan's histogram (order NULL: keys only): outputs, sort keys, positions
+    cr_plan_info_dev *info;
+    unsigned long long *ukey, *ucnt;
+    uint32_t *s[2], *o[2], *order;
+    uint32_t passes2;                // of the sort keys n_sum - count
+    unsigned long long n_sum;
+    unsigned long long n, skip_le;   // items (n_dev: at most), and the count up to which nothing is done
+    const unsigned long long *n_dev;
+    sort_counters *C;
+    unsigned long long *states[2];   // [tiles][256] of the even and the odd passes
+    uint32_t *status;
+};
+
+inline uint64_t sort_tiles(uint64_t n) { return (n + kSortTile - 1) / kSortTile; }
+
+// A tile's state of one digit: how far it is in the top two bits, a count below.
+constexpr unsigned long long kTileCount = 1ull << 62, kTilePrefix = 2ull << 62, kTileValue = kTileCount - 1ull;
+constexpr uint32_t kLookBack = 8;  // predecessors read at once
+
+struct sort_smem {
+    uint32_t wcnt[kSortBlock / 32][256];  // digit counts per warp (or per pass, in the counting phases)
+    uint32_t base[256], wsum[kSortBlock / 32];
+    uint32_t ticket, ok;
+};
+
+// One tile of a pass: the block ranks its 2048 items stably (warp w owns 256 consecutive
+// items, in rounds of 32), and thread d finds how many items of digit d the tiles before hold
+// by looking back over their states, eight at a time: a tile first publishes its own count,
+// without waiting, then the total through it.  What other blocks wrote is read past the L1.
 template <typename K>
-__global__ void __launch_bounds__(kSortBlock) k_radix_upsweep(const K *__restrict__ keys, uint64_t n, int shift,
-                                                              uint32_t ntiles, uint32_t *__restrict__ hist,
-                                                              const unsigned long long *n_dev,
-                                                              unsigned long long skip_le)
+__device__ __forceinline__ void sort_tile(sort_smem &S, uint32_t tile, const K *kin, const uint32_t *vin, K *kout,
+                                          uint32_t *vout, uint64_t n, int shift, const uint32_t *counts,
+                                          unsigned long long *states, unsigned long long *next_states,
+                                          sort_counters *C, uint32_t *status)
 {
-    if (n_dev && *n_dev <= skip_le) return;
-    if (n_dev && *n_dev < n) n = *n_dev;
-    __shared__ uint32_t cnt[256];
-    cnt[threadIdx.x] = 0;
+    constexpr int kWarps = kSortBlock / 32;
+    const uint32_t tid = threadIdx.x, lane = cr_lane(), warp = tid >> 5, lt = (1u << lane) - 1u;
+    const uint64_t i0 = (uint64_t)tile * kSortTile + warp * 256u + lane;
+    K key[kSortItems];
+    uint32_t rank[kSortItems];
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) key[j] = i0 + 32u * j < n ? __ldcg(kin + i0 + 32u * j) : (K)0;
+    const uint32_t total = __ldcg(counts + tid);
+    next_states[(uint64_t)tile * 256 + tid] = 0;  // of the pass before: no longer read
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) S.wcnt[w][tid] = 0;
     __syncthreads();
-    const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
 #pragma unroll
     for (int j = 0; j < kSortItems; ++j) {
-        uint64_t i = base + (uint64_t)j * kSortBlock + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(uint32_t)(keys[i] >> shift) & 0xffu], 1u);
+        const uint32_t d = (uint32_t)(key[j] >> shift) & 0xffu;
+        const bool in = i0 + 32u * j < n;
+        uint32_t peers = __ballot_sync(0xffffffffu, in);  // valid lanes of the round with this digit
+#pragma unroll
+        for (int bt = 0; bt < 8; ++bt) {
+            const uint32_t B = __ballot_sync(0xffffffffu, (d >> bt) & 1u);
+            peers &= ((d >> bt) & 1u) ? B : ~B;
+        }
+        const uint32_t before = S.wcnt[warp][d];
+        __syncwarp();
+        rank[j] = before + (uint32_t)__popc(peers & lt);
+        if (in && (peers & lt) == 0) S.wcnt[warp][d] = before + (uint32_t)__popc(peers);
+        __syncwarp();
     }
+    // items of the smaller digits: exclusive scan of the pass's 256 counts
+    uint32_t incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+    }
+    if (lane == 31) S.wsum[warp] = incl;
     __syncthreads();
-    hist[(uint64_t)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
+    uint32_t smaller = incl - total;
+    for (uint32_t w = 0; w < warp; ++w) smaller += S.wsum[w];
+    // thread d: digit d's items in the warps before, and in the tile
+    uint32_t mine = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const uint32_t c = S.wcnt[w][tid];
+        S.wcnt[w][tid] = mine;
+        mine += c;
+    }
+    volatile unsigned long long *st = states + tid;
+    unsigned long long before = 0;
+    if (tile) {
+        st[(uint64_t)tile * 256] = kTileCount | mine;
+        uint32_t t = tile, spin = 0;  // tiles t .. tile - 1 are counted
+        for (bool more = true; more;) {
+            unsigned long long s[kLookBack];
+#pragma unroll
+            for (uint32_t x = 0; x < kLookBack; ++x) {  // (tile 0's state is its prefix: none before it is needed)
+                s[x] = kTilePrefix;
+                if (x < t) s[x] = st[(uint64_t)(t - 1u - x) * 256];
+            }
+#pragma unroll
+            for (uint32_t x = 0; x < kLookBack; ++x) {
+                if (!more || !(s[x] >> 62)) break;  // (not there yet)
+                before += s[x] & kTileValue;
+                --t;
+                more = !(s[x] & kTilePrefix);
+            }
+            if (more && ++spin >= kSortSpin) {  // never: the items then go too low, not out of range
+                C->gave_up = 1;
+                atomicOr(status, CR_FLAG_TIMEOUT);
+                break;
+            }
+        }
+    }
+    st[(uint64_t)tile * 256] = kTilePrefix | (before + mine);
+    S.base[tid] = smaller + (uint32_t)before;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const uint64_t i = i0 + 32u * j;
+        if (i >= n) continue;
+        const uint32_t d = (uint32_t)(key[j] >> shift) & 0xffu, pos = S.base[d] + S.wcnt[warp][d] + rank[j];
+        kout[pos] = key[j];
+        vout[pos] = vin ? __ldcg(vin + i) : (uint32_t)i;
+    }
 }
 
-template <typename K>
-__global__ void __launch_bounds__(kSortBlock) k_radix_downsweep(const K *__restrict__ kin,
-                                                                const uint32_t *__restrict__ vin,
-                                                                K *__restrict__ kout, uint32_t *__restrict__ vout,
-                                                                uint64_t n, int shift, uint32_t ntiles,
-                                                                const uint32_t *__restrict__ offs,
-                                                                const unsigned long long *n_dev,
-                                                                unsigned long long skip_le)
+// Bound: the chain of phases (the wait for the one before, a tile's loads, its look-back), 5-7
+// us each.  Builds of one plan from 500,000 requests, C = 16,384, this sort in them: 500,000 keys
+// 282 us (304 with a launch per pass, 486 with three: tile counts, scan, scatter); 145 keys,
+// which it leaves alone, 82 us (142, 315: launches that find nothing to do are not free).
+__global__ void __launch_bounds__(kSortBlock, 3) k_sort(const __grid_constant__ sort_job J)
 {
-    if (n_dev && *n_dev <= skip_le) return;
-    if (n_dev && *n_dev < n) n = *n_dev;
-    constexpr int kWarps = kSortBlock / 32;
-    __shared__ uint32_t base_s[256];
-    __shared__ uint32_t wcnt[kWarps][257];
-    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5;
-    base_s[threadIdx.x] = offs[(uint64_t)threadIdx.x * ntiles + blockIdx.x];
-    uint32_t run = 0;  // items of digit threadIdx.x already placed in this tile
-    const uint64_t tbase = (uint64_t)blockIdx.x * kSortTile;
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    for (int j = 0; j < kSortItems; ++j) {
-        for (int w = 0; w < kWarps; ++w) wcnt[w][threadIdx.x] = 0;
-        if (threadIdx.x == 0)
-            for (int w = 0; w < kWarps; ++w) wcnt[w][256] = 0;
-        __syncthreads();
-        const uint64_t i = tbase + (uint64_t)j * kSortBlock + threadIdx.x;
-        const bool valid = i < n;
-        K key = valid ? kin[i] : (K)0;
-        uint32_t d = valid ? ((uint32_t)(key >> shift) & 0xffu) : 256u;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        uint32_t rank = __popc(peers & lt_mask);
-        if (rank == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        {
-            uint32_t dd = threadIdx.x;
-            for (int w = 0; w < kWarps; ++w) {
-                uint32_t c = wcnt[w][dd];
-                wcnt[w][dd] = run;
-                run += c;
+    uint64_t n = J.n;
+    if (J.n_dev) {
+        const uint64_t u = *J.n_dev;
+        if (u <= J.skip_le) return;
+        n = u < n ? u : n;
+    }
+    __shared__ sort_smem S;
+    uint32_t *cnt = &S.wcnt[0][0];  // [8 * 256]
+    sort_counters *C = J.C;
+    const uint32_t tid = threadIdx.x, lt = (1u << cr_lane()) - 1u;
+    const uint32_t tiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
+    const uint32_t phases = J.order ? 10u + J.passes2 : 9u;
+    for (;;) {
+        __syncthreads();  // (the shared memory of the item before)
+        if (tid == 0) {
+            const uint32_t t = atomicAdd(&C->ticket, 1u), phase = t / tiles;
+            S.ticket = t;
+            S.ok = 1;
+            if (phase > 0 && phase < phases) {
+                const volatile uint32_t *done = &C->done[phase - 1u];
+                uint32_t spin = 0;
+                while (*done < tiles && ++spin < kSortSpin) {}
+                if (*done < tiles) {  // never
+                    S.ok = 0;
+                    C->gave_up = 1;
+                    atomicOr(J.status, CR_FLAG_TIMEOUT);
+                }
+                __threadfence();
             }
         }
         __syncthreads();
-        if (valid) {
-            uint32_t pos = base_s[d] + wcnt[warp][d] + rank;
-            kout[pos] = key;
-            if (vout) vout[pos] = vin ? vin[i] : (uint32_t)i;
+        const uint32_t phase = S.ticket / tiles, tile = S.ticket - phase * tiles;
+        if (phase >= phases || !S.ok) return;
+        const uint64_t i0 = (uint64_t)tile * kSortTile + tid;
+        if (phase == 0) {
+            for (uint32_t x = tid; x < 8u * 256u; x += kSortBlock) cnt[x] = 0;
+            J.states[0][(uint64_t)tile * 256 + tid] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < kSortItems; ++j) {
+                const uint64_t i = i0 + (uint64_t)j * kSortBlock;
+                if (i >= n) break;
+                const unsigned long long key = J.k_in[i];
+#pragma unroll
+                for (int p = 0; p < 8; ++p) atomicAdd(&cnt[256 * p + ((uint32_t)(key >> (8 * p)) & 0xffu)], 1u);
+            }
+            __syncthreads();
+            for (uint32_t x = tid; x < 8u * 256u; x += kSortBlock)
+                if (cnt[x]) atomicAdd(&C->digits[0][0] + x, cnt[x]);
+        } else if (phase <= 8) {
+            const uint32_t p = phase - 1u, w = p & 1u;
+            sort_tile<unsigned long long>(S, tile, p ? J.k[w ^ 1u] : J.k_in, p ? J.v[w ^ 1u] : J.v_in, J.k[w], J.v[w], n,
+                                          (int)(8u * p), C->digits[p], J.states[w], J.states[w ^ 1u], C, J.status);
+        } else if (phase == 9) {
+            // the sorted pairs as the plan's histogram, the second sort's keys and their digits
+            for (uint32_t x = tid; x < 4u * 256u; x += kSortBlock) cnt[x] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < kSortItems; ++j) {
+                const uint64_t u = i0 + (uint64_t)j * kSortBlock;
+                const bool in = u < n;
+                uint32_t key = 0;
+                if (in) {
+                    const uint32_t c = __ldcg(J.v[1] + u);
+                    J.ukey[u] = __ldcg(J.k[1] + u);
+                    J.ucnt[u] = c;
+                    J.s[1][u] = key = (uint32_t)(J.n_sum - c);
+                }
+                // most counts are equal: one atomic per distinct sort key of the warp
+                const uint32_t peers = __match_any_sync(0xffffffffu, key) & __ballot_sync(0xffffffffu, in);
+                if (in && (peers & lt) == 0)
+                    for (uint32_t p = 0; p < J.passes2; ++p)
+                        atomicAdd(&cnt[256u * p + ((key >> (8u * p)) & 0xffu)], (uint32_t)__popc(peers));
+            }
+            __syncthreads();
+            for (uint32_t x = tid; x < 256u * J.passes2; x += kSortBlock)
+                if (cnt[x]) atomicAdd(&C->digits[8][0] + x, cnt[x]);
+        } else {
+            const uint32_t p = phase - 10u, w = p & 1u;
+            sort_tile<uint32_t>(S, tile, J.s[w ^ 1u], p ? J.o[w ^ 1u] : nullptr, J.s[w],
+                                p + 1u == J.passes2 ? J.order : J.o[w], n, (int)(8u * p), C->digits[8u + p], J.states[w],
+                                J.states[w ^ 1u], C, J.status);
         }
         __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            const uint32_t d = atomicAdd(&C->done[phase], 1u) + 1u;
+            // the order is whole (S stays 0 if a wait gave up: nothing is admitted then)
+            if (J.order && phase + 1u == phases && d == tiles && !*(volatile uint32_t *)&C->gave_up) J.info->S = n;
+        }
     }
 }
 
-template <typename K>
-int radix_impl(cr_ctx *ctx, const K *k_in, const uint32_t *v_in, uint64_t n, int bits, const K **k_out,
-               const uint32_t **v_out, int kslot0, int kslot1)
+int sort_launch(cr_ctx *ctx, sort_job &J, bool zero)
 {
-    const int want_vals = v_out != nullptr;
-    *k_out = k_in;
-    if (v_out) *v_out = v_in;
-    if (n == 0 || bits <= 0) return CR_OK;
-    if (n >= (1ull << 32)) return cr_fail(ctx, CR_EINVAL, "radix sort: n >= 2^32");
-    const uint32_t ntiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
-    void *kb0, *kb1, *vb0 = nullptr, *vb1 = nullptr, *hist;
-    CR_TRY(cr_scratch(ctx, kslot0, n * sizeof(K), &kb0));
-    CR_TRY(cr_scratch(ctx, kslot1, n * sizeof(K), &kb1));
-    if (want_vals) {
-        CR_TRY(cr_scratch(ctx, SCR_SORT_V0, n * sizeof(uint32_t), &vb0));
-        CR_TRY(cr_scratch(ctx, SCR_SORT_V1, n * sizeof(uint32_t), &vb1));
-    }
-    CR_TRY(cr_scratch(ctx, SCR_SORT_HIST, (size_t)256 * ntiles * sizeof(uint32_t), &hist));
-    const K *ksrc = k_in;
-    const uint32_t *vsrc = v_in;
-    int pass = 0;
-    for (int shift = 0; shift < bits; shift += 8, ++pass) {
-        K *kdst = reinterpret_cast<K *>((pass & 1) ? kb1 : kb0);
-        uint32_t *vdst = want_vals ? reinterpret_cast<uint32_t *>((pass & 1) ? vb1 : vb0) : nullptr;
-        CR_LAUNCH(ctx, k_radix_upsweep<K>, ntiles, kSortBlock, 0, ksrc, n, shift, ntiles, (uint32_t *)hist,
-                  (const unsigned long long *)nullptr, 0ull);
-        CR_TRY(scan_impl<uint32_t>(ctx, (const uint32_t *)hist, (uint32_t *)hist, (uint64_t)256 * ntiles, 0,
-                                   (uint32_t *)nullptr));
-        CR_LAUNCH(ctx, k_radix_downsweep<K>, ntiles, kSortBlock, 0, ksrc, vsrc, kdst, vdst, n, shift, ntiles,
-                  (const uint32_t *)hist, (const unsigned long long *)nullptr, 0ull);
-        ksrc = kdst;
-        vsrc = vdst;
-    }
-    *k_out = ksrc;
-    if (v_out) *v_out = vsrc;
-    return CR_OK;
-}
-
-// (key, value) pairs ping-ponged between caller buffers 0 and 1, bits
-// [0, bits) in 8-bit passes; the item count is read from n_dev (<= n_max).
-// With iota the input values are not read: they are the items' positions.
-template <typename K>
-int radix_pairs_dev(cr_ctx *ctx, K *k0, uint32_t *v0, K *k1, uint32_t *v1, uint64_t n_max,
-                    const unsigned long long *n_dev, unsigned long long skip_le, int bits, int iota, int *in1)
-{
-    *in1 = 0;
-    if (n_max == 0 || bits <= 0) return CR_OK;
-    if (n_max >= (1ull << 32)) return cr_fail(ctx, CR_EINVAL, "radix sort: n >= 2^32");
-    const uint32_t ntiles = (uint32_t)((n_max + kSortTile - 1) / kSortTile);
-    void *hist;
-    CR_TRY(cr_scratch(ctx, SCR_SORT_HIST, (size_t)256 * ntiles * sizeof(uint32_t), &hist));
-    int cur = 0;
-    for (int shift = 0; shift < bits; shift += 8) {
-        K *ks = cur ? k1 : k0, *kd = cur ? k0 : k1;
-        const uint32_t *vs = (shift == 0 && iota) ? nullptr : (cur ? v1 : v0);
-        uint32_t *vd = cur ? v0 : v1;
-        CR_LAUNCH(ctx, k_radix_upsweep<K>, ntiles, kSortBlock, 0, (const K *)ks, n_max, shift, ntiles,
-                  (uint32_t *)hist, n_dev, skip_le);
-        if ((uint64_t)256 * ntiles <= kScanOne)
-            CR_LAUNCH(ctx, k_scan_one<uint32_t>, 1, kScanBlock, 0, (const uint32_t *)hist, (uint32_t *)hist,
-                      (uint64_t)256 * ntiles, 0, (uint32_t *)nullptr, n_dev, skip_le);
-        else
-            CR_TRY(scan_impl<uint32_t>(ctx, (const uint32_t *)hist, (uint32_t *)hist, (uint64_t)256 * ntiles, 0,
-                                       (uint32_t *)nullptr));
-        CR_LAUNCH(ctx, k_radix_downsweep<K>, ntiles, kSortBlock, 0, (const K *)ks, vs, kd, vd, n_max, shift, ntiles,
-                  (const uint32_t *)hist, n_dev, skip_le);
-        cur ^= 1;
-    }
-    *in1 = cur;
+    uint4 *p;
+    uint32_t quads;
+    CR_TRY(cr_sort_counters(ctx, J.n, &p, &quads));
+    J.C = (sort_counters *)p;
+    J.states[0] = (unsigned long long *)(J.C + 1);
+    J.states[1] = J.states[0] + sort_tiles(J.n) * 256;
+    J.status = ctx->d_status;
+    if (zero) CR_CUDA(ctx, cudaMemsetAsync(J.C, 0, sizeof(sort_counters), ctx->stream));
+    CR_LAUNCH(ctx, k_sort, cr_blocks(sort_tiles(J.n), 1, (unsigned int)ctx->num_sms * 3u), kSortBlock, 0, J);
     return CR_OK;
 }
 
 }  // namespace
-
-int cr_radix_pairs_u64_dev(cr_ctx *ctx, unsigned long long *k0, uint32_t *v0, unsigned long long *k1, uint32_t *v1,
-                           uint64_t n_max, const unsigned long long *n_dev, unsigned long long skip_le, int bits,
-                           int iota, int *in1)
-{
-    return radix_pairs_dev<unsigned long long>(ctx, k0, v0, k1, v1, n_max, n_dev, skip_le, bits, iota, in1);
-}
-
-int cr_radix_pairs_u32_dev(cr_ctx *ctx, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, uint64_t n_max,
-                           const unsigned long long *n_dev, unsigned long long skip_le, int bits, int iota,
-                           int *in1)
-{
-    return radix_pairs_dev<uint32_t>(ctx, k0, v0, k1, v1, n_max, n_dev, skip_le, bits, iota, in1);
-}
 
 int cr_scan_u32(cr_ctx *ctx, const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *d_total)
 {
@@ -343,14 +433,62 @@ int cr_scan_u64_inclusive(cr_ctx *ctx, const unsigned long long *in, unsigned lo
     return scan_impl<unsigned long long>(ctx, in, out, n, 1, (unsigned long long *)nullptr);
 }
 
-int cr_radix_sort_u64(cr_ctx *ctx, const unsigned long long *k_in, const uint32_t *v_in, uint64_t n, int bits,
-                      const unsigned long long **k_out, const uint32_t **v_out)
+int cr_sort_counters(cr_ctx *ctx, uint64_t n, uint4 **counters, uint32_t *quads)
 {
-    return radix_impl<unsigned long long>(ctx, k_in, v_in, n, bits, k_out, v_out, SCR_SORT_K0, SCR_SORT_K1);
+    if (n >= (1ull << 32)) return cr_fail(ctx, CR_EINVAL, "radix sort: n >= 2^32");
+    void *p;
+    CR_TRY(cr_scratch(ctx, SCR_SORT_HIST, sizeof(sort_counters) + 2 * sort_tiles(n) * 256 * sizeof(unsigned long long), &p));
+    *counters = (uint4 *)p;
+    *quads = (uint32_t)(sizeof(sort_counters) / sizeof(uint4));
+    return CR_OK;
 }
 
-int cr_radix_sort_u32(cr_ctx *ctx, const uint32_t *k_in, const uint32_t *v_in, uint64_t n, int bits,
-                      const uint32_t **k_out, const uint32_t **v_out)
+int cr_radix_sort_u64(cr_ctx *ctx, const unsigned long long *k_in, uint64_t n, const unsigned long long **k_out,
+                      const uint32_t **pos_out)
 {
-    return radix_impl<uint32_t>(ctx, k_in, v_in, n, bits, k_out, v_out, SCR_SORT_K0, SCR_SORT_K1);
+    *k_out = k_in;
+    *pos_out = nullptr;
+    if (n == 0) return CR_OK;
+    sort_job J = {};
+    J.k_in = k_in;
+    J.n = n;
+    for (int x = 0; x < 2; ++x) {
+        void *k, *v;
+        CR_TRY(cr_scratch(ctx, x ? SCR_SORT_K1 : SCR_SORT_K0, n * sizeof(unsigned long long), &k));
+        CR_TRY(cr_scratch(ctx, x ? SCR_SORT_V1 : SCR_SORT_V0, n * sizeof(uint32_t), &v));
+        J.k[x] = (unsigned long long *)k;
+        J.v[x] = (uint32_t *)v;
+    }
+    CR_TRY(sort_launch(ctx, J, true));
+    *k_out = J.k[1];  // eight passes: the last one writes buffers 1
+    *pos_out = J.v[1];
+    return CR_OK;
+}
+
+int cr_plan_sort_histogram(cr_ctx *ctx, cr_plan_info_dev *info, uint64_t n, unsigned long long skip_le,
+                           unsigned long long *k0, uint32_t *v0, unsigned long long *k1, uint32_t *v1,
+                           unsigned long long *ukey, unsigned long long *ucnt, uint32_t *sA, uint32_t *sB,
+                           uint32_t *oB, uint32_t *order)
+{
+    sort_job J = {};
+    J.k_in = k0;
+    J.v_in = v0;
+    J.k[0] = k1;
+    J.v[0] = v1;
+    J.k[1] = k0;
+    J.v[1] = v0;
+    J.info = info;
+    J.ukey = ukey;
+    J.ucnt = ucnt;
+    J.s[0] = sB;  // pass p of the second sort reads s[p & 1 ^ 1]: sA first
+    J.s[1] = sA;
+    J.o[0] = oB;
+    J.o[1] = v0;  // (the counts have been copied out by then)
+    J.order = order;
+    J.passes2 = 1;
+    while (J.passes2 < 4 && (n >> (8 * J.passes2))) ++J.passes2;  // n - count < 2^(8 passes)
+    J.n_sum = J.n = n;
+    J.n_dev = &info->U;
+    J.skip_le = skip_le;
+    return sort_launch(ctx, J, false);
 }

@@ -1163,6 +1163,48 @@ def test_every_plan_exports_its_histogram(P, ctx, n, U):
         assert (got["ukey"] == uk).all() and (got["ucnt"] == uc).all()
 
 
+@pytest.mark.parametrize("pattern", ["random", "small", "high", "equal"])
+@pytest.mark.parametrize("U", [4097, 6144, 6145, 32768, 32769, 70001])
+def test_plan_wide_sort(P, ctx, U, pattern):
+    # the sort of more than 4,096 keys by the whole GPU, at the edges of its tiles of 2,048: keys
+    # that differ in every digit, only in the low or the high ones, counts of one to four digits
+    # or all equal
+    rng = np.random.default_rng(U)
+    pool = {"random": rng.choice(2**62, U, replace=False).astype(np.uint64) * np.uint64(3),
+            "small": np.arange(U, dtype=np.uint64), "high": np.arange(U, dtype=np.uint64) << np.uint64(44),
+            "equal": np.arange(U, dtype=np.uint64) * np.uint64(2**46 + 1)}[pattern]
+    cnt = np.ones(U, np.int64) if pattern == "equal" else 1 + (rng.pareto(1.0, U) * 0.7).astype(np.int64).clip(0, 70000)
+    keys = np.repeat(pool, cnt)
+    rng.shuffle(keys)
+    n, R, W = keys.size, 64, 70  # C = 4,480
+    got = P.build_plan(ctx, d_u64(keys), P.plan_params(R, W, 5 * n, 4 * R)).export()
+    _cmp_plan(got, O.build_plan(keys, R, W, 5 * n, 4 * R))
+    uk, uc = O.histogram(keys)
+    assert (got["ukey"] == uk).all() and (got["ucnt"] == uc).all()
+
+
+def test_plan_wide_sort_on_many_streams(P):
+    # eight builds at once on streams of their own: a block of the sort waits only for work that
+    # a running block holds, so they do not need the whole GPU to themselves
+    rng = np.random.default_rng(8)
+    n, R, W = 600000, 256, 256
+    keys = rng.integers(0, 400000, n).astype(np.uint64) * np.uint64(0x9e3779b97f4a7c15)
+    dk = d_u64(keys)
+    torch.cuda.synchronize()
+    ctxs = [P.Context(0, torch.cuda.Stream(DEV)) for _ in range(8)]
+    plans = [P.Plan(c) for c in ctxs]
+    prm = P.plan_params(R, W, 5 * n, 4 * R)
+    for _ in range(5):
+        for c, p in zip(ctxs, plans):
+            P.build_plans(c, dk, [prm], [p])
+    ref = O.build_plan(keys, R, W, 5 * n, 4 * R)
+    for p in plans:
+        _cmp_plan(p.export(), ref)
+    for c, p in zip(ctxs, plans):
+        p.close()
+        c.close()
+
+
 @pytest.mark.parametrize("R,W,kinds", [(1024, 66, ("SLOTCAP", "LPT")), (2048, 33, ("SLOTCAP", "LPT")),
                                        (2048, 33, ("SLOTCAP", "RANDOM")), (4096, 33, ("SLOTCAP", "SLOTCAP", "LPT", "RANDOM"))])
 def test_plans_beside_a_trimmed_slotcap(P, ctx, R, W, kinds):
