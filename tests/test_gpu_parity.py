@@ -109,6 +109,21 @@ def test_hash_every_start_and_remainder(P, ctx, shift):
     assert (h_u64(got) == ref).all()
 
 
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_hash_short_spans(P, ctx, shift):
+    # the lengths that are read word by word (8 to 192 tokens, unless they are whole vectors) and
+    # their neighbours, at every start within a vector, the arena itself `shift` tokens into one
+    plens = np.repeat(np.concatenate([np.arange(0, 12), np.arange(60, 70), np.arange(124, 132), np.arange(186, 204)]), 4)
+    offs = np.cumsum(np.concatenate([[0], plens[:-1] + 5])) // 4 * 4 + np.tile(np.arange(4), plens.size // 4)
+    tok = np.random.default_rng(shift).integers(-2**31, 2**31, int(offs[-1] + 300), dtype=np.int64).astype(np.int32)
+    ref = O.hash_prefixes(tok, offs.astype(np.uint64), plens.astype(np.uint32), salt=7)
+    dev = torch.zeros(tok.size + 3, dtype=torch.int32, device=DEV)[shift:shift + tok.size]
+    dev.copy_(torch.from_numpy(tok))
+    got = P.hash_prefixes(ctx, dev, d_u64(offs), d_u32(plens), salt=7)
+    ctx.sync()
+    assert (h_u64(got) == ref).all()
+
+
 def test_hash_empty(P, ctx):
     t = torch.zeros(4, dtype=torch.int32, device=DEV)
     out = P.hash_prefixes(ctx, t, torch.zeros(0, dtype=torch.int64, device=DEV),
