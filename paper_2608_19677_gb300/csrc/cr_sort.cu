@@ -92,32 +92,76 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_block(const T *__restrict__
     if (total_out && threadIdx.x == kScanBlock - 1 && blockIdx.x == gridDim.x - 1) *total_out = pre;
 }
 
-// Scan of up to kScanOne elements by one CTA, kScanOne / 1024 consecutive elements per
-// thread: one launch instead of three.
+// Eight consecutive elements, in 16-byte accesses where all of them are there (`in` on a
+// 16-byte boundary, i a multiple of 8).
+template <typename T>
+__device__ __forceinline__ void load8(T (&x)[8], const T *__restrict__ in, uint64_t i, uint64_t n)
+{
+    if (i + 8 <= n) {
+        constexpr int kQuads = (int)(8 * sizeof(T) / sizeof(uint4));
+        union {
+            uint4 q[kQuads];
+            T t[8];
+        } u;
+#pragma unroll
+        for (int j = 0; j < kQuads; ++j) u.q[j] = reinterpret_cast<const uint4 *>(in + i)[j];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = u.t[j];
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = i + j < n ? in[i + j] : (T)0;
+    }
+}
+template <typename T>
+__device__ __forceinline__ void store8(const T (&x)[8], T *__restrict__ out, uint64_t i, uint64_t n)
+{
+    if (i + 8 <= n) {
+        constexpr int kQuads = (int)(8 * sizeof(T) / sizeof(uint4));
+        union {
+            uint4 q[kQuads];
+            T t[8];
+        } u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) u.t[j] = x[j];
+#pragma unroll
+        for (int j = 0; j < kQuads; ++j) reinterpret_cast<uint4 *>(out + i)[j] = u.q[j];
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (i + j < n) out[i + j] = x[j];
+    }
+}
+
+// Scan of up to kScanOne elements (arrays on 16-byte boundaries) by one CTA, eight consecutive
+// elements per thread and round, the next round's loads in flight: one launch instead of three.
 constexpr uint32_t kScanOne = 32768;
 template <typename T>
-__global__ void __launch_bounds__(kScanBlock) k_scan_one(const T *__restrict__ in, T *__restrict__ out, uint64_t n,
-                                                         int inclusive, T *__restrict__ total_out)
+__global__ void __launch_bounds__(kScanBlock) k_scan_one(const T *in, T *out, uint64_t n, int inclusive,
+                                                         T *__restrict__ total_out)
 {
     __shared__ T tot;
-    T carry = 0;
-    for (uint64_t t0 = 0; t0 < n; t0 += 4ull * kScanBlock * 2) {  // 8,192 elements a round
-        const uint64_t base = t0 + (uint64_t)threadIdx.x * 8;
-        T x[8], s = 0;
+    T carry = 0, x[8];
+    const uint64_t i0 = (uint64_t)threadIdx.x * 8;
+    load8(x, in, i0, n);
+    for (uint64_t t0 = 0; t0 < n; t0 += 8ull * kScanBlock) {
+        const uint64_t i = t0 + i0;
+        T y[8], s = 0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            x[j] = base + j < n ? in[base + j] : (T)0;
+            y[j] = x[j];
             s += x[j];
         }
+        load8(x, in, i + 8ull * kScanBlock, n);  // (elements that this round does not write)
         T pre = carry + block_excl_scan<T>(s, &tot);
         carry += tot;
         __syncthreads();  // (tot is written again)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const T nx = pre + x[j];
-            if (base + j < n) out[base + j] = inclusive ? nx : pre;
+            const T nx = pre + y[j];
+            y[j] = inclusive ? nx : pre;
             pre = nx;
         }
+        store8(y, out, i, n);
     }
     if (total_out && threadIdx.x == 0) *total_out = carry;
 }
@@ -142,7 +186,7 @@ int scan_rec(cr_ctx *ctx, const T *in, T *out, uint64_t n, int inclusive, T *d_t
         CR_LAUNCH(ctx, k_scan_block<T>, 1, kScanBlock, 0, in, out, n, (const T *)nullptr, inclusive, d_total);
         return CR_OK;
     }
-    if (n <= kScanOne) {
+    if (n <= kScanOne && (((uintptr_t)in | (uintptr_t)out) & 15u) == 0) {
         CR_LAUNCH(ctx, k_scan_one<T>, 1, kScanBlock, 0, in, out, n, inclusive, d_total);
         return CR_OK;
     }
