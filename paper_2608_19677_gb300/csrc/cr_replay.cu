@@ -301,8 +301,25 @@ __global__ void k_chunk_counts(const uint32_t *__restrict__ start, uint32_t ns, 
     if ((threadIdx.x & 31u) == 0 && nf) atomicAdd(&next[2], nf);
 }
 
-// map[x] and map[items_max + x]: item x's stream and chunk.  coff[s]: chunks of the streams
-// before s; next[0], next[1]: long and other items placed so far.
+// map[x] and map[items_max + x]: item x's stream and chunk.  f / b: places of the stream's long
+// / other chunks.
+struct item_map {
+    uint32_t *__restrict__ map;
+    uint64_t items_max;
+    uint32_t CL, longer;
+    __device__ __forceinline__ void put(uint32_t s, uint32_t len, uint32_t n, uint32_t f, uint32_t b, uint32_t c) const
+    {
+        const bool full = CL > longer;  // all chunks but the last have CL requests
+        uint32_t x = (full ? f : b) + c;
+        if (c + 1u == n) x = len - c * CL > longer ? f + (full ? c : 0u) : b + (full ? 0u : c);
+        if (x < items_max) {
+            map[x] = s;
+            map[items_max + x] = c;
+        }
+    }
+};
+
+// coff[s]: chunks of the streams before s; next[0], next[1]: long and other items placed so far.
 __global__ void k_item_map(const uint32_t *__restrict__ start, const uint32_t *__restrict__ coff, uint32_t ns,
                            uint32_t CL, uint32_t longer, uint32_t *next, uint32_t *__restrict__ map,
                            uint64_t items_max)
@@ -321,61 +338,75 @@ __global__ void k_item_map(const uint32_t *__restrict__ start, const uint32_t *_
         }
         f0 = __shfl_sync(0xffffffffu, f0, 31) + fi - nf;
         b0 = __shfl_sync(0xffffffffu, b0, 31) + first + bi - (nch - nf);
-        for (uint32_t c = 0; c < nch; ++c) {
-            const uint32_t x = min(len - c * CL, CL) > longer ? f0++ : b0++;
-            if (x < items_max) {
-                map[x] = s;
-                map[items_max + x] = c;
-            }
-        }
+        const item_map M = {map, items_max, CL, longer};
+        for (uint32_t c = 0; c < nch; ++c) M.put(s, len, nch, f0, b0, c);
     }
 }
 
 // The same for up to kItemsCta streams by one CTA, stream starts included: one launch in
-// place of k_part_starts, k_chunk_counts, a scan and k_item_map.  Thread t takes `per`
-// consecutive streams.  30 replicas x 133,333 requests, 64 destinations,
-// with the records packed in the count launch: 212 -> 192 us a call; one interval of 20,000
-// requests, two replicas 154 -> 142 us.
-constexpr uint32_t kItemsCta = 32768;
+// place of k_part_starts, k_chunk_counts, a scan and k_item_map.  A warp takes 32 consecutive
+// streams at a time; the chunks of a stream with more than a few are left for a warp of their
+// own (one lane took 120 us over the 3,907 chunks of a call on one stream).  30 replicas x
+// 133,333 requests, 64 destinations, with the records packed in the count launch: 212 -> 192 us
+// a call; one interval of 20,000 requests, two replicas 154 -> 142 us.  8,000 / 12,288 / 20,480
+// / 30,720 streams of a few requests, partition: 38 / 46 / 58 / 70 us, in four launches 38 (from
+// 8,193) / 46 / 50 / 50.
+constexpr uint32_t kItemsCta = 8192, kItemsMany = 512;
 __global__ void __launch_bounds__(1024) k_items_cta(const uint32_t *__restrict__ off, uint32_t ns, uint32_t ntiles,
                                                     const uint32_t *__restrict__ total_in, uint32_t *start, uint32_t CL,
                                                     uint32_t longer, uint32_t *__restrict__ total,
                                                     uint32_t *__restrict__ map, uint64_t items_max)
 {
-    extern __shared__ uint32_t st[];  // [ns + 1] the starts again: the loops below are serial
-    __shared__ uint32_t wf[32], wb[32];
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    extern __shared__ uint32_t st[];  // [ns + 1] the starts again
+    __shared__ uint32_t s_long, s_other, n_long;  // places given out, long items
+    __shared__ uint3 many[kItemsMany];            // streams of many chunks: stream, f, b
+    __shared__ uint32_t n_many;
+    const uint32_t lane = threadIdx.x & 31u;
+    if (threadIdx.x == 0) s_long = s_other = n_long = n_many = 0;
+#pragma unroll 4
     for (uint32_t s = threadIdx.x; s <= ns; s += 1024u)
         start[s] = st[s] = s < ns ? off[(unsigned long long)s * ntiles] : *total_in;
     __syncthreads();
-    const uint32_t per = (ns + 1023u) / 1024u, s0 = min(threadIdx.x * per, ns), s1 = min(s0 + per, ns);
-    uint32_t nf = 0, nb = 0;  // long and other chunks of this thread's streams
-    for (uint32_t s = s0; s < s1; ++s) {
-        const uint32_t len = st[s + 1] - st[s], nch = len ? (len + CL - 1u) / CL : 1u;
-        const uint32_t f = long_chunks(len, nch, CL, longer);
-        nf += f;
-        nb += nch - f;
+    auto chunks = [&](uint32_t s, uint32_t &len, uint32_t &nch, uint32_t &nf) {
+        const bool in = s < ns;
+        len = in ? st[s + 1] - st[s] : 0u;
+        nch = in ? (len ? (len + CL - 1u) / CL : 1u) : 0u;
+        nf = nch ? long_chunks(len, nch, CL, longer) : 0u;
+    };
+    const item_map M = {map, items_max, CL, longer};
+    uint32_t len, nch, nf, sum = 0;
+    for (uint32_t s0 = threadIdx.x & ~31u; s0 < ns; s0 += 1024u) {
+        chunks(s0 + lane, len, nch, nf);
+        sum += nf;
     }
-    const uint32_t fi = warp_incl_scan(nf, lane), bi = warp_incl_scan(nb, lane);
-    if (lane == 31) {
-        wf[warp] = fi;
-        wb[warp] = bi;
-    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0 && sum) atomicAdd(&n_long, sum);
     __syncthreads();
-    const uint32_t fw = warp_incl_scan(wf[lane], lane), bw = warp_incl_scan(wb[lane], lane);  // over the 32 warps
-    const uint32_t first = __shfl_sync(0xffffffffu, fw, 31);
-    const uint32_t fp = __shfl_sync(0xffffffffu, fw, (warp + 31u) & 31u), bp = __shfl_sync(0xffffffffu, bw, (warp + 31u) & 31u);
-    uint32_t f0 = fi - nf + (warp ? fp : 0u), b0 = first + bi - nb + (warp ? bp : 0u);
-    if (threadIdx.x == 1023) *total = b0 + nb;
-    for (uint32_t s = s0; s < s1; ++s) {
-        const uint32_t len = st[s + 1] - st[s], nch = len ? (len + CL - 1u) / CL : 1u;
-        for (uint32_t c = 0; c < nch; ++c) {
-            const uint32_t x = min(len - c * CL, CL) > longer ? f0++ : b0++;
-            if (x < items_max) {
-                map[x] = s;
-                map[items_max + x] = c;
+    for (uint32_t s0 = threadIdx.x & ~31u; s0 < ns; s0 += 1024u) {
+        chunks(s0 + lane, len, nch, nf);
+        const uint32_t fi = warp_incl_scan(nf, lane), bi = warp_incl_scan(nch - nf, lane);
+        uint32_t f0 = 0, b0 = 0;
+        if (lane == 31) {
+            if (fi) f0 = atomicAdd(&s_long, fi);
+            if (bi) b0 = atomicAdd(&s_other, bi);
+        }
+        f0 = __shfl_sync(0xffffffffu, f0, 31) + fi - nf;
+        b0 = __shfl_sync(0xffffffffu, b0, 31) + n_long + bi - (nch - nf);
+        if (nch > 4u) {
+            const uint32_t i = atomicAdd(&n_many, 1u);
+            if (i < kItemsMany) {
+                many[i] = make_uint3(s0 + lane, f0, b0);
+                nch = 0;
             }
         }
+        for (uint32_t c = 0; c < nch; ++c) M.put(s0 + lane, len, nch, f0, b0, c);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *total = n_long + s_other;
+    for (uint32_t i = threadIdx.x >> 5; i < min(n_many, kItemsMany); i += 32u) {
+        const uint3 e = many[i];
+        chunks(e.x, len, nch, nf);
+        for (uint32_t c = lane; c < nch; c += 32u) M.put(e.x, len, nch, e.y, e.z, c);
     }
 }
 

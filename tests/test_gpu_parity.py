@@ -1465,6 +1465,27 @@ def test_replay_partition_edges(P, ctx, R, n):
     assert (h_u64(ctr) == orp.ctr).all()
 
 
+@pytest.mark.parametrize("R,n,hot", [(1, 10007, 0.0), (3, 9001, 0.0), (600, 800000, 0.0), (8192, 60000, 0.5),
+                                     (8191, 60000, 0.5), (2731, 50000, 0.3)])
+def test_replay_items_of_many_chunks(P, ctx, R, n, hot):
+    # streams of more than a few chunks (of 256 requests): one, three, 600 of them (more than one
+    # CTA lists), a hot one among thousands; around 8,192 streams in one CTA or in four launches
+    rng = np.random.default_rng(R)
+    dest = rng.integers(0, R, (3 if R == 2731 else 1, n)).astype(np.uint16)
+    dest[:, rng.random(n) < hot] = R // 2
+    keys = rng.integers(1, 9, n).astype(np.uint64)
+    plen = rng.integers(1, 5000, n).astype(np.uint32)
+    slen = np.full(n, 64, np.uint32)
+    orp = O.Replay(dest.shape[0], R, [3])
+    rp = P.Replay(ctx, dest.shape[0], R, [3])
+    ctr = torch.zeros((dest.shape[0], 1, R, 5), dtype=torch.int64, device=DEV)
+    for _ in range(2):
+        orp.step(keys, plen, slen, dest)
+        P.shadow_replay(ctx, rp, d_u64(keys), d_u32(plen), d_u32(slen), d_u16(dest), ctr)
+    ctx.sync()
+    assert (h_u64(ctr) == orp.ctr).all()
+
+
 @pytest.mark.parametrize("tokens", [False, True])
 @pytest.mark.parametrize("R,hot", [(40, [7]), (700, [3, 200, 699]), (700, list(range(0, 700, 9))), (33, [])])
 def test_replay_items_of_long_streams(P, ctx, tokens, R, hot):
