@@ -45,11 +45,7 @@ enum cr_scratch_slot {
     SCR_PLAN_A,        // plan-build temporaries
     SCR_PLAN_B,
     SCR_PLAN_C,
-    SCR_REPLAY_IDX,    // partitioned request indices
-    SCR_REPLAY_START,  // per-stream start offsets
-    SCR_REPLAY_REC,    // request indices in stream order
-    SCR_REPLAY_RECS,   // (key, prefix, suffix) record of each request
-    SCR_REPLAY_CHUNK,  // per-stream chunk counts -> offsets, and their total
+    SCR_REPLAY_REST,   // replay items left to the window kernels, and their number
     SCR_ROUTE_DESC,    // per-replica route descriptors
     SCR_DIFF,          // plan-difference counters
     SCR_NUM

@@ -410,12 +410,154 @@ __global__ void __launch_bounds__(1024) k_items_cta(const uint32_t *__restrict__
     }
 }
 
+// State before and after a call: [stream][cmax] (token capacities: [stream][kTokMax]), most
+// recent first.
 struct replay_state {
-    const unsigned long long *keys_in;  // [stream][cmax], most recent first
+    const unsigned long long *keys_in;
+    const uint32_t *cum_in;  // token capacities: tokens of entries 0 .. j
     const uint32_t *fill_in;
     unsigned long long *keys_out;
+    uint32_t *cum_out;
     uint32_t *fill_out;
 };
+
+inline replay_state state_of(const cr_replay *rp)
+{
+    return {rp->d_keys[rp->cur],     rp->d_size[rp->cur],     rp->d_fill[rp->cur],
+            rp->d_keys[rp->cur ^ 1], rp->d_size[rp->cur ^ 1], rp->d_fill[rp->cur ^ 1]};
+}
+
+__device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b)
+{
+    const uint32_t v = a + b;
+    return v < a ? 0xffffffffu : v;
+}
+
+// ---- replay of calls whose streams are mostly empty or a few requests long ----------
+// One warp per item, the list in registers (lane j holds entry j), one request at a time: items
+// whose carried-in keys and requests are at most 32 together; empty streams carry their state
+// over whatever its size; the others are left in rest[1 ..], their number in rest[0].  Nothing
+// in shared memory, so that the chain of dependent reads (item, stream, state, indices,
+// records) overlaps over three to five times the warps that the windows below leave room for,
+// which an item of two requests pays for without using them.  Simulation alone, 24 replicas x
+// 1,000 requests over 8,192 destinations, 24,576 tokens 289 -> 53 us, capacity 128 107 -> 55;
+// 48 x 4,096 over 1,024, 24,576 tokens 125 -> 37 (prefixes of 175 tokens on average, lists of
+// 140: 216 -> 212).
+template <bool TOKENS>
+__global__ void __launch_bounds__(256) k_replay_short(const __grid_constant__ replay_caps caps, uint32_t lim, uint32_t stride,
+                                                      uint32_t R, uint32_t ns, const uint32_t *__restrict__ start,
+                                                      const uint32_t *__restrict__ map, uint32_t items_max,
+                                                      const uint32_t *__restrict__ total, const uint32_t *__restrict__ idx,
+                                                      const rec16 *__restrict__ recs, uint32_t nrec, const replay_state st,
+                                                      unsigned long long *__restrict__ ctr, uint32_t *rest, uint32_t *status)
+{
+    __shared__ uint32_t s_rest, s_at;
+    const uint32_t lane = cr_lane(), w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (threadIdx.x == 0) s_rest = 0;
+    __syncthreads();
+    const bool mine = w < *total;
+    uint32_t s = 0, ci = 0, b = 0, e = 0, fin = 0;
+    if (mine) {
+        s = min(map[w], ns - 1u);
+        ci = map[items_max + w];
+        b = start[s];
+        e = start[s + 1];
+        fin = min(st.fill_in[s], stride);
+    }
+    const uint32_t n = e - b;
+    const bool few = mine && n && ci == 0 && n <= 32u && fin <= 32u - n;
+    uint32_t at = 0;
+    if (mine && n && !few && lane == 0) at = atomicAdd(&s_rest, 1u);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_rest) s_at = atomicAdd(rest, s_rest);
+    __syncthreads();
+    if (mine && n && !few && lane == 0) rest[1u + s_at + at] = w;
+    const unsigned long long *kin = st.keys_in + (size_t)s * stride;
+    unsigned long long *kout = st.keys_out + (size_t)s * stride;
+    const uint32_t *cin = TOKENS ? st.cum_in + (size_t)s * stride : nullptr;
+    uint32_t *cout = TOKENS ? st.cum_out + (size_t)s * stride : nullptr;
+    if (mine && n == 0) {
+        for (uint32_t j = lane; j < fin; j += 32) {
+            kout[j] = kin[j];
+            if (TOKENS) cout[j] = cin[j];
+        }
+        if (lane == 0) st.fill_out[s] = fin;
+    }
+    if (!few) return;  // (whole warps: no barrier follows)
+    const uint32_t mycap = lane < caps.n_caps ? caps.cap[lane] : 0u;
+    rec16 r = {0ull, 0u, 0u};
+    if (lane < n) r = recs[min(idx[b + lane], nrec - 1u)];
+    unsigned long long kr = lane < fin ? kin[lane] : 0ull;
+    uint32_t cr = TOKENS && lane < fin ? cin[lane] : 0u, f = fin;  // tokens through the entry; entries
+    uint32_t hits = 0;
+    unsigned long long hit_tok = 0;
+    for (uint32_t q = 0; q < n; ++q) {  // uniform
+        const unsigned long long x = __shfl_sync(0xffffffffu, r.key, q);
+        const uint32_t P = __shfl_sync(0xffffffffu, r.P, q);
+        const uint32_t match = __ballot_sync(0xffffffffu, lane < f && kr == x);
+        const bool found = match != 0;
+        const uint32_t pos = found ? (uint32_t)__ffs(match) - 1u : f;  // f <= 31 when it is not found
+        uint32_t depth = pos + 1u;
+        if (TOKENS) {
+            depth = __shfl_sync(0xffffffffu, cr, pos);
+            const uint32_t before = __shfl_sync(0xffffffffu, cr, pos ? pos - 1u : 0u);
+            if (found && depth - (pos ? before : 0u) != P && lane == 0) atomicOr(status, CR_FLAG_BADSIZE);
+        }
+        if (found && depth <= mycap) {  // lane c: capacity c
+            ++hits;
+            hit_tok += P;
+        }
+        // entries [0, pos) move down one place and now follow x
+        const unsigned long long ku = __shfl_up_sync(0xffffffffu, kr, 1);
+        const uint32_t cu = TOKENS ? __shfl_up_sync(0xffffffffu, cr, 1) : 0u;
+        if (lane <= pos) {
+            kr = lane ? ku : x;
+            cr = TOKENS ? (lane ? sat_add(cu, P) : P) : 0u;
+        }
+        f += found ? 0u : 1u;
+        if (TOKENS) {
+            const uint32_t over = __ballot_sync(0xffffffffu, lane < f && cr > lim);
+            if (over) f = (uint32_t)__ffs(over) - 1u;
+        } else {
+            f = min(f, lim);
+        }
+    }
+    if (lane < f) {
+        kout[lane] = kr;
+        if (TOKENS) cout[lane] = cr;
+    }
+    if (lane == 0) st.fill_out[s] = f;
+    const unsigned long long prompt = cr_warp_sum_u64(lane < n ? (unsigned long long)r.P + r.S : 0ull);
+    if (lane < caps.n_caps) {
+        unsigned long long *C = ctr + (((unsigned long long)(s / R) * caps.n_caps + lane) * R + s % R) * CR_CTR_FIELDS;
+        atomicAdd(&C[0], (unsigned long long)n);
+        if (hits) atomicAdd(&C[1], (unsigned long long)hits);
+        if (hit_tok) atomicAdd(&C[2], hit_tok);
+        atomicAdd(&C[3], prompt);
+        atomicAdd(&C[4], prompt - hit_tok);
+    }
+}
+
+// Which calls start with it (*rest != NULL then): streams of up to two requests on average, or,
+// for token capacities whose lists seldom pass 32 prefixes, of up to eight.  Once lists are
+// longer its launch is lost: ten replicas x 3,000 requests over 1,000 destinations, capacity
+// 128, lists full 19 -> 29 us; four x 60,000 over 8,192 54 -> 89.
+template <bool TOKENS>
+int launch_short(cr_ctx *ctx, const cr_replay *rp, const replay_caps &caps, uint32_t lim, const uint32_t *start,
+                 const uint32_t *map, uint32_t items_max, const uint32_t *total, uint64_t m, uint64_t items,
+                 const uint32_t *idx, const rec16 *recs, uint64_t *d_ctr, uint32_t **rest)
+{
+    *rest = nullptr;
+    if (m > (TOKENS && lim <= (1u << 16) ? 8u : 2u) * rp->n_streams) return CR_OK;
+    void *p;
+    CR_TRY(cr_scratch(ctx, SCR_REPLAY_REST, (items + 1) * sizeof(uint32_t), &p));
+    *rest = (uint32_t *)p;
+    CR_CUDA(ctx, cudaMemsetAsync(p, 0, sizeof(uint32_t), ctx->stream));
+    CR_LAUNCH(ctx, k_replay_short<TOKENS>, (unsigned int)((items + 7) / 8), 256, 0, caps, lim, rp->cmax, rp->R,
+              (uint32_t)rp->n_streams, start, map, items_max, total, idx, recs, (uint32_t)(m / rp->n_rep), state_of(rp),
+              (unsigned long long *)d_ctr, *rest, ctx->d_status);
+    return CR_OK;
+}
 
 // ---- replay: batched stack distances over access times -------------------------
 // One warp per (stream, chunk) holds the LRU stack in shared memory, indexed by
@@ -690,20 +832,20 @@ __device__ __forceinline__ void sl_compact(const window_lru &X, uint32_t live, u
     }
 }
 
+// One work item.
 template <int NC, int NG, bool SMALL>
-__global__ void __launch_bounds__(128, 5)
-k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t nb, uint32_t R,
-             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ map, uint32_t items_max,
-             const uint32_t *__restrict__ total, const uint32_t *__restrict__ idx, const rec16 *__restrict__ recs,
-             uint32_t nrec, const replay_state st, unsigned long long *__restrict__ ctr, uint32_t *status)
+__device__ __forceinline__ void lru_item(uint32_t w, const replay_caps &caps, uint32_t cmax, uint32_t nw, uint32_t nb,
+                                         uint32_t R, uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start,
+                                         const uint32_t *__restrict__ map, uint32_t items_max,
+                                         const uint32_t *__restrict__ idx, const rec16 *__restrict__ recs,
+                                         uint32_t nrec, const replay_state &st, unsigned long long *__restrict__ ctr,
+                                         uint32_t *status)
 {
     extern __shared__ uint4 smb[];
-    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5;
     const window_lru X =
         window_lru_at(reinterpret_cast<unsigned char *>(smb) + window_lru_bytes(nw, nb) * warp, nw, nb);
 
-    const uint32_t w = blockIdx.x * wpb + warp;
-    if (w >= *total) return;
     const uint32_t s = min(map[w], ns - 1u), ci = map[items_max + w];  // the item's stream and chunk
     const uint32_t b = start[s], e = start[s + 1];
     const uint32_t p0 = b + ci * CL;
@@ -924,6 +1066,24 @@ k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw
     }
 }
 
+// The items 0 .. *total - 1, or those that `list` names (k_replay_short's leftovers, whose
+// number the host does not know: the grid then is what the GPU holds at once).
+template <int NC, int NG, bool SMALL>
+__global__ void __launch_bounds__(128, 5)
+k_lru_stamp(const __grid_constant__ replay_caps caps, uint32_t cmax, uint32_t nw, uint32_t nb, uint32_t R,
+             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ map, uint32_t items_max,
+             const uint32_t *__restrict__ total, const uint32_t *__restrict__ list, const uint32_t *__restrict__ idx,
+             const rec16 *__restrict__ recs, uint32_t nrec, const replay_state st, unsigned long long *__restrict__ ctr,
+             uint32_t *status)
+{
+    const uint32_t wpb = blockDim.x >> 5, n = *total;
+    for (uint32_t w = blockIdx.x * wpb + (threadIdx.x >> 5); w < n; w += gridDim.x * wpb) {
+        lru_item<NC, NG, SMALL>(list ? list[w] : w, caps, cmax, nw, nb, R, ns, CL, start, map, items_max, idx, recs, nrec,
+                                st, ctr, status);
+        __syncwarp();
+    }
+}
+
 // Words of the window: the cmax keys that a compaction leaves plus twelve steps before the
 // next one.  More steps cost warps per SM, fewer cost compactions: at cmax 1024, 4 / 8 / 12 / 17 /
 // 20 / 32 steps measured 1.80 / 1.73 / 1.73 / 1.83 / 1.80 / 2.02 ms, at cmax 128 223 / 217 / 215 /
@@ -965,6 +1125,13 @@ uint32_t window_warps(size_t per_warp, uint32_t regs, uint32_t *per_sm)
     return wpb;
 }
 
+// Blocks of a replay launch: one warp per item, or for leftovers what the GPU holds at once.
+inline unsigned int item_grid(const cr_ctx *ctx, uint64_t items, uint32_t wpb, uint32_t per_sm, const uint32_t *rest)
+{
+    const uint64_t all = (items + wpb - 1) / wpb, held = (uint64_t)ctx->num_sms * (per_sm / wpb);
+    return (unsigned int)(rest && held < all ? held : all);
+}
+
 template <int NC, int NG, bool SMALL>
 int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t CL, const uint32_t *start,
                   const uint32_t *map, uint32_t items_max, const uint32_t *total, uint64_t m, const uint32_t *idx,
@@ -985,16 +1152,12 @@ int launch_stamp(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t C
                                           (int)smem));
     const uint32_t ns = rp->n_rep * rp->R;
     const uint64_t items = (uint64_t)ns + (m + CL - 1) / CL;  // upper bound on work items
-    replay_state st;
-    st.keys_in = rp->d_keys[rp->cur];
-    st.fill_in = rp->d_fill[rp->cur];
-    st.keys_out = rp->d_keys[rp->cur ^ 1];
-    st.fill_out = rp->d_fill[rp->cur ^ 1];
     const int pr = cr_prof_begin(ctx, ctx->stream, CR_PROF_REPLAY);
-    CR_LAUNCH(ctx, (k_lru_stamp<NC, NG, SMALL>), (unsigned int)((items + wpb - 1) / wpb), wpb * 32, smem, caps, cmax,
-              nw, nb, rp->R, ns, CL, start, map, items_max, total, idx, recs, (uint32_t)(m / rp->n_rep), st,
-              (unsigned long long *)d_ctr,
-              ctx->d_status);
+    uint32_t *rest;
+    CR_TRY(launch_short<false>(ctx, rp, caps, cmax, start, map, items_max, total, m, items, idx, recs, d_ctr, &rest));
+    CR_LAUNCH(ctx, (k_lru_stamp<NC, NG, SMALL>), item_grid(ctx, items, wpb, per_sm, rest), wpb * 32, smem, caps, cmax, nw,
+              nb, rp->R, ns, CL, start, map, items_max, rest ? rest : total, rest ? rest + 1 : nullptr, idx, recs,
+              (uint32_t)(m / rp->n_rep), state_of(rp), (unsigned long long *)d_ctr, ctx->d_status);
     cr_prof_end(ctx, ctx->stream, pr);
     rp->cur ^= 1;
     return CR_OK;
@@ -1047,12 +1210,6 @@ constexpr uint32_t kTokMax = CR_MAX_CAP;  // prefixes per list
 // Below this largest capacity a step's sums of prefixes cut to it cannot pass 2^32.
 constexpr uint32_t kTokNarrow = 1u << 26;
 
-__device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b)
-{
-    const uint32_t v = a + b;
-    return v < a ? 0xffffffffu : v;
-}
-
 // Inclusive sum over the lanes from this one up.
 __device__ __forceinline__ uint32_t warp_sat_suffix(uint32_t v, uint32_t lane)
 {
@@ -1063,15 +1220,6 @@ __device__ __forceinline__ uint32_t warp_sat_suffix(uint32_t v, uint32_t lane)
     }
     return v;
 }
-
-struct token_state {
-    const unsigned long long *keys_in;  // [stream][kTokMax], most recent first
-    const uint32_t *cum_in;             // [stream][kTokMax], tokens of entries 0..j
-    const uint32_t *fill_in;
-    unsigned long long *keys_out;
-    uint32_t *cum_out;
-    uint32_t *fill_out;
-};
 
 // Each word's live tokens from the bitmap and the times' tokens (words below `wend`;
 // cleared above).
@@ -1113,20 +1261,19 @@ __device__ __forceinline__ uint32_t tk_list(const window_lru &X, uint32_t wend, 
     return n;
 }
 
+// One work item.
 template <int NC>
-__global__ void __launch_bounds__(128, 4)
-k_lru_tokens(const __grid_constant__ replay_caps caps, uint32_t capmax, uint32_t nw, uint32_t nb, uint32_t R,
-             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ map,
-             uint32_t items_max, const uint32_t *__restrict__ total, const uint32_t *__restrict__ idx,
-             const rec16 *__restrict__ recs, uint32_t nrec, const token_state st,
-             unsigned long long *__restrict__ ctr, uint32_t *status)
+__device__ __forceinline__ void token_item(uint32_t w, const replay_caps &caps, uint32_t capmax, uint32_t nw, uint32_t nb,
+                                           uint32_t R, uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start,
+                                           const uint32_t *__restrict__ map, uint32_t items_max,
+                                           const uint32_t *__restrict__ idx, const rec16 *__restrict__ recs,
+                                           uint32_t nrec, const replay_state &st, unsigned long long *__restrict__ ctr,
+                                           uint32_t *status)
 {
     extern __shared__ uint4 smb[];
-    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const uint32_t lane = cr_lane(), warp = threadIdx.x >> 5;
     const window_lru X =
         window_lru_at(reinterpret_cast<unsigned char *>(smb) + window_lru_bytes(nw, nb, true) * warp, nw, nb);
-    const uint32_t w = blockIdx.x * wpb + warp;
-    if (w >= *total) return;  // whole warps only; the kernel has no block-wide barrier
     const uint32_t s = min(map[w], ns - 1u), ci = map[items_max + w];  // the item's stream and chunk
     const uint32_t b = start[s], e = start[s + 1];
     const uint32_t p0 = b + ci * CL;
@@ -1404,6 +1551,22 @@ k_lru_tokens(const __grid_constant__ replay_caps caps, uint32_t capmax, uint32_t
 }
 
 template <int NC>
+__global__ void __launch_bounds__(128, 4)
+k_lru_tokens(const __grid_constant__ replay_caps caps, uint32_t capmax, uint32_t nw, uint32_t nb, uint32_t R,
+             uint32_t ns, uint32_t CL, const uint32_t *__restrict__ start, const uint32_t *__restrict__ map,
+             uint32_t items_max, const uint32_t *__restrict__ total, const uint32_t *__restrict__ list,
+             const uint32_t *__restrict__ idx, const rec16 *__restrict__ recs, uint32_t nrec, const replay_state st,
+             unsigned long long *__restrict__ ctr, uint32_t *status)
+{
+    const uint32_t wpb = blockDim.x >> 5, n = *total;
+    for (uint32_t w = blockIdx.x * wpb + (threadIdx.x >> 5); w < n; w += gridDim.x * wpb) {
+        token_item<NC>(list ? list[w] : w, caps, capmax, nw, nb, R, ns, CL, start, map, items_max, idx, recs, nrec, st, ctr,
+                       status);
+        __syncwarp();
+    }
+}
+
+template <int NC>
 int launch_tokens(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t CL, const uint32_t *start,
                   const uint32_t *map, uint32_t items_max, const uint32_t *total, uint64_t m, const uint32_t *idx,
                   const rec16 *recs, uint64_t *d_ctr)
@@ -1423,18 +1586,13 @@ int launch_tokens(cr_ctx *ctx, cr_replay *rp, const replay_caps &caps, uint32_t 
     if (smem > kDefaultSmem)
         CR_CUDA(ctx, cudaFuncSetAttribute(k_lru_tokens<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const uint32_t ns = rp->n_rep * rp->R;
-    token_state st;
-    st.keys_in = rp->d_keys[rp->cur];
-    st.cum_in = rp->d_size[rp->cur];
-    st.fill_in = rp->d_fill[rp->cur];
-    st.keys_out = rp->d_keys[rp->cur ^ 1];
-    st.cum_out = rp->d_size[rp->cur ^ 1];
-    st.fill_out = rp->d_fill[rp->cur ^ 1];
     const uint64_t items = (uint64_t)ns + (m + CL - 1) / CL;  // upper bound on work items
     const int pt = cr_prof_begin(ctx, ctx->stream, CR_PROF_REPLAY);
-    CR_LAUNCH(ctx, (k_lru_tokens<NC>), (unsigned int)((items + wpb - 1) / wpb), wpb * 32, smem, caps, capmax, nw, nb,
-              rp->R, ns, CL, start, map, items_max, total, idx, recs, (uint32_t)(m / rp->n_rep), st,
-              (unsigned long long *)d_ctr, ctx->d_status);
+    uint32_t *rest;
+    CR_TRY(launch_short<true>(ctx, rp, caps, capmax, start, map, items_max, total, m, items, idx, recs, d_ctr, &rest));
+    CR_LAUNCH(ctx, (k_lru_tokens<NC>), item_grid(ctx, items, wpb, per_sm, rest), wpb * 32, smem, caps, capmax, nw, nb, rp->R,
+              ns, CL, start, map, items_max, rest ? rest : total, rest ? rest + 1 : nullptr, idx, recs,
+              (uint32_t)(m / rp->n_rep), state_of(rp), (unsigned long long *)d_ctr, ctx->d_status);
     cr_prof_end(ctx, ctx->stream, pt);
     rp->cur ^= 1;
     return CR_OK;

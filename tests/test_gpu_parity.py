@@ -1487,6 +1487,35 @@ def test_replay_items_of_many_chunks(P, ctx, R, n, hot):
 
 
 @pytest.mark.parametrize("tokens", [False, True])
+@pytest.mark.parametrize("R,n,hot,caps", [(900, 1800, 0.0, [64]), (900, 1801, 0.1, [2, 40, 1000]), (8192, 500, 0.0, [8]),
+                                          (300, 600, 0.3, [33]), (50, 100, 0.0, [32, 31]), (400, 3200, 0.0, [100]),
+                                          (400, 3201, 0.0, [5])])
+def test_replay_short_streams(P, ctx, tokens, R, n, hot, caps):
+    # streams of a few requests or none: lists that fit 32 entries with the call's requests, that
+    # outgrow them over the calls, empty streams with longer lists; averages at and past the
+    # lines of the kernel for them (two requests, eight for token capacities); a hot stream of
+    # several chunks beside
+    rng = np.random.default_rng(R + n)
+    if tokens:
+        caps = [c * 500 for c in caps]
+    orp, rp = O.Replay(2, R, caps, tokens=tokens), P.Replay(ctx, 2, R, caps, tokens=tokens)
+    ctr = torch.zeros((2, len(caps), R, 5), dtype=torch.int64, device=DEV)
+    for call in range(12):
+        dest = rng.integers(0, R, (2, n)).astype(np.uint16)
+        dest[:, rng.random(n) < hot] = 1
+        keys = rng.integers(1, 40 if call % 3 else 4000, n).astype(np.uint64)
+        plen = (keys * np.uint64(7919) % np.uint64(900)).astype(np.uint32)  # 0 for some, above the least capacity for others
+        slen = np.full(n, 64, np.uint32)
+        orp.step(keys, plen, slen, dest)
+        P.shadow_replay(ctx, rp, d_u64(keys), d_u32(plen), d_u32(slen), d_u16(dest), ctr)
+    ctx.sync()
+    assert (h_u64(ctr) == orp.ctr).all()
+    top = int(np.argmax(caps))
+    for r in list(range(0, R, max(1, R // 20))) + [1]:
+        assert (rp.state(1, r) == orp.state(1, top, r)).all()
+
+
+@pytest.mark.parametrize("tokens", [False, True])
 @pytest.mark.parametrize("R,hot", [(40, [7]), (700, [3, 200, 699]), (700, list(range(0, 700, 9))), (33, [])])
 def test_replay_items_of_long_streams(P, ctx, tokens, R, hot):
     # streams longer than twice the mean take the first work items: none, a few, and one in
