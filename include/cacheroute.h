@@ -112,10 +112,12 @@ CR_API int cr_set_stream(cr_ctx *ctx, void *cuda_stream);
 /* Routing split over two streams: with a non-NULL stream, cr_route_batch runs
  * the per-request candidates (and the load counts of RR / HASH replicas) on
  * the context's stream and the load-dependent resolution on `cuda_stream`,
- * ordered by an event; the resolution's end (on `cuda_stream`) then covers all
- * of the call's writes to d_dest and d_load, and the next call's candidates
- * wait for it.  Callers order later readers of d_dest / d_load after
- * `cuda_stream`.  NULL restores single-stream routing.  Setting the stream the
+ * ordered by an event (batches of at most 32 requests: the candidates of the
+ * load-dependent replicas too, from a copy of the keys); the resolution's end
+ * (on `cuda_stream`) then covers all of the call's writes to d_dest and d_load
+ * and its reads of the plans and rings, and the next call's candidates wait for
+ * it.  Callers order later readers of d_dest / d_load, and calls that rebuild or
+ * destroy a plan or ring of the call, after `cuda_stream`.  NULL restores single-stream routing.  Setting the stream the
  * context already has does nothing; switching waits for the old stream.
  * cr_sync also waits for the last resolution enqueued on `cuda_stream`, so an
  * error it raised is reported by the first blocking call after it.
@@ -191,8 +193,8 @@ CR_API int cr_profile_read(cr_ctx *ctx, uint32_t tag, uint64_t *launches, double
  *   n         number of requests (0 allowed: nothing is enqueued)
  *   salt      64-bit salt
  *   d_key_out uint64[n] receives b_r
- * Requests whose prefix starts on a 16-byte boundary (d_off[r] % 4 == 0) take
- * the vectorised path; any other offset is still exact, only slower.
+ * Spans may start anywhere in the arena and end anywhere; those of whole
+ * 16-byte vectors are read fastest.
  * Errors: CR_EINVAL (NULL pointer with n > 0). */
 CR_API int cr_hash_prefixes(cr_ctx *ctx, const int32_t *d_tokens, const uint64_t *d_off,
                      const uint32_t *d_plen, uint64_t n, uint64_t salt, uint64_t *d_key_out);
@@ -371,9 +373,10 @@ typedef struct {
  *     at the first ring point >= fmix64(b ^ seed) (wrapping to the first
  *     point), walk the ring and take the first owner whose load is < cap.
  *     The least-loaded destination is always below cap, so the walk ends.
- * Batches of at most 32 requests are resolved by one warp per replica that
- * takes 32 // batch_B whole batches per step; longer batches by one CTA per
- * replica.  Both give the sequential result defined above.
+ * Batches of at most 32 requests are resolved by one CTA per replica, a warp of
+ * which takes 32 // batch_B whole batches per step while the others prepare
+ * later steps; longer batches by one CTA per replica, a batch at a time.  Both
+ * give the sequential result defined above.
  * Errors: CR_EINVAL (R == 0 or > CR_MAX_R, n_rep > CR_MAX_REPLICAS, missing
  * or mismatched plan or ring, batch_B == 0, n >= 2^40).  A load sum that
  * has wrapped past 2^64 can leave no destination below cap: the request then

@@ -40,13 +40,13 @@ enum cr_scratch_slot {
     SCR_SORT_K1,       // radix-sort keys (pong)
     SCR_SORT_V0,       // radix-sort values (ping)
     SCR_SORT_V1,       // radix-sort values (pong)
-    SCR_SORT_HIST,     // per-tile digit counts / offsets
+    SCR_SORT_HIST,     // radix sort: counters and tile states
     SCR_SCAN,          // block partials of the device-wide scan
     SCR_PLAN_A,        // plan-build temporaries
     SCR_PLAN_B,
     SCR_PLAN_C,
     SCR_REPLAY_REST,   // replay items left to the window kernels, and their number
-    SCR_ROUTE_DESC,    // per-replica route descriptors
+    SCR_ROUTE_DESC,    // route candidates, or the keys of a split route call
     SCR_DIFF,          // plan-difference counters
     SCR_NUM
 };

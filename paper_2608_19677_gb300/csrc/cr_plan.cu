@@ -93,7 +93,6 @@ __global__ void k_hist_insert(const unsigned long long *__restrict__ keys, uint6
     }
 }
 
-// Occupied slots -> a dense list (order immaterial: it is sorted next).
 // Occupied slots appended to a dense list (order free: the list is sorted next).
 // A warp takes 8 x 32 consecutive slots and claims their places with one atomic:
 // one atomic per 32 slots on the single counter serialised the launch.
@@ -274,8 +273,6 @@ __device__ void cta_radix_pass(const K *kin, const uint32_t *vin, K *kout, uint3
     }
 }
 
-// Sorts the U distinct (key, count) pairs: key ascending into (ukey, ucnt), then
-// stably by (n - count) into `order` = admission order (count desc, key asc).
 // Stable LSD sort of U (key, count) pairs in one CTA: by key (8 passes), the
 // sorted pairs written to ukey/ucnt, then by n - count (ceil(cbits/8) passes)
 // giving order = positions in ukey/ucnt by (count desc, key asc).  The pairs
@@ -1730,10 +1727,6 @@ int bits_for(uint64_t v)  // smallest b with v < 2^b
     while (b < 64 && (v >> b) != 0) ++b;
     return b;
 }
-
-struct plan_caps {
-    uint64_t n, adm, mem, load;
-};
 
 static_assert(offsetof(cr_plan_info_dev, by_rate) == offsetof(cr_plan_info_dev, U) + 16, "U, S, by_rate: one copy");
 

@@ -136,8 +136,8 @@ __host__ __device__ inline size_t part_scatter_smem(uint32_t R)
 constexpr uint32_t kPartSparse = 192;
 
 // Bound: instructions (ranking about half).  51 M destinations, R = 1024: 345 -> 239 us;
-// ranks are kept in registers instead of shared memory (a pass less; 80 registers, three
-// blocks per SM: four with 64 spill and take 315 us), and the lane numbers take about 20
+// ranks are kept in registers instead of shared memory (a pass less; 80 registers and 32
+// bytes of spills, three blocks per SM: four with 64 registers spill more and take 315 us), and the lane numbers take about 20
 // instructions per 32 requests where a ballot per destination bit takes 50.
 template <bool BALLOTS>
 __global__ void __launch_bounds__(kPartBlock, 3) k_part_scatter(const uint16_t *__restrict__ dest, unsigned long long n,

@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(kRouteBlock, 1) k_route_resolve(const __grid_c
 // ms, plan replicas 0.68 ms, bounded loads 1.58 ms; all fifteen 1.42 ms, where one
 // warp that did all of it (every iteration re-reading loads and masks from shared
 // memory, bound computed by division inside the chain) took 3.7 ms.  256 requests,
-// one plan replica at R = 64: 64.8 -> 19.0 us a call (no staging of member lists, no
+// one plan replica at R = 64: 62 -> 15 us a call (no staging of member lists, no
 // candidate launch).  Bounded loads on R > 32 cost 1.87 ms (masked_step).
 constexpr int kPrepWarps = 8;
 // warps 4 and 8 stay idle: the resolver has its SM sub-partition's issue slots to itself
@@ -1249,7 +1249,7 @@ k_route_resolve_warp(const __grid_constant__ route_args args, const unsigned lon
             mi = v < mi ? v : mi;
         }
         // one 64-bit shared atomic (a compare-and-swap loop) per warp, not per thread: five
-        // requests at R = 520 17.3 -> 9.4 us, 256 at R = 64 17.4 -> 13.3
+        // requests at R = 520 17.3 -> 9.4 us
         if ((threadIdx.x & ~31u) < R) {
             tot = cr_warp_sum_u64(tot);
             mx = ~cr_warp_min_u64(~mx);
