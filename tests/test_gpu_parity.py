@@ -1143,10 +1143,12 @@ def test_plan_parity_slotcap(P, ctx, R, W, nkeys, total, skew):
 
 @pytest.mark.parametrize("n,R,W,n_rand", [(24576, 1024, 200, 1), (24577, 1024, 8, 1), (24577, 1024, 9, 1),
                                           (70000, 1024, 64, 1), (70000, 1024, 65, 1), (70000, 1024, 65, 3),
-                                          (130000, 1024, 200, 1), (130000, 16, 300, 5)])
+                                          (130000, 1024, 200, 1), (130000, 16, 300, 5), (4096, 1024, 200, 1),
+                                          (4097, 1024, 200, 1), (24577, 1024, 4, 1), (24577, 241, 17, 1)])
 def test_plan_parity_sort_and_admission_rules(P, ctx, n, R, W, n_rand):
-    # both sides of the rules on interval and slot budget: histogram sorted by one CTA or in
-    # device-wide passes, admission of all plans by one CTA each or plan by plan
+    # both sides of the rules on interval and slot budget: histogram sorted by one CTA (up to
+    # 4,096 requests or slots) or by the whole GPU, admission of all plans by one CTA each or
+    # plan by plan
     rng = np.random.default_rng(n + R + W)
     pool = rng.integers(1, 2**63, n, dtype=np.int64).astype(np.uint64)
     keys = pool[np.minimum((rng.random(n) ** 2 * n).astype(np.int64), n - 1)]
